@@ -35,6 +35,26 @@ constexpr int RC_THREADS = 256;
 
 template <class R> struct CX { R re, im; };
 
+// entry Z[m][n] in FP32 by G::PARTS neighbouring lanes, lane `part` evaluating its part; the
+// parts are added in the order of entry(), to the same result, in every lane (all lanes of
+// the warp take part)
+template <class G> __device__ __forceinline__ CX<float> entry_parts(const G &g, int m, int n, int part)
+{
+    if constexpr (G::PARTS == 1) {
+        return g.template entry<float>(m, n);
+    } else {
+        const CX<float> v = g.part(m, n, part);
+        CX<float> z{0, 0};
+        const int base = (threadIdx.x & 31) - part;
+#pragma unroll
+        for (int p = 0; p < G::PARTS; ++p) {
+            z.re += __shfl_sync(0xffffffffu, v.re, base + p);
+            z.im += __shfl_sync(0xffffffffu, v.im, base + p);
+        }
+        return g.scale(m, n, z);
+    }
+}
+
 __device__ __forceinline__ float sqrtR(float v) { return sqrtf(v); }
 __device__ __forceinline__ double sqrtR(double v) { return sqrt(v); }
 __device__ __forceinline__ float logR(float v) { return logf(v); }
@@ -117,37 +137,46 @@ __device__ void block_argmax(float v, int idx, float *sv, int *si, float &ov, in
     __syncthreads();
     if (lane == 0) { sv[w] = v; si[w] = idx; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float bv = sv[0];
-        int bi = si[0];
-        for (int q = 1; q < nw; ++q)
-            if (sv[q] > bv || (sv[q] == bv && si[q] < bi)) { bv = sv[q]; bi = si[q]; }
-        sv[0] = bv; si[0] = bi;
-    }
-    __syncthreads();
     ov = sv[0];
     oi = si[0];
+    for (int q = 1; q < nw; ++q)
+        if (sv[q] > ov || (sv[q] == ov && si[q] < oi)) { ov = sv[q]; oi = si[q]; }
 }
 
-// block-wide sum of a complex value (double accumulation across the block)
-__device__ double2 block_sum(double2 v, double2 *sbuf)
+// warp-wide sums (FP64 accumulation of FP32 products) over conj(a[i]) b[i], i < n
+__device__ __forceinline__ double2 warp_cdot(const float2 *a, const float2 *b, int n, int lane)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int s = 16; s >= 1; s >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, s);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, s);
-    }
-    __syncthreads();
-    if (lane == 0) sbuf[w] = v;
-    __syncthreads();
     double2 r = make_double2(0, 0);
-    for (int q = 0; q < nw; ++q) { r.x += sbuf[q].x; r.y += sbuf[q].y; }
-    __syncthreads();
+    for (int i = lane; i < n; i += 32) {
+        const float2 t = cconjmul(a[i], b[i]);
+        r.x += t.x;
+        r.y += t.y;
+    }
+    for (int s = 16; s >= 1; s >>= 1) {
+        r.x += __shfl_xor_sync(0xffffffffu, r.x, s);
+        r.y += __shfl_xor_sync(0xffffffffu, r.y, s);
+    }
+    return r;
+}
+__device__ __forceinline__ double warp_norm2(const float2 *a, int n, int lane)
+{
+    double r = 0.0;
+    for (int i = lane; i < n; i += 32) r += cabs2(a[i]);
+    for (int s = 16; s >= 1; s >>= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
     return r;
 }
 
 // Partially pivoted ACA: Z[rows, cols] ~ sum_l u_l v_l^T with u_l stored as the
 // row l of U^T (length m) and v_l as row l of V (length n).
+//
+// Bound by the entry evaluations (a few thousand FP32 instructions each, in dependent
+// chains): G::PARTS lanes share one entry (the RWG's four triangle pairs), so that the
+// short rows of a block (15 to 64 entries) fill the CTA's warps and a row takes a
+// quarter of the chain; the CTA has 64 threads for blocks of up to 32 x 32 (launcher).
+// The cross terms of |S_k|_F^2 take one warp per earlier row and no barrier between
+// them: FP64 adds run at 2 lanes per clock and SM here, and block-wide sums spent six
+// times as many of them.  7,680-unknown sphere (100,000 blocks of 15 x 15): see the
+// launcher in assemble().
 template <class G>
 __global__ void __launch_bounds__(ACA_THREADS)
 k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, float tol)
@@ -157,10 +186,12 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
     float2 *V = UT + (int64_t)J.kmax * J.m;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *used = smem_raw;           // [m]
-    __shared__ float sv[32];
-    __shared__ int si[32];
-    __shared__ double2 sb[32];
-    for (int i = threadIdx.x; i < J.m; i += blockDim.x) used[i] = 0;
+    __shared__ float sv[ACA_THREADS / 32];
+    __shared__ int si[ACA_THREADS / 32];
+    __shared__ double s_nu, s_nv, s_cross[ACA_KCAP];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    const int part = tid % G::PARTS, e0 = tid / G::PARTS, ne = blockDim.x / G::PARTS;
+    for (int i = tid; i < J.m; i += blockDim.x) used[i] = 0;
     __syncthreads();
     int k = 0, istar = 0;
     double s2 = 0.0;
@@ -169,11 +200,14 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
         ++guard;
         float2 *v = V + (int64_t)k * J.n;
         float2 *u = UT + (int64_t)k * J.m;
-        // residual row istar
+        // residual row istar (the lanes of a warp run the same rounds: the parts of an entry are shuffled)
         float best = -1.f;
         int bj = 0;
-        for (int j = threadIdx.x; j < J.n; j += blockDim.x) {
-            const CX<float> z = g.template entry<float>(g.perm[J.r0 + istar], g.perm[J.c0 + j]);
+        for (int j0 = 0; j0 < J.n; j0 += ne) {
+            const int j = j0 + e0;
+            if (j0 + (tid & ~31) / G::PARTS >= J.n) continue;   // the whole warp is past the row
+            const CX<float> z = entry_parts(g, g.perm[J.r0 + istar], g.perm[J.c0 + min(j, J.n - 1)], part);
+            if (part != 0 || j >= J.n) continue;
             float2 r = make_float2(z.re, z.im);
             for (int l = 0; l < k; ++l) {
                 const float2 p = cmulf(UT[(int64_t)l * J.m + istar], V[(int64_t)l * J.n + j]);
@@ -185,7 +219,7 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
             if (a > best) { best = a; bj = j; }
         }
         __syncthreads();
-        if (threadIdx.x == 0) used[istar] = 1;
+        if (tid == 0) used[istar] = 1;
         float pv;
         int jstar;
         block_argmax(best, bj, sv, si, pv, jstar);
@@ -202,10 +236,13 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
         __syncthreads();
         const float pn = cabs2(piv);
         const float2 ipiv = make_float2(piv.x / pn, -piv.y / pn);
-        for (int j = threadIdx.x; j < J.n; j += blockDim.x) v[j] = cmulf(v[j], ipiv);
+        for (int j = tid; j < J.n; j += blockDim.x) v[j] = cmulf(v[j], ipiv);
         // residual column jstar
-        for (int i = threadIdx.x; i < J.m; i += blockDim.x) {
-            const CX<float> z = g.template entry<float>(g.perm[J.r0 + i], g.perm[J.c0 + jstar]);
+        for (int i0 = 0; i0 < J.m; i0 += ne) {
+            const int i = i0 + e0;
+            if (i0 + (tid & ~31) / G::PARTS >= J.m) continue;
+            const CX<float> z = entry_parts(g, g.perm[J.r0 + min(i, J.m - 1)], g.perm[J.c0 + jstar], part);
+            if (part != 0 || i >= J.m) continue;
             float2 c = make_float2(z.re, z.im);
             for (int l = 0; l < k; ++l) {
                 const float2 p = cmulf(V[(int64_t)l * J.n + jstar], UT[(int64_t)l * J.m + i]);
@@ -215,33 +252,28 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
             u[i] = c;
         }
         __syncthreads();
-        // norms and the cross terms of |S_k|_F^2
-        double2 a = make_double2(0, 0);
-        for (int i = threadIdx.x; i < J.m; i += blockDim.x) a.x += cabs2(u[i]);
-        for (int j = threadIdx.x; j < J.n; j += blockDim.x) a.y += cabs2(v[j]);
-        const double2 nuv = block_sum(a, sb);
-        double cross = 0.0;
-        for (int l = 0; l < k; ++l) {
-            double2 pu = make_double2(0, 0), pv2 = make_double2(0, 0);
-            for (int i = threadIdx.x; i < J.m; i += blockDim.x) {
-                const float2 t = cconjmul(UT[(int64_t)l * J.m + i], u[i]);
-                pu.x += t.x; pu.y += t.y;
+        // norms and the cross terms of |S_k|_F^2: l = k is the new pair itself
+        for (int l = k - w; l >= 0; l -= nw) {
+            if (l == k) {
+                const double nu = warp_norm2(u, J.m, lane), nv = warp_norm2(v, J.n, lane);
+                if (lane == 0) { s_nu = nu; s_nv = nv; }
+            } else {
+                const double2 su = warp_cdot(UT + (int64_t)l * J.m, u, J.m, lane);
+                const double2 svv = warp_cdot(V + (int64_t)l * J.n, v, J.n, lane);
+                if (lane == 0) s_cross[l] = su.x * svv.x - su.y * svv.y;   // Re(su * svv)
             }
-            const double2 su = block_sum(pu, sb);
-            for (int j = threadIdx.x; j < J.n; j += blockDim.x) {
-                const float2 t = cconjmul(V[(int64_t)l * J.n + j], v[j]);
-                pv2.x += t.x; pv2.y += t.y;
-            }
-            const double2 svv = block_sum(pv2, sb);
-            cross += su.x * svv.x - su.y * svv.y;   // Re(su * svv)
         }
-        s2 += 2.0 * cross + nuv.x * nuv.y;
+        __syncthreads();
+        double cross = 0.0;
+        for (int l = 0; l < k; ++l) cross += s_cross[l];
+        const double nuv = s_nu * s_nv;
+        s2 += 2.0 * cross + nuv;
         ++k;
-        if (sqrt(nuv.x * nuv.y) <= (double)tol * sqrt(fmax(s2, 0.0))) break;
+        if (sqrt(nuv) <= (double)tol * sqrt(fmax(s2, 0.0))) break;
         // next pivot row: largest |u_i| over unused rows
         float bu = -1.f;
         int bi = -1;
-        for (int i = threadIdx.x; i < J.m; i += blockDim.x)
+        for (int i = tid; i < J.m; i += blockDim.x)
             if (!used[i]) {
                 const float a2 = cabs2(u[i]);
                 if (a2 > bu) { bu = a2; bi = i; }
@@ -253,42 +285,52 @@ k_aca(G g, const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, flo
         istar = oi;
         __syncthreads();
     }
-    if (threadIdx.x == 0) ranks[blockIdx.x] = k;
+    if (tid == 0) ranks[blockIdx.x] = k;
 }
 
 // ------------------------------------------------------------ re-compression ----
-// One CTA per block.  Orthonormalise the rows of U^T (k x m) and of V (k x n) in
-// place by Gram-Schmidt applied twice (R factors in shared memory, FP64), form
-// the core C = R_U R_V^T, orthogonalise its columns by one-sided Jacobi
-// rotations (C W = [sigma_i w_i]), keep the smallest rank r whose discarded
-// singular values have Frobenius norm <= tol * total, and overwrite the rows:
+// One group of NT threads (a warp, or a CTA of 256 threads for high ranks and long
+// blocks) per block.  Orthonormalise the rows of U^T (k x m) and of V (k x n) in place
+// by Gram-Schmidt applied twice (R factors in shared memory, FP64), form the core
+// C = R_U R_V^T, orthogonalise its columns by one-sided Jacobi rotations
+// (C W = [sigma_i w_i]), keep the smallest rank r whose discarded singular values have
+// Frobenius norm <= tol * total, and overwrite the rows:
 //   U'^T[l] = sum_t (C W)[t][p_l] q_t      V'[l] = sum_t conj(W[t][p_l]) q'_t
 // (p = singular values sorted descending), so that U'^T^T V' = Q_U C Q_V^T.
-__device__ void gram_schmidt_rows(float2 *Q, int k, int len, double2 *Rm /* k x k, Rm[t*k + l] */,
-                                  double2 *coef, double2 *sb)
+//
+// Bound by latency (barriers, FP64 at 2 lanes per clock and SM), so the work is cut to
+// need few barriers: the dots of one Gram-Schmidt row run side by side (one warp each),
+// and a Jacobi sweep takes its pairs in round-robin steps of k / 2 disjoint pairs
+// (Brent & Luk 1985), a group of JG lanes each, instead of k (k - 1) / 2 rotations one
+// after another.  A rank of up to 16 takes one warp per block (no CTA barrier at all).
+// All blocks of the 7,680-unknown sphere: 59 ms; the pairs one by one, a CTA of 256 threads
+// per block and a block-wide sum per dot took 636 ms.
+template <int NT> __device__ __forceinline__ void group_sync()
 {
-    for (int l = 0; l < k; ++l)
-        for (int t = threadIdx.x; t < k; t += blockDim.x) Rm[t * k + l] = make_double2(0, 0);
-    __syncthreads();
+    if (NT == 32) __syncwarp();
+    else __syncthreads();
+}
+
+template <int NT>
+__device__ void gram_schmidt_rows(float2 *Q, int k, int len, double2 *Rm /* k x k, Rm[t*k + l] */, double2 *coef,
+                                  int tid)
+{
+    const int lane = tid & 31, w = tid >> 5;
+    for (int t = tid; t < k * k; t += NT) Rm[t] = make_double2(0, 0);
+    group_sync<NT>();
     for (int l = 0; l < k; ++l) {
         float2 *ql = Q + (int64_t)l * len;
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int t = 0; t < l; ++t) {
-                const float2 *qt = Q + (int64_t)t * len;
-                double2 a = make_double2(0, 0);
-                for (int i = threadIdx.x; i < len; i += blockDim.x) {
-                    const float2 c = cconjmul(qt[i], ql[i]);
-                    a.x += c.x; a.y += c.y;
-                }
-                const double2 s = block_sum(a, sb);
-                if (threadIdx.x == 0) {
+        for (int pass = 0; pass < 2 && l > 0; ++pass) {
+            for (int t = w; t < l; t += NT / 32) {
+                const double2 s = warp_cdot(Q + (int64_t)t * len, ql, len, lane);
+                if (lane == 0) {
                     coef[t] = s;
                     Rm[t * k + l].x += s.x;
                     Rm[t * k + l].y += s.y;
                 }
             }
-            __syncthreads();
-            for (int i = threadIdx.x; i < len; i += blockDim.x) {
+            group_sync<NT>();
+            for (int i = tid; i < len; i += NT) {
                 float2 v = ql[i];
                 for (int t = 0; t < l; ++t) {
                     const float2 q = Q[(int64_t)t * len + i];
@@ -298,122 +340,134 @@ __device__ void gram_schmidt_rows(float2 *Q, int k, int len, double2 *Rm /* k x 
                 }
                 ql[i] = v;
             }
-            __syncthreads();
+            group_sync<NT>();
         }
-        double2 a = make_double2(0, 0);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) a.x += cabs2(ql[i]);
-        const double nrm = sqrt(block_sum(a, sb).x);
-        if (threadIdx.x == 0) Rm[l * k + l] = make_double2(nrm, 0.0);
+        // every warp forms the norm (the same sum)
+        const double nrm = sqrt(warp_norm2(ql, len, lane));
+        if (tid == 0) Rm[l * k + l] = make_double2(nrm, 0.0);
         const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.f;
-        for (int i = threadIdx.x; i < len; i += blockDim.x) {
+        group_sync<NT>();                     // every warp has read the row
+        for (int i = tid; i < len; i += NT) {
             ql[i].x *= inv;
             ql[i].y *= inv;
         }
-        __syncthreads();
+        group_sync<NT>();
     }
 }
 
 __device__ __forceinline__ double2 zmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 __device__ __forceinline__ double2 zcmul(double2 a, double2 b) { return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }  // conj(a) b
 
-__global__ void __launch_bounds__(RC_THREADS)
-k_recompress(const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, float tol)
+constexpr int RC_BIG_LEN = 256;   // blocks with a longer side take a CTA (a warp would walk it alone)
+
+// shared bytes of one block of rank up to kc
+__host__ __device__ constexpr size_t rc_smem(int kc)
 {
-    const AcaJob J = jobs[blockIdx.x];
-    const int k = ranks[blockIdx.x];
+    return 4 * (size_t)kc * kc * sizeof(double2) + (((size_t)kc * (sizeof(double2) + sizeof(double) + sizeof(int)) + 3 * sizeof(int) + 15) & ~(size_t)15);
+}
+
+// WPC blocks per CTA, NT threads each; kc = the largest rank of the launch
+template <int NT, int WPC, int JG>
+__global__ void __launch_bounds__(NT * WPC)
+k_recompress(const AcaJob *__restrict__ jobs, int njobs, float2 *scratch, int32_t *ranks, float tol, int kc)
+{
+    const int sub = threadIdx.x / NT, tid = threadIdx.x % NT;
+    const int job = blockIdx.x * WPC + sub;
+    if (job >= njobs) return;                 // whole warps (NT = 32) or the CTA
+    const AcaJob J = jobs[job];
+    const int k = ranks[job];
     if (k <= 1) return;
     float2 *UT = scratch + J.off;
     float2 *V = UT + (int64_t)J.kmax * J.m;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2 *Ru = reinterpret_cast<double2 *>(smem_raw);   // k x k
+    double2 *Ru = reinterpret_cast<double2 *>(smem_raw + sub * rc_smem(kc));   // k x k
     double2 *Rv = Ru + k * k;                              // k x k
     double2 *C = Rv + k * k;                               // k x k, column-major C[col*k + row]
     double2 *W = C + k * k;                                // k x k, column-major
     double2 *coef = W + k * k;                             // k
     double *sig = reinterpret_cast<double *>(coef + k);    // k
     int *order = reinterpret_cast<int *>(sig + k);         // k
-    __shared__ double2 sb[32];
-    __shared__ int s_r;
-    __shared__ int s_rot;
-    gram_schmidt_rows(UT, k, J.m, Ru, coef, sb);
-    gram_schmidt_rows(V, k, J.n, Rv, coef, sb);
+    int *flags = order + k;                                // rotated in this sweep (two, alternating); kept rank
+    gram_schmidt_rows<NT>(UT, k, J.m, Ru, coef, tid);
+    gram_schmidt_rows<NT>(V, k, J.n, Rv, coef, tid);
     // C = Ru Rv^T (both upper triangular, Rm[t*k + l] = R[t][l])
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
+    for (int e = tid; e < k * k; e += NT) {
         const int row = e % k, col = e / k;
         double2 s = make_double2(0, 0);
-        for (int t = 0; t < k; ++t) {
+        for (int t = max(row, col); t < k; ++t) {
             const double2 p = zmul(Ru[row * k + t], Rv[col * k + t]);
             s.x += p.x; s.y += p.y;
         }
         C[col * k + row] = s;
         W[col * k + row] = make_double2(row == col ? 1.0 : 0.0, 0.0);
     }
-    __syncthreads();
-    // one-sided Jacobi on the columns of C (cyclic sweeps over pairs p < q);
-    // warp 0 forms the 2x2 Gram entries, the whole CTA applies the rotation
+    if (tid < 2) flags[tid] = 0;
+    group_sync<NT>();
+    // one-sided Jacobi on the columns of C: step s of a sweep pairs (k2 - 1, s) and
+    // (s + i, s - i) mod (k2 - 1), i = 1 .. k2/2 - 1, k2 = k rounded up to even (a pair with
+    // the column k that is not there is skipped); JG lanes form a pair's 2x2 Gram entries
+    // and rotate its rows
+    const int k2 = (k + 1) & ~1, jl = tid % JG;
     for (int sweep = 0; sweep < 20; ++sweep) {
-        if (threadIdx.x == 0) s_rot = 0;
-        __syncthreads();
-        for (int p = 0; p < k - 1; ++p)
-            for (int q = p + 1; q < k; ++q) {
-                if (threadIdx.x < 32) {
-                    double al = 0, be = 0, gr = 0, gi = 0;
-                    for (int t = threadIdx.x; t < k; t += 32) {
+        if (tid == 0) flags[(sweep + 1) & 1] = 0;
+        for (int s = 0; s < k2 - 1; ++s) {
+            for (int i0 = 0; i0 < k2 / 2; i0 += NT / JG) {
+                const int i = i0 + tid / JG;
+                int p = k2 - 1, q = s;
+                if (i > 0) { p = (s + i) % (k2 - 1); q = (s + k2 - 1 - i) % (k2 - 1); }
+                if (p > q) { const int t = p; p = q; q = t; }
+                const bool on = i < k2 / 2 && q < k;
+                double al = 0, be = 0, gr = 0, gi = 0;
+                if (on)
+                    for (int t = jl; t < k; t += JG) {
                         const double2 cp = C[p * k + t], cq = C[q * k + t];
                         al += cp.x * cp.x + cp.y * cp.y;
                         be += cq.x * cq.x + cq.y * cq.y;
                         gr += cp.x * cq.x + cp.y * cq.y;
                         gi += cp.x * cq.y - cp.y * cq.x;
                     }
-                    for (int o = 16; o >= 1; o >>= 1) {
-                        al += __shfl_xor_sync(0xffffffffu, al, o);
-                        be += __shfl_xor_sync(0xffffffffu, be, o);
-                        gr += __shfl_xor_sync(0xffffffffu, gr, o);
-                        gi += __shfl_xor_sync(0xffffffffu, gi, o);
-                    }
-                    if (threadIdx.x == 0) {
-                        const double gabs = sqrt(gr * gr + gi * gi);
-                        double c = 1.0, sr = 0.0, si = 0.0;
-                        if (gabs > 1e-12 * sqrt(al * be) && gabs > 0.0) {
-                            const double zeta = (be - al) / (2.0 * gabs);
-                            const double tt = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                            c = 1.0 / sqrt(1.0 + tt * tt);
-                            const double sv_ = c * tt;
-                            sr = sv_ * gr / gabs;   // s = |s| gamma / |gamma|
-                            si = sv_ * gi / gabs;
-                            s_rot = 1;
-                        }
-                        coef[0] = make_double2(c, 0.0);
-                        coef[1] = make_double2(sr, si);
-                    }
+#pragma unroll
+                for (int o = JG / 2; o >= 1; o >>= 1) {
+                    al += __shfl_xor_sync(0xffffffffu, al, o);
+                    be += __shfl_xor_sync(0xffffffffu, be, o);
+                    gr += __shfl_xor_sync(0xffffffffu, gr, o);
+                    gi += __shfl_xor_sync(0xffffffffu, gi, o);
                 }
-                __syncthreads();
-                const double c = coef[0].x;
-                const double2 sv2 = coef[1];
-                if (c != 1.0)
-                    for (int t = threadIdx.x; t < 2 * k; t += blockDim.x) {
+                const double g2 = gr * gr + gi * gi;
+                if (on && g2 > 1e-24 * (al * be) && g2 > 0.0) {
+                    const double gabs = sqrt(g2);
+                    const double zeta = (be - al) / (2.0 * gabs);
+                    const double tt = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+                    const double c = 1.0 / sqrt(1.0 + tt * tt);
+                    const double sg = c * tt / gabs;
+                    const double2 sv = make_double2(sg * gr, sg * gi);   // s = |s| gamma / |gamma|
+                    for (int t = jl; t < 2 * k; t += JG) {
                         double2 *M = t < k ? C : W;
                         const int r = t < k ? t : t - k;
                         const double2 a = M[p * k + r], b = M[q * k + r];
                         // [a b] <- [a b] [[c, s], [-conj(s), c]]
-                        const double2 csb = zcmul(sv2, b);   // conj(s) b
-                        const double2 sa = zmul(sv2, a);
+                        const double2 csb = zcmul(sv, b);   // conj(s) b
+                        const double2 sa = zmul(sv, a);
                         M[p * k + r] = make_double2(c * a.x - csb.x, c * a.y - csb.y);
                         M[q * k + r] = make_double2(sa.x + c * b.x, sa.y + c * b.y);
                     }
-                __syncthreads();
+                    if (jl == 0) flags[sweep & 1] = 1;
+                }
             }
-        if (!s_rot) break;
-        __syncthreads();
+            group_sync<NT>();
+        }
+        const int rot = flags[sweep & 1];
+        group_sync<NT>();
+        if (!rot) break;
     }
     // singular values and truncation
-    for (int l = threadIdx.x; l < k; l += blockDim.x) {
+    for (int l = tid; l < k; l += NT) {
         double a = 0;
         for (int t = 0; t < k; ++t) a += C[l * k + t].x * C[l * k + t].x + C[l * k + t].y * C[l * k + t].y;
         sig[l] = sqrt(a);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    group_sync<NT>();
+    if (tid == 0) {
         for (int l = 0; l < k; ++l) order[l] = l;
         for (int a = 1; a < k; ++a) {   // insertion sort, descending
             const int key = order[a];
@@ -430,15 +484,15 @@ k_recompress(const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, f
             tail -= sig[order[l]] * sig[order[l]];
         }
         if (r < 1) r = 1;
-        s_r = r;
+        flags[2] = r;
     }
-    __syncthreads();
-    const int r = s_r;
+    group_sync<NT>();
+    const int r = flags[2];
     // rows of U'^T and V' : each thread owns one position and transforms its k-vector
     for (int side = 0; side < 2; ++side) {
         float2 *Q = side == 0 ? UT : V;
         const int len = side == 0 ? J.m : J.n;
-        for (int i = threadIdx.x; i < len; i += blockDim.x) {
+        for (int i = tid; i < len; i += NT) {
             float2 qv[ACA_KCAP];
             for (int t = 0; t < k; ++t) qv[t] = Q[(int64_t)t * len + i];
             for (int l = 0; l < r; ++l) {
@@ -454,8 +508,27 @@ k_recompress(const AcaJob *__restrict__ jobs, float2 *scratch, int32_t *ranks, f
             }
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) ranks[blockIdx.x] = r;
+    if (tid == 0) ranks[job] = r;
+}
+
+// re-compression of the blocks jb (ranks rb, on the device), all of rank at most kc
+inline hm_status launch_recompress(const AcaJob *jb, int n, float2 *scr, int32_t *rb, float tol, int kc, bool big,
+                                   cudaStream_t s)
+{
+    constexpr int WPC = 4;
+    auto go = [&](auto kern, int wpc, int threads) -> hm_status {
+        const size_t sm = wpc * rc_smem(kc);
+        HM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        kern<<<(unsigned)((n + wpc - 1) / wpc), threads, sm, s>>>(jb, n, scr, rb, tol, kc);
+        return HM_OK;
+    };
+    hm_status st;
+    if (kc <= 8 && !big) st = go(k_recompress<32, WPC, 8>, WPC, 32 * WPC);
+    else if (kc <= 16 && !big) st = go(k_recompress<32, WPC, 4>, WPC, 32 * WPC);
+    else st = go(k_recompress<RC_THREADS, 1, 8>, 1, RC_THREADS);
+    if (st != HM_OK) return st;
+    HM_CUDA(cudaGetLastError());
+    return HM_OK;
 }
 
 // copy rank-r factors from the ACA scratch into the padded pool
@@ -650,6 +723,17 @@ struct TmpBuffers {
     }
 };
 
+// each double as the pair (hi, lo) of floats, hi the nearest float, lo the nearest to the rest
+inline std::vector<float2> float_pairs(const std::vector<double> &v)
+{
+    std::vector<float2> r(v.size());
+    for (size_t i = 0; i < v.size(); ++i) {
+        r[i].x = (float)v[i];
+        r[i].y = (float)(v[i] - (double)r[i].x);
+    }
+    return r;
+}
+
 // Host description of the unknowns of one basis: the point each unknown is
 // sorted by in the tree and its support box, plus what the operator keeps for
 // plane-wave excitation (b_m = sum over the two sides of ucoef * sum_q w_q
@@ -724,29 +808,43 @@ hm_status assemble(BasisData &B, G g, const hm_build_opts *o, TmpBuffers &tmp, c
         if ((st = tmp.up(&d_aj, aj, s)) != HM_OK) return st;
         int64_t maxm = 0;
         for (auto &j : aj) maxm = std::max<int64_t>(maxm, j.m);
-        k_aca<G><<<(unsigned)fars.size(), ACA_THREADS, maxm, s>>>(g, d_aj, d_scr, d_ranks, (float)o->aca_tol);
+        // two warps a block up to 32 x 32 (its rows are 15 to 32 entries of PARTS lanes), four above
+        const int at = maxm <= 32 ? 64 : ACA_THREADS;
+        k_aca<G><<<(unsigned)fars.size(), at, maxm, s>>>(g, d_aj, d_scr, d_ranks, (float)o->aca_tol);
         HM_CUDA(cudaGetLastError());
         HM_CUDA(cudaMemcpyAsync(ranks.data(), d_ranks, sizeof(int32_t) * fars.size(), cudaMemcpyDeviceToHost, s));
         HM_CUDA(cudaStreamSynchronize(s));
-        // re-compression, launched per rank bucket so that shared memory fits the bucket
+        // re-compression, launched per rank bucket so that shared memory fits the bucket, blocks
+        // of a long side apart; one read-back of the new ranks at the end
         const int bounds[] = {8, 16, 32, ACA_KCAP};
+        std::vector<AcaJob> jb;
+        std::vector<int32_t> rb;
+        std::vector<size_t> where;
+        struct Launch { size_t first, n; int kc; bool big; };
+        std::vector<Launch> ls;
         int lo = 1;
         for (int bk : bounds) {
-            std::vector<AcaJob> jb;
-            std::vector<int32_t> rb;
-            std::vector<size_t> where;
-            for (size_t b = 0; b < fars.size(); ++b)
-                if (ranks[b] > lo && ranks[b] <= bk) { jb.push_back(aj[b]); rb.push_back(ranks[b]); where.push_back(b); }
+            for (bool big : {false, true}) {
+                const size_t first = where.size();
+                for (size_t b = 0; b < fars.size(); ++b)
+                    if (ranks[b] > lo && ranks[b] <= bk && (std::max(aj[b].m, aj[b].n) > RC_BIG_LEN) == big) {
+                        jb.push_back(aj[b]);
+                        rb.push_back(ranks[b]);
+                        where.push_back(b);
+                    }
+                if (where.size() > first) ls.push_back({first, where.size() - first, bk, big});
+            }
             lo = bk;
-            if (jb.empty()) continue;
+        }
+        if (!where.empty()) {
             AcaJob *d_jb = nullptr;
             int32_t *d_rb = nullptr;
             if ((st = tmp.up(&d_jb, jb, s)) != HM_OK) return st;
             if ((st = tmp.up(&d_rb, rb, s)) != HM_OK) return st;
-            const size_t rsm = 4 * (size_t)bk * bk * sizeof(double2) + bk * (sizeof(double2) + sizeof(double) + sizeof(int)) + 64;
-            HM_CUDA(cudaFuncSetAttribute(k_recompress, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-            k_recompress<<<(unsigned)jb.size(), RC_THREADS, rsm, s>>>(d_jb, d_scr, d_rb, (float)o->aca_tol);
-            HM_CUDA(cudaGetLastError());
+            for (const Launch &l : ls)
+                if ((st = launch_recompress(d_jb + l.first, (int)l.n, d_scr, d_rb + l.first, (float)o->aca_tol, l.kc,
+                                            l.big, s)) != HM_OK)
+                    return st;
             HM_CUDA(cudaMemcpyAsync(rb.data(), d_rb, sizeof(int32_t) * rb.size(), cudaMemcpyDeviceToHost, s));
             HM_CUDA(cudaStreamSynchronize(s));
             for (size_t q = 0; q < where.size(); ++q) ranks[where[q]] = rb[q];

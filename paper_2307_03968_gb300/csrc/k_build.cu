@@ -35,10 +35,42 @@ struct Geo {
     const double *elen;   // ne
     const int32_t *perm;  // tree position -> original edge index
     double k, eta;
+    // the same points as pairs of floats (hi, lo), hi + lo within 2^-49 of the double, for the
+    // FP32 entries: their local coordinates p - o are then formed without the FP64 pipe, which
+    // runs at 1/64 of the FP32 rate here and which 96 subtractions and conversions per triangle
+    // pair made the bound of the fill and of the ACA
+    const float2 *vtx32;  // nv x 3
+    const float2 *qpd32;  // nt x NQ x 3
+    float kf, ik2f;       // k and 1/k^2, rounded
+    static constexpr int PARTS = 4;
     template <class R> __device__ CX<R> entry(int m, int n) const;
+    __device__ CX<float> part(int m, int n, int p) const;              // the signed triangle pair p of an entry
+    __device__ CX<float> scale(int m, int n, const CX<float> &z) const;
 };
 
 __constant__ double c_qw[NQ];
+__constant__ float c_qwf[NQ];
+
+template <class R> __device__ __forceinline__ R qweight(int q);
+template <> __device__ __forceinline__ double qweight<double>(int q) { return c_qw[q]; }
+template <> __device__ __forceinline__ float qweight<float>(int q) { return c_qwf[q]; }
+
+// (p - o) for vertex or quadrature points (index i of p64 / p32, vertex o): FP64 subtraction
+// for the FP64 entries; for FP32 the difference of the two (hi, lo) pairs, the leading parts
+// subtracted error-free (TwoDiff) and rounded once
+__device__ __forceinline__ void rel_point(const Geo &g, const double *p64, const float2 *, int i, int o, double (&out)[3])
+{
+    for (int d = 0; d < 3; ++d) out[d] = p64[3 * (int64_t)i + d] - g.vtx[3 * (int64_t)o + d];
+}
+__device__ __forceinline__ void rel_point(const Geo &g, const double *, const float2 *p32, int i, int o, float (&out)[3])
+{
+    for (int d = 0; d < 3; ++d) {
+        const float2 a = p32[3 * (int64_t)i + d], b = g.vtx32[3 * (int64_t)o + d];
+        const float s = __fsub_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
+        const float e = __fsub_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fadd_rn(b.x, bb));
+        out[d] = __fadd_rn(s, __fadd_rn(e, __fsub_rn(a.y, b.y)));
+    }
+}
 
 // The singular-extraction predicate, evaluated in FP64 without contractions so
 // that it takes the same decision as any other IEEE FP64 evaluation of
@@ -61,8 +93,7 @@ __device__ void potential(const Geo &g, int tn, const R r[3], R &s0, R s1[3])
 {
     const int32_t *tv = g.tri + 3 * tn;
     R P[3][3];
-    for (int a = 0; a < 3; ++a)
-        for (int d = 0; d < 3; ++d) P[a][d] = (R)(g.vtx[3 * tv[a] + d] - g.vtx[3 * tv[0] + d]);
+    for (int a = 0; a < 3; ++a) rel_point(g, g.vtx, g.vtx32, tv[a], tv[0], P[a]);
     R n[3];
     for (int d = 0; d < 3; ++d) n[d] = (R)g.nrm[3 * tn + d];
     const R dd = n[0] * r[0] + n[1] * r[1] + n[2] * r[2];
@@ -102,19 +133,20 @@ __device__ void potential(const Geo &g, int tn, const R r[3], R &s0, R s1[3])
 template <class R>
 __device__ CX<R> pair_integral(const Geo &g, int tm, int vmi, int tn, int vni)
 {
-    const R k = (R)g.k, ik2 = (R)(1.0 / (g.k * g.k));
+    R k, ik2;
+    if constexpr (sizeof(R) == 4) { k = g.kf; ik2 = g.ik2f; }
+    else { k = g.k; ik2 = 1.0 / (g.k * g.k); }
     const R inv4pi = (R)(0.25 / 3.14159265358979323846);
     const bool extract = extract_pair(g, tm, tn);
-    const double *o = g.vtx + 3 * g.tri[3 * tn];
-    const R vm[3] = {(R)(g.vtx[3 * vmi] - o[0]), (R)(g.vtx[3 * vmi + 1] - o[1]), (R)(g.vtx[3 * vmi + 2] - o[2])};
-    const R vn[3] = {(R)(g.vtx[3 * vni] - o[0]), (R)(g.vtx[3 * vni + 1] - o[1]), (R)(g.vtx[3 * vni + 2] - o[2])};
-    R qn[NQ][3];
-    for (int j = 0; j < NQ; ++j)
-        for (int d = 0; d < 3; ++d) qn[j][d] = (R)(g.qpd[(tn * NQ + j) * 3 + d] - o[d]);
+    const int o = g.tri[3 * tn];
+    R vm[3], vn[3], qn[NQ][3];
+    rel_point(g, g.vtx, g.vtx32, vmi, o, vm);
+    rel_point(g, g.vtx, g.vtx32, vni, o, vn);
+    for (int j = 0; j < NQ; ++j) rel_point(g, g.qpd, g.qpd32, tn * NQ + j, o, qn[j]);
     CX<R> acc{0, 0};
     for (int i = 0; i < NQ; ++i) {
         R ri[3];
-        for (int d = 0; d < 3; ++d) ri[d] = (R)(g.qpd[(tm * NQ + i) * 3 + d] - o[d]);
+        rel_point(g, g.qpd, g.qpd32, tm * NQ + i, o, ri);
         const R a[3] = {ri[0] - vm[0], ri[1] - vm[1], ri[2] - vm[2]};
         CX<R> inner{0, 0};
         for (int j = 0; j < NQ; ++j) {
@@ -136,7 +168,7 @@ __device__ CX<R> pair_integral(const Geo &g, int tm, int vmi, int tn, int vni)
                 gre = c * inv4pi / Rr;
                 gim = -s * inv4pi / Rr;
             }
-            const R w = (R)c_qw[j] * fac;
+            const R w = qweight<R>(j) * fac;
             inner.re += w * gre;
             inner.im += w * gim;
         }
@@ -150,8 +182,8 @@ __device__ CX<R> pair_integral(const Geo &g, int tm, int vmi, int tn, int vni)
             inner.re += ((R)0.25 * (a[0] * S1[0] + a[1] * S1[1] + a[2] * S1[2]) - ik2 * s0) * inv4pi /
                         (R)g.area[tn];
         }
-        acc.re += (R)c_qw[i] * inner.re;
-        acc.im += (R)c_qw[i] * inner.im;
+        acc.re += qweight<R>(i) * inner.re;
+        acc.im += qweight<R>(i) * inner.im;
     }
     return acc;
 }
@@ -177,6 +209,19 @@ __device__ CX<R> rwg_entry(const Geo &g, int m, int n)
 }
 
 template <class R> __device__ CX<R> Geo::entry(int m, int n) const { return rwg_entry<R>(*this, m, n); }
+
+__device__ CX<float> Geo::part(int m, int n, int p) const
+{
+    const int a = 2 * m + (p >> 1), b = 2 * n + (p & 1);
+    const CX<float> v = pair_integral<float>(*this, etri[a], efree[a], etri[b], efree[b]);
+    const float s = ((p >> 1) == (p & 1)) ? 1.f : -1.f;
+    return CX<float>{s * v.re, s * v.im};
+}
+__device__ CX<float> Geo::scale(int m, int n, const CX<float> &z) const
+{
+    const float f = (float)(k * eta * elen[m] * elen[n]);
+    return CX<float>{-f * z.im, f * z.re};
+}
 
 
 // b[r*ldb + m] = sum_s ucoef[m][s] sum_q w_q (r_q - v_s) . p_hat exp(-jk k_hat . r_q): the
@@ -353,6 +398,9 @@ hm_status build_from_mesh(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
                 qpd[(t * NQ + q) * 3 + d] = bary[q][0] * p0[d] + bary[q][1] * p1[d] + bary[q][2] * p2[d];
     }
     HM_CUDA(cudaMemcpyToSymbol(c_qw, qw, sizeof(qw)));
+    float qwf[NQ];
+    for (int q = 0; q < NQ; ++q) qwf[q] = (float)qw[q];
+    HM_CUDA(cudaMemcpyToSymbol(c_qwf, qwf, sizeof(qwf)));
     TmpBuffers tmp;
     Geo g{};
     std::vector<double> vtx(mesh->xyz, mesh->xyz + 3 * nv);
@@ -368,6 +416,12 @@ hm_status build_from_mesh(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
     g.etri = d_etri; g.efree = d_efree; g.elen = d_elen;
     g.k = 2.0 * 3.14159265358979323846 / mesh->wavelength;
     g.eta = 376.730313461770655;
+    float2 *d_vtx32, *d_qpd32;
+    if ((st = tmp.up(&d_vtx32, float_pairs(vtx), s)) || (st = tmp.up(&d_qpd32, float_pairs(qpd), s))) return st;
+    g.vtx32 = d_vtx32;
+    g.qpd32 = d_qpd32;
+    g.kf = (float)g.k;
+    g.ik2f = (float)(1.0 / (g.k * g.k));
 
     B.nq = NQ;
     B.qw.assign(qw, qw + NQ);

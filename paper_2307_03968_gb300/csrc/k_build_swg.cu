@@ -57,6 +57,7 @@ struct VGeo {
     const double *fqs;      // nf surface charge kappa(T+) - kappa(T-)
     const int32_t *perm;    // tree position -> original face index
     double k;
+    static constexpr int PARTS = 1;
     template <class R> __device__ CX<R> entry(int m, int n) const;
 };
 
