@@ -530,8 +530,7 @@ static void copy_vec(SolveCtx &c, void *dst, const void *src)
 static void last_leaf_update(SolveCtx &c, const void *Y, void *Z, void *dst)
 {
     if (!c.rec && !c.fp64 && c.fin_target == dst) {
-        launch_leaf_finish(c.h, (const float2 *)Y, (float2 *)Z, (float2 *)dst, c.fin_base, c.fin_x, c.fin_ldx, c.nrhs,
-                           c.s);
+        launch_leaf_finish(c.h, (const float2 *)Y, (float2 *)Z, c.fin_base, c.fin_x, c.fin_ldx, c.nrhs, c.s);
         c.launches++;
         c.bytes += leaf_update_bytes(c);
         c.fin_done = true;
@@ -744,7 +743,7 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
             c.launches += launch_apply_items_partials(h, it->second, x, h->ws.d_part, h->partial_elems, nr, c.s,
                                                       c.res_rb);
         }
-        if (y_next && nr == c.nrhs) {
+        if (y_next && nr == c.nrhs && leaf_chunks(h, nr) == 1) {
             launch_gather_leaf_update(h, x, c.m, h->ws.d_part, h->partial_elems, bt, out, norms, y_next, nr, c.s);
             c.bytes += leaf_update_bytes(c);
             c.y_ready = out;

@@ -102,7 +102,7 @@ __device__ bool run_phases(const Phase *phases, int n_phases, const PersistCtx &
         }
         case PH_LEAF: {
             float2 *zs = reinterpret_cast<float2 *>(sm);
-            float2(*part)[64] = reinterpret_cast<float2(*)[64]>(sm + PERSIST_MAX_NP * sizeof(float2));
+            float2 *part = reinterpret_cast<float2 *>(sm + PERSIST_MAX_NP * sizeof(float2));
             const int64_t nvb = c.n_leaves * P.nrhs;
             for (int64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
                 const int leaf = (int)(vb % c.n_leaves), r = (int)(vb / c.n_leaves);
@@ -143,7 +143,7 @@ __device__ bool run_phases(const Phase *phases, int n_phases, const PersistCtx &
                 const int leaf = (int)(vb % c.n_leaves), r = (int)(vb / c.n_leaves);
                 gather_leaf(leaf, r, c.pleaf_off, c.dinv_off, c.self32, (const float2 *)P.a, c.pN, c.csr_off,
                             c.csr_stride, P.m, c.csr_idx, (const cdf *)P.d, P.ld, (const float2 *)P.b,
-                            (float2 *)P.c, P.norms, acc_s, xs);
+                            (float2 *)P.c, P.norms, acc_s, xs, 0, 64);
             }
             break;
         }

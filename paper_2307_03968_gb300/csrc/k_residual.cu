@@ -58,8 +58,9 @@ k_item_bounds(const Item *__restrict__ items, int64_t n_items, const float2 *__r
     }
 }
 
-// Per leaf (blockIdx.x) and right-hand side (blockIdx.y): acc = D_I x_I +
-// sum of the leaf's partial slots of levels 1..m (gather_leaf).
+// Per leaf (blockIdx.x), right-hand side (blockIdx.y) and row chunk (blockIdx.z, where the
+// leaves are few and long: leaf_chunks): acc = D_I x_I + sum of the leaf's partial slots of
+// levels 1..m (gather_leaf).
 __global__ void __launch_bounds__(GW * 32)
 k_gather_acc64(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict__ dinv_off,
                const float2 *__restrict__ self32, const float2 *__restrict__ x, int64_t ld,
@@ -70,7 +71,7 @@ k_gather_acc64(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict_
     __shared__ cdf acc_s[GW][64];
     extern __shared__ __align__(16) unsigned char gsm[];
     gather_leaf(blockIdx.x, blockIdx.y, pleaf_off, dinv_off, self32, x, ld, csr_off, csr_stride, m, csr_idx, part,
-                pstride, b, out, norms, acc_s, reinterpret_cast<float2 *>(gsm));
+                pstride, b, out, norms, acc_s, reinterpret_cast<float2 *>(gsm), 64 * blockIdx.z, 64 * gridDim.z);
 }
 
 // The gather, then the next series step of the refinement in the same CTA: out = b - acc
@@ -84,10 +85,10 @@ k_gather_leaf_update(const int32_t *__restrict__ pleaf_off, const int64_t *__res
                      const float2 *__restrict__ b, float2 *out, double *norms, float2 *y)
 {
     __shared__ cdf acc_s[GW][64];
-    __shared__ float2 lpart[8][64];
+    __shared__ float2 lpart[8 * 64];
     extern __shared__ __align__(16) unsigned char gsm[];
     gather_leaf(blockIdx.x, blockIdx.y, pleaf_off, dinv_off, self32, x, ld, csr_off, csr_stride, m, csr_idx, part,
-                pstride, b, out, norms, acc_s, reinterpret_cast<float2 *>(gsm));
+                pstride, b, out, norms, acc_s, reinterpret_cast<float2 *>(gsm), 0, 64);
     __syncthreads();                                       // this CTA's writes of out_i, read back below
     leaf_update_leaf<float>(blockIdx.x, blockIdx.y, pleaf_off, dinv_off, dinv32, nullptr, out, y, ld, 0,
                             reinterpret_cast<float2 *>(gsm), lpart);
@@ -155,7 +156,7 @@ void launch_item_bounds(const Item *items, int64_t n, const float2 *pool, float4
 void launch_gather_acc64(hm_matrix h, const float2 *x, int m, const cdf *part, int64_t pstride,
                          const float2 *b, float2 *out, double *norms, int nrhs, cudaStream_t s)
 {
-    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs);
+    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs, (unsigned)leaf_chunks(h, nrhs));
     const int64_t maxnp = [&] {
         int64_t v = 0;
         for (int64_t i = 0; i < h->n_leaves; ++i) v = std::max<int64_t>(v, h->pleaf_off[i + 1] - h->pleaf_off[i]);

@@ -491,14 +491,16 @@ __device__ __forceinline__ void resid_item(const Item &it, const float4 *__restr
 // rounded to complex64) and |r|^2, |b|^2 go to norms; else out = acc (complex64).
 // No atomics on sums.
 // The body for one (leaf, right-hand side) pair, run by a CTA of GW warps;
-// acc_s and xs (the leaf's x, np entries) are shared-memory buffers of the caller.
+// acc_s and xs (the leaf's x, np entries) are shared-memory buffers of the caller; rows
+// rc0 .. rc0 + 63, then every rcs rows on.
 constexpr int GW = 8;   // warps per leaf
 __device__ __forceinline__ void gather_leaf(int leaf, int r, const int32_t *__restrict__ pleaf_off,
                                             const int64_t *__restrict__ dinv_off, const float2 *__restrict__ self32,
                                             const float2 *HM_XR x, int64_t ld, const int64_t *__restrict__ csr_off,
                                             int csr_stride, int m, const int64_t *__restrict__ csr_idx,
                                             const cdf *HM_XR part, int64_t pstride, const float2 *HM_XR b,
-                                            float2 *HM_XR out, double *norms, cdf (*acc_s)[64], float2 *xs)
+                                            float2 *HM_XR out, double *norms, cdf (*acc_s)[64], float2 *xs, int rc0,
+                                            int rcs)
 {
     const int o = pleaf_off[leaf], np = pleaf_off[leaf + 1] - o;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -507,7 +509,7 @@ __device__ __forceinline__ void gather_leaf(int leaf, int r, const int32_t *__re
     const cdf *P = part + r * pstride;
     const int64_t e0 = csr_off[(int64_t)leaf * csr_stride], e1 = csr_off[(int64_t)leaf * csr_stride + m];
     const float2 *S = self32 + dinv_off[leaf];                      // column-major np x np
-    for (int rc = 0; rc < np; rc += 64) {
+    for (int rc = rc0; rc < np; rc += rcs) {
         const int i = rc + 2 * lane;
         cdf a0 = cdf_zero(), a1 = cdf_zero();
         if (i < np) {

@@ -13,18 +13,49 @@ namespace {
 
 using namespace kc;
 
-// Per leaf (blockIdx.x) and right-hand side (blockIdx.y): leaf_update_leaf.
-template <class T>
+// The leaf passes: a CTA per leaf (blockIdx.x), group of RB right-hand sides (blockIdx.y)
+// and, where the leaves are few and long, row chunk (blockIdx.z; leaf_grid gives the
+// split and the reasons).
+
+// the leaf's vectors of RB right-hand sides (nr of them given, zero past them) into zs, all
+// loads before the first store, then cleared if asked
+template <int RB, class C>
+__device__ __forceinline__ void leaf_vectors(C *z, int64_t ld, int np, int nr, int clear, C *zs)
+{
+    for (int j = threadIdx.x; j < np; j += 256) {
+        C v[RB];
+#pragma unroll
+        for (int q = 0; q < RB; ++q) v[q] = q < nr ? z[q * ld + j] : czero(C());
+#pragma unroll
+        for (int q = 0; q < RB; ++q) zs[q * np + j] = v[q];
+    }
+    __syncthreads();
+    if (clear)
+        for (int j = threadIdx.x; j < np; j += 256)
+#pragma unroll
+            for (int q = 0; q < RB; ++q)
+                if (q < nr) z[q * ld + j] = czero(C());
+}
+
+// out = y ? y - D_i^{-1} zin_i : D_i^{-1} zin_i; zin_i cleared if zero_in (one row chunk only)
+template <class T, int RB>
 __global__ void __launch_bounds__(256)
 k_leaf_update(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict__ dinv_off,
               const typename CT<T>::C *__restrict__ dinv, const typename CT<T>::C *y,
-              typename CT<T>::C *zin, typename CT<T>::C *out, int64_t ld, int zero_in)
+              typename CT<T>::C *zin, typename CT<T>::C *out, int64_t ld, int nrhs, int zero_in)
 {
     using C = typename CT<T>::C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ C part[8][64];
-    leaf_update_leaf<T>(blockIdx.x, blockIdx.y, pleaf_off, dinv_off, dinv, y, zin, out, ld, zero_in,
-                        reinterpret_cast<C *>(smem_raw), part);
+    __shared__ C part[8 * RB * 64];
+    C *zs = reinterpret_cast<C *>(smem_raw);
+    const int leaf = blockIdx.x, r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);
+    const int o = pleaf_off[leaf], np = pleaf_off[leaf + 1] - o;
+    leaf_vectors<RB>(zin + (int64_t)r0 * ld + o, ld, np, nr, zero_in, zs);
+    leaf_product<T, RB>(dinv + dinv_off[leaf], np, 64 * blockIdx.z, 64 * gridDim.z, zs, part, [&](int q, int i, C s) {
+        if (q >= nr) return;
+        const int64_t g = (int64_t)(r0 + q) * ld + o + i;
+        out[g] = y ? csub(y[g], s) : s;
+    });
 }
 
 // acc += D x for the complex64 self blocks (column-major, like D^{-1}), with
@@ -79,25 +110,36 @@ __global__ void k_permute_in(const C *__restrict__ b, int64_t ldb, C *__restrict
     }
 }
 
-// Per leaf (blockIdx.x) and right-hand side (blockIdx.y), complex64: the leaf's rows
-// of bt = P b (0 at pads), then y = D_i^{-1} bt_i (the first step of the series, eq. 12
-// applied to the permuted right-hand side) in the same CTA.
+// complex64: the leaf's rows of bt = P b (0 at pads) and y = D_i^{-1} bt_i (the first step
+// of the series, eq. 12 applied to the permuted right-hand side)
+template <int RB>
 __global__ void __launch_bounds__(256)
 k_permute_leaf(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict__ dinv_off,
                const float2 *__restrict__ dinv, const int32_t *__restrict__ pperm, const float2 *__restrict__ b,
-               int64_t ldb, float2 *bt, float2 *y, int64_t pN)
+               int64_t ldb, float2 *bt, float2 *y, int64_t pN, int nrhs)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float2 part[8][64];
-    const int leaf = blockIdx.x, r = blockIdx.y;
+    __shared__ float2 part[8 * RB * 64];
+    float2 *zs = reinterpret_cast<float2 *>(smem_raw);
+    const int leaf = blockIdx.x, r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);
     const int o = pleaf_off[leaf], np = pleaf_off[leaf + 1] - o;
-    for (int j = threadIdx.x; j < np; j += blockDim.x) {
+    for (int j = threadIdx.x; j < np; j += 256) {
         const int32_t src = pperm[o + j];
-        bt[r * pN + o + j] = src >= 0 ? b[r * ldb + src] : make_float2(0.f, 0.f);
+        float2 v[RB];
+#pragma unroll
+        for (int q = 0; q < RB; ++q)
+            v[q] = src >= 0 && q < nr ? b[(int64_t)(r0 + q) * ldb + src] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+            zs[q * np + j] = v[q];
+            if (blockIdx.z == 0 && q < nr) bt[(int64_t)(r0 + q) * pN + o + j] = v[q];
+        }
     }
-    __syncthreads();                                       // this CTA's writes of bt_i, read back below
-    leaf_update_leaf<float>(leaf, r, pleaf_off, dinv_off, dinv, nullptr, bt, y, pN, 0,
-                            reinterpret_cast<float2 *>(smem_raw), part);
+    __syncthreads();
+    leaf_product<float, RB>(dinv + dinv_off[leaf], np, 64 * blockIdx.z, 64 * gridDim.z, zs, part,
+                            [&](int q, int i, float2 s) {
+                                if (q < nr) y[(int64_t)(r0 + q) * pN + o + i] = s;
+                            });
 }
 
 template <class C>
@@ -156,31 +198,33 @@ __global__ void k_finish(const float2 *__restrict__ xt, const float2 *__restrict
     if (bad) atomicCAS(status, 0, (int)HM_ERR_DIVERGED);
 }
 
-// The last series step of a complex64 solve and the end of the solve, per leaf
-// (blockIdx.x) and right-hand side (blockIdx.y): out_i = y_i - D_i^{-1} z_i (z_i cleared),
-// then v = (base ? base_i + out_i : out_i), non-finite v -> HM_ERR_DIVERGED, and
-// x[r * ldx + pperm[p]] = v (k_leaf_update followed by k_finish, in one CTA).
+// The last series step of a complex64 solve and the end of the solve:
+// v = (base ? base_i : 0) + (y_i - D_i^{-1} z_i) (z_i cleared if zero_in), non-finite v ->
+// HM_ERR_DIVERGED, x[r * ldx + pperm[p]] = v.
+template <int RB>
 __global__ void __launch_bounds__(256)
 k_leaf_finish(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict__ dinv_off,
-              const float2 *__restrict__ dinv, const float2 *y, float2 *z, float2 *out, const float2 *base,
-              int64_t pN, float2 *__restrict__ x, int64_t ldx, const int32_t *__restrict__ pperm, int *status)
+              const float2 *__restrict__ dinv, const float2 *__restrict__ y, float2 *z, const float2 *__restrict__ base,
+              int64_t pN, int nrhs, float2 *__restrict__ x, int64_t ldx, const int32_t *__restrict__ pperm, int *status,
+              int zero_in)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float2 part[8][64];
-    const int leaf = blockIdx.x, r = blockIdx.y;
-    leaf_update_leaf<float>(leaf, r, pleaf_off, dinv_off, dinv, y, z, out, pN, 1,
-                            reinterpret_cast<float2 *>(smem_raw), part);
-    __syncthreads();                                       // this CTA's writes of out_i, read back below
+    __shared__ float2 part[8 * RB * 64];
+    float2 *zs = reinterpret_cast<float2 *>(smem_raw);
+    const int leaf = blockIdx.x, r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);
     const int o = pleaf_off[leaf], np = pleaf_off[leaf + 1] - o;
+    leaf_vectors<RB>(z + (int64_t)r0 * pN + o, pN, np, nr, zero_in, zs);
     bool bad = false;
-    for (int j = threadIdx.x; j < np; j += blockDim.x) {
-        const int64_t g = r * pN + o + j;
-        float2 v = out[g];
-        if (base) v = cadd(v, base[g]);
-        bad |= !isfinite(v.x) || !isfinite(v.y);
-        const int32_t dst = pperm[o + j];
-        if (dst >= 0) x[r * ldx + dst] = v;
-    }
+    leaf_product<float, RB>(dinv + dinv_off[leaf], np, 64 * blockIdx.z, 64 * gridDim.z, zs, part,
+                            [&](int q, int i, float2 s) {
+                                if (q >= nr) return;
+                                const int64_t g = (int64_t)(r0 + q) * pN + o + i;
+                                float2 v = csub(y[g], s);
+                                if (base) v = cadd(v, base[g]);
+                                bad |= !isfinite(v.x) || !isfinite(v.y);
+                                const int32_t dst = pperm[o + i];
+                                if (dst >= 0) x[(int64_t)(r0 + q) * ldx + dst] = v;
+                            });
     if (bad) atomicCAS(status, 0, (int)HM_ERR_DIVERGED);
 }
 
@@ -242,26 +286,64 @@ void launch_apply_self_f32(hm_matrix h, const float2 *x, float2 *acc, int nrhs, 
                                                                               h->d_self32, x, acc, h->pN);
 }
 
+// Grid of a leaf pass over nrhs right-hand sides.
+//  - Row chunks (chunks > 1): one CTA per leaf and right-hand side leaves the GPU idle when
+//    the leaves are few: the 64 leaves of 1,050 unknowns of a 67,200-unknown plate took 0.63 ms
+//    a pass on 64 of 152 SMs, 0.11 ms in chunks of 64 rows (their 564 MB of inverses need
+//    0.083 ms at the measured copy bandwidth).  Above 8 CTAs an SM there is nothing to gain
+//    and the chunks would only re-read z, so the split is for fewer CTAs than that.
+//  - RB right-hand sides a CTA: the inverse is read (from L2) once for RB of them, where the
+//    pass still has 4 CTAs an SM then: 512 leaves of 60 with 181 right-hand sides take 0.177 ms
+//    an update, 0.155 the last one and 0.135 the first, instead of 0.31, 0.52 and 0.29.
+struct LeafGrid { dim3 grid; int rb, chunks; size_t maxnp; };
+static LeafGrid leaf_grid(hm_matrix h, int nrhs, bool batch)
+{
+    LeafGrid g;
+    g.maxnp = (size_t)std::max<int64_t>(max_padded_leaf(h), 1);
+    const int64_t sms = h->num_sms > 0 ? h->num_sms : 1;
+    g.chunks = leaf_chunks(h, nrhs);
+    g.rb = batch && g.chunks == 1 && g.maxnp <= 256 && h->n_leaves * ((nrhs + 3) / 4) >= 4 * sms ? 4 : 1;
+    g.grid = dim3((unsigned)h->n_leaves, (unsigned)((nrhs + g.rb - 1) / g.rb), (unsigned)g.chunks);
+    return g;
+}
+
+int leaf_chunks(hm_matrix h, int nrhs)
+{
+    const int64_t maxnp = max_padded_leaf(h), sms = h->num_sms > 0 ? h->num_sms : 1;
+    return h->n_leaves * nrhs < 8 * sms ? (int)std::max<int64_t>((maxnp + 63) / 64, 1) : 1;
+}
+
 void launch_permute_leaf(hm_matrix h, const float2 *b, int64_t ldb, float2 *bt, float2 *y, int nrhs, cudaStream_t s)
 {
-    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs);
-    k_permute_leaf<<<grid, 256, max_padded_leaf(h) * sizeof(float2), s>>>(h->d_pleaf_off, h->d_dinv_off, h->d_dinv32,
-                                                                          h->d_pperm, b, ldb, bt, y, h->pN);
+    const LeafGrid g = leaf_grid(h, nrhs, true);
+    auto go = [&](auto kern) {
+        kern<<<g.grid, 256, g.rb * g.maxnp * sizeof(float2), s>>>(h->d_pleaf_off, h->d_dinv_off, h->d_dinv32, h->d_pperm,
+                                                                  b, ldb, bt, y, h->pN, nrhs);
+    };
+    if (g.rb == 4) go(k_permute_leaf<4>);
+    else go(k_permute_leaf<1>);
 }
 
 void launch_leaf_update(hm_matrix h, const void *y, void *zin, void *out, int nrhs, bool zero_in, bool fp64,
                         cudaStream_t s)
 {
-    const int64_t maxnp = max_padded_leaf(h);
-    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs);
-    if (fp64)
-        k_leaf_update<double><<<grid, 256, maxnp * sizeof(double2), s>>>(
-            h->d_pleaf_off, h->d_dinv_off, h->d_dinv64, (const double2 *)y, (double2 *)zin, (double2 *)out, h->pN,
-            zero_in ? 1 : 0);
-    else
-        k_leaf_update<float><<<grid, 256, maxnp * sizeof(float2), s>>>(
-            h->d_pleaf_off, h->d_dinv_off, h->d_dinv32, (const float2 *)y, (float2 *)zin, (float2 *)out, h->pN,
-            zero_in ? 1 : 0);
+    const LeafGrid g = leaf_grid(h, nrhs, !fp64);
+    const int clear = zero_in && g.chunks == 1;    // else the row chunks of a leaf read z side by side
+    if (fp64) {
+        k_leaf_update<double, 1><<<g.grid, 256, g.maxnp * sizeof(double2), s>>>(
+            h->d_pleaf_off, h->d_dinv_off, h->d_dinv64, (const double2 *)y, (double2 *)zin, (double2 *)out, h->pN, nrhs,
+            clear);
+    } else {
+        auto go = [&](auto kern) {
+            kern<<<g.grid, 256, g.rb * g.maxnp * sizeof(float2), s>>>(h->d_pleaf_off, h->d_dinv_off, h->d_dinv32,
+                                                                      (const float2 *)y, (float2 *)zin, (float2 *)out,
+                                                                      h->pN, nrhs, clear);
+        };
+        if (g.rb == 4) go(k_leaf_update<float, 4>);
+        else go(k_leaf_update<float, 1>);
+    }
+    if (zero_in && !clear)
+        cudaMemsetAsync(zin, 0, (fp64 ? sizeof(double2) : sizeof(float2)) * (size_t)h->pN * nrhs, s);
 }
 
 void launch_sub(const void *y, const void *w, void *out, int64_t n, bool fp64, cudaStream_t s)
@@ -285,13 +367,18 @@ void launch_check_finite(const void *x, int64_t n, bool fp64, int *status, cudaS
     else k_check_finite<float2><<<g, 256, 0, s>>>((const float2 *)x, n, status);
 }
 
-void launch_leaf_finish(hm_matrix h, const float2 *y, float2 *z, float2 *out, const float2 *base, float2 *x,
-                        int64_t ldx, int nrhs, cudaStream_t s)
+void launch_leaf_finish(hm_matrix h, const float2 *y, float2 *z, const float2 *base, float2 *x, int64_t ldx, int nrhs,
+                        cudaStream_t s)
 {
-    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs);
-    k_leaf_finish<<<grid, 256, max_padded_leaf(h) * sizeof(float2), s>>>(h->d_pleaf_off, h->d_dinv_off, h->d_dinv32, y,
-                                                                         z, out, base, h->pN, x, ldx, h->d_pperm,
-                                                                         h->d_status);
+    const LeafGrid g = leaf_grid(h, nrhs, true);
+    const int clear = g.chunks == 1;
+    auto go = [&](auto kern) {
+        kern<<<g.grid, 256, g.rb * g.maxnp * sizeof(float2), s>>>(h->d_pleaf_off, h->d_dinv_off, h->d_dinv32, y, z, base,
+                                                                  h->pN, nrhs, x, ldx, h->d_pperm, h->d_status, clear);
+    };
+    if (g.rb == 4) go(k_leaf_finish<4>);
+    else go(k_leaf_finish<1>);
+    if (!clear) cudaMemsetAsync(z, 0, sizeof(float2) * (size_t)h->pN * nrhs, s);
 }
 
 void launch_finish(const float2 *xt, const float2 *dx, int64_t pN, float2 *x, int64_t ldx, const int32_t *pperm,
