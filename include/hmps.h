@@ -430,14 +430,17 @@ hm_status hm_get_info(hm_matrix h, hm_info *info);
  * bucket (the next power of two >= nrhs, at least 4).  The first complex64
  * solve, product or residual in a bucket on an operator times the candidate
  * kernels on that operator at the bucket's size (with CUDA events on the
- * caller's stream, which it synchronises once) and keeps the fastest: for the product and for the
- * FP64-class residual products, 0 = one right-hand side at a time, 8 / 16 / 32 =
- * blocks staged once in shared memory per chunk of that many right-hand sides,
- * 1016 (product only, timed from 32 right-hand sides on) = the blocks of at most
- * 64 x 64 (rank <= 32) on the tensor cores in tiles of 128 right-hand sides;
+ * caller's stream, which it synchronises once) and keeps the fastest: 0 = one right-hand side at
+ * a time, 8 / 16 = blocks staged once in shared memory per chunk of that many right-hand sides,
+ * 32 (product only) = the blocks of at most 64 x 64 (rank <= 32) on the matrix instructions, in
+ * FP16 halves and tiles of 16 or 32 right-hand sides (its first call packs the blocks a second
+ * time, twice their bytes, counted in hm_info.device_bytes, with its workspace);
  * 1017 (residual only, where every level of the call holds only such blocks) =
  * owner-computes FP64-class products, one CTA per output cluster and group of 16
- * right-hand sides, no partial slots.  res_ms of the owner kernel covers all
+ * right-hand sides, no partial slots.  A refined solve whose levels hold only such blocks and
+ * whose choice is not pinned has a choice of its own: the owner-computes form on the matrix
+ * instructions (exact integer digits; errors relative to an output cluster's largest
+ * terms; reported as 1017), above 16 right-hand sides always.  res_ms of the owner kernel covers all
  * nrhs right-hand sides at once, of the others one chunk of at most 16.
  * prod_ms / res_ms: the measured time of one leaf-level launch of the choice.
  * Any output pointer may be NULL.  HM_ERR_STATE if no call with that nrhs has
@@ -448,8 +451,8 @@ hm_status hm_get_tuning(hm_matrix h, int nrhs, int *prod_rb, int *res_rb, double
 /*
  * Pin the kernel choice for the bucket of `nrhs` right-hand sides instead of
  * letting the autotuner time it (e.g. for reproducible benchmarks or to test a
- * kernel): prod_rb 0 (one right-hand side at a time), 8 / 16 / 32 (shared-memory
- * SIMT chunks) or 1016 (tensor-core products of the blocks of at most 64 x 64 and
+ * kernel): prod_rb 0 (one right-hand side at a time), 8 / 16 (shared-memory
+ * SIMT chunks), 32 (matrix instructions) or 1016 (tensor-core products of the blocks of at most 64 x 64 and
  * rank <= 32, dense and low-rank, tiles of 128 right-hand sides, tcgen05 3xTF32;
  * the first call that runs it allocates its stage-1 workspace: the low-rank
  * intermediates, 8 KB per 8 rank rows of every low-rank block side and per tile,

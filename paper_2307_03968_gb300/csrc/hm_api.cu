@@ -63,26 +63,6 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         }
         L.n_small = (int64_t)small.size();
         L.n_big = (int64_t)big.size();
-        const std::map<int32_t, std::vector<TcProd>> by_out = directed_products(small);
-        std::vector<TcUnit> rcu;
-        std::vector<TcProd> rcp;
-        build_owner_lists(by_out, rcu, rcp);
-        TcLists tc;
-        if (!build_tc_lists(by_out, tc)) return fail(HM_ERR_STATE, "tensor-core work lists out of their index bounds");
-        L.n_rcu = (int64_t)rcu.size();
-        if ((st = upload(h, &L.d_rcu, rcu, s)) != HM_OK) return st;
-        if ((st = upload(h, &L.d_rcp, rcp, s)) != HM_OK) return st;
-        if ((st = dev_alloc(h, (void **)&L.d_rcb, sizeof(float2) * rcp.size())) != HM_OK) return st;
-        launch_prod_bounds(L.d_rcp, (int64_t)rcp.size(), h->d_pool32, L.d_rcb, s);
-        L.n_tcu = (int64_t)tc.units.size();
-        L.n_tco = (int64_t)tc.ops.size();
-        L.n_xch = (int64_t)tc.xch.size();
-        L.n_tcb = (int64_t)tc.batches.size();
-        L.n_tcr = (int64_t)tc.rows.size();
-        L.n_tchunk = tc.n_tchunk;
-        h->tc_max_xch = std::max(h->tc_max_xch, L.n_xch);
-        h->tc_max_tchunk = std::max(h->tc_max_tchunk, L.n_tchunk);
-        if ((st = upload(h, &L.d_xch, tc.xch, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_items, L.items, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_small, small, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_big, big, s)) != HM_OK) return st;
@@ -95,11 +75,6 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         launch_item_bounds(L.d_res, (int64_t)res.size(), h->d_pool32, L.d_bnd, s);
         launch_item_bounds(L.d_big, L.n_big, h->d_pool32, L.d_bnd_big, s);
         HM_CUDA(cudaGetLastError());
-        if ((st = upload(h, &L.d_tcu, tc.units, s)) != HM_OK) return st;
-        if ((st = upload(h, &L.d_tco, tc.ops, s)) != HM_OK) return st;
-        if ((st = upload(h, &L.d_tcb, tc.batches, s)) != HM_OK) return st;
-        if ((st = upload(h, &L.d_tcr, tc.rows, s)) != HM_OK) return st;
-        if ((st = upload(h, &L.d_tcc, tc.tchunks, s)) != HM_OK) return st;
         // the product's lists with tall dense blocks cut into row panels: a panel of rows
         // [r, r + mr) of a row-major block is itself a dense item with the same row stride
         auto panels = [](const std::vector<Item> &in, std::vector<Item> &out) {
@@ -132,6 +107,141 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
     return HM_OK;
 }
 
+// the items the multi-right-hand-side kernels take
+static std::vector<Item> small_items(const LevelList &L)
+{
+    std::vector<Item> small;
+    for (const Item &it : L.items)
+        if (it.m <= MRHS_MAX_DIM && it.n <= MRHS_MAX_DIM && it.k <= MRHS_MAX_RANK) small.push_back(it);
+    return small;
+}
+
+// the tcgen05 product's lists, made by the first call that runs it (a pinned choice)
+static hm_status ensure_tc_lists(hm_matrix h, cudaStream_t s)
+{
+    hm_status st;
+    for (auto &kv : h->levels) {
+        LevelList &L = kv.second;
+        if (L.tc_built) continue;
+        TcLists tc;
+        if (!build_tc_lists(directed_products(small_items(L)), tc))
+            return fail(HM_ERR_STATE, "tensor-core work lists out of their index bounds");
+        L.n_tcu = (int64_t)tc.units.size();
+        L.n_tco = (int64_t)tc.ops.size();
+        L.n_xch = (int64_t)tc.xch.size();
+        L.n_tcb = (int64_t)tc.batches.size();
+        L.n_tcr = (int64_t)tc.rows.size();
+        L.n_tchunk = tc.n_tchunk;
+        if ((st = upload(h, &L.d_xch, tc.xch, s)) != HM_OK || (st = upload(h, &L.d_tcu, tc.units, s)) != HM_OK ||
+            (st = upload(h, &L.d_tco, tc.ops, s)) != HM_OK || (st = upload(h, &L.d_tcb, tc.batches, s)) != HM_OK ||
+            (st = upload(h, &L.d_tcr, tc.rows, s)) != HM_OK || (st = upload(h, &L.d_tcc, tc.tchunks, s)) != HM_OK)
+            return st;
+        HM_CUDA(cudaStreamSynchronize(s));        // the host lists end here
+        h->tc_max_xch = std::max(h->tc_max_xch, L.n_xch);
+        h->tc_max_tchunk = std::max(h->tc_max_tchunk, L.n_tchunk);
+        L.tc_built = true;
+    }
+    return HM_OK;
+}
+
+// the lists of the owner-computes residual on the FP32 pipes, made by the first call that runs it
+static hm_status ensure_own_lists(hm_matrix h, cudaStream_t s)
+{
+    hm_status st;
+    for (auto &kv : h->levels) {
+        LevelList &L = kv.second;
+        if (L.own_built) continue;
+        std::vector<TcUnit> rcu;
+        std::vector<TcProd> rcp;
+        build_owner_lists(directed_products(small_items(L)), rcu, rcp);
+        L.n_rcu = (int64_t)rcu.size();
+        if ((st = upload(h, &L.d_rcu, rcu, s)) != HM_OK || (st = upload(h, &L.d_rcp, rcp, s)) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_rcb, sizeof(float2) * rcp.size())) != HM_OK)
+            return st;
+        launch_prod_bounds(L.d_rcp, (int64_t)rcp.size(), h->d_pool32, L.d_rcb, s);
+        HM_CUDA(cudaStreamSynchronize(s));        // the host lists end here
+        L.own_built = true;
+    }
+    return HM_OK;
+}
+
+// a device array of the current call, freed with it
+struct TmpArray {
+    void *p = nullptr;
+    ~TmpArray() { if (p) cudaFree(p); }
+    hm_status make(const void *src, size_t bytes, cudaStream_t s)
+    {
+        HM_CUDA(cudaMalloc(&p, std::max<size_t>(bytes, 16)));
+        if (src && bytes) HM_CUDA(cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, s));
+        else HM_CUDA(cudaMemsetAsync(p, 0, std::max<size_t>(bytes, 16), s));
+        return HM_OK;
+    }
+};
+
+// the matrix-instruction products' lists and operand streams, made by the first call that runs them
+static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
+{
+    hm_status st;
+    for (int lev = 1; lev <= m; ++lev) {
+        auto it = h->levels.find(lev);
+        if (it == h->levels.end() || it->second.mm_built || it->second.n_small == 0) continue;
+        LevelList &L = it->second;
+        MmLists mm;
+        // about four CTAs an SM for one tile of right-hand sides
+        if (!build_mm_lists(directed_products(small_items(L)), 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), mm))
+            return fail(HM_ERR_STATE, "matrix-product work lists out of their index bounds");
+        TmpArray sets, chunks, rows, pairs, wscale, rscale;
+        struct Undo {   // a level's arrays go again if the last of them cannot be had
+            hm_matrix h;
+            LevelList &L;
+            int64_t bytes;
+            ~Undo()
+            {
+                if (L.mm_built) return;
+                void **p[] = {(void **)&L.d_mm_unit, (void **)&L.d_mm_unit2, (void **)&L.d_mm_runit, (void **)&L.d_mm_batch,
+                              (void **)&L.d_mm_xch, (void **)&L.d_mm_ca, (void **)&L.d_mm_tdst, (void **)&L.d_mm_eout,
+                              (void **)&L.d_mm_os, (void **)&L.d_mm_ws};
+                for (void **q : p) {
+                    if (*q) cudaFree(*q);
+                    *q = nullptr;
+                }
+                h->device_bytes = bytes;
+            }
+        } undo{h, L, h->device_bytes};
+        if ((st = upload(h, &L.d_mm_unit, mm.units, s)) != HM_OK || (st = upload(h, &L.d_mm_unit2, mm.units2, s)) != HM_OK ||
+             (st = upload(h, &L.d_mm_runit, mm.runits, s)) != HM_OK ||
+            (st = upload(h, &L.d_mm_batch, mm.batches, s)) != HM_OK || (st = upload(h, &L.d_mm_xch, mm.xch, s)) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_ca, sizeof(int32_t) * mm.chunks.size())) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_tdst, sizeof(int32_t) * mm.pairs.size())) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_eout, sizeof(int) * (size_t)mm.n_cl)) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_os, mm_stream_bytes(mm.n_out))) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_ws, mm_stream_bytes(mm.n_w))) != HM_OK ||
+            (st = sets.make(mm.sets.data(), mm.sets.size() * sizeof(MmSet), s)) != HM_OK ||
+            (st = chunks.make(mm.chunks.data(), mm.chunks.size() * sizeof(MmChunk), s)) != HM_OK ||
+            (st = rows.make(mm.rows.data(), mm.rows.size() * sizeof(int64_t), s)) != HM_OK ||
+            (st = pairs.make(mm.pairs.data(), mm.pairs.size() * sizeof(MmPair), s)) != HM_OK ||
+            (st = wscale.make(nullptr, 2 * mm.pairs.size() * sizeof(float), s)) != HM_OK ||
+            (st = rscale.make(nullptr, mm.rows.size() * sizeof(float), s)) != HM_OK)
+            return st;
+        L.mm_n_unit = (int64_t)mm.units.size();
+        L.mm_n_unit2 = (int64_t)mm.units2.size();
+        L.mm_n_chunk = (int64_t)mm.chunks.size();
+        L.mm_n_runit = (int64_t)mm.runits.size();
+        L.mm_n_batch = (int64_t)mm.batches.size();
+        L.mm_n_xch = (int64_t)mm.xch.size();
+        L.mm_n_tch = mm.n_tch;
+        L.mm_parts = mm.n_cl > 0 ? mm.parts : 0;
+        launch_mm_pack(L, MmPackArgs{(const MmSet *)sets.p, (const MmChunk *)chunks.p, (const int64_t *)rows.p,
+                                     (const MmPair *)pairs.p, (float *)wscale.p, (float *)rscale.p, (int64_t)mm.sets.size(),
+                                     (int64_t)mm.chunks.size(), mm.n_cl},
+                       h->d_pool32, s);
+        HM_CUDA(cudaGetLastError());
+        HM_CUDA(cudaStreamSynchronize(s));        // the lists end here
+        L.mm_built = true;
+    }
+    return HM_OK;
+}
+
 static void clear_graphs(hm_matrix h)
 {
     for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second);
@@ -155,7 +265,7 @@ static void free_handle(hm_matrix h)
     void *ptrs[] = {h->d_pperm, h->d_pleaf_off, h->d_dinv_off, h->d_leaf_n, h->d_self_off, h->d_bad_leaf,
                     h->d_self64, h->d_self32, h->d_dinv32, h->d_dinv64, h->d_pool32, h->d_pool64, h->d_status,
                     h->ws.d_acc64, h->ws.d_io, h->ws.d_part, h->d_csr_off, h->d_csr_idx, h->ws.d_xpl, h->ws.d_tct,
-                    h->ws.d_own};
+                    h->ws.d_own, h->ws.d_mm};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &kv : h->levels) {
@@ -173,9 +283,11 @@ static void free_handle(hm_matrix h)
         if (kv.second.d_tcr) cudaFree(kv.second.d_tcr);
         if (kv.second.d_tcc) cudaFree(kv.second.d_tcc);
         if (kv.second.d_xch) cudaFree(kv.second.d_xch);
-        if (kv.second.d_rcu) cudaFree(kv.second.d_rcu);
-        if (kv.second.d_rcp) cudaFree(kv.second.d_rcp);
-        if (kv.second.d_rcb) cudaFree(kv.second.d_rcb);
+        const LevelList &L = kv.second;
+        void *mm[] = {L.d_rcu, L.d_rcp, L.d_rcb, L.d_mm_unit, L.d_mm_unit2, L.d_mm_runit, L.d_mm_batch, L.d_mm_xch, L.d_mm_ca, L.d_mm_tdst,
+                      L.d_mm_eout, L.d_mm_os, L.d_mm_ws};
+        for (void *p : mm)
+            if (p) cudaFree(p);
     }
     for (void *p : h->ws.vec32) if (p) cudaFree(p);
     for (void *p : h->ws.vec64) if (p) cudaFree(p);
@@ -367,26 +479,41 @@ static hm_status ensure_workspace(hm_matrix h, int nrhs, int m)
     if (ws.d_own) cudaFree(ws.d_own);   // owner sums: ensure_own
     ws.d_own = nullptr;
     ws.own_bytes = 0;
-    if (ws.d_tct) cudaFree(ws.d_tct);   // stage-1 results of the tensor-core product: ensure_tct
+    if (ws.d_tct) cudaFree(ws.d_tct);   // workspaces of the tcgen05 product: ensure_tct
     ws.d_tct = nullptr;
     ws.tct_bytes = 0;
-    if (r >= MRHS_MIN_RHS && h->tc_max_xch > 0) {   // split x of the tensor-core product (it can be pinned from 4 RHS)
-        ws.xpl_bytes = tc_xplane_bytes(h->tc_max_xch, r);
-        HM_CUDA(cudaMalloc((void **)&ws.d_xpl, ws.xpl_bytes));
-        ws.dev_bytes += (int64_t)ws.xpl_bytes;
-    }
+    if (ws.d_mm) ws.dev_bytes += (int64_t)ws.mm_bytes;   // kept: it does not depend on the workspace's size (ensure_mm)
     ws.part_rhs = std::min(r, RESID_CHUNK);   // the partial slots themselves: ensure_partials
     ws.nrhs = r;
     return HM_OK;
 }
 
-// FP64 owner sums of the owner-computes residual ([level][RHS][pN] for the
+// FP64 owner sums of the owner-computes residual ([level][part][RHS][pN] for the
 // workspace's RHS count and m levels); allocated only by the calls that form a
 // residual with that kernel, before any capture
-static hm_status ensure_own(hm_matrix h, int m)
+// owner-sum arrays of levels 1..m: one a level, or its mm_parts on the matrix instructions
+static int own_arrays(hm_matrix h, int m, bool mm)
+{
+    int n = 0;
+    for (int lev = 1; lev <= m; ++lev) {
+        auto it = h->levels.find(lev);
+        if (it != h->levels.end() && !it->second.items.empty()) n += mm ? it->second.mm_parts : 1;
+    }
+    return n;
+}
+static size_t own_bytes(hm_matrix h, int m, int nrhs, bool mm)
+{
+    return sizeof(double2) * (size_t)std::max(own_arrays(h, m, mm), 1) * (size_t)nrhs * (size_t)h->pN;
+}
+
+static hm_status ensure_own(hm_matrix h, int m, bool mm, cudaStream_t s)
 {
     hm::Workspace &ws = h->ws;
-    const size_t bytes = sizeof(double2) * (size_t)std::max(m, 1) * (size_t)ws.nrhs * (size_t)h->pN;
+    if (!mm) {
+        const hm_status st = ensure_own_lists(h, s);
+        if (st != HM_OK) return st;
+    }
+    const size_t bytes = own_bytes(h, m, ws.nrhs, mm);
     if (ws.d_own && ws.own_bytes >= bytes) return HM_OK;
     clear_graphs(h);   // graphs hold the old pointer
     if (ws.d_own) {
@@ -401,23 +528,53 @@ static hm_status ensure_own(hm_matrix h, int m)
     return HM_OK;
 }
 
-// stage-1 results of the tensor-core product (T chunks of the largest level for the
-// workspace's RHS tiles); allocated only by the calls that run that product, before
-// any capture
-static hm_status ensure_tct(hm_matrix h)
+// split x and stage-1 results of the tcgen05 product (the largest level, the workspace's RHS
+// tiles) with its lists; allocated only by the calls that run that product, before any capture
+static hm_status ensure_tct(hm_matrix h, cudaStream_t s)
 {
     hm::Workspace &ws = h->ws;
-    const size_t bytes = tc_t_bytes(h->tc_max_tchunk, ws.nrhs);
-    if (bytes == 0 || (ws.d_tct && ws.tct_bytes >= bytes)) return HM_OK;
-    clear_graphs(h);   // graphs hold the old pointer
-    if (ws.d_tct) {
-        cudaFree(ws.d_tct);
-        ws.dev_bytes -= (int64_t)ws.tct_bytes;
+    const hm_status st = ensure_tc_lists(h, s);
+    if (st != HM_OK) return st;
+    const size_t xb = tc_xplane_bytes(h->tc_max_xch, ws.nrhs), tb = tc_t_bytes(h->tc_max_tchunk, ws.nrhs);
+    struct { float **p; size_t *have, need; } bufs[] = {{&ws.d_xpl, &ws.xpl_bytes, xb}, {&ws.d_tct, &ws.tct_bytes, tb}};
+    for (auto &q : bufs) {
+        if (q.need == 0 || (*q.p && *q.have >= q.need)) continue;
+        clear_graphs(h);   // graphs hold the old pointer
+        if (*q.p) {
+            cudaFree(*q.p);
+            ws.dev_bytes -= (int64_t)*q.have;
+        }
+        *q.p = nullptr;
+        *q.have = 0;
+        HM_CUDA(cudaMalloc((void **)q.p, q.need));
+        *q.have = q.need;
+        ws.dev_bytes += (int64_t)q.need;
     }
-    ws.d_tct = nullptr;
-    ws.tct_bytes = 0;
-    HM_CUDA(cudaMalloc((void **)&ws.d_tct, bytes));
-    ws.tct_bytes = bytes;
+    return HM_OK;
+}
+
+// operand tiles of the matrix-instruction products for nrhs right-hand sides (a pass of them),
+// levels 1..m; allocated only by the calls that run them, before any capture
+static hm_status ensure_mm(hm_matrix h, int m, int nrhs, bool res, cudaStream_t s)
+{
+    hm::Workspace &ws = h->ws;
+    const hm_status st = ensure_mm_lists(h, m, s);
+    if (st != HM_OK) return st;
+    size_t bytes = 0;
+    for (int lev = 1; lev <= m; ++lev) {
+        auto it = h->levels.find(lev);
+        if (it != h->levels.end() && it->second.n_small > 0) bytes = std::max(bytes, mm_ws_bytes(it->second, nrhs, res));
+    }
+    if (bytes == 0 || (ws.d_mm && ws.mm_bytes >= bytes)) return HM_OK;
+    clear_graphs(h);   // graphs hold the old pointer
+    if (ws.d_mm) {
+        cudaFree(ws.d_mm);
+        ws.dev_bytes -= (int64_t)ws.mm_bytes;
+    }
+    ws.d_mm = nullptr;
+    ws.mm_bytes = 0;
+    HM_CUDA(cudaMalloc(&ws.d_mm, bytes));
+    ws.mm_bytes = bytes;
     ws.dev_bytes += (int64_t)bytes;
     return HM_OK;
 }
@@ -691,19 +848,28 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
                        float2 *y_next = nullptr)
 {
     hm_matrix h = c.h;
-    if (!c.rec && c.res_rb == RB_OWN && h->ws.d_own &&
-        h->ws.own_bytes >= sizeof(double2) * (size_t)c.m * (size_t)c.nrhs * (size_t)h->pN && own_applies(h, c.m)) {
-        // owner-computes: each level's sums into its own FP64 [RHS][pN] array, then one gather
+    const bool mm = c.res_rb == RB_MM;
+    if (!c.rec && (mm || c.res_rb == RB_OWN) && h->ws.d_own && h->ws.own_bytes >= own_bytes(h, c.m, c.nrhs, mm) &&
+        own_applies(h, c.m)) {
+        // owner-computes: each level's sums into its own FP64 [part][RHS][pN] arrays, then one gather
         const int64_t lstride = (int64_t)c.nrhs * h->pN;
-        cudaMemsetAsync(h->ws.d_own, 0, sizeof(double2) * (size_t)c.m * (size_t)lstride, c.s);
+        const int arrays = own_arrays(h, c.m, mm);
+        cudaMemsetAsync(h->ws.d_own, 0, sizeof(double2) * (size_t)arrays * (size_t)lstride, c.s);
+        int at = 0;
         for (int lev = 1; lev <= c.m; ++lev) {
             auto it = h->levels.find(lev);
             if (it == h->levels.end() || it->second.items.empty()) continue;
-            launch_resid_own(h, it->second, xt, h->ws.d_own + (int64_t)(lev - 1) * lstride, c.nrhs, c.s);
-            c.launches++;
+            if (mm) {
+                c.launches += launch_mm_resid(h, it->second, xt, h->ws.d_own + at * lstride, lstride, c.nrhs, h->ws.d_mm, c.s);
+                at += it->second.mm_parts;
+            } else {
+                launch_resid_own(h, it->second, xt, h->ws.d_own + at * lstride, c.nrhs, c.s);
+                c.launches++;
+                at++;
+            }
         }
-        launch_gather_own(h, xt, c.m, h->ws.d_own, lstride, bt, out, norms, c.nrhs, c.s);
-        c.launches += 2;
+        launch_gather_own(h, xt, arrays, h->ws.d_own, lstride, bt, out, norms, c.nrhs, c.s);
+        c.launches += 1;
         return;
     }
     const int chunk = std::max(1, h->ws.part_rhs);
@@ -758,12 +924,15 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
 // Autotuner of the many-right-hand-side kernels.  On the first complex64 solve,
 // product or residual with a given right-hand-side count (>= MRHS_MIN_RHS), time
 // on this operator, with CUDA events on the caller's stream, the leaf-level
-// product with every candidate kernel (one right-hand side at a time; shared-
-// memory chunks of 8, 16, 32) and the FP64-class residual products likewise (one
-// at a time; chunks of 8, 16), and keep the fastest of each.  The candidates
-// compute the same sums (up to the order of FP32 atomics), so the choice changes
-// speed only.  It runs before any graph capture, so captured solves replay the
-// chosen kernels.
+// product with the candidate kernels for that count (one right-hand side at a time;
+// shared-memory chunks of 8, 16; the matrix instructions) and, for hm_residual and
+// hm_apply, the FP64-class residual products likewise (one at a time; chunks of 8, 16;
+// owner-computes), and keep the fastest of each.  The candidates compute the same
+// sums up to FP32 rounding, so the choice changes speed only.  It runs before any graph
+// capture, so captured solves replay the chosen kernels.  A refined solve's residual on levels
+// of small blocks is on the matrix instructions above 16 right-hand sides (faster at every
+// size measured, 300 to 30,720 unknowns: 76 against 83 us the solve to 8.8 against 16.6 ms at
+// 32) and up to 16 timed against the partial-slot kernels (use_solve_residual).
 // right-hand-side counts share a kernel choice per power-of-two bucket
 static int tune_bucket(int nrhs)
 {
@@ -811,13 +980,18 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
         return HM_OK;
     };
     double best = 1e30;
-    const int prod_c[] = {0, 8, 16, 32, RB_TC};
+    // candidates: up to 8 right-hand sides one at a time, chunks of 8 and the matrix instructions;
+    // above, those and (up to 16, or on small operators, where launches count) chunks of 16
+    const int prod_c[] = {0, 8, 16, 32};
     for (int rb : prod_c) {
         if (!do_prod) break;
-        if (rb == RB_TC ? (nrhs < TC_MIN_RHS || L.n_tcu == 0) : (rb > 8 && rb / 2 >= nrhs))
-            continue;   // a chunk of twice the RHS count or more only adds idle work; tensor tiles of 128 from 32 RHS
+        if (rb < 16 ? nrhs > 8 : rb == 16 && (nrhs <= 8 || (nrhs > 16 && L.elems > 4000000))) continue;
         double ms = 0;
-        if (rb == RB_TC && (st = ensure_tct(h)) != HM_OK) break;
+        if (rb == 32) {
+            st = ensure_mm(h, m, nrhs, false, s);
+            if (st == HM_ERR_OOM) { st = HM_OK; continue; }   // no room for the operand streams: the other kernels
+            if (st != HM_OK) break;
+        }
         if ((st = time_it([&] { launch_apply_items(h, L, x, z, nrhs, false, s, rb); }, ms)) != HM_OK) break;
         if (ms < best) { best = ms; t.prod_rb = rb; t.prod_ms = ms; }
     }
@@ -829,8 +1003,8 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     for (int rb : res_c) {
         if (st != HM_OK || !residual) break;
         if (rb == RB_OWN) {
-            if (!own_applies(h, m) || L.n_rcu == 0) continue;
-            if ((st = ensure_own(h, m)) != HM_OK) break;
+            if (!own_applies(h, m)) continue;
+            if ((st = ensure_own(h, m, false, s)) != HM_OK) break;
         } else if (rb > 8 && rb / 2 >= nr) {
             continue;
         }
@@ -852,7 +1026,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
 
 // the autotuner's (or hm_set_tuning's) kernel choices for the call, with the
 // workspace the chosen product needs
-static hm_status use_tuning(SolveCtx &c)
+static hm_status use_tuning(SolveCtx &c, bool residual)
 {
     if (c.nrhs < MRHS_MIN_RHS) return HM_OK;
     auto tn = c.h->tune.find(tune_bucket(c.nrhs));
@@ -860,7 +1034,61 @@ static hm_status use_tuning(SolveCtx &c)
         c.prod_rb = tn->second.prod_rb;
         c.res_rb = tn->second.res_rb;
     }
-    return c.prod_rb == RB_TC ? ensure_tct(c.h) : HM_OK;
+    hm_status st = HM_OK;
+    if (c.prod_rb == RB_TC) st = ensure_tct(c.h, c.s);
+    else if (c.prod_rb == 32) st = ensure_mm(c.h, c.m, c.nrhs, false, c.s);
+    if (st == HM_ERR_OOM && c.prod_rb == 32) {   // no room for the operand streams: chunks in shared memory
+        c.prod_rb = -1;
+        st = HM_OK;
+    }
+    if (st != HM_OK || !residual || c.res_rb != RB_OWN || !own_applies(c.h, c.m)) return st;
+    return ensure_own(c.h, c.m, false, c.s);
+}
+
+// the residual kernel of a refined solve on levels of small blocks that is not pinned: the matrix
+// instructions, up to 16 right-hand sides if faster than the partial-slot kernels (one right-hand
+// side at a time, chunks of 8 or 16), timed with the gather; without room for them, those
+static hm_status use_solve_residual(SolveCtx &c)
+{
+    hm_matrix h = c.h;
+    hm_matrix_s::Tune &t = h->tune[tune_bucket(c.nrhs)];
+    c.res_rb = t.solve_rb;
+    hm_status st = c.res_rb < 0 || c.res_rb == RB_MM ? ensure_mm(h, c.m, c.nrhs, true, c.s) : HM_OK;
+    if (st == HM_OK && (c.res_rb < 0 || c.res_rb == RB_MM)) st = ensure_own(h, c.m, true, c.s);
+    const bool room = st != HM_ERR_OOM;
+    if (st == HM_ERR_OOM) st = HM_OK;
+    if (st != HM_OK) return st;
+    if (c.res_rb == RB_MM && !room) c.res_rb = -1;
+    if (t.solve_rb >= 0) return HM_OK;
+    if (c.nrhs > 16) {
+        c.res_rb = t.solve_rb = room ? RB_MM : -1;
+        return HM_OK;
+    }
+    float2 *x = (float2 *)h->ws.vec32[0], *r = (float2 *)h->ws.vec32[1];
+    HM_CUDA(cudaMemsetAsync(x, 0, sizeof(float2) * h->pN * c.nrhs, c.s));
+    struct Events {
+        cudaEvent_t a = nullptr, b = nullptr;
+        ~Events() { if (a) cudaEventDestroy(a); if (b) cudaEventDestroy(b); }
+    } ev;
+    HM_CUDA(cudaEventCreate(&ev.a));
+    HM_CUDA(cudaEventCreate(&ev.b));
+    const int cand[] = {RB_MM, 0, c.nrhs <= 8 ? 8 : 16};
+    double best = 1e30;
+    for (int rb : cand) {
+        if (rb == RB_MM && !room) continue;
+        SolveCtx q = c;
+        q.res_rb = rb;
+        residual64(q, x, x, r, nullptr);                // warm-up (also sets kernel attributes)
+        HM_CUDA(cudaEventRecord(ev.a, c.s));
+        for (int i = 0; i < 3; ++i) residual64(q, x, x, r, nullptr);
+        HM_CUDA(cudaEventRecord(ev.b, c.s));
+        HM_CUDA(cudaEventSynchronize(ev.b));
+        float ms = 0.f;
+        HM_CUDA(cudaEventElapsedTime(&ms, ev.a, ev.b));
+        if (ms < best) { best = ms; t.solve_rb = rb; }
+    }
+    c.res_rb = t.solve_rb;
+    return HM_OK;
 }
 
 // permutations and vector updates of a solve, launched or recorded
@@ -949,9 +1177,13 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     const bool persist = (o->persistent || rec_out) && !c.fp64 && persist_supported(h);
     if (rec_out && !persist) return fail(HM_ERR_ARG, "the operator does not fit the one-launch solve");
     if (!c.fp64 && !persist) {
-        if ((st = autotune(h, nrhs, c.m, s, resid)) != HM_OK) return st;
-        if ((st = use_tuning(c)) != HM_OK) return st;
-        if (resid && c.res_rb == RB_OWN && own_applies(h, c.m) && (st = ensure_own(h, c.m)) != HM_OK) return st;
+        if ((st = autotune(h, nrhs, c.m, s, resid && !own_applies(h, c.m))) != HM_OK) return st;
+        if ((st = use_tuning(c, resid)) != HM_OK) return st;
+        if (resid && (st = ensure_partials(h)) != HM_OK) return st;   // the tuning may have grown the workspace
+        if (resid && nrhs >= MRHS_MIN_RHS && own_applies(h, c.m)) {
+            auto tn = h->tune.find(tune_bucket(nrhs));
+            if ((tn == h->tune.end() || !tn->second.pinned) && (st = use_solve_residual(c)) != HM_OK) return st;
+        }
     }
     if (persist) {   // the one-launch solve runs the one-right-hand-side-at-a-time block bodies
         c.prod_rb = 0;
@@ -1435,9 +1667,7 @@ hm_status hm_apply(hm_matrix h, const void *x, int64_t ldx, void *y, int64_t ldy
     if (st != HM_OK) return st;
     if (fp64_accumulate && (st = ensure_partials(h)) != HM_OK) return st;
     if ((st = autotune(h, nrhs, c.m, s, fp64_accumulate != 0)) != HM_OK) return st;
-    if ((st = use_tuning(c)) != HM_OK) return st;
-    if (fp64_accumulate && c.res_rb == RB_OWN && own_applies(h, c.m) && (st = ensure_own(h, c.m)) != HM_OK)
-        return st;
+    if ((st = use_tuning(c, fp64_accumulate != 0)) != HM_OK) return st;
     void *xt = h->ws.vec32[0], *yt = h->ws.vec32[1];
     launch_permute_in(x, ldx, xt, h->pN, h->d_pperm, nrhs, false, s);
     if (fp64_accumulate) {
@@ -1469,8 +1699,7 @@ hm_status hm_residual(hm_matrix h, const void *b, int64_t ldb, const void *x, in
     if (st != HM_OK) return st;
     if ((st = ensure_partials(h)) != HM_OK) return st;
     if ((st = autotune(h, nrhs, c.m, s, true)) != HM_OK) return st;
-    if ((st = use_tuning(c)) != HM_OK) return st;
-    if (c.res_rb == RB_OWN && own_applies(h, c.m) && (st = ensure_own(h, c.m)) != HM_OK) return st;
+    if ((st = use_tuning(c, true)) != HM_OK) return st;
     void *bt = h->ws.vec32[0], *xt = h->ws.vec32[1], *rt = h->ws.vec32[3];
     launch_permute_in(b, ldb, bt, h->pN, h->d_pperm, nrhs, false, s);
     launch_permute_in(x, ldx, xt, h->pN, h->d_pperm, nrhs, false, s);
@@ -1548,6 +1777,7 @@ hm_status hm_set_tuning(hm_matrix h, int nrhs, int prod_rb, int res_rb)
     hm_matrix_s::Tune t;
     t.prod_rb = prod_rb;
     t.res_rb = res_rb;
+    t.pinned = true;
     h->tune[tune_bucket(nrhs)] = t;
     clear_graphs(h);   // captured solves hold the previous choice
     return HM_OK;
@@ -1568,7 +1798,9 @@ hm_status hm_get_tuning(hm_matrix h, int nrhs, int *prod_rb, int *res_rb, double
     auto it = nrhs < MRHS_MIN_RHS ? h->tune.end() : h->tune.find(tune_bucket(nrhs));
     if (it == h->tune.end()) return fail(HM_ERR_STATE, "no tuned kernel choice for this right-hand-side count");
     if (prod_rb) *prod_rb = it->second.prod_rb;
-    if (res_rb) *res_rb = it->second.res_rb;
+    // a choice made for refined solves alone: the matrix-instruction form is the owner-computes one
+    const int solve_rb = it->second.solve_rb == RB_MM ? RB_OWN : it->second.solve_rb;
+    if (res_rb) *res_rb = it->second.res_rb < 0 ? solve_rb : it->second.res_rb;
     if (prod_ms) *prod_ms = it->second.prod_ms;
     if (res_ms) *res_ms = it->second.res_ms;
     return HM_OK;

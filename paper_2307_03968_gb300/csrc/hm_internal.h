@@ -32,6 +32,7 @@ constexpr int RESID_CHUNK = 16;     // right-hand sides per chunk of the FP64-cl
 constexpr int RB_TC = 1016;         // product choice: tensor-core products of the small items, RHS tiles of 128
 constexpr int TC_MIN_RHS = 32;      // the autotuner times the tensor-core product from this many RHS on
 constexpr int RB_OWN = 1017;        // residual choice: owner-computes FP64-class products (levels of small items)
+constexpr int RB_MM = 1018;         // the same on the matrix instructions (refined solves; not a choice of hm_set_tuning)
 
 // Double-float numbers of the FP64-class residual (hi + lo, |lo| a few ulps of hi at
 // most): a real one, and a complex one of 16 bytes, which is also the element of
@@ -67,12 +68,27 @@ struct LevelList {
     int64_t *d_tcr = nullptr;         // row table: W row offsets (-1 = zero row)
     int32_t *d_tcc = nullptr;         // chunk table: T chunk of each 8-row group
     int64_t n_tcb = 0, n_tcr = 0, n_tchunk = 0;   // batches, rows, T chunks per RHS tile
+    bool tc_built = false;        // the tensor-core product's lists above (made by the first call that runs it)
     // the same directed products with one unit per output cluster (the owner-computes
-    // FP64-class residual: each output row summed by one CTA in a fixed order)
+    // FP64-class residual: each output row summed by one CTA in a fixed order), made by the
+    // first call that runs it
+    bool own_built = false;
     TcProd *d_rcp = nullptr;
     TcUnit *d_rcu = nullptr;
     int64_t n_rcu = 0;
     float2 *d_rcb = nullptr;      // per product of d_rcp: its common-grid bounds (k_prod_bounds)
+    // the same directed products as two dense products on the matrix instructions (k_mm.cu,
+    // hm_lists.h build_mm_lists): product units, residual units (mm_parts a cluster at most), scales
+    // and operand streams, made by the first call that runs them
+    bool mm_built = false;
+    MmUnit *d_mm_unit = nullptr, *d_mm_unit2 = nullptr, *d_mm_runit = nullptr;
+    MmBatch *d_mm_batch = nullptr;
+    XChunk *d_mm_xch = nullptr;
+    int32_t *d_mm_ca = nullptr, *d_mm_tdst = nullptr;   // per chunk its operand tile, per stage-1 pair its T pair
+    unsigned char *d_mm_os = nullptr, *d_mm_ws = nullptr;   // output and stage-1 streams
+    int *d_mm_eout = nullptr;
+    int64_t mm_n_unit = 0, mm_n_unit2 = 0, mm_n_runit = 0, mm_n_chunk = 0, mm_n_batch = 0, mm_n_xch = 0, mm_n_tch = 0;
+    int mm_parts = 0;
     // the input clusters' K chunks of 8 unknowns (padded-tree offset, valid length):
     // the tensor-core product splits x once per launch into these chunks
     XChunk *d_xch = nullptr;
@@ -179,8 +195,10 @@ struct Workspace {
     size_t xpl_bytes = 0;
     float *d_tct = nullptr;       // stage-1 results T of the tensor-core product (TC_T_CHUNK floats per chunk and tile)
     size_t tct_bytes = 0;
-    double2 *d_own = nullptr;     // FP64 owner sums of the residual, [level][RHS][pN]
+    double2 *d_own = nullptr;     // FP64 owner sums of the residual, [level][part][RHS][pN]
     size_t own_bytes = 0;
+    void *d_mm = nullptr;         // operand tiles of the matrix-instruction products (mm_ws_bytes)
+    size_t mm_bytes = 0;
 };
 
 } // namespace hm
@@ -263,7 +281,7 @@ struct hm_matrix_s {
     unsigned *d_bar = nullptr;
 
     // kernel choices measured on this operator per right-hand-side count (hm_api.cu autotune)
-    struct Tune { int prod_rb = -1, res_rb = -1; double prod_ms = 0.0, res_ms = 0.0; };   // res_rb < 0: not tuned
+    struct Tune { int prod_rb = -1, res_rb = -1; double prod_ms = 0.0, res_ms = 0.0; bool pinned = false; int solve_rb = -1; };   // res_rb < 0: not tuned; solve_rb: a refined solve's residual
     std::map<int, Tune> tune;
 
     // estimates of the level operators U_l = D^{-1} M_l (index l - 1), made by hm_factor_leaf /
@@ -375,11 +393,29 @@ void launch_apply_items_mrhs(hm_matrix h, const LevelList &L, const float2 *x, f
 // the same for an explicit list of small items (k_mrhs.cu)
 void launch_apply_list_mrhs(hm_matrix h, const LevelList &L, const Item *items, int64_t n_items, const float2 *x,
                             float2 *z, int nrhs, int rb, cudaStream_t s);
-// owner-computes FP64-class products of a level's small items into own ([RHS][pN]) and the gather
-// out = b - (D x + sum of the m levels' owner sums) (k_resid_own.cu)
+// matrix-instruction products of a level's small items (k_mm.cu): z += M_level x (vector atomics),
+// and the owner-computes FP64-class sums into own[part][RHS][pN]; both return the kernels
+// enqueued and need a workspace of mm_ws_bytes; the scales and operand streams of a level, once
+int launch_mm_product(hm_matrix h, const LevelList &L, const float2 *x, float2 *z, int nrhs, void *ws, cudaStream_t s);
+int launch_mm_resid(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int64_t pstride, int nrhs, void *ws,
+                    cudaStream_t s);
+size_t mm_ws_bytes(const LevelList &L, int nrhs, bool res);
+// owner-computes FP64-class products of a level's small items into own ([RHS][pN]) on the FP32
+// pipes (k_resid_own.cu), and their common-grid bounds of prods[0 .. n)
 void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int nrhs, cudaStream_t s);
-// the owner-computes products' common-grid bounds of prods[0 .. n) (k_resid_own.cu)
 void launch_prod_bounds(const TcProd *prods, int64_t n, const float2 *pool, float2 *out, cudaStream_t s);
+struct MmPackArgs {
+    const MmSet *sets;
+    const MmChunk *chunks;
+    const int64_t *rows;
+    const MmPair *pairs;
+    float *wscale, *rscale;
+    int64_t n_sets, n_chunks;
+    int n_cl;
+};
+void launch_mm_pack(const LevelList &L, const MmPackArgs &M, const float2 *pool, cudaStream_t s);
+size_t mm_stream_bytes(int64_t tiles);
+// out = b - (D x + sum of the m owner-sum arrays, lstride apart) (k_resid_own.cu)
 void launch_gather_own(hm_matrix h, const float2 *x, int m, const double2 *own, int64_t lstride, const float2 *b,
                        float2 *out, double *norms, int nrhs, cudaStream_t s);
 // level-operator norm estimate (k_norm.cu): start vector (zero pads), |v|^2 into one device double

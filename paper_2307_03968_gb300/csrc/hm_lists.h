@@ -270,6 +270,181 @@ inline bool build_tc_lists(const std::map<int32_t, std::vector<TcProd>> &by_out,
     return true;
 }
 
+// The matrix-instruction products' lists (k_mm.cu): the small items of a level as two
+// dense matrix products.
+//  - Stage 1, per input cluster J: T = W X_J with the W rows (rank rows) of every low-rank
+//    directed product from J stacked, two at a time (MmPair), eight to a tile; MmBatch is
+//    a run of tiles over one input cluster.
+//  - Output, per output cluster: Z = [B_1 B_2 ... Y_1 Y_2 ...] [X; X; ... T_1; T_2; ...], K in
+//    chunks of 16 (MmChunk): chunks of the dense products over split-x chunks, then the rank
+//    rows of all low-rank products one after another (pairs, T in that order, so that no
+//    rank is padded beyond an even number of rows), MmUnit a run of chunks.
+constexpr int MM_K = 16;            // K per chunk (one matrix instruction)
+struct MmChunk {
+    int64_t src;     // kind 0: element (out 0, k 0); 1: the same (rows are K); 2: first of the chunk's 16 row offsets
+    int32_t a;       // split-x chunk (kinds 0, 1) or T chunk (2)
+    int32_t ld;      // row stride (kinds 0, 1)
+    int16_t kind;    // 0 dense, element (i, k) = src[i ld + k]; 1 dense mirrored, src[k ld + i]; 2 rank rows, pool[row[k] + i]
+    int16_t klen;    // valid K of the chunk
+    int16_t olen;    // valid outputs
+    int16_t tiles;   // tiles of 8 outputs of its cluster
+    int32_t cl;      // its output cluster
+    int32_t pos;     // its first tile in the operand stream
+};
+static_assert(sizeof(MmChunk) == 32, "MmChunk layout");
+// chunks [c0, c1) of output cluster cl, the first at tile pos of the stream; part: the unit's
+// index among the cluster's units
+struct MmUnit { int32_t out0, mlen, c0, c1, cl, part, pos; };
+struct MmPair { int64_t w; int32_t ld, dst; };   // W rows at w and w + ld (ld 0: one row; w -1: none) -> T pair dst (-1: no store)
+struct MmBatch { int32_t xg0, klen, tile0, ntiles, pos; };   // pos: first 8 x 16 tile in the stream (chunk fastest)
+struct MmSet {       // one directed product, for the scales: rank > 0: W (rank x klen) and Y (rank x olen); 0: the block at w
+    int64_t w, y;
+    int32_t w_ld, y_ld, rank, wlen, ylen;   // rank 0: y_ld = rows
+    int32_t t0, p0, cl;  // first T pair, first stage-1 pair, output cluster
+};
+struct MmLists {
+    std::vector<MmChunk> chunks;
+    std::vector<int64_t> rows;       // 16 per T chunk: pool offsets of the Y rows (-1: none)
+    std::vector<MmUnit> units, units2, runits;
+    std::vector<MmPair> pairs;       // four to a tile
+    std::vector<MmBatch> batches;
+    std::vector<XChunk> xch;
+    std::vector<MmSet> sets;
+    int64_t n_tch = 0;               // T chunks
+    int64_t n_out = 0, n_w = 0;      // 8 x 16 tiles of the output and of the stage-1 stream
+    int32_t n_cl = 0, parts = 1;     // output clusters; residual units of a cluster, at most
+};
+
+// target: work units wanted for one tile of right-hand sides (a few CTAs per SM)
+inline bool build_mm_lists(const std::map<int32_t, std::vector<TcProd>> &by_out, int64_t target, MmLists &L)
+{
+    std::map<int32_t, int32_t> in_len, in_g0;
+    for (auto &kv : by_out)
+        for (const TcProd &p : kv.second) {
+            int32_t &v = in_len[p.in0];
+            v = std::max(v, p.klen);
+        }
+    for (auto &kv : in_len) {
+        in_g0[kv.first] = (int32_t)L.xch.size();
+        for (int32_t c = 0; c < kv.second; c += MM_K) L.xch.push_back(XChunk{kv.first + c, std::min(MM_K, kv.second - c)});
+    }
+    std::map<std::pair<int32_t, int32_t>, std::vector<MmPair>> by_in;
+    std::map<std::pair<int32_t, int32_t>, std::vector<size_t>> sets_in;    // sets in the order of their pairs
+    struct C { int32_t out0, mlen, c0, c1; };
+    std::vector<C> cls;
+    for (auto &kv : by_out) {
+        C c{kv.first, 0, (int32_t)L.chunks.size(), 0};
+        const int32_t cl = (int32_t)cls.size();
+        for (const TcProd &p : kv.second) {
+            c.mlen = std::max(c.mlen, p.olen);
+            if (p.rank > 0) continue;
+            for (int32_t k = 0; k < p.klen; k += MM_K)
+                L.chunks.push_back(MmChunk{p.b_off + (p.trans ? (int64_t)k * p.b_ld : k), in_g0[p.in0] + k / MM_K, p.b_ld,
+                                           (int16_t)(p.trans ? 1 : 0), (int16_t)std::min(MM_K, p.klen - k), (int16_t)p.olen, 0, cl, 0});
+            L.sets.push_back(MmSet{p.b_off, 0, p.b_ld, p.trans ? p.klen : p.olen, 0, p.trans ? p.olen : p.klen, 0, 0, 0, cl});
+        }
+        // rank rows: pairs in product order; a chunk holds rows of one output length
+        int fill = MM_K, olen = -1;
+        std::pair<int32_t, int32_t> last{0, 0};
+        auto pad = [&] {
+            for (; fill < MM_K; fill += 2)
+                by_in[last].push_back(MmPair{-1, 0, (int32_t)((L.n_tch - 1) * (MM_K / 2) + fill / 2)});
+        };
+        for (const TcProd &p : kv.second) {
+            if (p.rank == 0) continue;
+            if (p.olen != olen) pad();
+            olen = p.olen;
+            MmSet st{p.b_off, p.y_off, p.b_ld, p.y_ld, p.rank, p.klen, p.olen, 0, 0, cl};
+            last = {p.in0, p.klen};
+            std::vector<MmPair> &in = by_in[last];
+            st.p0 = (int32_t)in.size();
+            for (int32_t l = 0; l < p.rank; l += 2) {
+                if (fill == MM_K) {
+                    L.chunks.push_back(MmChunk{(int64_t)L.rows.size(), (int32_t)L.n_tch, 0, 2, MM_K, (int16_t)p.olen, 0, cl, 0});
+                    L.rows.insert(L.rows.end(), MM_K, -1);
+                    ++L.n_tch;
+                    fill = 0;
+                }
+                const int32_t dst = (int32_t)((L.n_tch - 1) * (MM_K / 2) + fill / 2);
+                if (l == 0) st.t0 = dst;
+                in.push_back(MmPair{p.b_off + (int64_t)l * p.b_ld, l + 1 < p.rank ? p.b_ld : 0, dst});
+                int64_t *row = &L.rows[(size_t)dst * 2];
+                row[0] = p.y_off + (int64_t)l * p.y_ld;
+                if (l + 1 < p.rank) row[1] = row[0] + p.y_ld;
+                fill += 2;
+            }
+            sets_in[last].push_back(L.sets.size());
+            L.sets.push_back(st);
+        }
+        pad();
+        c.c1 = (int32_t)L.chunks.size();
+        for (int32_t q = c.c0; q < c.c1; ++q) {
+            L.chunks[q].tiles = (int16_t)((c.mlen + 7) / 8);
+            L.chunks[q].pos = (int32_t)L.n_out;
+            L.n_out += L.chunks[q].tiles;
+        }
+        if (L.n_out > INT32_MAX) return false;
+        cls.push_back(c);
+    }
+    if (L.n_tch > INT32_MAX / MM_K || L.chunks.size() > (size_t)INT32_MAX) return false;
+    L.n_cl = (int32_t)cls.size();
+    // units: enough for the SMs; the residual keeps its sums per unit ([part][RHS][pN]), so few a cluster
+    const int64_t n_ch = (int64_t)L.chunks.size();
+    // product units of at most cap chunks: fine ones, enough for the SMs with one tile of right-hand
+    // sides; coarse ones where more tiles give the CTAs, 32 chunks for each of the K groups that share
+    // a unit there (k_mm_out: 8 warps, 16 outputs a warp, two groups of right-hand sides)
+    const int64_t cap = std::min<int64_t>(256, std::max<int64_t>(8, (n_ch + target - 1) / target));
+    L.parts = (int32_t)std::min<int64_t>(8, std::max<int64_t>(1, (target + L.n_cl - 1) / std::max<int32_t>(L.n_cl, 1)));
+    for (int32_t i = 0; i < L.n_cl; ++i) {
+        const C &c = cls[i];
+        const int64_t n = c.c1 - c.c0;
+        auto cut = [&](std::vector<MmUnit> &us, int64_t np) {
+            for (int64_t q = 0; q < np; ++q)
+                us.push_back(MmUnit{c.out0, c.mlen, (int32_t)(c.c0 + n * q / np), (int32_t)(c.c0 + n * (q + 1) / np), i, (int32_t)q, 0});
+        };
+        cut(L.units, (n + cap - 1) / cap);
+        const int64_t cap2 = std::max<int64_t>(cap, 32 * (8 / (2 * ((c.mlen + 15) / 16))));
+        cut(L.units2, (n + cap2 - 1) / cap2);
+        cut(L.runits, std::max<int64_t>(1, std::min<int64_t>(L.parts, (n + 7) / 8)));
+    }
+    for (auto *us : {&L.units, &L.units2, &L.runits})
+        for (MmUnit &u : *us) u.pos = u.c0 < u.c1 ? L.chunks[u.c0].pos : 0;
+    auto longest = [](const MmUnit &a, const MmUnit &b) { return a.c1 - a.c0 > b.c1 - b.c0; };
+    std::stable_sort(L.units.begin(), L.units.end(), longest);
+    std::stable_sort(L.units2.begin(), L.units2.end(), longest);
+    std::stable_sort(L.runits.begin(), L.runits.end(), longest);
+    // stage 1: whole tiles of four pairs per input cluster, batches of at most 32 tiles
+    for (auto &kv : by_in) {
+        std::vector<MmPair> &v = kv.second;
+        const int32_t base = (int32_t)L.pairs.size();
+        for (size_t q : sets_in[kv.first]) L.sets[q].p0 += base;
+        while (v.size() & 3) v.push_back(MmPair{-1, 0, -1});
+        const int32_t t0 = base / 4, nt = (int32_t)(v.size() / 4);
+        const int32_t nch = (kv.first.second + MM_K - 1) / MM_K;
+        for (int32_t t = 0; t < nt; t += 32) {
+            L.batches.push_back(MmBatch{in_g0[kv.first.first], kv.first.second, t0 + t, std::min(32, nt - t), (int32_t)L.n_w});
+            L.n_w += (int64_t)nch * std::min(32, nt - t);
+        }
+        if (L.n_w > INT32_MAX) return false;
+        L.pairs.insert(L.pairs.end(), v.begin(), v.end());
+    }
+    // the bounds the kernels index by
+    const int64_t n_x = (int64_t)L.xch.size();
+    for (const MmChunk &c : L.chunks)
+        if (c.klen < 1 || c.klen > MM_K || c.olen < 1 || c.olen > MRHS_MAX_DIM || c.a < 0 ||
+            c.a >= (c.kind == 2 ? L.n_tch : n_x) || (c.kind == 2 && c.src + MM_K > (int64_t)L.rows.size()))
+            return false;
+    for (const MmPair &p : L.pairs)
+        if (p.dst >= L.n_tch * (MM_K / 2)) return false;
+    for (const MmBatch &b : L.batches)
+        if (b.klen < 1 || b.klen > MRHS_MAX_DIM || b.xg0 + (b.klen + MM_K - 1) / MM_K > n_x ||
+            4 * ((int64_t)b.tile0 + b.ntiles) > (int64_t)L.pairs.size())
+            return false;
+    for (const MmUnit &u : L.units)
+        if (u.mlen > MRHS_MAX_DIM || u.c0 > u.c1) return false;
+    return true;
+}
+
 // items reordered for a persistent kernel whose nw warps take items t, t + nw, ...:
 // sorted by cost, largest first, and every odd round of nw reversed (a snake), so that
 // the warps' sums match.  Cost of the product: stored bytes plus a fixed 2 KB for the

@@ -1,0 +1,935 @@
+// Block products for many right-hand sides on the matrix instructions (arxiv 2307.03968
+// eqs. 6 and 8 with the half storage of §III, blocks of up to 64 x 64 and rank 32):
+//     Z_I += B X_J, Z_J += B^T X_I;   Z_I += U (V X_J), Z_J += V^T (U^T X_I)
+// as two dense products over lists (hm_lists.h, build_mm_lists): stage 1, per input cluster,
+// T = W X_J with the rank rows of all its low-rank products stacked; then per output
+// cluster [B_1 B_2 .. Y_1 Y_2 ..] [X; X; .. T_1; T_2; ..], the ranks concatenated along K, so that
+// neither a rank nor a block is padded to an instruction's shape (only the 16 of a chunk
+// and the 8 of a cluster's outputs).
+//
+// Why mma.sync m16n8k16 with FP16 operands.  FP32 accuracy takes 3 products of 11-bit
+// halves whatever the type; FP16 has TF32's 11 bits at twice its rate (measured, registers
+// only: 606 against 302 TFLOP/s; the tcgen05 kernel of k_mrhs_tc.cu, 1952 TFLOP/s in bf16,
+// reaches 28 % of its TF32 roof on the hand-offs of its operand pipeline), and a call of 4 to
+// 64 right-hand sides fills its tiles of 16, which a tile of 128 does not.
+//
+// Operand streams.  The first call repacks the blocks (k_mm_pack_*): for each chunk of 16 K and
+// tile of 8 outputs the 128 values in the order the lanes of the instruction take them, FP32,
+// scaled, both directions of every block: twice the blocks' bytes.  A unit's blocks are then
+// one contiguous stream, copied with a few cp.async a thread, and what is left beside the
+// instructions is the split into halves or digits in registers.  (Gathered from the blocks
+// in place, by rows and by columns, the same kernels spent 500 instructions on 24 products:
+// 0.60 ms instead of 0.31 for 16 right-hand sides of the 12,600-unknown cube.)
+//
+// Measured (GB300): a product of the 30,720-unknown sphere with 181 right-hand sides 6.0 ms, of
+// which stage 1 1.6 (the tcgen05 kernels: 7.3); 16 right-hand sides of the 12,600-unknown
+// cube 0.34 ms (SIMT chunks of 16: 0.66); the FP64-class residual of those 24 ms (SIMT
+// owner kernel: 68) and 1.2 ms (2.3).
+//
+// Right-hand sides are the instruction's M, so an accumulator pair of stage 1 is, in place,
+// an operand pair of the output stage (its K are the W rows): T is stored in operand layout.
+// Operand tile of 16 right-hand sides x 16 K: one plane per half (product: re hi, re lo, im
+// hi, im lo; residual: re 1..4, im 1..4), each 4 registers x 32 words; word t * 8 + g of
+// register r is the pair of K 2t, 2t + 1 (+ 8 for r >= 2) of right-hand side g (+ 8 for odd r):
+// what lane (g, t) holds, and 32 bytes per t, so that stage 1 writes whole sectors.
+//
+// Scales (powers of two, exact).  FP16 has 5 exponent bits, so every operand is brought to
+// at most 1: x by 2^ex per right-hand side (k_mm_max), W row l by 2^et(l), |T_l| <= |W_l|_1 |x|_inf
+// <= 1 with it, and Y row l (dense blocks: the block) by 2^(E - et(l)), E per output cluster the
+// largest that keeps all its terms at most 1 (k_mm_prep, once per operator).  Sums of one
+// output then share the factor 2^(ex + E).
+//
+// Product: a = hi + lo, hi = fp16(2^15 a), lo = fp16(2^15 a - hi): 22 bits for a >= 2^-17, an
+// absolute 2^-40 below; hi hi + hi lo + lo hi.  The tensor core truncates its FP32 sums, so each
+// chunk's six products start from zero and are added to the running sum in FP32 outside.
+//
+// FP64-class residual: a = 2^-8 d1 + 2^-17 d2 + 2^-26 d3 + 2^-35 r, the digits integers of at most
+// 2^8, r a FP16 of at most 2^8: 38 bits below the scale, exact for every FP32 a >= 2^-14 (integer
+// digits on a common grid follow Ozaki, Ogita, Oishi & Rump 2012).  Thirteen products:
+//     H0 = d1 e1;  H1 = d1 e2 + d2 e1;  H2 = d1 e3 + d2 e2 + d3 e1;
+//     A = d1 s + d2 e3 + d3 e2 + r e1;  C = d2 s + d3 e3 + r e2
+// of weights 2^-16, 2^-25, 2^-34, 2^-43, 2^-52 (the dropped ones are below 2^-44).  H0, H1, H2
+// are sums of integers of at most 2^16, exact in the tensor core's truncating FP32 sums up to
+// 64 K per accumulation (256 real products a pair): every 4 chunks they join a double-float
+// sum.  With the digits past d2 left as floats (two FP16 of 22 bits, also 13 products), the
+// truncation of d1 s cost 2^-38 of sum |a b| instead of being exact.
+#include "k_dot2.cuh"
+
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+namespace hm {
+namespace {
+
+using namespace kc;
+using namespace dot2;
+
+constexpr int MMW = 8;                    // warps per CTA
+constexpr int MM_PLANE = 128;             // words of one plane of an operand tile
+template <bool RES> constexpr int planes() { return RES ? 8 : 4; }
+template <bool RES> constexpr int tile_words() { return planes<RES>() * MM_PLANE; }
+constexpr int MM_PASS_MIN = 64;           // right-hand sides per pass, at least (mm_pass)
+constexpr size_t MM_PASS_BYTES = size_t(4) << 30;   // operand tiles of a pass, above that many
+constexpr int MM_DRAIN = 4;               // residual: chunks per exact accumulation
+constexpr float MM_TOP = 32768.f;         // product: operands are scaled to at most 2^15
+
+__device__ __forceinline__ void mma16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+__device__ __forceinline__ uint32_t h2(float a, float b)
+{
+    const __half2 v = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+__device__ __forceinline__ float2 f2(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2 *>(&v)); }
+
+// the planes of a pair of normalised values (product: already times 2^15)
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[2])
+{
+    p[0] = h2(a, b);
+    const float2 h = f2(p[0]);
+    p[1] = h2(__fsub_rn(a, h.x), __fsub_rn(b, h.y));
+}
+// the nearest integer of |v| < 2^22 (ties to even)
+__device__ __forceinline__ float nearest(float v) { return __fsub_rn(__fadd_rn(v, 12582912.f), 12582912.f); }
+// digits of v + lo, |v| <= 1, lo below v's last bits: d1, d2, d3 and the rest r
+__device__ __forceinline__ void digits(float v, float lo, float &d1, float &d2, float &d3, float &r)
+{
+    const float t = v * 256.f;
+    d1 = nearest(t);
+    const float q = __fsub_rn(t, d1) * 512.f, l = lo * 131072.f;
+    d2 = nearest(__fadd_rn(q, l));
+    const float w = __fadd_rn(__fsub_rn(q, d2), l) * 512.f;
+    d3 = nearest(w);
+    r = __fsub_rn(w, d3) * 512.f;
+}
+__device__ __forceinline__ void split_pair(float a, float al, float b, float bl, uint32_t (&p)[4])
+{
+    float a1, a2, a3, ar, b1, b2, b3, br;
+    digits(a, al, a1, a2, a3, ar);
+    digits(b, bl, b1, b2, b3, br);
+    p[0] = h2(a1, b1);
+    p[1] = h2(a2, b2);
+    p[2] = h2(a3, b3);
+    p[3] = h2(ar, br);
+}
+
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
+// the least e with v <= 2^e (0 for 0 and for values that are not finite), within +-120
+__device__ __forceinline__ int ceil_exp(float v)
+{
+    if (!(v > 0.f) || !isfinite(v)) return 0;
+    int e;
+    const float f = frexpf(v, &e);
+    if (f == 0.5f) --e;
+    return min(max(e, -120), 120);
+}
+
+// ---- x: scale per right-hand side, operand tiles --------------------------------
+
+// xs[2 r] = 2^ex, xs[2 r + 1] = 2^-ex with 2^ex |x_r|_inf <= 1; one CTA per right-hand side
+// (245 KB of x at 30,720 unknowns: a few us beside products of milliseconds)
+__global__ void __launch_bounds__(1024)
+k_mm_max(const float2 *__restrict__ x, int64_t pN, float *__restrict__ xs)
+{
+    __shared__ float sm[32];
+    const float4 *v = reinterpret_cast<const float4 *>(x + blockIdx.x * pN);   // pN is even
+    float m = 0.f;
+    for (int64_t i = threadIdx.x; i < pN / 2; i += 1024) {
+        const float4 a = v[i];
+        m = fmaxf(fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
+    }
+    m = warp_max(m);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = warp_max(sm[threadIdx.x]);
+        if (threadIdx.x == 0) {
+            const int e = ceil_exp(m);
+            xs[2 * blockIdx.x] = pow2f(-e);
+            xs[2 * blockIdx.x + 1] = pow2f(e);
+        }
+    }
+}
+
+// operand tiles of x: chunk of 16 unknowns (a warp each) x tile of 16 right-hand sides (blockIdx.y)
+template <bool RES>
+__global__ void __launch_bounds__(128)
+k_mm_split(const XChunk *__restrict__ xch, int n_xch, const float2 *__restrict__ x, int64_t pN, int nrhs,
+           const float *__restrict__ xs, uint32_t *__restrict__ xt)
+{
+    const int ch = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    if (ch >= n_xch) return;
+    const XChunk c = xch[ch];
+    uint32_t *w = xt + ((int64_t)blockIdx.y * n_xch + ch) * tile_words<RES>() + t * 8 + g;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int q = blockIdx.y * 16 + g + 8 * (r & 1), k = 2 * t + 8 * (r >> 1);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q < nrhs && k < c.len) {
+            v = *reinterpret_cast<const float4 *>(x + q * pN + c.off + k);
+            if (k + 1 >= c.len) v.z = v.w = 0.f;
+            const float s = xs[2 * q];
+            v.x *= s; v.y *= s; v.z *= s; v.w *= s;
+        }
+        if constexpr (RES) {
+            uint32_t re[4], im[4];
+            split_pair(v.x, 0.f, v.z, 0.f, re);
+            split_pair(v.y, 0.f, v.w, 0.f, im);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                w[p * MM_PLANE + r * 32] = re[p];
+                w[(4 + p) * MM_PLANE + r * 32] = im[p];
+            }
+        } else {
+            uint32_t re[2], im[2];
+            split_pair(v.x * MM_TOP, v.z * MM_TOP, re);
+            split_pair(v.y * MM_TOP, v.w * MM_TOP, im);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                w[p * MM_PLANE + r * 32] = re[p];
+                w[(2 + p) * MM_PLANE + r * 32] = im[p];
+            }
+        }
+    }
+}
+
+// ---- operands of the blocks -------------------------------------------------------
+
+// the B operands of one chunk and 8 outputs from the lane's four complex values (K 2t, 2t + 1,
+// 2t + 8, 2t + 9 of output g, times 2^15): planes [half or digit][register]
+template <bool RES> struct BFrag { uint32_t re[planes<RES>() / 2][2], im[planes<RES>() / 2][2]; };
+
+// tile: an 8 x 16 tile of an operand stream in shared memory, two planes of 16 bytes a lane
+template <bool RES>
+__device__ __forceinline__ void make_b(const unsigned char *tile, int lane, BFrag<RES> &b)
+{
+    constexpr int H = planes<RES>() / 2;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float4 v = *reinterpret_cast<const float4 *>(tile + q * 512 + lane * 16);
+        uint32_t re[H], im[H];
+        if constexpr (RES) {
+            split_pair(v.x * (1.f / MM_TOP), 0.f, v.z * (1.f / MM_TOP), 0.f, re);
+            split_pair(v.y * (1.f / MM_TOP), 0.f, v.w * (1.f / MM_TOP), 0.f, im);
+        } else {
+            split_pair(v.x, v.z, re);
+            split_pair(v.y, v.w, im);
+        }
+#pragma unroll
+        for (int p = 0; p < H; ++p) {
+            b.re[p][q] = re[p];
+            b.im[p][q] = im[p];
+        }
+    }
+}
+constexpr int MM_TILE = 1024;             // bytes of an 8 x 16 tile of a stream
+
+__device__ __forceinline__ void negate(uint32_t (&n)[2], const uint32_t (&b)[2])
+{
+    n[0] = b[0] ^ 0x80008000u;
+    n[1] = b[1] ^ 0x80008000u;
+}
+
+// plane p of an operand tile in shared memory (`tile`: the lane's word)
+__device__ __forceinline__ void load_plane(uint32_t (&a)[4], const uint32_t *tile, int p)
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a[r] = tile[p * MM_PLANE + r * 32];
+}
+
+// sums of one tile of 16 right-hand sides x 8 outputs
+template <bool RES> struct Acc;
+template <> struct Acc<false> {
+    float s[2][4], c[2][4];     // re, im: the running sums, and what the tensor core holds since the last drain
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[0][i] = s[1][i] = c[0][i] = c[1][i] = 0.f;
+    }
+    __device__ __forceinline__ void drain()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s[0][i] += c[0][i];
+            s[1][i] += c[1][i];
+            c[0][i] = c[1][i] = 0.f;
+        }
+    }
+};
+// one chunk into N tiles of 8 outputs (the products of the N tiles interleaved: a tile alone is
+// two chains of dependent instructions): A operand planes at `tile` (the lane's word), B operands b
+template <int N>
+__device__ __forceinline__ void mm_chunk(Acc<false> (&s)[N], const uint32_t *tile, const BFrag<false> (&b)[N])
+{
+    uint32_t xr[4], xi[4];
+    auto terms = [&](int q) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            mma16(s[n].c[0], xr, b[n].re[q]);
+            mma16(s[n].c[1], xr, b[n].im[q]);
+        }
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            uint32_t m[2];
+            negate(m, b[n].im[q]);
+            mma16(s[n].c[0], xi, m);
+            mma16(s[n].c[1], xi, b[n].re[q]);
+        }
+    };
+    // the small products first: only the last two instructions truncate at the sum's own size
+    load_plane(xr, tile, 1);
+    load_plane(xi, tile, 3);
+    terms(0);
+    load_plane(xr, tile, 0);
+    load_plane(xi, tile, 2);
+    terms(1);
+    terms(0);
+}
+template <> struct Acc<true> {
+    float h0[2][4], h1[2][4], h2[2][4], a[2][4], c[2][4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h0[p][i] = h1[p][i] = h2[p][i] = a[p][i] = c[p][i] = 0.f;
+    }
+    // one digit of x (xr, xi) times digits 0 .. Q - 1 of the block into d[0 .. Q - 1]
+    template <int Q>
+    __device__ __forceinline__ static void terms(float (*const (&d)[Q])[4], const uint32_t (&xr)[4], const uint32_t (&xi)[4],
+                                                 const BFrag<true> &f)
+    {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            mma16(d[q][0], xr, f.re[q]);
+            mma16(d[q][1], xr, f.im[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            uint32_t n[2];
+            negate(n, f.im[q]);
+            mma16(d[q][0], xi, n);
+            mma16(d[q][1], xi, f.re[q]);
+        }
+    }
+    __device__ __forceinline__ void chunk(const uint32_t *tile, const BFrag<true> &f)
+    {
+        uint32_t xr[4], xi[4];
+        load_plane(xr, tile, 0);
+        load_plane(xi, tile, 4);
+        terms<4>({h0, h1, h2, a}, xr, xi, f);
+        load_plane(xr, tile, 1);
+        load_plane(xi, tile, 5);
+        terms<4>({h1, h2, a, c}, xr, xi, f);
+        load_plane(xr, tile, 2);
+        load_plane(xi, tile, 6);
+        terms<3>({h2, a, c}, xr, xi, f);
+        load_plane(xr, tile, 3);
+        load_plane(xi, tile, 7);
+        terms<2>({a, c}, xr, xi, f);
+    }
+    // value (p, i) of the accumulations, in units of 2^-16, as hi + lo
+    __device__ __forceinline__ void value(int p, int i, float &hi, float &lo) const
+    {
+        float s, e, e2;
+        two_sum(h0[p][i], h1[p][i] * 0x1p-9f, s, e);
+        two_sum(s, h2[p][i] * 0x1p-18f, hi, e2);
+        lo = __fadd_rn(__fmaf_rn(c[p][i], 0x1p-36f, a[p][i] * 0x1p-27f), __fadd_rn(e, e2));
+    }
+};
+
+// ---- copies ------------------------------------------------------------------------
+
+__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// waits until at most N of this thread's latest groups are in flight
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// ---- stage 1: T = W X --------------------------------------------------------------
+
+template <bool RES, int MT> constexpr int s1_smem() { return 4 * MT * tile_words<RES>() * 4 + MMW * 2 * 4 * MM_TILE; }
+
+// One batch of W row tiles over an input cluster (blockIdx.x / groups) and MT tiles of 16
+// right-hand sides (blockIdx.x % groups: the CTAs that read the same blocks run together, from L2): the cluster's x tiles are copied to shared memory once, each warp takes
+// every 8th tile of 8 rows, the next one in flight while one is multiplied.
+template <bool RES, int MT>
+__global__ void __launch_bounds__(MMW * 32, 2)
+k_mm_stage1(const MmBatch *__restrict__ batches, const int32_t *__restrict__ tdst, const unsigned char *__restrict__ ws,
+            const uint32_t *__restrict__ xt, int n_xch, uint32_t *__restrict__ tt, int64_t n_tch, int n_tiles, int groups)
+{
+    extern __shared__ __align__(128) unsigned char sm1[];
+    constexpr int TW = tile_words<RES>();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const MmBatch B = batches[blockIdx.x / groups];
+    const int nch = (B.klen + MM_K - 1) / MM_K;
+    const int m0 = blockIdx.x % groups * MT;
+    uint32_t *xs = reinterpret_cast<uint32_t *>(sm1);
+    unsigned char *wr = sm1 + 4 * MT * TW * 4 + w * 8 * MM_TILE;
+    auto fetch = [&](int it, int h) {
+        const unsigned char *src = ws + ((int64_t)B.pos + (int64_t)it * nch) * MM_TILE + lane * 16;
+        const uint32_t d = su32(wr + h * 4 * MM_TILE + lane * 16);
+        for (int c = 0; c < 2 * nch; ++c) cp16(d + c * 512, src + c * 512);
+    };
+    for (int i = threadIdx.x; i < nch * MT * (TW / 4); i += MMW * 32) {
+        const int c = i / (MT * (TW / 4)), m = i / (TW / 4) % MT, o = i % (TW / 4);
+        if (m0 + m < n_tiles)
+            cp16(su32(xs + (c * MT + m) * TW + 4 * o), xt + ((int64_t)(m0 + m) * n_xch + B.xg0 + c) * TW + 4 * o);
+    }
+    if (w < B.ntiles) fetch(w, 0);
+    cp_commit();
+    cp_wait<0>();
+    __syncthreads();
+    const uint32_t *xw = xs + t * 8 + g;
+    int h = 0;
+    for (int it = w; it < B.ntiles; it += MMW, h ^= 1) {
+        const int dst = tdst[4 * (B.tile0 + it) + t];
+        __syncwarp();                              // every lane is done with the half the next copy fills
+        if (it + MMW < B.ntiles) fetch(it + MMW, h ^ 1);
+        cp_commit();
+        cp_wait<1>();
+        __syncwarp();                              // the warp's copies of this tile have landed
+        Acc<RES> acc[MT][1];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) acc[m][0].zero();
+        for (int c = 0; c < nch; ++c) {
+            BFrag<RES> f[1];
+            make_b<RES>(wr + (4 * h + c) * MM_TILE, lane, f[0]);
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                if constexpr (RES) {
+                    acc[m][0].chunk(xw + (c * MT + m) * TW, f[0]);
+                } else {
+                    mm_chunk<1>(acc[m], xw + (c * MT + m) * TW, f);
+                    acc[m][0].drain();
+                }
+            }
+        }
+        if (dst < 0) continue;
+        // accumulators 0, 1 (right-hand side g) and 2, 3 (g + 8) are the K pair dst of T
+        const int pr = dst & 7;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            if (m0 + m >= n_tiles) break;
+            uint32_t *o = tt + ((int64_t)(m0 + m) * n_tch + (dst >> 3)) * TW + (pr >> 2) * 64 + (pr & 3) * 8 + g;
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {   // re, im
+                    if constexpr (RES) {
+                        float a, al, b, bl;
+                        acc[m][0].value(c, 2 * q, a, al);
+                        acc[m][0].value(c, 2 * q + 1, b, bl);
+                        uint32_t p[4];
+                        split_pair(a * 0x1p-16f, al * 0x1p-16f, b * 0x1p-16f, bl * 0x1p-16f, p);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) __stcs(o + (4 * c + j) * MM_PLANE + q * 32, p[j]);
+                    } else {
+                        uint32_t p[2];
+                        split_pair(acc[m][0].s[c][2 * q] * (1.f / MM_TOP), acc[m][0].s[c][2 * q + 1] * (1.f / MM_TOP), p);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) __stcs(o + (2 * c + j) * MM_PLANE + q * 32, p[j]);
+                    }
+                }
+        }
+    }
+}
+
+// ---- output stage ------------------------------------------------------------------
+
+struct MmOutArgs {
+    const MmUnit *units;
+    const int32_t *ca;       // per chunk: its split-x chunk, or -1 - its T chunk
+    const int *eout;         // per output cluster: E
+    const unsigned char *os; // operand stream
+    const uint32_t *xt, *tt;
+    int n_xch, n_tiles, nrhs;
+    int64_t n_tch;
+    const float *xs;
+    int groups;              // CTAs of a unit, over the right-hand sides
+};
+
+// The copies of a K group: T threads that work on the same chunks, each chunk's stream tiles and
+// the operand tiles of `mtiles` tiles of right-hand sides in one of the stages of the group's
+// shared memory.  The operand tile index of the next chunk is loaded one chunk ahead.
+template <bool RES> struct Pipe {
+    static constexpr int NB = RES ? 2 : 4;        // 16-byte pieces of a chunk's stream per thread, at most
+    static constexpr int TW = tile_words<RES>();
+    uint32_t base;
+    const unsigned char *smem, *src;               // src: the thread's piece of the chunk to copy next
+    int gt, T, tiles, mtiles, m0, n_tiles, stages, bsz, ssz, a, step;
+    __device__ __forceinline__ void init(const MmOutArgs &A, const MmUnit &U, unsigned char *region, int bytes, int gt_, int T_,
+                                         int room, int mt, int m0_, int kw, int ks)
+    {
+        base = su32(region);
+        smem = region;
+        gt = gt_; T = T_; mtiles = mt; m0 = m0_; n_tiles = A.n_tiles;
+        tiles = (U.mlen + 7) / 8;
+        bsz = room * MM_TILE;
+        ssz = bsz + mtiles * TW * 4;
+        stages = min(6, bytes / ssz);
+        step = ks * tiles * MM_TILE;
+        src = A.os + ((int64_t)U.pos + kw * tiles) * MM_TILE + gt * 16;
+    }
+    __device__ __forceinline__ void copy(const MmOutArgs &A, int stage)
+    {
+        const uint32_t st = base + stage * ssz;
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+            if (gt + T * j < tiles * (MM_TILE / 16)) cp16(st + (gt + T * j) * 16, src + T * j * 16);
+        src += step;
+        const uint32_t *tl = a < 0 ? A.tt + (int64_t)(-1 - a) * TW : A.xt + (int64_t)a * TW;
+        const int64_t stride = (a < 0 ? A.n_tch : A.n_xch) * TW;
+        for (int q = gt; q < mtiles * (TW / 4); q += T) {
+            const int m = q / (TW / 4), o = q % (TW / 4);
+            if (m0 + m < n_tiles) cp16(st + bsz + q * 16, tl + (m0 + m) * stride + 4 * o);
+        }
+    }
+    __device__ __forceinline__ const uint32_t *tile(int stage, int m) const
+    {
+        return reinterpret_cast<const uint32_t *>(smem + stage * ssz + bsz) + m * TW;
+    }
+    __device__ __forceinline__ const unsigned char *values(int stage, int n) const { return smem + stage * ssz + n * MM_TILE; }
+    // the pipeline over chunks c0, c0 + ks, ... < c1: body(stage) for each; the group's threads meet at
+    // the named barrier `bar` once a chunk
+    template <class Body>
+    __device__ __forceinline__ void run(const MmOutArgs &A, int c0, int c1, int ks, int bar, Body body)
+    {
+        if (stages >= 5) run_stages<5>(A, c0, c1, ks, bar, body);
+        else if (stages >= 3) run_stages<3>(A, c0, c1, ks, bar, body);
+        else run_stages<2>(A, c0, c1, ks, bar, body);
+    }
+    template <int S, class Body>
+    __device__ __forceinline__ void run_stages(const MmOutArgs &A, int c0, int c1, int ks, int bar, Body body)
+    {
+        const int n = c0 < c1 ? (c1 - c0 + ks - 1) / ks : 0;
+        const int32_t *ca = A.ca + c0;
+        if (n > 0) a = *ca;
+#pragma unroll
+        for (int q = 0; q < S - 1; ++q) {
+            if (q < n) copy(A, q);
+            cp_commit();
+            ca += ks;
+            if (q + 1 < n) a = *ca;
+        }
+        int st = 0, nx = S - 1;                    // the stage of chunk q, and of chunk q + S - 1
+        for (int q = 0; q < n; ++q) {
+            cp_wait<S - 2>();
+            asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
+            if (q + S - 1 < n) copy(A, nx);
+            cp_commit();
+            ca += ks;
+            if (q + S < n) a = *ca;
+            body(st);
+            st = st + 1 == S ? 0 : st + 1;
+            nx = nx + 1 == S ? 0 : nx + 1;
+        }
+        cp_wait<0>();
+    }
+};
+
+constexpr int MM_SMEM = 112 * 1024;               // two CTAs an SM
+
+// Product: one unit (blockIdx.x / groups) for MT x mw tiles of 16 right-hand sides.  The 8
+// warps: 16 outputs each (the fastest index), mw groups of MT right-hand-side tiles, and what
+// is left of them along K; every warp adds its sums into z (vector atomics).
+// `drain`: chunks the tensor core adds up before their sum leaves it.
+template <int MT>
+__global__ void __launch_bounds__(MMW * 32, 2)
+k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
+{
+    extern __shared__ __align__(128) unsigned char smo[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const MmUnit U = p.units[blockIdx.x / p.groups];
+    const int nt = (U.mlen + 15) / 16, gw = nt * mw, ks = MMW / gw, kw = w / gw, wi = w - kw * gw;
+    if (kw >= ks) return;
+    const int n0 = 16 * (wi % nt), mi = (wi / nt) * MT, mb = (int)(blockIdx.x % p.groups) * mw * MT, m0 = mb + mi;
+    const int E = p.eout[U.cl];
+    Acc<false> acc[MT][2];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) { acc[m][0].zero(); acc[m][1].zero(); }
+    Pipe<false> P;
+    const int region = MM_SMEM / ks / 128 * 128;
+    P.init(p, U, smo + kw * region, region, wi * 32 + lane, gw * 32, 2 * nt, MT * mw, mb, kw, ks);
+    int held = 0;
+    P.run(p, U.c0 + kw, U.c1, ks, 1 + kw, [&](int st) {
+        BFrag<false> f[2];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) make_b<false>(P.values(st, n0 / 8 + n), lane, f[n]);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            if (m0 + m >= p.n_tiles) break;
+            const uint32_t *tile = P.tile(st, mi + m) + t * 8 + g;
+            mm_chunk<2>(acc[m], tile, f);
+        }
+        if (++held == drain) {
+            held = 0;
+#pragma unroll
+            for (int m = 0; m < MT; ++m) { acc[m][0].drain(); acc[m][1].drain(); }
+        }
+    });
+    const float ci = pow2f(-E) * (1.f / (MM_TOP * MM_TOP));
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = 16 * (m0 + m) + g + 8 * h;
+            if (r >= p.nrhs) continue;
+            const float xi = p.xs[2 * r + 1];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                if (h == 0) acc[m][n].drain();
+                const int i = n0 + 8 * n + 2 * t;
+                const float2 a = make_float2(acc[m][n].s[0][2 * h] * ci * xi, acc[m][n].s[1][2 * h] * ci * xi);
+                const float2 b = make_float2(acc[m][n].s[0][2 * h + 1] * ci * xi, acc[m][n].s[1][2 * h + 1] * ci * xi);
+                float2 *zz = z + (int64_t)r * pN + U.out0 + i;
+                if (i + 1 < U.mlen) red2(zz, a, b);
+                else if (i < U.mlen) red1(zz, a);
+            }
+        }
+}
+
+// FP64-class residual products: one unit (blockIdx.x / groups) for a tile of 16 right-hand
+// sides.  The 8 warps: 8 outputs each, the rest along K; the K groups' double-float
+// sums are added in a fixed order, the unit's sums stored once in FP64: no atomics, the
+// result does not depend on scheduling.
+__global__ void __launch_bounds__(MMW * 32, 2)
+k_mm_resid(MmOutArgs p, double2 *__restrict__ own, int64_t pstride, int64_t pN)
+{
+    extern __shared__ __align__(128) unsigned char smo[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const MmUnit U = p.units[blockIdx.x / p.groups];
+    const int nt = (U.mlen + 7) / 8, ks = MMW / nt, kw = w / nt, wi = w - kw * nt, m0 = (int)(blockIdx.x % p.groups);
+    const int n0 = 8 * wi;
+    const int E = p.eout[U.cl];
+    float hi[8], lo[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) hi[i] = lo[i] = 0.f;
+    if (kw < ks) {
+        Acc<true> acc;
+        acc.zero();
+        auto drain = [&] {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float vh, vl, s, e;
+                acc.value(i >> 2, i & 3, vh, vl);
+                two_sum(hi[i], vh, s, e);
+                hi[i] = s;
+                lo[i] = __fadd_rn(lo[i], __fadd_rn(e, vl));
+            }
+            acc.zero();
+        };
+        Pipe<true> P;
+        const int region = MM_SMEM / ks / 128 * 128;
+        P.init(p, U, smo + kw * region, region, wi * 32 + lane, nt * 32, nt, 1, m0, kw, ks);
+        int held = 0;
+        P.run(p, U.c0 + kw, U.c1, ks, 1 + kw, [&](int st) {
+            BFrag<true> f;
+            make_b<true>(P.values(st, wi), lane, f);
+            acc.chunk(P.tile(st, 0) + t * 8 + g, f);
+            if (++held == MM_DRAIN) {
+                held = 0;
+                drain();
+            }
+        });
+        if (held) drain();
+    }
+    if (ks > 1) {
+        float(*sm)[16][32] = reinterpret_cast<float(*)[16][32]>(smo);
+        __syncthreads();                            // every group is done with its stages
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            sm[w][2 * i][lane] = hi[i];
+            sm[w][2 * i + 1][lane] = lo[i];
+        }
+        __syncthreads();
+        if (kw == 0)
+            for (int q = 1; q < ks; ++q)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const df v = df_add(df{hi[i], lo[i]}, df{sm[w + q * nt][2 * i][lane], sm[w + q * nt][2 * i + 1][lane]});
+                    hi[i] = v.hi;
+                    lo[i] = v.lo;
+                }
+    }
+    if (kw != 0) return;
+    const double cs = ldexp(1.0, -16 - E);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = 16 * m0 + g + 8 * h;
+        if (r >= p.nrhs) continue;
+        const double sc = cs * (double)p.xs[2 * r + 1];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int i = n0 + 2 * t + j, a = 2 * h + j;
+            if (i < U.mlen)
+                own[(int64_t)U.part * pstride + (int64_t)r * pN + U.out0 + i] =
+                    make_double2(sc * ((double)hi[a] + (double)lo[a]), sc * ((double)hi[4 + a] + (double)lo[4 + a]));
+        }
+    }
+}
+
+// ---- scales, once per operator -------------------------------------------------------
+
+// Per directed product (a warp each): low-rank, et of every W row from its 1-norm (FP32, rounded
+// up) into wscale and, negated, into rscale, and E's bound et - exponent(max Y row); dense,
+// E's bound from the block's largest component.
+__global__ void __launch_bounds__(256)
+k_mm_prep(const MmSet *__restrict__ sets, int64_t n, const float2 *__restrict__ pool, float *__restrict__ wscale,
+          float *__restrict__ rscale, int *__restrict__ eout)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < n; q += nw) {
+        const MmSet S = sets[q];
+        int bound = 1000;
+        if (S.rank == 0) {
+            float m = 0.f;
+            for (int i = 0; i < S.y_ld; ++i)
+                for (int j = lane; j < S.wlen; j += 32) m = fmaxf(m, linf(pool[S.w + (int64_t)i * S.w_ld + j]));
+            m = warp_max(m);
+            if (m > 0.f) bound = -ceil_exp(m);
+        }
+        for (int l = 0; l < S.rank; ++l) {
+            float a = 0.f, m = 0.f;
+            for (int j = lane; j < S.wlen; j += 32) {
+                const float2 v = pool[S.w + (int64_t)l * S.w_ld + j];
+                a = __fadd_ru(a, __fadd_ru(fabsf(v.x), fabsf(v.y)));
+            }
+            for (int i = lane; i < S.ylen; i += 32) m = fmaxf(m, linf(pool[S.y + (int64_t)l * S.y_ld + i]));
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1) a = __fadd_ru(a, __shfl_xor_sync(FULL, a, s));
+            m = warp_max(m);
+            const int et = min(-ceil_exp(a), 100);
+            if (lane == 0) {
+                wscale[2 * (int64_t)S.p0 + l] = pow2f(et);
+                rscale[2 * (int64_t)S.t0 + l] = pow2f(-et);
+            }
+            if (m > 0.f) bound = min(bound, et - ceil_exp(m));
+        }
+        if (lane == 0 && bound < 1000) atomicMin(eout + S.cl, min(max(bound, -120), 100));
+    }
+}
+// rscale = 2^(E - et) of every T row; clusters with nothing but zeros get E = 0
+__global__ void __launch_bounds__(256)
+k_mm_rscale(const MmSet *__restrict__ sets, int64_t n, float *__restrict__ rscale, const int *__restrict__ eout)
+{
+    for (int64_t q = blockIdx.x * 256ll + threadIdx.x; q < n; q += gridDim.x * 256ll) {
+        const MmSet S = sets[q];
+        for (int l = 0; l < S.rank; ++l) {
+            float &v = rscale[2 * (int64_t)S.t0 + l];
+            v = pow2f(min(eout[S.cl] + ((__float_as_int(v) >> 23) - 127), 110));
+        }
+    }
+}
+__global__ void k_mm_eout(int *eout, int n, int set)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < n && (set || eout[i] == 1000)) eout[i] = set ? 1000 : 0;
+}
+
+// ---- operand streams, once per operator ---------------------------------------------
+
+__device__ __forceinline__ void pack_tile(float4 *dst, const float2 (&v)[4], const float (&s)[4], int lane)
+{
+    dst[lane] = make_float4(v[0].x * s[0] * MM_TOP, v[0].y * s[0] * MM_TOP, v[1].x * s[1] * MM_TOP, v[1].y * s[1] * MM_TOP);
+    dst[32 + lane] = make_float4(v[2].x * s[2] * MM_TOP, v[2].y * s[2] * MM_TOP, v[3].x * s[3] * MM_TOP, v[3].y * s[3] * MM_TOP);
+}
+
+// the output stream, a warp per chunk
+__global__ void __launch_bounds__(256)
+k_mm_pack_out(const MmChunk *__restrict__ chunks, int64_t n, const int64_t *__restrict__ rows, const float *__restrict__ rscale,
+              const int *__restrict__ eout, const float2 *__restrict__ pool, unsigned char *__restrict__ os,
+              int32_t *__restrict__ ca)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    for (int64_t c = blockIdx.x * 8ll + (threadIdx.x >> 5); c < n; c += gridDim.x * 8ll) {
+        const MmChunk C = chunks[c];
+        if (lane == 0) ca[c] = C.kind == 2 ? -1 - C.a : C.a;
+        int64_t off[4];
+        float s[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int k = 2 * t + (q & 1) + 8 * (q >> 1);
+            off[q] = C.kind == 2 ? rows[C.src + k] : k < C.klen ? C.src + (C.kind == 0 ? k : (int64_t)k * C.ld) : -1;
+            s[q] = C.kind == 2 ? rscale[C.src + k] : pow2f(eout[C.cl]);
+        }
+        for (int tl = 0; tl < C.tiles; ++tl) {
+            const int i = 8 * tl + g;
+            float2 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[q] = off[q] >= 0 && i < C.olen ? pool[off[q] + (C.kind == 0 ? (int64_t)i * C.ld : i)] : make_float2(0.f, 0.f);
+            pack_tile(reinterpret_cast<float4 *>(os + ((int64_t)C.pos + tl) * MM_TILE), v, s, lane);
+        }
+    }
+}
+
+// the stage-1 stream, a CTA per batch, a warp per tile of 8 W rows
+__global__ void __launch_bounds__(256)
+k_mm_pack_w(const MmBatch *__restrict__ batches, const MmPair *__restrict__ pairs, const float *__restrict__ wscale,
+            const float2 *__restrict__ pool, unsigned char *__restrict__ ws, int32_t *__restrict__ tdst)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const MmBatch B = batches[blockIdx.x];
+    const int nch = (B.klen + MM_K - 1) / MM_K;
+    for (int it = threadIdx.x >> 5; it < B.ntiles; it += 8) {
+        const int tile = B.tile0 + it;
+        const MmPair P = pairs[4 * tile + (g >> 1)];
+        const int64_t off = P.w < 0 || ((g & 1) && P.ld == 0) ? -1 : P.w + (g & 1) * (int64_t)P.ld;
+        const float sw = wscale[8 * tile + g];
+        const float s[4] = {sw, sw, sw, sw};
+        if (lane < 4) tdst[4 * tile + lane] = pairs[4 * tile + lane].dst;
+        for (int c = 0; c < nch; ++c) {
+            float2 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = c * MM_K + 2 * t + (q & 1) + 8 * (q >> 1);
+                v[q] = off >= 0 && k < B.klen ? pool[off + k] : make_float2(0.f, 0.f);
+            }
+            pack_tile(reinterpret_cast<float4 *>(ws + ((int64_t)B.pos + (int64_t)it * nch + c) * MM_TILE), v, s, lane);
+        }
+    }
+}
+
+} // namespace
+
+// scales and operand streams of a level's lists (device copies M; wscale, rscale zeroed by the caller)
+void launch_mm_pack(const LevelList &L, const MmPackArgs &M, const float2 *pool, cudaStream_t s)
+{
+    const int n_cl = M.n_cl;
+    if (M.n_sets <= 0 || n_cl <= 0) return;
+    k_mm_eout<<<(n_cl + 255) / 256, 256, 0, s>>>(L.d_mm_eout, n_cl, 1);
+    k_mm_prep<<<(unsigned)std::min<int64_t>((M.n_sets + 7) / 8, 152 * 16), 256, 0, s>>>(M.sets, M.n_sets, pool, M.wscale, M.rscale,
+                                                                                      L.d_mm_eout);
+    k_mm_eout<<<(n_cl + 255) / 256, 256, 0, s>>>(L.d_mm_eout, n_cl, 0);
+    k_mm_rscale<<<(unsigned)std::min<int64_t>((M.n_sets + 255) / 256, 4096), 256, 0, s>>>(M.sets, M.n_sets, M.rscale, L.d_mm_eout);
+    k_mm_pack_out<<<(unsigned)std::min<int64_t>((M.n_chunks + 7) / 8, 152 * 32), 256, 0, s>>>(
+        M.chunks, M.n_chunks, M.rows, M.rscale, L.d_mm_eout, pool, L.d_mm_os, L.d_mm_ca);
+    if (L.mm_n_batch > 0)
+        k_mm_pack_w<<<(unsigned)L.mm_n_batch, 256, 0, s>>>(L.d_mm_batch, M.pairs, M.wscale, pool, L.d_mm_ws, L.d_mm_tdst);
+}
+size_t mm_stream_bytes(int64_t tiles) { return (size_t)tiles * MM_TILE; }
+
+// right-hand sides per pass: all of them while x and T in operand layout fit MM_PASS_BYTES (a
+// pass streams the blocks from HBM once), else whole groups of 64 that do
+static int mm_pass(const LevelList &L, int nrhs, bool res)
+{
+    const size_t words = res ? tile_words<true>() : tile_words<false>();
+    const size_t tile = words * sizeof(uint32_t) * ((size_t)L.mm_n_xch + (size_t)L.mm_n_tch);
+    const int64_t fit = (int64_t)(MM_PASS_BYTES / std::max<size_t>(tile, 1)) * 16 / MM_PASS_MIN * MM_PASS_MIN;
+    return (int)std::min<int64_t>(nrhs, std::max<int64_t>(fit, MM_PASS_MIN));
+}
+
+// bytes of the operand tiles (x, then T, then the right-hand sides' scales) of a pass over nrhs
+size_t mm_ws_bytes(const LevelList &L, int nrhs, bool res)
+{
+    const int pass = mm_pass(L, nrhs, res);
+    const size_t tiles = (size_t)(pass + 15) / 16;
+    const size_t words = res ? tile_words<true>() : tile_words<false>();
+    return tiles * words * sizeof(uint32_t) * ((size_t)L.mm_n_xch + (size_t)L.mm_n_tch) + 2 * sizeof(float) * (size_t)pass;
+}
+
+namespace {
+// shared memory of a kernel beyond the default, two CTAs an SM
+void mm_attr(const void *kern, int smem)
+{
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+}
+
+// x of a pass into operand tiles, then stage 1
+template <bool RES>
+int mm_inputs(hm_matrix h, const LevelList &L, const float2 *x, int nr, uint32_t *xt, uint32_t *tt, float *xs, cudaStream_t s)
+{
+    const int tiles = (nr + 15) / 16;
+    k_mm_max<<<nr, 1024, 0, s>>>(x, h->pN, xs);
+    k_mm_split<RES><<<dim3((unsigned)((L.mm_n_xch + 3) / 4), (unsigned)tiles), 128, 0, s>>>(L.d_mm_xch, (int)L.mm_n_xch, x,
+                                                                                           h->pN, nr, xs, xt);
+    if (L.mm_n_batch == 0) return 2;
+    auto go = [&](auto kern, int mt, int smem) {
+        mm_attr((const void *)kern, smem);
+        const int groups = (tiles + mt - 1) / mt;
+        kern<<<(unsigned)(groups * L.mm_n_batch), MMW * 32, smem, s>>>(
+            L.d_mm_batch, L.d_mm_tdst, L.d_mm_ws, xt, (int)L.mm_n_xch, tt, L.mm_n_tch, tiles, groups);
+    };
+    if constexpr (!RES) {
+        if (tiles > 1) {
+            go(k_mm_stage1<RES, 2>, 2, s1_smem<RES, 2>());
+            return 3;
+        }
+    }
+    go(k_mm_stage1<RES, 1>, 1, s1_smem<RES, 1>());
+    return 3;
+}
+} // namespace
+
+// z += M_level x for the level's small items and all right-hand sides; ws as mm_ws_bytes
+int launch_mm_product(hm_matrix h, const LevelList &L, const float2 *x, float2 *z, int nrhs, void *ws, cudaStream_t s)
+{
+    if (L.mm_n_unit == 0 || nrhs <= 0) return 0;
+    int n = 0;
+    // Chunks of 16 K the tensor core adds up before the sum is taken out.  It truncates, so a sum
+    // shrinks a little with every product: one chunk, and the product errs by 2.8e-7 (30,720-unknown
+    // sphere; the FP32 kernels 5.0e-7), 32 and it errs by 4.2e-6 and takes 6 % less time.  32 is for
+    // the calls of many right-hand sides that had the tcgen05 product (7.5e-6, sums of 512 K):
+    // above 32 of them, or above 16 on operators large enough.
+    const bool many = (nrhs > 32 && L.mm_n_chunk > 3000) || (nrhs > 16 && L.mm_n_chunk > 60000);
+    const int drain = many ? 32 : 1;
+    const bool coarse = many && nrhs > 32;
+    const int pass = mm_pass(L, nrhs, false);
+    const size_t tiles_max = (size_t)(pass + 15) / 16;
+    uint32_t *xt = (uint32_t *)ws, *tt = xt + tiles_max * tile_words<false>() * L.mm_n_xch;
+    float *xs = (float *)(tt + tiles_max * tile_words<false>() * L.mm_n_tch);
+    for (int r0 = 0; r0 < nrhs; r0 += pass) {
+        const int nr = std::min(pass, nrhs - r0), tiles = (nr + 15) / 16;
+        const float2 *xp = x + (int64_t)r0 * h->pN;
+        n += mm_inputs<false>(h, L, xp, nr, xt, tt, xs, s) + 1;
+        // tiles of 16 right-hand sides a warp up to 16 of them, 32 above, two such groups a CTA above 32
+        const int mw = tiles > 2 ? 2 : 1, mt = tiles > 1 ? 2 : 1, groups = (tiles + mt * mw - 1) / (mt * mw);
+        MmOutArgs a{coarse ? L.d_mm_unit2 : L.d_mm_unit, L.d_mm_ca, L.d_mm_eout, L.d_mm_os, xt, tt, (int)L.mm_n_xch,
+                    tiles, nr, L.mm_n_tch, xs, groups};
+        float2 *zp = z + (int64_t)r0 * h->pN;
+        const unsigned units = (unsigned)(coarse ? L.mm_n_unit2 : L.mm_n_unit);
+        auto go = [&](auto kern) {
+            mm_attr((const void *)kern, MM_SMEM);
+            kern<<<units * (unsigned)groups, MMW * 32, MM_SMEM, s>>>(a, mw, drain, zp, h->pN);
+        };
+        if (mt == 1) go(k_mm_out<1>);
+        else go(k_mm_out<2>);
+    }
+    return n;
+}
+
+// own[part][r][p] = the FP64-class sums of the level's small items' products, by part of the
+// output cluster's units (rows no unit covers are left as they are)
+int launch_mm_resid(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int64_t pstride, int nrhs, void *ws,
+                    cudaStream_t s)
+{
+    if (L.mm_n_runit == 0 || nrhs <= 0) return 0;
+    int n = 0;
+    const int pass = mm_pass(L, nrhs, true);
+    const size_t tiles_max = (size_t)(pass + 15) / 16;
+    uint32_t *xt = (uint32_t *)ws, *tt = xt + tiles_max * tile_words<true>() * L.mm_n_xch;
+    float *xs = (float *)(tt + tiles_max * tile_words<true>() * L.mm_n_tch);
+    for (int r0 = 0; r0 < nrhs; r0 += pass) {
+        const int nr = std::min(pass, nrhs - r0), tiles = (nr + 15) / 16;
+        n += mm_inputs<true>(h, L, x + (int64_t)r0 * h->pN, nr, xt, tt, xs, s) + 1;
+        MmOutArgs a{L.d_mm_runit, L.d_mm_ca, L.d_mm_eout, L.d_mm_os, xt, tt, (int)L.mm_n_xch,
+                    tiles, nr, L.mm_n_tch, xs, tiles};
+        mm_attr((const void *)k_mm_resid, MM_SMEM);
+        k_mm_resid<<<(unsigned)(tiles * L.mm_n_runit), MMW * 32, MM_SMEM, s>>>(a, own + (int64_t)r0 * h->pN,
+                                                                                           pstride, h->pN);
+    }
+    return n;
+}
+
+} // namespace hm

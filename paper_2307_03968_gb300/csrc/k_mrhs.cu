@@ -507,8 +507,7 @@ void launch_apply_list_mrhs(hm_matrix h, const LevelList &L, const Item *items, 
 {
     if (n_items == 0 || nrhs <= 0) return;
     if (rb <= 8) launch_rb<8>(h, L, items, n_items, x, z, nrhs, s);
-    else if (rb <= 16) launch_rb<16>(h, L, items, n_items, x, z, nrhs, s);
-    else launch_rb<32>(h, L, items, n_items, x, z, nrhs, s);
+    else launch_rb<16>(h, L, items, n_items, x, z, nrhs, s);
 }
 
 } // namespace hm

@@ -84,7 +84,7 @@ int launch_apply_items(hm_matrix h, const LevelList &L, const void *x, void *z, 
         // tall dense blocks go as row panels (LevelList::d_prod), one warp each
         const Item *list = L.d_prod ? L.d_prod : L.d_items;
         int64_t cnt = L.d_prod ? L.n_prod : n;
-        if (rb < 0) rb = nrhs < MRHS_MIN_RHS ? 0 : nrhs <= 8 ? 8 : nrhs <= 16 ? 16 : 32;
+        if (rb < 0) rb = nrhs < MRHS_MIN_RHS ? 0 : nrhs <= 8 ? 8 : 16;
         if (rb == RB_TC && nrhs > 1) {
             // the small blocks (dense and low-rank) on the tensor cores
             launched += launch_apply_tc(h, L, (const float2 *)x, (float2 *)z, nrhs, s);
@@ -92,9 +92,13 @@ int launch_apply_items(hm_matrix h, const LevelList &L, const void *x, void *z, 
             cnt = L.d_prod ? L.n_prod_big : L.n_big;
             if (cnt == 0) return launched;
         } else if (rb > 0 && nrhs > 1 && L.n_small > 0) {
-            // many right-hand sides: blocks that fit shared memory are read once per RHS chunk
-            launch_apply_items_mrhs(h, L, (const float2 *)x, (float2 *)z, nrhs, rb, s);
-            launched += 1;
+            // many right-hand sides: on the matrix instructions, or blocks staged in shared memory once per chunk
+            if (rb == 32 && h->ws.d_mm && h->ws.mm_bytes >= mm_ws_bytes(L, nrhs, false)) {
+                launched += launch_mm_product(h, L, (const float2 *)x, (float2 *)z, nrhs, h->ws.d_mm, s);
+            } else {
+                launch_apply_items_mrhs(h, L, (const float2 *)x, (float2 *)z, nrhs, std::min(rb, 16), s);
+                launched += 1;
+            }
             list = L.d_prod ? L.d_prod_big : L.d_big;
             cnt = L.d_prod ? L.n_prod_big : L.n_big;
             if (cnt == 0) return launched;
