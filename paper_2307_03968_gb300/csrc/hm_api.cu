@@ -1205,7 +1205,8 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     c.Y.assign(c.m + 1, nullptr); c.X = c.Y; c.Z = c.Y; c.W = c.Y;
     for (int l = 1; l <= c.m; ++l) { c.Y[l] = V[vi++]; c.X[l] = V[vi++]; c.Z[l] = V[vi++]; c.W[l] = V[vi++]; }
     void *bt = V[vi++], *xt = V[vi++], *rt = V[vi++], *dx = V[vi++];
-    double *norms = o->refine ? h->ws.d_acc64 : nullptr;
+    // |r|^2, |b|^2 are formed only for a caller that gets them (a memset and the gather's atomics less)
+    double *norms = o->refine && info ? h->ws.d_acc64 : nullptr;
     // the solve's steps, launched or recorded (the one-launch solve) through c
     auto steps = [&](SolveCtx &cc) {
         // complex64, launched: the permutation of b and the series' first step in one pass
@@ -1233,7 +1234,7 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
         else Pflat(cc, bt, xt);
         cc.fin_target = nullptr;
         if (o->refine) {
-            zero_vec(cc, norms, 2 * sizeof(double) * nrhs);
+            if (norms) zero_vec(cc, norms, 2 * sizeof(double) * nrhs);
             residual64(cc, (const float2 *)xt, (const float2 *)bt, (float2 *)rt, norms,
                        fuse ? (float2 *)cc.Y[1] : nullptr);
             finish_with(dx, (const float2 *)xt);
