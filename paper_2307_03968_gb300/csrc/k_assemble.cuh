@@ -919,9 +919,13 @@ hm_status assemble(BasisData &B, G g, const hm_build_opts *o, TmpBuffers &tmp, c
     if ((st = tmp.up(&d_fj, fj, s)) != HM_OK) return st;
     if ((st = tmp.up(&d_fs, fs, s)) != HM_OK) return st;
     if (flat > 0) {
+      if constexpr (G::BLOCK_FILL) {   // the basis fills whole blocks (its element integrals serve many entries)
+        if ((st = g.fill_near(fj, h->d_pool32, tmp, s)) != HM_OK) return st;
+      } else {
         const int grid = (int)std::min<int64_t>((flat + 255) / 256, 152 * 64);
         k_fill<G, false><<<grid, 256, 0, s>>>(g, d_fj, (int)fj.size(), flat, h->d_pool32, h->d_self64);
         HM_CUDA(cudaGetLastError());
+      }
     }
     if (flat_self > 0) {
         const int grid = (int)std::min<int64_t>((flat_self + 255) / 256, 152 * 64);

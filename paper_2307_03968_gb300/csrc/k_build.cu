@@ -43,6 +43,7 @@ struct Geo {
     const float2 *qpd32;  // nt x NQ x 3
     float kf, ik2f;       // k and 1/k^2, rounded
     static constexpr int PARTS = 4;
+    static constexpr bool BLOCK_FILL = false;
     template <class R> __device__ CX<R> entry(int m, int n) const;
     __device__ CX<float> part(int m, int n, int p) const;              // the signed triangle pair p of an entry
     __device__ CX<float> scale(int m, int n, const CX<float> &z) const;

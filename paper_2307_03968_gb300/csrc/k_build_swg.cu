@@ -21,7 +21,7 @@
 // theorem, Int_T 1/R dV' = 1/2 sum_f ((p_f - r) . n_f) Int_f 1/R dS' and
 // Int_T (r' - r)/R dV' = sum_f n_f Int_f R dS' with outward face normals n_f.
 // Coordinates are taken relative to a vertex of the column face.  The near
-// blocks (complex64) take the quadrature in FP32 but the analytic singular
+// blocks (complex64, k_fill_swg) take the quadrature in FP32 but the analytic singular
 // terms in FP64: the four tetrahedron pairs of one function pair cancel like a
 // dipole-dipole interaction, which turns the ~1e-6 FP32 error of the edge
 // formulas two or three element sizes away into ~1e-4 of the entry.  The leaf
@@ -37,6 +37,9 @@ constexpr double EXTRACT_FACTOR = 2.0;
 constexpr double INV4PI = 0.25 / 3.14159265358979323846;
 
 __constant__ double c_fw[NQF];
+
+constexpr int FGEO = 31;                 // P[3][3], n[3], dir[3][3], out[3][3], 2 area
+constexpr int TGEO = 12 + 4 * (3 + 9 + 1) + 6 * 4;   // P[4][3]; faces: n[3], out[3][3], 2 area; edges: dir[3], length
 
 struct VGeo {
     const double *vtx;      // nv x 3
@@ -58,6 +61,12 @@ struct VGeo {
     const int32_t *perm;    // tree position -> original face index
     double k;
     static constexpr int PARTS = 1;
+    static constexpr bool BLOCK_FILL = true;
+    // for the near fill by blocks (k_fill_swg)
+    const float2 *vtx32, *tqp32, *fqp32;   // the points as pairs of floats (hi, lo)
+    const double *fgeo;     // nf x FGEO: vertices, unit normal away from T+'s free vertex, per edge direction and outward in-plane normal
+    const double *tgeo;     // nt x TGEO: vertices; per face (opposite vertex a): outward normal, per edge of the face its outward in-plane normal; the 6 edge directions and lengths
+    hm_status fill_near(const std::vector<FillJob> &jobs, float2 *pool, TmpBuffers &tmp, cudaStream_t s) const;
     template <class R> __device__ CX<R> entry(int m, int n) const;
 };
 
@@ -363,6 +372,395 @@ template <class R> __device__ CX<R> VGeo::entry(int m, int n) const
     return z;
 }
 
+// ---- near fill by blocks ------------------------------------------------------------
+//
+// The 4 + 4 + 1 element integrals of an entry (tetrahedron pairs, tetrahedron-face pairs, face
+// pair) hang on the elements, and an element belongs to several of the block's functions: a
+// chunk of 32 x 32 faces has about 32 tetrahedra a side, so each tetrahedron pair serves four
+// to five entries and each tetrahedron-face pair two.  A CTA takes one such chunk, evaluates each
+// pair once (phase 1: quadrature values of G and, for close pairs, the FP64 analytic parts at
+// the four outer points) and then forms the entries from them (phase 2).
+//
+// The FP64 analytic parts bound it (FP64 runs at 1/64 of the FP32 rate here).  Over a
+// tetrahedron at one point they take 4 vertex distances, 6 edge logarithms (an edge's logarithm
+// is the same in both of its faces) and 4 arc tangents (the sum over a face's edges is the
+// solid angle of the face: Van Oosterom & Strackee 1983), with all directions and normals from
+// a table, where the entry function evaluates each face by itself from its vertices (24 distances,
+// 12 logarithms, 24 arc tangents and 48 square roots and quotients for the directions).
+// 2,808 unknowns (6^3 voxels, leaves of 44): 60 ms; one thread per entry with its own element
+// integrals took 400 ms.
+constexpr int FB = 32;                    // faces of a chunk side
+constexpr int FG = 4;                     // inner tetrahedra per round
+
+struct SwgJob { int64_t out; int32_t r0, c0, m, n, ld, pad; };
+
+__device__ __forceinline__ void diff_points(const float2 *a, const float2 *b, float (&d)[3])
+{
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        const float s = __fsub_rn(a[x].x, b[x].x), bb = __fsub_rn(s, a[x].x);
+        const float e = __fsub_rn(__fsub_rn(a[x].x, __fsub_rn(s, bb)), __fadd_rn(b[x].x, bb));
+        d[x] = __fadd_rn(s, __fadd_rn(e, __fsub_rn(a[x].y, b[x].y)));
+    }
+}
+
+__device__ __forceinline__ double edge_log(double lm, double lp, double Rm, double Rp)
+{
+    return (lm < 0 && lp < 0) ? log((Rm - lm) / (Rp - lp)) : log((Rp + lp) / (Rm + lm));
+}
+__device__ __forceinline__ double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
+
+// |d| times the solid angle of a triangle with vertices v0, v1, v2 relative to the point (lengths R),
+// d = distance of its plane, a2 = twice its area (|det(v0, v1, v2)| = a2 |d|)
+__device__ __forceinline__ double plane_angle(double d, double a2, const double *v0, const double *v1, const double *v2,
+                                              double R0, double R1, double R2)
+{
+    const double ad = fabs(d);
+    if (!(ad > 0)) return 0.0;
+    const double den = R0 * R1 * R2 + dot3(v0, v1) * R2 + dot3(v0, v2) * R1 + dot3(v1, v2) * R0;
+    return ad * 2.0 * atan2(a2 * ad, den);
+}
+
+// Int_f 1/R dS' over face f at r
+__device__ double face_s0(const double *__restrict__ F, const double *r)
+{
+    double v[3][3], R[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) v[a][x] = F[3 * a + x] - r[x];
+        R[a] = sqrt(dot3(v[a], v[a]));
+    }
+    const double d = dot3(v[0], F + 9);
+    double s0 = 0.0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int b = (e + 1) % 3;
+        const double t = dot3(v[e], F + 21 + 3 * e);
+        if (t * t + d * d > 0) s0 += t * edge_log(dot3(v[e], F + 12 + 3 * e), dot3(v[b], F + 12 + 3 * e), R[e], R[b]);
+    }
+    return s0 - plane_angle(d, F[30], v[0], v[1], v[2], R[0], R[1], R[2]);
+}
+
+// faces of a tetrahedron (opposite vertex a): their vertices; edges 01 02 03 12 13 23 by vertex pair
+__device__ constexpr int TFV[4][3] = {{1, 2, 3}, {0, 2, 3}, {0, 1, 3}, {0, 1, 2}};
+__device__ constexpr int TEV[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
+// the edges of face a in the order (v0 v1), (v1 v2), (v0 v2)
+__device__ constexpr int TFE[4][3] = {{3, 5, 4}, {1, 5, 2}, {0, 4, 2}, {0, 3, 1}};
+
+// Int_T 1/R dV' (out[0]) and Int_T (r' - r)/R dV' (out[1..3])
+__device__ void tet_s0_s1(const double *__restrict__ G, const double *r, double *out)
+{
+    double v[4][3], R[4], f[6], g[6];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) v[a][x] = G[3 * a + x] - r[x];
+        R[a] = sqrt(dot3(v[a], v[a]));
+    }
+    const double *E = G + 12 + 4 * 13;
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+        const int a = TEV[e][0], b = TEV[e][1];
+        const double lm = dot3(v[a], E + 4 * e), lp = lm + E[4 * e + 3];
+        f[e] = edge_log(lm, lp, R[a], R[b]);
+        g[e] = lp * R[b] - lm * R[a];
+    }
+    double s0v = 0, s1[3] = {0, 0, 0};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const double *F = G + 12 + 13 * a;
+        const double d = dot3(v[TFV[a][0]], F);
+        double s0 = 0, eR = 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int e = TFE[a][q];
+            const double t = dot3(v[TEV[e][0]], F + 3 + 3 * q), r02 = t * t + d * d;
+            if (r02 > 0) {
+                s0 += t * f[e];
+                eR += t * 0.5 * (r02 * f[e] + g[e]);
+            } else {
+                eR += t * 0.5 * g[e];
+            }
+        }
+        s0 -= plane_angle(d, F[12], v[TFV[a][0]], v[TFV[a][1]], v[TFV[a][2]], R[TFV[a][0]], R[TFV[a][1]], R[TFV[a][2]]);
+        const double sR = (d * d * s0 + eR) / 3.0;
+        s0v += 0.5 * d * s0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) s1[x] += F[x] * sR;
+    }
+    out[0] = s0v;
+    out[1] = s1[0];
+    out[2] = s1[1];
+    out[3] = s1[2];
+}
+
+struct SwgSide {                          // one side (rows or columns) of a chunk
+    int face[FB];
+    int tl[FB][2], tf[FB][2];             // local tetrahedron and free vertex of each half (-1: none)
+    int tet[2 * FB], nt;
+    double cm[FB][2], qm[FB][2], qs[FB];  // s a / 3V kappa and -kappa s a / V of the halves; face charge
+    float pt[FB][2][NQT][3];              // quadrature points relative to the half's free vertex
+};
+struct SwgSmem {
+    SwgSide r, c;
+    int ex[2 * FB * FG];
+    union {
+        struct {                          // phase 1 and 2, one round
+            double an[2 * FB * FG][NQT][4];   // analytic parts of (outer tetrahedron, inner of the round) at the outer points
+            float2 G[2 * FB * FG][NQT][NQT];
+        } v;
+        double2 k[2][2 * FB][FB];         // Int_t Int_f G: row tetrahedra x column faces, column tetrahedra x row faces
+    };
+};
+
+__device__ void load_side(SwgSide &S, const VGeo &g, int p0, int n)
+{
+    const int tid = threadIdx.x;
+    if (tid < FB) S.face[tid] = tid < n ? g.perm[p0 + tid] : -1;
+    __syncthreads();
+    if (tid < 2 * FB) {
+        const int i = tid >> 1, p = tid & 1, f = S.face[i];
+        const int t = f >= 0 ? g.ftet[2 * f + p] : -1;
+        S.tf[i][p] = t >= 0 ? g.ffree[2 * f + p] : -1;
+        S.tl[i][p] = t;                   // the tetrahedron for now
+        const double s = p == 0 ? 1.0 : -1.0;
+        S.cm[i][p] = t >= 0 ? g.kappa[t] * (s * g.farea[f] / (3.0 * g.tvol[t])) : 0.0;
+        S.qm[i][p] = t >= 0 ? -g.kappa[t] * s * g.farea[f] / g.tvol[t] : 0.0;
+        if (p == 0) S.qs[i] = f >= 0 ? g.fqs[f] : 0.0;
+    }
+    __syncthreads();
+    // local numbers: a half is first if no earlier half has its tetrahedron
+    int mine = -1, first = -1, rank = 0;
+    if (tid < 2 * FB) {
+        mine = S.tl[tid >> 1][tid & 1];
+        for (int k = 0; k < tid && mine >= 0; ++k)
+            if (S.tl[k >> 1][k & 1] == mine) { first = k; break; }
+        if (mine >= 0 && first < 0) first = tid;
+    }
+    __syncthreads();
+    __shared__ int isf[2 * FB];
+    if (tid < 2 * FB) isf[tid] = mine >= 0 && first == tid;
+    __syncthreads();
+    if (tid < 2 * FB && mine >= 0) {
+        for (int k = 0; k < first; ++k) rank += isf[k];
+        S.tl[tid >> 1][tid & 1] = rank;
+        if (first == tid) S.tet[rank] = mine;
+    }
+    if (tid == 0) {
+        int k = 0;
+        for (int q = 0; q < 2 * FB; ++q) k += isf[q];
+        S.nt = k;
+    }
+    __syncthreads();
+    for (int e = tid; e < 2 * FB * NQT; e += blockDim.x) {
+        const int i = e / (2 * NQT), p = e / NQT % 2, q = e % NQT;
+        if (S.tl[i][p] < 0) continue;
+        diff_points(g.tqp32 + 3 * ((int64_t)S.tet[S.tl[i][p]] * NQT + q), g.vtx32 + 3 * (int64_t)S.tf[i][p], S.pt[i][p][q]);
+    }
+    __syncthreads();
+}
+
+// Int_t Int_f G, outer point i of the four: the quad's lanes (i = lane % 4) each one point, summed
+// in point order (the analytic parts in FP64)
+__device__ double2 volface_quad(const VGeo &g, int t, int f, int i, float k)
+{
+    const bool ex = near_pair(g.tcen + 3 * (int64_t)t, g.thmax[t], g.fcen + 3 * (int64_t)f, g.fhmax[f]);
+    CX<float> K{0, 0};
+    for (int j = 0; j < NQF; ++j) {
+        float dr[3];
+        diff_points(g.tqp32 + 3 * ((int64_t)t * NQT + i), g.fqp32 + 3 * ((int64_t)f * NQF + j), dr);
+        const CX<float> G = green<float>(k, sqrtf(dot(dr, dr)), ex);
+        const float w = (float)c_fw[j];
+        K.re += w * G.re;
+        K.im += w * G.im;
+    }
+    double s0 = 0.0;
+    if (ex) s0 = face_s0(g.fgeo + (int64_t)f * FGEO, g.tqp + 3 * ((int64_t)t * NQT + i)) * INV4PI;
+    const int base = (threadIdx.x & 31) & ~3;
+    float re = 0.f, im = 0.f;
+    double an = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        re += 0.25f * __shfl_sync(0xffffffffu, K.re, base + q);
+        im += 0.25f * __shfl_sync(0xffffffffu, K.im, base + q);
+        an += 0.25 * __shfl_sync(0xffffffffu, s0, base + q);
+    }
+    const double V = g.tvol[t], A = g.farea[f];
+    return make_double2(V * (A * re + an), V * A * im);
+}
+
+__global__ void __launch_bounds__(256)
+k_fill_swg(VGeo g, const SwgJob *__restrict__ jobs, float2 *pool)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    SwgSmem &S = *reinterpret_cast<SwgSmem *>(smraw);
+    const SwgJob J = jobs[blockIdx.x];
+    const int tid = threadIdx.x;
+    const float k = (float)g.k;
+    const double k2 = g.k * g.k;
+    load_side(S.r, g, J.r0, J.m);
+    load_side(S.c, g, J.c0, J.n);
+    const int n = tid % FB, m0 = tid / FB;         // the thread's entries: column n, rows m0 + 8 e
+    // the entries in FP64: their element integrals cancel like the charges of a dipole
+    double2 z[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) z[e] = make_double2(0.0, 0.0);
+    const int nr = S.r.nt, nc = S.c.nt;
+    for (int b0 = 0; b0 < nc; b0 += FG) {
+        const int nb = min(FG, nc - b0);
+        // phase 1: outer tetrahedron a, inner b0 + b, outer point i
+        for (int q = tid; q < nr * nb * NQT; q += blockDim.x) {
+            const int i = q % NQT, a = q / NQT % nr, b = q / (NQT * nr);
+            const int t = S.r.tet[a], tp = S.c.tet[b0 + b];
+            const bool ex = near_pair(g.tcen + 3 * (int64_t)t, g.thmax[t], g.tcen + 3 * (int64_t)tp, g.thmax[tp]);
+            const int at = b * nr + a;
+            for (int j = 0; j < NQT; ++j) {
+                float dr[3];
+                diff_points(g.tqp32 + 3 * ((int64_t)t * NQT + i), g.tqp32 + 3 * ((int64_t)tp * NQT + j), dr);
+                const CX<float> G = green<float>(k, sqrtf(dot(dr, dr)), ex);
+                S.v.G[at][i][j] = make_float2(G.re, G.im);
+            }
+            if (ex) tet_s0_s1(g.tgeo + (int64_t)tp * TGEO, g.tqp + 3 * ((int64_t)t * NQT + i), S.v.an[at][i]);
+            if (i == 0) S.ex[at] = ex;
+        }
+        __syncthreads();
+        // phase 2
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int m = m0 + 8 * e;
+            if (m >= J.m || n >= J.n) continue;
+            for (int q = 0; q < 2; ++q) {
+                const int bl = S.c.tl[n][q] - b0;
+                if (S.c.tl[n][q] < 0 || bl < 0 || bl >= nb) continue;
+                const int tp = S.c.tet[b0 + bl];
+                const double *vn = g.vtx + 3 * (int64_t)S.c.tf[n][q];
+                for (int p = 0; p < 2; ++p) {
+                    const int al = S.r.tl[m][p];
+                    if (al < 0) continue;
+                    const int t = S.r.tet[al], at = bl * nr + al;
+                    const bool ex = S.ex[at];
+                    CX<float> I{0, 0}, Jc{0, 0};
+                    double aI = 0.0, aJ = 0.0;         // the analytic parts
+                    for (int i = 0; i < NQT; ++i) {
+                        const float *a = S.r.pt[m][p][i];
+                        CX<float> Ii{0, 0}, Ji{0, 0};
+#pragma unroll
+                        for (int j = 0; j < NQT; ++j) {
+                            const float2 G = S.v.G[at][i][j];
+                            const float *b = S.c.pt[n][q][j];
+                            const float w = a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+                            Ii.re += w * G.x; Ii.im += w * G.y;
+                            Ji.re += G.x; Ji.im += G.y;
+                        }
+                        I.re += Ii.re; I.im += Ii.im;
+                        Jc.re += Ji.re; Jc.im += Ji.im;
+                        if (ex) {
+                            const double *rd = g.tqp + 3 * ((int64_t)t * NQT + i), *vm = g.vtx + 3 * (int64_t)S.r.tf[m][p];
+                            const double *an = S.v.an[at][i];
+#pragma unroll
+                            for (int x = 0; x < 3; ++x) aI += (rd[x] - vm[x]) * (an[1 + x] + (rd[x] - vn[x]) * an[0]);
+                            aJ += an[0];
+                        }
+                    }
+                    // weights 1/4 of each point; times the volumes (the analytic parts hold the inner one)
+                    const double Vt = g.tvol[t], W = Vt * g.tvol[tp] * 0.0625, Wa = Vt * 0.25 * INV4PI;
+                    const double ca = -k2 * S.r.cm[m][p] * S.c.cm[n][q], cb = S.r.qm[m][p] * S.c.qm[n][q];
+                    z[e].x += ca * (W * I.re + Wa * aI) + cb * (W * Jc.re + Wa * aJ);
+                    z[e].y += W * (ca * I.im + cb * Jc.im);
+                    if (t == tp && g.kappa[t] != 0.0) {   // Int (kappa/eps_r) f_m . f_n dV: degree 2, exact with the 4-point rule
+                        float acc = 0.f;
+                        for (int i = 0; i < NQT; ++i) {
+                            const float *a = S.r.pt[m][p][i], *b = S.c.pt[n][q][i];
+                            acc += 0.25f * (a[0] * b[0] + a[1] * b[1] + a[2] * b[2]);
+                        }
+                        z[e].x += S.r.cm[m][p] * S.c.cm[n][q] * g.tvol[t] / (g.kappa[t] * g.epsr[t]) * acc;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    // tetrahedron-face integrals, both ways (a quad of lanes each; all lanes run the same rounds)
+    for (int side = 0; side < 2; ++side) {
+        const SwgSide &T = side ? S.c : S.r, &F = side ? S.r : S.c;
+        const int nf = side ? J.m : J.n, total = T.nt * nf;
+        for (int q0 = 0; q0 < total; q0 += blockDim.x / 4) {
+            const int q = min(q0 + tid / 4, total - 1), a = q / nf, f = q % nf;
+            const double2 K = volface_quad(g, T.tet[a], F.face[f], tid & 3, k);
+            if ((tid & 3) == 0) S.k[side][a][f] = K;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int m = m0 + 8 * e;
+        if (m >= J.m || n >= J.n) continue;
+        const double qsm = S.r.qs[m], qsn = S.c.qs[n];
+        for (int p = 0; p < 2; ++p) {
+            const int al = S.r.tl[m][p], bl = S.c.tl[n][p];
+            if (qsn != 0.0 && al >= 0) {
+                const double2 K = S.k[0][al][n];
+                const double c = S.r.qm[m][p] * qsn;
+                z[e].x += c * K.x;
+                z[e].y += c * K.y;
+            }
+            if (qsm != 0.0 && bl >= 0) {
+                const double2 K = S.k[1][bl][m];
+                const double c = qsm * S.c.qm[n][p];
+                z[e].x += c * K.x;
+                z[e].y += c * K.y;
+            }
+        }
+        if (qsm != 0.0 && qsn != 0.0) {     // Int_m Int_n G
+            const int f = S.r.face[m], fp = S.c.face[n];
+            const bool ex = near_pair(g.fcen + 3 * (int64_t)f, g.fhmax[f], g.fcen + 3 * (int64_t)fp, g.fhmax[fp]);
+            CX<float> L{0, 0};
+            double an = 0.0;
+            for (int i = 0; i < NQF; ++i) {
+                CX<float> Li{0, 0};
+                for (int j = 0; j < NQF; ++j) {
+                    float dr[3];
+                    diff_points(g.fqp32 + 3 * ((int64_t)f * NQF + i), g.fqp32 + 3 * ((int64_t)fp * NQF + j), dr);
+                    const CX<float> G = green<float>(k, sqrtf(dot(dr, dr)), ex);
+                    const float w = (float)c_fw[j];
+                    Li.re += w * G.re;
+                    Li.im += w * G.im;
+                }
+                if (ex) an += c_fw[i] * face_s0(g.fgeo + (int64_t)fp * FGEO, g.fqp + 3 * ((int64_t)f * NQF + i));
+                const float w = (float)c_fw[i];
+                L.re += w * Li.re;
+                L.im += w * Li.im;
+            }
+            const double A = g.farea[f], Ap = g.farea[fp], c = qsm * qsn * A;
+            z[e].x += c * (Ap * L.re + INV4PI * an);
+            z[e].y += c * Ap * L.im;
+        }
+        pool[J.out + (int64_t)m * J.ld + n] = make_float2((float)z[e].x, (float)z[e].y);
+    }
+}
+
+hm_status VGeo::fill_near(const std::vector<FillJob> &fj, float2 *pool, TmpBuffers &tmp, cudaStream_t s) const
+{
+    std::vector<SwgJob> jobs;
+    for (const FillJob &f : fj) {         // even chunks of at most FB faces a side
+        const int nm = (f.m + FB - 1) / FB, nn = (f.n + FB - 1) / FB;
+        for (int a = 0; a < nm; ++a)
+            for (int b = 0; b < nn; ++b) {
+                const int i0 = f.m * a / nm, i1 = f.m * (a + 1) / nm, j0 = f.n * b / nn, j1 = f.n * (b + 1) / nn;
+                jobs.push_back({f.out + (int64_t)i0 * f.ld + j0, f.r0 + i0, f.c0 + j0, i1 - i0, j1 - j0, f.ld, 0});
+            }
+    }
+    if (jobs.empty()) return HM_OK;
+    SwgJob *d_jobs = nullptr;
+    const hm_status st = tmp.up(&d_jobs, jobs, s);
+    if (st != HM_OK) return st;
+    HM_CUDA(cudaFuncSetAttribute(k_fill_swg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SwgSmem)));
+    k_fill_swg<<<(unsigned)jobs.size(), 256, sizeof(SwgSmem), s>>>(*this, d_jobs, pool);
+    HM_CUDA(cudaGetLastError());
+    return HM_OK;
+}
+
 static double norm3(const double *d) { return std::sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]); }
 
 static double max_edge(const double *const *p, int np)
@@ -490,6 +888,76 @@ hm_status build_from_tets(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
             B.bhi.push_back(hi);
         }
     }
+    // geometry of the analytic integrals (k_fill_swg): directions, in-plane outward normals, areas
+    std::vector<double> fgeo((size_t)N * FGEO), tgeo((size_t)nt * TGEO);
+    auto sub = [](const double *a, const double *b, double *o) { for (int d = 0; d < 3; ++d) o[d] = a[d] - b[d]; };
+    auto unit = [](double *a) {
+        const double l = norm3(a);
+        for (int d = 0; d < 3; ++d) a[d] /= l;
+        return l;
+    };
+    auto cross = [](const double *a, const double *b, double *o) {
+        o[0] = a[1] * b[2] - a[2] * b[1]; o[1] = a[2] * b[0] - a[0] * b[2]; o[2] = a[0] * b[1] - a[1] * b[0];
+    };
+    auto dotd = [](const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+    // unit normal of the triangle (p0, p1, p2) and twice its area
+    auto plane = [&](const double *p0, const double *p1, const double *p2, double *n) {
+        double a[3], b[3];
+        sub(p1, p0, a);
+        sub(p2, p0, b);
+        cross(a, b, n);
+        return unit(n);
+    };
+    // the in-plane unit normal of the edge a b of a triangle with normal n, away from its vertex c
+    auto outward = [&](const double *a, const double *b, const double *c, const double *n, double *u) {
+        double l[3], w[3];
+        sub(b, a, l);
+        unit(l);
+        cross(l, n, u);
+        sub(c, a, w);
+        if (dotd(u, w) > 0)
+            for (int d = 0; d < 3; ++d) u[d] = -u[d];
+    };
+    for (int64_t f = 0; f < N; ++f) {
+        double *G = &fgeo[(size_t)f * FGEO];
+        const double *p[3];
+        for (int a = 0; a < 3; ++a) {
+            p[a] = X + 3 * fv[3 * f + a];
+            for (int d = 0; d < 3; ++d) G[3 * a + d] = p[a][d];
+        }
+        G[30] = plane(p[0], p[1], p[2], G + 9);
+        for (int e = 0; e < 3; ++e) {
+            sub(p[(e + 1) % 3], p[e], G + 12 + 3 * e);
+            unit(G + 12 + 3 * e);
+            outward(p[e], p[(e + 1) % 3], p[(e + 2) % 3], G + 9, G + 21 + 3 * e);
+        }
+    }
+    static const int TV[4][3] = {{1, 2, 3}, {0, 2, 3}, {0, 1, 3}, {0, 1, 2}};
+    static const int TE[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
+    for (int64_t t = 0; t < nt; ++t) {
+        double *G = &tgeo[(size_t)t * TGEO];
+        const double *p[4];
+        for (int a = 0; a < 4; ++a) {
+            p[a] = X + 3 * mesh->cells[4 * t + a];
+            for (int d = 0; d < 3; ++d) G[3 * a + d] = p[a][d];
+        }
+        for (int a = 0; a < 4; ++a) {
+            const double *v0 = p[TV[a][0]], *v1 = p[TV[a][1]], *v2 = p[TV[a][2]];
+            double *F = G + 12 + 13 * a, w[3];
+            F[12] = plane(v0, v1, v2, F);
+            sub(p[a], v0, w);
+            if (dotd(F, w) > 0)
+                for (int d = 0; d < 3; ++d) F[d] = -F[d];
+            outward(v0, v1, v2, F, F + 3);
+            outward(v1, v2, v0, F, F + 6);
+            outward(v0, v2, v1, F, F + 9);
+        }
+        for (int e = 0; e < 6; ++e) {
+            double *E = G + 12 + 52 + 4 * e;
+            sub(p[TE[e][1]], p[TE[e][0]], E);
+            E[3] = unit(E);
+        }
+    }
     HM_CUDA(cudaMemcpyToSymbol(c_fw, fw, sizeof(fw)));
     TmpBuffers tmp;
     std::vector<double> vtx(X, X + 3 * nv);
@@ -508,6 +976,12 @@ hm_status build_from_tets(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
     g.kappa = d_kappa; g.epsr = d_epsr; g.fv = d_fv; g.ftet = d_ftet; g.ffree = d_ffree; g.fqp = d_fqp;
     g.fcen = d_fcen; g.fhmax = d_fhmax; g.farea = d_farea; g.fqs = d_fqs;
     g.k = 2.0 * 3.14159265358979323846 / mesh->wavelength;
+    float2 *d_vtx32, *d_tqp32, *d_fqp32;
+    double *d_fgeo, *d_tgeo;
+    if ((st = tmp.up(&d_vtx32, float_pairs(vtx), s)) || (st = tmp.up(&d_tqp32, float_pairs(tqp), s)) ||
+        (st = tmp.up(&d_fqp32, float_pairs(fqp), s)) || (st = tmp.up(&d_fgeo, fgeo, s)) || (st = tmp.up(&d_tgeo, tgeo, s)))
+        return st;
+    g.vtx32 = d_vtx32; g.tqp32 = d_tqp32; g.fqp32 = d_fqp32; g.fgeo = d_fgeo; g.tgeo = d_tgeo;
 
     // excitation: b_m = sum_s (s kappa_s a / 3) sum_q (1/4) (r_q - v_s) . p exp(-jk k . r_q)
     B.nq = NQT;
