@@ -50,11 +50,12 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
     hm_status st;
     for (auto &kv : h->levels) {
         LevelList &L = kv.second;
-        std::vector<Item> small, big;
+        std::vector<Item> small, big, wide, rest;
         L.small_dim = 2;
         L.small_rank = 0;
         for (const Item &it : L.items) {
             const bool fits = it.m <= MRHS_MAX_DIM && it.n <= MRHS_MAX_DIM && it.k <= MRHS_MAX_RANK;
+            (wide_item(it) ? wide : rest).push_back(it);
             (fits ? small : big).push_back(it);
             if (fits) {
                 L.small_dim = std::max<int>(L.small_dim, (int)std::max(even(it.m), even(it.n)));
@@ -65,40 +66,38 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         L.n_big = (int64_t)big.size();
         if ((st = upload(h, &L.d_items, L.items, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_small, small, s)) != HM_OK) return st;
+        // the residual's own list (the long low-rank blocks, a CTA each, largest first; then the
+        // rest, balanced for the round-robin warps) and the block bounds of that list and of the big part
+        L.n_wide = (int64_t)wide.size();
+        std::vector<Item> res = balanced_order(wide, L.n_wide, residual_cost);
+        std::stable_partition(big.begin(), big.end(), wide_item);
+        const std::vector<Item> narrow = balanced_order(rest, residual_warps(h), residual_cost);
+        res.insert(res.end(), narrow.begin(), narrow.end());
         if ((st = upload(h, &L.d_big, big, s)) != HM_OK) return st;
-        // the residual's own list (balanced for its round-robin warps) and the block bounds
-        // of that list and of the big part
-        const std::vector<Item> res = balanced_order(L.items, residual_warps(h), residual_cost);
         if ((st = upload(h, &L.d_res, res, s)) != HM_OK) return st;
         if ((st = dev_alloc(h, (void **)&L.d_bnd, sizeof(float4) * res.size())) != HM_OK) return st;
         if ((st = dev_alloc(h, (void **)&L.d_bnd_big, sizeof(float4) * big.size())) != HM_OK) return st;
         launch_item_bounds(L.d_res, (int64_t)res.size(), h->d_pool32, L.d_bnd, s);
         launch_item_bounds(L.d_big, L.n_big, h->d_pool32, L.d_bnd_big, s);
         HM_CUDA(cudaGetLastError());
-        // the product's lists with tall dense blocks cut into row panels: a panel of rows
-        // [r, r + mr) of a row-major block is itself a dense item with the same row stride
-        auto panels = [](const std::vector<Item> &in, std::vector<Item> &out) {
-            bool cut = false;
-            for (const Item &it : in) {
-                if (it.k != 0 || it.m <= PROD_PANEL) { out.push_back(it); continue; }
-                cut = true;
-                for (int32_t r = 0; r < it.m; r += PROD_PANEL) {
-                    Item q = it;
-                    q.off = it.off + (int64_t)r * even(it.n);
-                    q.row0 = it.row0 + r;
-                    q.m = std::min<int32_t>(PROD_PANEL, it.m - r);
-                    out.push_back(q);
-                }
-            }
-            return cut;
-        };
-        std::vector<Item> pa, pb;
-        panels(L.items, pa);
-        panels(big, pb);
-        // the product kernel hands items to its warps round-robin: sorted by cost, largest
+        // the product's lists with tall dense blocks cut into row panels, long low-rank ones into rank panels
+        std::vector<Item> pw, pa, pb;
+        product_panels(wide, pw);
+        pw = balanced_order(pw, (int64_t)pw.size(), product_cost);
+        L.prod_long = (int64_t)pw.size() >= product_warps(h);
+        if (L.prod_long) pw.clear();
+        L.n_prod_wide = (int64_t)pw.size();
+        // the product kernel hands the rest to its warps round-robin: sorted by cost, largest
         // first, with every other round reversed, each warp gets an even share
-        pa = balanced_order(pa, product_warps(h), product_cost);
-        pb = balanced_order(pb, product_warps(h), product_cost);
+        auto lists = [&](const std::vector<Item> &in, std::vector<Item> &out) {
+            std::vector<Item> p;
+            product_panels(in, p);
+            p = balanced_order(p, product_warps(h), product_cost);
+            out = pw;
+            out.insert(out.end(), p.begin(), p.end());
+        };
+        lists(L.prod_long ? L.items : rest, pa);
+        lists(std::vector<Item>(big.begin() + (L.prod_long ? 0 : L.n_wide), big.end()), pb);
         L.n_prod = (int64_t)pa.size();
         L.n_prod_big = (int64_t)pb.size();
         if ((st = upload(h, &L.d_prod, pa, s)) != HM_OK) return st;
@@ -604,6 +603,14 @@ static hm_status ensure_partials(hm_matrix h)
     return HM_OK;
 }
 
+std::vector<const LevelList *> used_levels(hm_matrix h, int m)
+{
+    std::vector<const LevelList *> v;
+    for (const auto &kv : h->levels)
+        if (kv.first >= 1 && kv.first <= m && !kv.second.items.empty()) v.push_back(&kv.second);
+    return v;
+}
+
 static int64_t level_bytes(hm_matrix h, int lev, bool fp64)
 {
     auto it = h->levels.find(lev);
@@ -619,8 +626,8 @@ static void apply_level(SolveCtx &c, int lev, const void *x, void *z)
     if (c.rec) {
         Phase q = phase(PH_APPLY, c.nrhs);
         q.a = x; q.c = z;
-        q.items = it->second.d_prod ? it->second.d_prod : it->second.d_items;
-        q.n = it->second.d_prod ? it->second.n_prod : (int64_t)it->second.items.size();
+        q.items = it->second.d_prod;
+        q.n = it->second.n_prod;
         c.rec->push_back(q);
         c.units = std::max<int64_t>(c.units, (q.n + 7) / 8);   // a block per warp
         c.launches++;
@@ -903,12 +910,9 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
             c.launches++;
             continue;
         }
-        for (int lev = 1; lev <= c.m; ++lev) {
-            auto it = h->levels.find(lev);
-            if (it == h->levels.end() || it->second.items.empty()) continue;
-            c.launches += launch_apply_items_partials(h, it->second, x, h->ws.d_part, h->partial_elems, nr, c.s,
-                                                      c.res_rb);
-        }
+        const std::vector<const LevelList *> used = used_levels(h, c.m);
+        c.launches += launch_apply_items_partials(h, used.data(), (int)used.size(), x, h->ws.d_part, h->partial_elems,
+                                                  nr, c.s, c.res_rb);
         if (y_next && nr == c.nrhs && leaf_chunks(h, nr) == 1) {
             launch_gather_leaf_update(h, x, c.m, h->ws.d_part, h->partial_elems, bt, out, norms, y_next, nr, c.s);
             c.bytes += leaf_update_bytes(c);
@@ -957,7 +961,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     }
     const bool do_prod = have == h->tune.end();
     if (!do_prod) t = have->second;
-    const LevelList &L = it1->second;
+    const LevelList &L = it1->second, *Lp = &L;
     hm_status st = ensure_workspace(h, nrhs, m);
     if (st != HM_OK) return st;
     if (residual && (st = ensure_partials(h)) != HM_OK) return st;
@@ -1012,7 +1016,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
         if (rb == RB_OWN)
             st = time_it([&] { launch_resid_own(h, L, x, h->ws.d_own, nrhs, s); }, ms);
         else
-            st = time_it([&] { launch_apply_items_partials(h, L, x, h->ws.d_part, h->partial_elems, nr, s, rb); }, ms);
+            st = time_it([&] { launch_apply_items_partials(h, &Lp, 1, x, h->ws.d_part, h->partial_elems, nr, s, rb); }, ms);
         if (st != HM_OK) break;
         const double per_rhs = ms / (rb == RB_OWN ? nrhs : nr);
         if (per_rhs < best) { best = per_rhs; t.res_rb = rb; t.res_ms = ms; }

@@ -53,9 +53,11 @@ struct LevelList {
     // in shared memory, and the rest
     Item *d_small = nullptr, *d_big = nullptr;
     int64_t n_small = 0, n_big = 0;
-    // the FP64-class residual's copy of the item list, in the order that balances its
-    // round-robin warps, and per item of it / of d_big the block bounds of the
+    // the FP64-class residual's copy of the item list: n_wide long low-rank blocks (wide_item;
+    // also the first n_wide of d_big), then the rest in the order that balances its
+    // round-robin warps; and per item of it / of d_big the block bounds of the
     // common-grid residual products (k_item_bounds: largest row and column 1-norms)
+    int64_t n_wide = 0;
     Item *d_res = nullptr;
     float4 *d_bnd = nullptr, *d_bnd_big = nullptr;
     int small_dim = 0, small_rank = 0;   // largest (even) side and rank among the small items
@@ -95,15 +97,15 @@ struct LevelList {
     int64_t n_xch = 0;
     int64_t n_dense = 0, n_lowrank = 0;
     int64_t elems = 0;            // stored complex elements
-    // the FP32 product's own copies of the item list and of its big part, with every dense
-    // block of more than PROD_PANEL rows cut into row panels (the product kernel gives each
-    // item to one warp: a leaf of ~1,000 unknowns would otherwise leave the GPU idle), in the
-    // order that balances the kernel's round-robin warps (largest first, snake rounds)
+    // the FP32 product's own copies of the item list and of its big part, long blocks cut into
+    // panels (product_panels): the n_prod_wide panels of long low-rank blocks, a CTA each, then
+    // the rest, a warp each, in the order that balances the kernel's round-robin warps (largest
+    // first, snake rounds).  Panels that fill the warps by their number go there (prod_long;
+    // plate of 67,200 unknowns: 2.13 ms a solve, a CTA each 2.17).
     Item *d_prod = nullptr, *d_prod_big = nullptr;
-    int64_t n_prod = 0, n_prod_big = 0;
+    int64_t n_prod = 0, n_prod_big = 0, n_prod_wide = 0;
+    bool prod_long = false;
 };
-constexpr int PROD_PANEL = 64;
-
 // One phase of the one-launch solve (k_persist.cu): every kernel the solve would
 // launch becomes a phase of one cooperative kernel, with a grid-wide barrier
 // between consecutive phases.
@@ -322,15 +324,18 @@ void launch_zero(void *p, size_t bytes, cudaStream_t s);
 // Returns the number of kernels it enqueued.
 int launch_apply_items(hm_matrix h, const LevelList &L, const void *x, void *z, int nrhs, bool fp64,
                         cudaStream_t s, int rb = -1);
-// FP64-class (Dot2) products of every block of a level into its partial slots (no atomics)
 // warps of the FP32 product kernel's persistent grid (k_product.cu) and of the
 // FP64-class residual kernel's (k_residual.cu)
 int64_t product_warps(hm_matrix h);
 int64_t residual_warps(hm_matrix h);
 // the residual products' block bounds of items[0 .. n) (k_residual.cu)
 void launch_item_bounds(const Item *items, int64_t n, const float2 *pool, float4 *bnd, cudaStream_t s);
-int launch_apply_items_partials(hm_matrix h, const LevelList &L, const float2 *x, dot2::cdf *part, int64_t pstride,
-                                int nrhs, cudaStream_t s, int rb = -1);   // returns the kernels enqueued
+// FP64-class products of every block of the n levels L into their partial slots (no atomics); returns
+// the kernels enqueued
+int launch_apply_items_partials(hm_matrix h, const LevelList *const *L, int n, const float2 *x, dot2::cdf *part,
+                                int64_t pstride, int nrhs, cudaStream_t s, int rb = -1);
+// the levels 1..m that have blocks
+std::vector<const LevelList *> used_levels(hm_matrix h, int m);
 // per leaf: acc = D x + sum of the leaf's partial slots of levels 1..m (double-float, fixed order);
 // out = b - acc (+ norms) when b is given, else out = acc (rounded to complex64)
 void launch_gather_acc64(hm_matrix h, const float2 *x, int m, const dot2::cdf *part, int64_t pstride,

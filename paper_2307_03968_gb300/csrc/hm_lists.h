@@ -445,6 +445,40 @@ inline bool build_mm_lists(const std::map<int32_t, std::vector<TcProd>> &by_out,
     return true;
 }
 
+// The FP32 product gives each item of its list to one warp, so long blocks are cut: a dense
+// block of more than PROD_PANEL rows into row panels (rows [r, r + mr) of a row-major block are
+// themselves a dense item of the same row stride), a low-rank block longer than 64 into panels of
+// PROD_RANK rank rows (their sum is the block's product; the kernel works in steps of that many
+// rank rows anyway, so the panels add no memory traffic).  A low-rank item's pad is half the
+// distance (m and n are even) from its U^T panel to its V panel (panel_voff).  (30,720-unknown sphere, level 2: 80 blocks of 480 x 480 and
+// more took 152 us on 80 warps.)
+constexpr int PROD_PANEL = 64;
+constexpr int PROD_RANK = 8;
+// low-rank blocks longer than 64 x 64
+inline bool wide_item(const Item &it) { return it.k > 0 && (it.m > 64 || it.n > 64); }
+HM_HD inline int64_t panel_voff(const Item &it) { return 2 * (int64_t)(uint32_t)it.pad; }
+inline void product_panels(const std::vector<Item> &in, std::vector<Item> &out)
+{
+    for (const Item &it : in) {
+        const int32_t step = it.k == 0 ? PROD_PANEL : wide_item(it) ? PROD_RANK : it.k;
+        const int32_t len = it.k == 0 ? it.m : it.k;
+        for (int32_t r = 0; r < len; r += step) {
+            Item q = it;
+            const int32_t c = std::min(step, len - r);
+            if (it.k == 0) {
+                q.off = it.off + (int64_t)r * even(it.n);
+                q.row0 = it.row0 + r;
+                q.m = c;
+            } else {
+                q.off = it.off + (int64_t)r * it.m;
+                q.pad = (int32_t)(uint32_t)(((int64_t)(it.k - r) * it.m + (int64_t)r * it.n) / 2);
+                q.k = c;
+            }
+            out.push_back(q);
+        }
+    }
+}
+
 // items reordered for a persistent kernel whose nw warps take items t, t + nw, ...:
 // sorted by cost, largest first, and every odd round of nw reversed (a snake), so that
 // the warps' sums match.  Cost of the product: stored bytes plus a fixed 2 KB for the

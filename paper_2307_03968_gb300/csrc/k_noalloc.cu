@@ -89,13 +89,10 @@ extern "C" hm_status hm_residual_noalloc(hm_matrix h, const void *b, int64_t ldb
     HM_CUDA(cudaMemsetAsync(dn, 0, 2 * sizeof(double) * nrhs, s));
     launch_permute_in(b, ldb, bt, h->pN, h->d_pperm, nrhs, false, s);
     launch_permute_in(x, ldx, xt, h->pN, h->d_pperm, nrhs, false, s);
+    const std::vector<const LevelList *> used = used_levels(h, m);
     for (int j = 0; j < nrhs; ++j) {   // one right-hand side at a time through the partial slots
         const float2 *xj = xt + (int64_t)j * h->pN;
-        for (int lev = 1; lev <= m; ++lev) {
-            auto it = h->levels.find(lev);
-            if (it == h->levels.end() || it->second.items.empty()) continue;
-            launch_apply_items_partials(h, it->second, xj, dpart, h->partial_elems, 1, s);
-        }
+        launch_apply_items_partials(h, used.data(), (int)used.size(), xj, dpart, h->partial_elems, 1, s);
         launch_gather_acc64(h, xj, m, dpart, h->partial_elems, bt + (int64_t)j * h->pN, rt + (int64_t)j * h->pN,
                             dn + 2 * j, 1, s);
     }

@@ -119,7 +119,7 @@ __device__ bool run_phases(const Phase *phases, int n_phases, const PersistCtx &
                 const Item it = P.items[t];
                 for (int r = 0; r < P.nrhs; ++r) {
                     if (it.k == 0) dense_item<float, float>(it, c.pool, x + r * c.pN, z + r * c.pN, xs, lane);
-                    else lowrank_item<float, float>(it, c.pool, x + r * c.pN, z + r * c.pN, lane);
+                    else lowrank_item<float, float, true>(it, panel_voff(it), c.pool, x + r * c.pN, z + r * c.pN, lane);
                 }
             }
             break;

@@ -77,9 +77,11 @@ __device__ __forceinline__ void dense_item(const Item &it, const typename CT<T>:
 }
 
 // Low-rank far block U V with U^T (k x m) and V (k x n) row-major, m and n the
-// padded (even) cluster lengths:  z_I += U (V x_J),  z_J += V^T (U^T x_I).
-template <class T, class A>
-__device__ __forceinline__ void lowrank_item(const Item &it, const typename CT<T>::C *__restrict__ pool,
+// padded (even) cluster lengths:  z_I += U (V x_J),  z_J += V^T (U^T x_I).  V starts
+// voff elements after U^T: k m for a whole block, further for a panel of its rank rows.
+// LONG: blocks longer than 64 are taken too.
+template <class T, class A, bool LONG>
+__device__ __forceinline__ void lowrank_item(const Item &it, int64_t voff, const typename CT<T>::C *__restrict__ pool,
                                              const typename CT<T>::C *HM_XR x,
                                              typename CT<A>::C *HM_XR z, int lane)
 {
@@ -87,9 +89,9 @@ __device__ __forceinline__ void lowrank_item(const Item &it, const typename CT<T
     using CA = typename CT<A>::C;
     const int m = it.m, n = it.n, k = it.k;
     const CTy *UT = pool + it.off;
-    const CTy *V = UT + (int64_t)k * m;
+    const CTy *V = UT + voff;
     const CA zero = czero(CA());
-    if (m <= 64 && n <= 64) {
+    if (!LONG || (m <= 64 && n <= 64)) {
         // registers hold a chunk of 8 rank rows of both panels
         const int i = 2 * lane;
         const bool iv = i < m, jv = i < n;

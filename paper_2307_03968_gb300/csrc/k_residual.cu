@@ -17,17 +17,45 @@ using namespace kc;
 using namespace dot2;
 constexpr int APPLY_WARPS = 8;
 
+// up to RESID_LEVELS item lists in one launch, so that the few blocks of the higher levels run
+// beside the first level's: the first `wide` CTAs take one long low-rank block (all the lists'
+// first n_wide items) and right-hand side each, the others the rest of the lists, a warp per block
+constexpr int RESID_LEVELS = 8;
+struct ResidLists {
+    const Item *items[RESID_LEVELS];
+    const float4 *bnd[RESID_LEVELS];
+    int32_t n_wide[RESID_LEVELS];
+    int64_t n_items[RESID_LEVELS];
+    int n;
+};
+
 __global__ void __launch_bounds__(APPLY_WARPS * 32, 2)
-k_residual_items(const Item *__restrict__ items, const float4 *__restrict__ bnd, int64_t n_items,
-                 const float2 *__restrict__ pool, const float2 *__restrict__ x, int64_t ldx, cdf *__restrict__ part,
-                 int64_t pstride, int nrhs)
+k_residual_items(const __grid_constant__ ResidLists R, int wide, const float2 *__restrict__ pool,
+                 const float2 *__restrict__ x, int64_t ldx, cdf *__restrict__ part, int64_t pstride, int nrhs)
 {
+    static_assert(WW == APPLY_WARPS, "a CTA takes one long block");
     __shared__ __align__(16) float2 xs_all[APPLY_WARPS][GRID_MAX];
+    __shared__ cdf ts[2][WK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t nw = (int64_t)gridDim.x * APPLY_WARPS;
-    for (int64_t t = (int64_t)blockIdx.x * APPLY_WARPS + w; t < n_items; t += nw) {
-        const Item it = items[t];
-        for (int r = 0; r < nrhs; ++r) resid_item(it, bnd, t, pool, x + r * ldx, part + r * pstride, xs_all[w], lane);
+    if ((int)blockIdx.x < wide) {
+        const int r = blockIdx.x % nrhs;
+        int t = blockIdx.x / nrhs, q = 0;
+        while (t >= R.n_wide[q]) t -= R.n_wide[q++];
+        lowrank_item_w(R.items[q][t], pool, x + r * ldx, part + r * pstride, ts, lane, w);
+        return;
+    }
+    const int64_t nw = (int64_t)(gridDim.x - wide) * APPLY_WARPS;
+    int64_t t = (int64_t)(blockIdx.x - wide) * APPLY_WARPS + w;
+    for (int q = 0; q < R.n; ++q) {
+        const Item *__restrict__ items = R.items[q];
+        const float4 *__restrict__ bnd = R.bnd[q];
+        const int64_t n_items = R.n_items[q];
+        for (t += R.n_wide[q]; t < n_items; t += nw) {
+            const Item it = items[t];
+            for (int r = 0; r < nrhs; ++r)
+                resid_item(it, bnd, t, pool, x + r * ldx, part + r * pstride, xs_all[w], lane);
+        }
+        t -= n_items;
     }
 }
 
@@ -107,27 +135,40 @@ void launch_gather_leaf_update(hm_matrix h, const float2 *x, int m, const cdf *p
         h->d_csr_idx, part, pstride, b, out, norms, y);
 }
 
-int launch_apply_items_partials(hm_matrix h, const LevelList &L, const float2 *x, cdf *part, int64_t pstride,
-                                int nrhs, cudaStream_t s, int rb)
+int launch_apply_items_partials(hm_matrix h, const LevelList *const *Ls, int n_lists, const float2 *x, cdf *part,
+                                int64_t pstride, int nrhs, cudaStream_t s, int rb)
 {
-    int launched = 0;
-    const Item *list = L.d_res;
-    const float4 *bnd = L.d_bnd;
-    int64_t n = (int64_t)L.items.size();
     if (rb < 0) rb = nrhs < MRHS_MIN_RHS ? 0 : nrhs <= 8 ? 8 : 16;
-    if (rb > 0 && nrhs > 1 && L.n_small > 0) {
-        // many right-hand sides: blocks that fit shared memory are read once per chunk
-        launch_apply_items_partials_mrhs(h, L, x, part, pstride, nrhs, s, rb);
-        launched = 1;
-        list = L.d_big;
-        bnd = L.d_bnd_big;
-        n = L.n_big;
+    int launched = 0, q = 0;
+    while (q < n_lists) {
+        ResidLists R{};
+        int64_t wide = 0, rest = 0;
+        for (; q < n_lists && R.n < RESID_LEVELS; ++q) {
+            const LevelList &L = *Ls[q];
+            // many right-hand sides: blocks that fit shared memory are read once per chunk
+            const bool m = rb > 0 && nrhs > 1 && L.n_small > 0;
+            if (m) {
+                launch_apply_items_partials_mrhs(h, L, x, part, pstride, nrhs, s, rb);
+                ++launched;
+            }
+            const int64_t n = m ? L.n_big : (int64_t)L.items.size();
+            if (n == 0) continue;
+            R.items[R.n] = m ? L.d_big : L.d_res;
+            R.bnd[R.n] = m ? L.d_bnd_big : L.d_bnd;
+            R.n_wide[R.n] = (int32_t)L.n_wide;
+            R.n_items[R.n] = n;
+            rest += n - L.n_wide;
+            wide += L.n_wide;
+            ++R.n;
+        }
+        if (R.n == 0) continue;
+        int64_t g = std::min(residual_warps(h) / APPLY_WARPS, (rest + APPLY_WARPS - 1) / APPLY_WARPS);
+        wide *= nrhs;
+        k_residual_items<<<(unsigned)(wide + g), APPLY_WARPS * 32, 0, s>>>(R, (int)wide, h->d_pool32, x, h->pN, part,
+                                                                           pstride, nrhs);
+        ++launched;
     }
-    if (n == 0) return launched;
-    int g = (int)(residual_warps(h) / APPLY_WARPS);
-    if ((int64_t)g * APPLY_WARPS > n) g = (int)((n + APPLY_WARPS - 1) / APPLY_WARPS);
-    k_residual_items<<<g, APPLY_WARPS * 32, 0, s>>>(list, bnd, n, h->d_pool32, x, h->pN, part, pstride, nrhs);
-    return launched + 1;
+    return launched;
 }
 
 int64_t residual_warps(hm_matrix h)

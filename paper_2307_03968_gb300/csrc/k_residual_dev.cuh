@@ -460,6 +460,68 @@ __device__ __forceinline__ void lowrank_item_c(const Item &it, const float2 *__r
     }
 }
 
+// The same block by a CTA of WW warps: stage 1 gives a warp four rank rows of one side, stage 2
+// 64 columns of one side over all the rank rows.  One warp for the whole block is a serial
+// chain of (m + n) k / 128 loads; here eight share it (7,500-unknown import with 984 such
+// blocks on levels 2 and 3: 24 us level 1, then 43 and 95 us, one warp each; 52 us now for
+// the three levels in one launch).
+// ts: 2 x WK intermediates of shared memory.
+constexpr int WW = 8, WK = 32;   // warps a block, rank rows a pass
+__device__ __forceinline__ void lowrank_item_w(const Item &it, const float2 *__restrict__ pool, const float2 *HM_XR x,
+                                               cdf *HM_XR part, cdf (*ts)[WK], int lane, int w)
+{
+    const int m = it.m, n = it.n, k = it.k;
+    const float2 *F[2] = {pool + it.off, pool + it.off + (int64_t)k * m};   // U^T, V
+    const int64_t len[2] = {m, n};
+    const float2 *xin[2] = {x + it.row0, x + it.col0};
+    for (int k0 = 0; k0 < k; k0 += WK) {
+        const int kc = min(WK, k - k0), ng = (kc + 3) / 4;
+        // ts[0] = U^T x_I, ts[1] = V x_J (rank rows k0 .. k0 + kc - 1)
+        for (int q = w; q < 2 * ng; q += WW) {
+            const int side = q & 1, l0 = 4 * (q >> 1);
+            const float2 *A = (side ? F[1] : F[0]) + (k0 + l0) * (side ? len[1] : len[0]);
+            const float2 *xs = side ? xin[1] : xin[0];
+            const int64_t ln = side ? len[1] : len[0];
+            cdf t[4];
+#pragma unroll
+            for (int l = 0; l < 4; ++l) t[l] = cdf_zero();
+            for (int64_t i = 2 * lane; i < ln; i += 64) {
+                const Pair<float> xp = ld_vec(xs + i);
+#pragma unroll
+                for (int l = 0; l < 4; ++l)
+                    if (l0 + l < kc) {
+                        const Pair<float> a = ld_cached(A + l * ln + i);
+                        cdot2(t[l], a.a, xp.a);
+                        cdot2(t[l], a.b, xp.b);
+                    }
+            }
+            reduce_cdf<4>(t, lane);
+            if (lane < 4) ts[side][l0 + lane] = t[0];
+        }
+        __syncthreads();
+        const int c_m = (m + 63) / 64, c_n = (n + 63) / 64;
+        for (int q = w; q < c_m + c_n; q += WW) {
+            const bool side = q >= c_m;
+            const int64_t ln = side ? len[1] : len[0];
+            const int64_t i = 64 * (int64_t)(side ? q - c_m : q) + 2 * lane;
+            if (i >= ln) continue;
+            const float2 *A = (side ? F[1] : F[0]) + k0 * ln + i;
+            cdf o0 = cdf_zero(), o1 = cdf_zero();
+#pragma unroll 4
+            for (int l = 0; l < kc; ++l) {
+                const Pair<float> a = ld_cached(A + l * ln);
+                const cdf t = ts[side ? 0 : 1][l];
+                cdot2_df(o0, a.a, t);
+                cdot2_df(o1, a.b, t);
+            }
+            cdf *d = part + it.pad + (side ? m : 0) + i;
+            if (k0 == 0) { d[0] = o0; d[1] = o1; }
+            else { d[0] = cdf_add(d[0], o0); d[1] = cdf_add(d[1], o1); }
+        }
+        __syncthreads();
+    }
+}
+
 // The residual products of one block (item t of a list with bounds bnd): on the
 // common grids where it fits (at most 64 x 64, rank <= 64), else the short-chain
 // and Dot2 bodies above.  xs: GRID_MAX float2 of the warp's shared memory.
