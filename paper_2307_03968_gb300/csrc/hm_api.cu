@@ -153,8 +153,10 @@ static hm_status ensure_own_lists(hm_matrix h, cudaStream_t s)
         std::vector<TcUnit> rcu;
         std::vector<TcProd> rcp;
         build_owner_lists(directed_products(small_items(L)), rcu, rcp);
-        L.n_rcu = (int64_t)rcu.size();
-        if ((st = upload(h, &L.d_rcu, rcu, s)) != HM_OK || (st = upload(h, &L.d_rcp, rcp, s)) != HM_OK ||
+        std::vector<RcUnit> parts;
+        L.own_parts = split_owner_units(rcu, rcp, 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), parts);
+        L.n_rcu = (int64_t)parts.size();
+        if ((st = upload(h, &L.d_rcu, parts, s)) != HM_OK || (st = upload(h, &L.d_rcp, rcp, s)) != HM_OK ||
             (st = dev_alloc(h, (void **)&L.d_rcb, sizeof(float2) * rcp.size())) != HM_OK)
             return st;
         launch_prod_bounds(L.d_rcp, (int64_t)rcp.size(), h->d_pool32, L.d_rcb, s);
@@ -490,13 +492,13 @@ static hm_status ensure_workspace(hm_matrix h, int nrhs, int m)
 // FP64 owner sums of the owner-computes residual ([level][part][RHS][pN] for the
 // workspace's RHS count and m levels); allocated only by the calls that form a
 // residual with that kernel, before any capture
-// owner-sum arrays of levels 1..m: one a level, or its mm_parts on the matrix instructions
+// owner-sum arrays of levels 1..m: a level's own_parts, or its mm_parts on the matrix instructions
 static int own_arrays(hm_matrix h, int m, bool mm)
 {
     int n = 0;
     for (int lev = 1; lev <= m; ++lev) {
         auto it = h->levels.find(lev);
-        if (it != h->levels.end() && !it->second.items.empty()) n += mm ? it->second.mm_parts : 1;
+        if (it != h->levels.end() && !it->second.items.empty()) n += mm ? it->second.mm_parts : it->second.own_parts;
     }
     return n;
 }
@@ -870,9 +872,9 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
                 c.launches += launch_mm_resid(h, it->second, xt, h->ws.d_own + at * lstride, lstride, c.nrhs, h->ws.d_mm, c.s);
                 at += it->second.mm_parts;
             } else {
-                launch_resid_own(h, it->second, xt, h->ws.d_own + at * lstride, c.nrhs, c.s);
+                launch_resid_own(h, it->second, xt, h->ws.d_own + at * lstride, lstride, c.nrhs, c.s);
                 c.launches++;
-                at++;
+                at += it->second.own_parts;
             }
         }
         launch_gather_own(h, xt, arrays, h->ws.d_own, lstride, bt, out, norms, c.nrhs, c.s);
@@ -1014,7 +1016,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
         }
         double ms = 0;
         if (rb == RB_OWN)
-            st = time_it([&] { launch_resid_own(h, L, x, h->ws.d_own, nrhs, s); }, ms);
+            st = time_it([&] { launch_resid_own(h, L, x, h->ws.d_own, (int64_t)nrhs * h->pN, nrhs, s); }, ms);
         else
             st = time_it([&] { launch_apply_items_partials(h, &Lp, 1, x, h->ws.d_part, h->partial_elems, nr, s, rb); }, ms);
         if (st != HM_OK) break;

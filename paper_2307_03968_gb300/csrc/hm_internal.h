@@ -76,8 +76,9 @@ struct LevelList {
     // first call that runs it
     bool own_built = false;
     TcProd *d_rcp = nullptr;
-    TcUnit *d_rcu = nullptr;
+    RcUnit *d_rcu = nullptr;
     int64_t n_rcu = 0;
+    int own_parts = 1;            // parts a cluster at most
     float2 *d_rcb = nullptr;      // per product of d_rcp: its common-grid bounds (k_prod_bounds)
     // the same directed products as two dense products on the matrix instructions (k_mm.cu,
     // hm_lists.h build_mm_lists): product units, residual units (mm_parts a cluster at most), scales
@@ -407,7 +408,8 @@ int launch_mm_resid(hm_matrix h, const LevelList &L, const float2 *x, double2 *o
 size_t mm_ws_bytes(const LevelList &L, int nrhs, bool res);
 // owner-computes FP64-class products of a level's small items into own ([RHS][pN]) on the FP32
 // pipes (k_resid_own.cu), and their common-grid bounds of prods[0 .. n)
-void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int nrhs, cudaStream_t s);
+void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int64_t lstride, int nrhs,
+                      cudaStream_t s);
 void launch_prod_bounds(const TcProd *prods, int64_t n, const float2 *pool, float2 *out, cudaStream_t s);
 struct MmPackArgs {
     const MmSet *sets;

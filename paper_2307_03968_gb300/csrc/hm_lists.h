@@ -144,6 +144,40 @@ inline void build_owner_lists(const std::map<int32_t, std::vector<TcProd>> &by_o
     }
 }
 
+// The owner units cut into parts of about equal cost, so that a call has `target` units a
+// right-hand-side group where there are fewer clusters than that (each part sums into an array of
+// its own, which the gather adds in order), parts of at least 8 products; returns the parts.
+struct RcUnit { int32_t out0, mlen, p0, p1, part; };
+inline int split_owner_units(const std::vector<TcUnit> &units, const std::vector<TcProd> &prods, int64_t target,
+                             std::vector<RcUnit> &out)
+{
+    auto cost = [](const TcProd &p) { return (int64_t)(p.rank > 0 ? 2 * p.rank + 24 : p.klen + 16); };
+    const int64_t want = units.empty() ? 1 : (target + (int64_t)units.size() - 1) / (int64_t)units.size();
+    int parts = 1;
+    std::vector<std::pair<int64_t, RcUnit>> rs;
+    for (const TcUnit &u : units) {
+        const int n = (int)std::max<int64_t>(1, std::min<int64_t>(want, (u.p1 - u.p0) / 8));
+        int64_t total = 0, run = 0, from = 0;
+        for (int32_t p = u.p0; p < u.p1; ++p) total += cost(prods[p]);
+        RcUnit r{u.out0, u.mlen, u.p0, u.p0, 0};
+        for (int32_t p = u.p0; p < u.p1; ++p) {
+            run += cost(prods[p]);
+            r.p1 = p + 1;
+            if (p + 1 == u.p1 || (r.part + 1 < n && run * n >= total * (r.part + 1))) {
+                rs.push_back({run - from, r});
+                parts = std::max(parts, r.part + 1);
+                r.p0 = p + 1;
+                ++r.part;
+                from = run;
+            }
+        }
+    }
+    std::stable_sort(rs.begin(), rs.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+    out.clear();
+    for (const auto &r : rs) out.push_back(r.second);
+    return parts;
+}
+
 // The tensor-core product's lists (k_mrhs_tc.cu), two launches.
 //  - Stage 1 of every low-rank directed product, T = W X_in (W = V forward, U^T mirrored),
 //    is batched over the products that share an input cluster: each product takes

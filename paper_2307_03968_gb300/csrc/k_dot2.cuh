@@ -91,8 +91,39 @@ __device__ __forceinline__ cdf cdf_add(const cdf &a, const cdf &b) { return {df_
 // within 2^-39, against a few units for Dot2 (an exact model of both is in the
 // tests).  That is 10^4 times and more below FP32 summation, and below the
 // complex64 rounding of the residual these sums feed.
-struct xacc { float tau, r; };
-struct cxacc { xacc re, im; };
+// The real and the imaginary part of a complex chain step take the same operations, so they
+// run as packed pairs (fma / add / sub.rn.f32x2: two IEEE operations an instruction, the
+// arithmetic unchanged): 8 instructions a complex product instead of 16.  The FMA units take
+// as long for a pair as for two single operations, but the kernels were bound by issue slots.
+struct cxacc { float2 tau, r; };   // (re, im)
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return reinterpret_cast<float2 &>(d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return reinterpret_cast<float2 &>(d);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return reinterpret_cast<float2 &>(d);
+}
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 rot(float2 a) { return make_float2(-a.y, a.x); }   // i a
 
 // the least power of two >= v for finite v >= 0 (0 for 0, 2^-126 for subnormals)
 __device__ __forceinline__ float pow2_ceil(float v)
@@ -108,41 +139,33 @@ __device__ __forceinline__ float linf(float2 a) { return fmaxf(fabsf(a.x), fabsf
 constexpr float CHAIN_MARGIN = 2.0f + 0x1p-16f;
 __device__ __forceinline__ float chain_sigma(float sa, float mb) { return pow2_ceil(CHAIN_MARGIN * sa * mb); }
 
-__device__ __forceinline__ void xfirst(xacc &c, float sigma, float a, float b)
+// both parts of one real factor: tau' - tau is exact, and so is its negative
+__device__ __forceinline__ void xstep(cxacc &c, float2 a, float2 b)
 {
-    c.tau = __fmaf_rn(a, b, sigma);
-    c.r = __fmaf_rn(a, b, -__fsub_rn(c.tau, sigma));
-}
-__device__ __forceinline__ void xstep(xacc &c, float a, float b)
-{
-    const float t2 = __fmaf_rn(a, b, c.tau);
-    c.r = __fadd_rn(c.r, __fmaf_rn(a, b, -__fsub_rn(t2, c.tau)));
+    const float2 t2 = fma2(a, b, c.tau);
+    c.r = add2(c.r, fma2(a, b, sub2(c.tau, t2)));
     c.tau = t2;
+}
+// c += a * b:  (re, im) += a b.re, then += (i a) b.im
+__device__ __forceinline__ void cxstep(cxacc &c, float2 a, float2 b)
+{
+    xstep(c, a, dup(b.x));
+    xstep(c, rot(a), dup(b.y));
 }
 // c = a * b (the chain's first complex term)
 __device__ __forceinline__ void cxfirst(cxacc &c, float sigma, float2 a, float2 b)
 {
-    xfirst(c.re, sigma, a.x, b.x);
-    xstep(c.re, -a.y, b.y);
-    xfirst(c.im, sigma, a.x, b.y);
-    xstep(c.im, a.y, b.x);
-}
-// c += a * b
-__device__ __forceinline__ void cxstep(cxacc &c, float2 a, float2 b)
-{
-    xstep(c.re, a.x, b.x);
-    xstep(c.re, -a.y, b.y);
-    xstep(c.im, a.x, b.y);
-    xstep(c.im, a.y, b.x);
+    const float2 s = dup(sigma);
+    c.tau = fma2(a, dup(b.x), s);
+    c.r = fma2(a, dup(b.x), sub2(s, c.tau));
+    xstep(c, rot(a), dup(b.y));
 }
 // c += a * (b.hi + b.lo) for a double-float b: the leading part through the
 // chain (its bound uses |b.hi|), the trailing part (2^-24 of it) into r
 __device__ __forceinline__ void cx_lo(cxacc &c, float2 a, const cdf &b)
 {
-    c.re.r = __fmaf_rn(a.x, b.re.lo, c.re.r);
-    c.re.r = __fmaf_rn(-a.y, b.im.lo, c.re.r);
-    c.im.r = __fmaf_rn(a.x, b.im.lo, c.im.r);
-    c.im.r = __fmaf_rn(a.y, b.re.lo, c.im.r);
+    c.r = fma2(a, dup(b.re.lo), c.r);
+    c.r = fma2(rot(a), dup(b.im.lo), c.r);
 }
 __device__ __forceinline__ void cxfirst_df(cxacc &c, float sigma, float2 a, const cdf &b)
 {
@@ -157,7 +180,8 @@ __device__ __forceinline__ void cxstep_df(cxacc &c, float2 a, const cdf &b)
 // the chain's sum as a double-float: the exact grid part and the remainder
 __device__ __forceinline__ cdf cxclose(const cxacc &c, float sigma)
 {
-    return {{__fsub_rn(c.re.tau, sigma), c.re.r}, {__fsub_rn(c.im.tau, sigma), c.im.r}};
+    const float2 g = sub2(c.tau, dup(sigma));
+    return {{g.x, c.r.x}, {g.y, c.r.y}};
 }
 // ---------------------------------------------------------------------------
 // Chains on a common grid.  When every chain that feeds one output sum takes the
@@ -174,7 +198,16 @@ __device__ __forceinline__ cdf cxclose(const cxacc &c, float sigma)
 // chain step, sigma being at most 4.01 times the bound of the sum.
 constexpr float GRID_MARGIN = 2.0f + 0x1p-10f;
 __device__ __forceinline__ float grid_sigma(float bound, float mb) { return pow2_ceil(GRID_MARGIN * bound * mb); }
-__device__ __forceinline__ void cx_start(cxacc &c, float sigma) { c = {{sigma, 0.f}, {sigma, 0.f}}; }
+__device__ __forceinline__ void cx_start(cxacc &c, float sigma) { c = {dup(sigma), dup(0.f)}; }
+// the four values a lane reduction of a chain sums: grid parts and remainders (re grid, re rem, im grid, im rem)
+__device__ __forceinline__ void cx_values(float *v, const cxacc &c, float sigma)
+{
+    const float2 g = sub2(c.tau, dup(sigma));
+    v[0] = g.x;
+    v[1] = c.r.x;
+    v[2] = g.y;
+    v[3] = c.r.y;
+}
 // one step of a transposing warp reduction: of the pair (v[j], v[j + H]) this lane
 // keeps the upper one when its lane bit `mask` is set, and adds the partner lane's
 // copy of it; after the steps for masks M, M/2, ..., 1 over V values, each lane

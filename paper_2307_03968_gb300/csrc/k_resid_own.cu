@@ -2,9 +2,10 @@
 // (the refinement residual r = b - A_m x of the solve; the block products are
 // eq. 6 and eq. 8 of arxiv 2307.03968 with the half storage of §III).
 //
-// A work unit is one output cluster O of a level and one group of RG right-hand
-// sides (16, or 8 for calls with few right-hand sides, so that there are enough
-// units to balance).  The CTA walks every directed product into O (the stored
+// A work unit is one output cluster O of a level, or a part of its products where there are few
+// clusters (split_owner_units: 7,500 unknowns, 128 clusters, 50 right-hand sides: 512 whole units
+// leave the 608 places of the chip a single uneven wave), and one group of RG right-hand
+// sides (16, or 8 for calls with few right-hand sides).  The CTA walks the directed products into O (the stored
 // blocks with O as row cluster, and mirrored, those with O as column cluster;
 // dense or low-rank), in a fixed order, and keeps the sums in registers as
 // double-float complex numbers.  Each directed product is summed, per output row
@@ -35,25 +36,60 @@ using namespace dot2;
 constexpr int RGMAX = 16;        // right-hand sides per unit (at most)
 constexpr int BS = 65;           // float2 stride of a staged K row of a block (odd: conflict-free staging)
 constexpr int WS = 33;           // float2 stride of a staged K row of W (rank <= 32)
-constexpr int XS = 18;           // float2 stride of a staged K row of x (16 RHS, 16-byte aligned rows)
+constexpr int XP = 9;            // float4 stride of a staged K row of x (8 pairs of right-hand sides)
 constexpr int SM_B = 64 * WS + 32 * BS;   // float2: W (64 x WS) then Y (32 x BS), or a dense block (64 x BS)
-constexpr int SM_X = 64 * XS;
-constexpr int SM_T = 32 * RGMAX; // cdf: T = W x (rank x RG RHS)
+constexpr int SM_X = 64 * XP;
+constexpr int SM_T = 32 * RGMAX; // float4: T = W x (rank x RG / 2 pairs of RHS x leading and trailing parts)
 static_assert(64 * BS <= SM_B, "a dense block fits the block area");
 
 struct alignas(16) Smem {
     float2 b[SM_B];
-    float2 x[SM_X];
-    cdf t[SM_T];
+    float4 x[SM_X];
+    float4 t[SM_T];
     float mx[2 * RGMAX];         // max |x|_inf over K indices 32h..32h+31 (h = 0, 1), per right-hand side
 };
 
-// stage x of the input cluster: xs[j * XS + q] = x[(r0 + q) * ldx + in0 + j] for j < klen, q < nr,
+// The chains of two right-hand sides q, q + 1 as packed pairs (k_dot2.cuh xstep): x is staged as
+// (re_q, re_q+1, im_q, im_q+1), so that the right-hand sides need no rearranged copies, and the
+// block element's duplicated parts serve all of a thread's pairs.  8 instructions a complex
+// product and right-hand side instead of 16: 0.845 to TODO ms at 7,500 unknowns, 50 right-hand sides.
+struct chain2 { float2 tr, rr, ti, ri; };   // real part: grid sum, remainder; imaginary part
+__device__ __forceinline__ void c2_start(chain2 &c, float2 sigma) { c = {sigma, dup(0.f), sigma, dup(0.f)}; }
+__device__ __forceinline__ void step2(float2 &tau, float2 &r, float2 a, float2 b)
+{
+    const float2 t2 = fma2(a, b, tau);
+    r = add2(r, fma2(a, b, sub2(tau, t2)));
+    tau = t2;
+}
+// c += a x for a block element a and the pair's x
+__device__ __forceinline__ void c2_step(chain2 &c, float2 a, float4 x)
+{
+    const float2 re = make_float2(x.x, x.y), im = make_float2(x.z, x.w);
+    step2(c.tr, c.rr, dup(a.x), re);
+    step2(c.tr, c.rr, dup(-a.y), im);
+    step2(c.ti, c.ri, dup(a.x), im);
+    step2(c.ti, c.ri, dup(a.y), re);
+}
+// the trailing parts of a double-float x into the remainders
+__device__ __forceinline__ void c2_lo(chain2 &c, float2 a, float4 x)
+{
+    const float2 re = make_float2(x.x, x.y), im = make_float2(x.z, x.w);
+    c.rr = fma2(dup(-a.y), im, fma2(dup(a.x), re, c.rr));
+    c.ri = fma2(dup(a.y), re, fma2(dup(a.x), im, c.ri));
+}
+__device__ __forceinline__ void c2_fold(cdf (&acc)[2], const chain2 &c, float2 sigma)
+{
+    const float2 gr = sub2(c.tr, sigma), gi = sub2(c.ti, sigma);
+    acc[0] = cdf_add(acc[0], {{gr.x, c.rr.x}, {gi.x, c.ri.x}});
+    acc[1] = cdf_add(acc[1], {{gr.y, c.rr.y}, {gi.y, c.ri.y}});
+}
+
+// stage x of the input cluster: pair q / 2 of xs[j * XP + ..] = x[(r0 + q) * ldx + in0 + j] for j < klen, q < nr,
 // 0 for the rest of j < roundup4(klen); mx[2 q + h] = max over j = 32h..32h+31 of |x|_inf.
 // Every thread runs the same number of iterations (RG * 64 is a multiple of RT), and a warp
 // covers 32 consecutive j of one q.
 template <int RG, int RT>
-__device__ __forceinline__ void stage_x(float2 *xs, float *mx, const float2 *__restrict__ x, int64_t ldx, int r0,
+__device__ __forceinline__ void stage_x(float4 *xs, float *mx, const float2 *__restrict__ x, int64_t ldx, int r0,
                                         int nr, int in0, int klen)
 {
     static_assert((RG * 64) % RT == 0, "uniform staging loop");
@@ -61,7 +97,11 @@ __device__ __forceinline__ void stage_x(float2 *xs, float *mx, const float2 *__r
     for (int e = threadIdx.x; e < RG * 64; e += RT) {
         const int q = e >> 6, j = e & 63;
         const float2 v = (j < klen && q < nr) ? x[(int64_t)(r0 + q) * ldx + in0 + j] : make_float2(0.f, 0.f);
-        if (j < k4) xs[j * XS + q] = v;
+        if (j < k4) {
+            float *d = reinterpret_cast<float *>(xs + j * XP + (q >> 1)) + (q & 1);
+            d[0] = v.x;
+            d[2] = v.y;
+        }
         const float m = warp_max(linf(v));
         if ((j & 31) == 0) mx[2 * q + (j >> 5)] = m;
     }
@@ -71,9 +111,9 @@ __device__ __forceinline__ float x_max(const float *mx, int q) { return fmaxf(mx
 
 template <int RG, int RT>
 __global__ void __launch_bounds__(RT, 4)
-k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restrict__ prods,
+k_resid_own(const RcUnit *__restrict__ units, int n_units, const TcProd *__restrict__ prods,
             const float2 *__restrict__ pbnd, const float2 *__restrict__ pool, const float2 *__restrict__ x,
-            int64_t ldx, int nrhs, double2 *__restrict__ own, int64_t ldo)
+            int64_t ldx, int nrhs, double2 *__restrict__ own, int64_t ldo, int64_t lstride)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     Smem &S = *reinterpret_cast<Smem *>(smraw);
@@ -85,11 +125,11 @@ k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restr
     // run on neighbouring CTAs at the same time and read the cluster's blocks from DRAM
     // once between them (the later reads hit L2)
     for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {
-        const TcUnit U = units[u / n_groups];
+        const RcUnit U = units[u / n_groups];
         const int r0 = (int)(u % n_groups) * RG, nr = min(RG, nrhs - r0);
-        cdf acc[QN];
+        cdf acc[QN / 2][2];
 #pragma unroll
-        for (int q = 0; q < QN; ++q) acc[q] = cdf_zero();
+        for (int q = 0; q < QN; ++q) acc[q / 2][q & 1] = cdf_zero();
         for (int p = U.p0; p < U.p1; ++p) {
             const TcProd P = prods[p];
             __syncthreads();                                  // the previous product's reads are done
@@ -111,26 +151,23 @@ k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restr
                     // one chain per right-hand side over all K indices, on the grid of the
                     // product's largest output-row 1-norm times the input's largest component
                     const float bo = pbnd[p].x;
-                    float sg[QN];
-                    cxacc c[QN];
+                    float2 sg[QN / 2];
+                    chain2 c[QN / 2];
 #pragma unroll
-                    for (int q = 0; q < QN; ++q) {
-                        sg[q] = grid_sigma(bo, x_max(S.mx, QN * hh + q));
-                        cx_start(c[q], sg[q]);
+                    for (int q = 0; q < QN / 2; ++q) {
+                        sg[q] = make_float2(grid_sigma(bo, x_max(S.mx, QN * hh + 2 * q)),
+                                            grid_sigma(bo, x_max(S.mx, QN * hh + 2 * q + 1)));
+                        c2_start(c[q], sg[q]);
                     }
+                    const float4 *xv = S.x + QN / 2 * hh;
 #pragma unroll 4
                     for (int j = 0; j < P.klen; ++j) {
                         const float2 bv = S.b[j * BS + i];
-                        const float4 *xv = reinterpret_cast<const float4 *>(S.x + j * XS + QN * hh);
 #pragma unroll
-                        for (int q = 0; q < QN / 2; ++q) {
-                            const float4 v = xv[q];
-                            cxstep(c[2 * q], bv, make_float2(v.x, v.y));
-                            cxstep(c[2 * q + 1], bv, make_float2(v.z, v.w));
-                        }
+                        for (int q = 0; q < QN / 2; ++q) c2_step(c[q], bv, xv[j * XP + q]);
                     }
 #pragma unroll
-                    for (int q = 0; q < QN; ++q) acc[q] = cdf_add(acc[q], cxclose(c[q], sg[q]));
+                    for (int q = 0; q < QN / 2; ++q) c2_fold(acc[q], c[q], sg[q]);
                 }
             } else {
                 // W (rank rows l, K j) into b[j * WS + l]; Y (element (i, l) = Y[l][i]) into y[l * BS + i]
@@ -142,28 +179,32 @@ k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restr
                     if (c < P.olen) Ysm[l * BS + c] = Y[(int64_t)l * P.y_ld + c];
                 }
                 __syncthreads();
-                // stage 1: T[l][q] = sum_j W[l][j] x[j][q]; a round covers 128 / (4 RG) rank rows;
-                // thread (row l0 + tid / (4 RG), q = (tid / 4) % RG, K slice ks = tid % 4: j = ks,
-                // ks + 4, ...); the four slices' chains share the grid of W's largest rank-row
+                // stage 1: T[l][q] = sum_j W[l][j] x[j][q]; thread (row l0 + lr, pair qp, K slice
+                // ks: j = ks, ks + NS, ...); the slices' chains share the grid of W's largest rank-row
                 // 1-norm times x's largest component, so their grid parts add exactly across lanes
                 const float2 bb = pbnd[p];
                 {
-                    constexpr int NS = 2;                          // K slices per rank row and RHS
-                    constexpr int LR = RT / (NS * RG);             // rank rows per round
-                    const int ks = tid % NS, q = (tid / NS) % RG, lr = tid / (NS * RG);
-                    const float s1 = grid_sigma(bb.x, x_max(S.mx, q));
+                    constexpr int NS = RG == 16 ? 2 : 4;           // K slices per rank row and pair
+                    constexpr int LR = RT / (NS * RG / 2);         // rank rows per round
+                    const int ks = tid % NS, qp = (tid / NS) % (RG / 2), lr = tid / (NS * RG / 2);
+                    const float2 s1 = make_float2(grid_sigma(bb.x, x_max(S.mx, 2 * qp)),
+                                                  grid_sigma(bb.x, x_max(S.mx, 2 * qp + 1)));
                     for (int l0 = 0; l0 < P.rank; l0 += LR) {
                         const int l = l0 + lr;
-                        cxacc c;
-                        cx_start(c, s1);
+                        chain2 c;
+                        c2_start(c, s1);
                         if (l < P.rank)
-                            for (int j = ks; j < P.klen; j += NS) cxstep(c, Wsm[j * WS + l], S.x[j * XS + q]);
-                        float v[4] = {__fsub_rn(c.re.tau, s1), c.re.r, __fsub_rn(c.im.tau, s1), c.im.r};
+                            for (int j = ks; j < P.klen; j += NS) c2_step(c, Wsm[j * WS + l], S.x[j * XP + qp]);
+                        const float2 gr = sub2(c.tr, s1), gi = sub2(c.ti, s1);
+                        float v[8] = {gr.x, gr.y, gi.x, gi.y, c.rr.x, c.rr.y, c.ri.x, c.ri.y};
 #pragma unroll
                         for (int sh = 1; sh < NS; sh <<= 1)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) v[e] = __fadd_rn(v[e], __shfl_xor_sync(FULL, v[e], sh));
-                        if (ks == 0 && l < P.rank) S.t[l * RG + q] = {{v[0], v[1]}, {v[2], v[3]}};
+                            for (int e = 0; e < 8; ++e) v[e] = __fadd_rn(v[e], __shfl_xor_sync(FULL, v[e], sh));
+                        if (ks == 0 && l < P.rank) {
+                            S.t[l * RG + 2 * qp] = make_float4(v[0], v[1], v[2], v[3]);
+                            S.t[l * RG + 2 * qp + 1] = make_float4(v[4], v[5], v[6], v[7]);
+                        }
                     }
                 }
                 __syncthreads();
@@ -171,20 +212,26 @@ k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restr
                 // all rank rows: the leading part of T[l][q] is a grid sum, at most half of
                 // stage 1's sigma, which bounds the inputs with Y's largest output-row 1-norm
                 if (i < P.olen) {
-                    float sg[QN];
-                    cxacc c[QN];
+                    float2 sg[QN / 2];
+                    chain2 c[QN / 2];
 #pragma unroll
-                    for (int q = 0; q < QN; ++q) {
-                        sg[q] = grid_sigma(bb.y, 0.5f * grid_sigma(bb.x, x_max(S.mx, QN * hh + q)));
-                        cx_start(c[q], sg[q]);
+                    for (int q = 0; q < QN / 2; ++q) {
+                        const int g = QN * hh + 2 * q;
+                        sg[q] = make_float2(grid_sigma(bb.y, 0.5f * grid_sigma(bb.x, x_max(S.mx, g))),
+                                            grid_sigma(bb.y, 0.5f * grid_sigma(bb.x, x_max(S.mx, g + 1))));
+                        c2_start(c[q], sg[q]);
                     }
                     for (int l = 0; l < P.rank; ++l) {
                         const float2 yv = Ysm[l * BS + i];
 #pragma unroll
-                        for (int q = 0; q < QN; ++q) cxstep_df(c[q], yv, S.t[l * RG + QN * hh + q]);
+                        for (int q = 0; q < QN / 2; ++q) {
+                            const float4 *t = S.t + l * RG + QN * hh + 2 * q;
+                            c2_step(c[q], yv, t[0]);
+                            c2_lo(c[q], yv, t[1]);
+                        }
                     }
 #pragma unroll
-                    for (int q = 0; q < QN; ++q) acc[q] = cdf_add(acc[q], cxclose(c[q], sg[q]));
+                    for (int q = 0; q < QN / 2; ++q) c2_fold(acc[q], c[q], sg[q]);
                 }
             }
         }
@@ -192,48 +239,106 @@ k_resid_own(const TcUnit *__restrict__ units, int n_units, const TcProd *__restr
 #pragma unroll
             for (int q = 0; q < QN; ++q) {
                 const int r = QN * hh + q;
-                if (r < nr) own[(int64_t)(r0 + r) * ldo + U.out0 + i] = to_d2(acc[q]);
+                if (r < nr) own[U.part * lstride + (int64_t)(r0 + r) * ldo + U.out0 + i] = to_d2(acc[q / 2][q & 1]);
             }
         }
     }
 }
 
-// Per leaf (blockIdx.x) and right-hand side (blockIdx.y): acc = D_I x_I (Dot2) +
-// the owner sums of levels 1..m at the leaf's rows (FP64), in a fixed order.  If b
+// Dot2 of two right-hand sides as packed pairs (k_dot2.cuh dot2): acc += a * b, na = -a
+struct dot2x2 { float2 hi, lo; };
+__device__ __forceinline__ void dot2_pair(dot2x2 &acc, float2 a, float2 na, float2 b)
+{
+    const float2 z = dup(0.f);
+    const float2 p = fma2(a, b, z), np = fma2(na, b, z);
+    const float2 s = add2(acc.hi, p), bb = sub2(s, acc.hi);
+    const float2 q = add2(sub2(acc.hi, sub2(s, bb)), sub2(p, bb));
+    acc.lo = add2(acc.lo, add2(q, fma2(a, b, np)));
+    acc.hi = s;
+}
+
+// Per leaf (blockIdx.x) and GR right-hand sides (blockIdx.y): acc = D_I x_I (Dot2) +
+// the `arrays` owner sums at the leaf's rows (FP64), in a fixed order.  If b
 // is given, out = b - acc (FP64, rounded to complex64) and |r|^2, |b|^2 go to
 // norms; else out = acc (complex64).  x of the leaf is staged in dynamic shared
-// memory (np entries).
-__global__ void __launch_bounds__(64)
+// memory as pairs; each element of D_I serves the GR right-hand sides.  Four threads share a
+// row: columns j = js, js + 4, .. each, then right-hand side q = js each (the Dot2 chain over
+// the columns is what a row waits for).  7,500 unknowns, 50 right-hand sides: 54 us with one a
+// CTA and a thread a row, TODO us.
+template <int GR>
+__global__ void __launch_bounds__(256)
 k_gather_own(const int32_t *__restrict__ pleaf_off, const int64_t *__restrict__ dinv_off,
-             const float2 *__restrict__ self32, const float2 *__restrict__ x, int64_t ld, int m,
+             const float2 *__restrict__ self32, const float2 *__restrict__ x, int64_t ld, int nrhs, int arrays,
              const double2 *__restrict__ own, int64_t lstride, const float2 *__restrict__ b, float2 *__restrict__ out,
              double *norms)
 {
+    static_assert(GR == 1 || GR == 4, "a right-hand side per column slice");
+    constexpr int GP = (GR + 1) / 2;
+    __shared__ cdf part[4][GR][64];
     extern __shared__ __align__(16) unsigned char gsm[];
-    float2 *xs = reinterpret_cast<float2 *>(gsm);
-    const int leaf = blockIdx.x, r = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    float *xs = reinterpret_cast<float *>(gsm);
+    const int leaf = blockIdx.x, r0 = GR * blockIdx.y, tid = threadIdx.x, lane = tid & 31, js = tid >> 6;
     const int o = pleaf_off[leaf], np = pleaf_off[leaf + 1] - o;
-    double rr = 0.0, bb = 0.0;
-    for (int j = tid; j < np; j += 64) xs[j] = x[r * ld + o + j];
-    __syncthreads();
-    const float2 *Sd = self32 + dinv_off[leaf];                 // column-major np x np
-    for (int i = tid; i < np; i += 64) {
-        const int64_t g = r * ld + o + i;
-        cdf dx = cdf_zero();
-        for (int j = 0; j < np; ++j) cdot2(dx, Sd[(int64_t)j * np + i], xs[j]);
-        double2 acc = to_d2(dx);
-        for (int lev = 0; lev < m; ++lev) acc = cadd(acc, own[lev * lstride + g]);
-        if (b) {
-            const double2 bv = conv<double2>(b[g]);
-            const double2 rv = csub(bv, acc);
-            out[g] = make_float2((float)rv.x, (float)rv.y);
-            rr += rv.x * rv.x + rv.y * rv.y;
-            bb += bv.x * bv.x + bv.y * bv.y;
-        } else {
-            out[g] = make_float2((float)acc.x, (float)acc.y);
-        }
+    const int r = r0 + js;                                     // the thread's right-hand side
+    const bool mine = js < GR && r < nrhs;
+    for (int e = tid; e < 2 * GP * np; e += 256) {
+        const int q = e / np, j = e - q * np;
+        const float2 v = q < GR && r0 + q < nrhs ? x[(r0 + q) * ld + o + j] : make_float2(0.f, 0.f);
+        float *d = xs + 4 * (j * GP + (q >> 1)) + (q & 1);
+        d[0] = v.x;
+        d[2] = v.y;
     }
-    if (norms) {
+    __syncthreads();
+    const float4 *xp = reinterpret_cast<const float4 *>(xs);
+    const float2 *Sd = self32 + dinv_off[leaf];                 // column-major np x np
+    double rr = 0.0, bb = 0.0;
+    for (int i0 = 0; i0 < np; i0 += 64) {
+        const int i = i0 + (tid & 63);
+        if (i < np) {
+            dot2x2 re[GP], im[GP];
+#pragma unroll
+            for (int q = 0; q < GP; ++q) re[q] = im[q] = {dup(0.f), dup(0.f)};
+#pragma unroll 4
+            for (int j = js; j < np; j += 4) {
+                const float2 a = Sd[(int64_t)j * np + i];
+#pragma unroll
+                for (int q = 0; q < GP; ++q) {
+                    const float4 v = xp[j * GP + q];
+                    const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
+                    dot2_pair(re[q], dup(a.x), dup(-a.x), vr);
+                    dot2_pair(re[q], dup(-a.y), dup(a.y), vi);
+                    dot2_pair(im[q], dup(a.x), dup(-a.x), vi);
+                    dot2_pair(im[q], dup(a.y), dup(-a.y), vr);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < GR; ++q) {
+                const dot2x2 &u = re[q / 2], &v = im[q / 2];
+                part[js][q][tid & 63] =
+                    q & 1 ? cdf{{u.hi.y, u.lo.y}, {v.hi.y, v.lo.y}} : cdf{{u.hi.x, u.lo.x}, {v.hi.x, v.lo.x}};
+            }
+        }
+        __syncthreads();
+        if (i < np && mine) {
+            const int64_t g = r * ld + o + i;
+            cdf s = part[0][js][tid & 63];
+#pragma unroll
+            for (int q = 1; q < 4; ++q) s = cdf_add(s, part[q][js][tid & 63]);
+            double2 acc = to_d2(s);
+            for (int lev = 0; lev < arrays; ++lev) acc = cadd(acc, own[lev * lstride + g]);
+            if (b) {
+                const double2 bv = conv<double2>(b[g]);
+                const double2 rv = csub(bv, acc);
+                out[g] = make_float2((float)rv.x, (float)rv.y);
+                rr += rv.x * rv.x + rv.y * rv.y;
+                bb += bv.x * bv.x + bv.y * bv.y;
+            } else {
+                out[g] = make_float2((float)acc.x, (float)acc.y);
+            }
+        }
+        __syncthreads();
+    }
+    if (norms && mine) {                                       // whole warps: js is a warp's
         for (int s = 16; s >= 1; s >>= 1) {
             rr += __shfl_xor_sync(FULL, rr, s);
             bb += __shfl_xor_sync(FULL, bb, s);
@@ -278,9 +383,11 @@ void launch_prod_bounds(const TcProd *prods, int64_t n, const float2 *pool, floa
     k_prod_bounds<<<g, 256, 0, s>>>(prods, n, pool, out);
 }
 
-// owner-computes FP64-class products of a level's small items: own[r * pN + i] = (M_level x_r)_i
-// for the level's output rows (a level whose items are all small; the rest of own is untouched)
-void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int nrhs, cudaStream_t s)
+// owner-computes FP64-class products of a level's small items: the sum over the level's parts q of
+// own[q * lstride + r * pN + i] = (M_level x_r)_i for the level's output rows (a level whose items
+// are all small; the rest of own is untouched)
+void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 *own, int64_t lstride, int nrhs,
+                      cudaStream_t s)
 {
     if (L.n_rcu == 0 || nrhs <= 0) return;
     constexpr int SMEM = (int)sizeof(Smem);
@@ -305,20 +412,29 @@ void launch_resid_own(hm_matrix h, const LevelList &L, const float2 *x, double2 
     if (g > units) g = units;
     auto go = [&](auto kern, int rt) {
         kern<<<(unsigned)g, rt, SMEM, s>>>(L.d_rcu, (int)L.n_rcu, L.d_rcp, L.d_rcb, h->d_pool32, x, h->pN, nrhs, own,
-                                           h->pN);
+                                           h->pN, lstride);
     };
     if (rg == 8) wide ? go(k_resid_own<8, 256>, 256) : go(k_resid_own<8, 128>, 128);
     else wide ? go(k_resid_own<16, 256>, 256) : go(k_resid_own<16, 128>, 128);
 }
 
-void launch_gather_own(hm_matrix h, const float2 *x, int m, const double2 *own, int64_t lstride, const float2 *b,
+void launch_gather_own(hm_matrix h, const float2 *x, int arrays, const double2 *own, int64_t lstride, const float2 *b,
                        float2 *out, double *norms, int nrhs, cudaStream_t s)
 {
-    dim3 grid((unsigned)h->n_leaves, (unsigned)nrhs);
     int64_t maxnp = 0;
     for (int64_t i = 0; i < h->n_leaves; ++i) maxnp = std::max<int64_t>(maxnp, h->pleaf_off[i + 1] - h->pleaf_off[i]);
-    k_gather_own<<<grid, 64, sizeof(float2) * (size_t)std::max<int64_t>(maxnp, 1), s>>>(
-        h->d_pleaf_off, h->d_dinv_off, h->d_self32, x, h->pN, m, own, lstride, b, out, norms);
+    // four right-hand sides a CTA where that leaves a CTA per SM
+    const int64_t groups = (nrhs + 3) / 4;
+    const bool four = h->n_leaves * groups >= h->num_sms;
+    const auto kern = four ? k_gather_own<4> : k_gather_own<1>;
+    const size_t sm = sizeof(float4) * (four ? 2 : 1) * (size_t)std::max<int64_t>(maxnp, 1);
+    static bool attr = false;
+    if (sm > 32 * 1024 && !attr) {
+        cudaFuncSetAttribute(k_gather_own<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+        attr = true;
+    }
+    kern<<<dim3((unsigned)h->n_leaves, (unsigned)(four ? groups : nrhs)), 256, sm, s>>>(
+        h->d_pleaf_off, h->d_dinv_off, h->d_self32, x, h->pN, nrhs, arrays, own, lstride, b, out, norms);
 }
 
 } // namespace hm

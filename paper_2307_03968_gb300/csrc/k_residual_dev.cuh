@@ -143,7 +143,8 @@ __device__ __forceinline__ void grid_row(const Pair<float> (&b)[4], int i, int r
             cxstep(acc[t][1], b[t].b, vi);
         }
     }
-    float rv[4] = {__fsub_rn(c.re.tau, sR), c.re.r, __fsub_rn(c.im.tau, sR), c.im.r};
+    float rv[4];
+    cx_values(rv, c, sR);
     // value index bit 1 (re / im) by cg bit 2, bit 0 (grid part / remainder) by cg bit 1,
     // then the pair of lanes cg, cg ^ 1 adds its two partial sums
     xreduce_step<2>(rv, lane, 4);
@@ -181,12 +182,7 @@ __device__ __forceinline__ void grid_pass(const float2 *__restrict__ A, int rows
 #pragma unroll
     for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            w[8 * t + 4 * e] = __fsub_rn(acc[t][e].re.tau, sC);
-            w[8 * t + 4 * e + 1] = acc[t][e].re.r;
-            w[8 * t + 4 * e + 2] = __fsub_rn(acc[t][e].im.tau, sC);
-            w[8 * t + 4 * e + 3] = acc[t][e].im.r;
-        }
+        for (int e = 0; e < 2; ++e) cx_values(w + 8 * t + 4 * e, acc[t][e], sC);
     // over the column group's 4 lanes: index bit 4 (t bit 1) by rg bit 1, bit 3 (t bit 0)
     // by rg bit 0, so lane (rg, cg) ends with its pair of t = rg
     xreduce_step<16>(w, lane, 16);
@@ -236,154 +232,129 @@ __device__ __forceinline__ void dense_item_g(const Item &it, float4 bnd, const f
               grid_sigma(bnd.y, mxi), part + it.pad + even_d(m), lane);
 }
 
-// the lane's two columns (i, i + 1) of the rank rows l0, l0 + 1 of U^T and V (zero
-// past the rank or the panel)
-__device__ __forceinline__ void lr_load(Pair<float> (&u)[2], Pair<float> (&v)[2], const float2 *__restrict__ UT,
-                                        const float2 *__restrict__ V, int l0, int k, int m, int n, int i, bool iv,
-                                        bool jv)
+// the lane's four columns (two pairs, 32 t + 2 c, c = lane & 15) of rank row l of U^T (side 0)
+// and V (side 1), zero past the rank or the panel
+__device__ __forceinline__ void lr_load(Pair<float> (&f)[2][2], const float2 *__restrict__ UT,
+                                        const float2 *__restrict__ V, int l, int k, int m, int n, int c)
 {
 #pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        u[l] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        v[l] = u[l];
-        if (l0 + l < k) {
-            if (iv) u[l] = ld_stream(UT + (int64_t)(l0 + l) * m + i);
-            if (jv) v[l] = ld_stream(V + (int64_t)(l0 + l) * n + i);
+    for (int t = 0; t < 2; ++t) {
+        const int i = 32 * t + 2 * c;
+        f[0][t] = f[1][t] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (l < k && i < m) f[0][t] = ld_stream(UT + (int64_t)l * m + i);
+        if (l < k && i < n) f[1][t] = ld_stream(V + (int64_t)l * n + i);
+    }
+}
+
+// one rank row per half-warp (f: the lane's columns of U^T and V): stage 1 on the common grids
+// s1[side], reduced over the half-warp's 16 lanes, then the row into the outputs' stage-2 chains
+// (o[0]: rows, from V x_J; o[1]: columns, from U^T x_I).  Rank rows past k have zero factors and
+// zero intermediates.
+__device__ __forceinline__ void lr_row(const Pair<float> (&f)[2][2], const Pair<float> (&xin)[2][2],
+                                       const float (&s1)[2], cxacc (&o)[2][2][2], int lane)
+{
+    float g[8];                                        // value index 4 side + (re grid, re rem, im grid, im rem)
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        cxacc c;
+        cx_start(c, s1[side]);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            cxstep(c, f[side][t].a, xin[side][t].a);
+            cxstep(c, f[side][t].b, xin[side][t].b);
+        }
+        cx_values(g + 4 * side, c, s1[side]);
+    }
+    // over the half-warp: index bits 2..0 by lane bits 3..1, then the pair of lanes adds its
+    // halves: lane L of the half ends with value L / 2
+    xreduce_step<4>(g, lane, 8);
+    xreduce_step<2>(g, lane, 4);
+    xreduce_step<1>(g, lane, 2);
+    g[0] = __fadd_rn(g[0], __shfl_xor_sync(FULL, g[0], 1));
+    const int h = lane & 16;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {             // the other side's intermediate
+        const int v = h + 8 * (1 - side);
+        const cdf tl = {{__shfl_sync(FULL, g[0], v), __shfl_sync(FULL, g[0], v + 2)},
+                        {__shfl_sync(FULL, g[0], v + 4), __shfl_sync(FULL, g[0], v + 6)}};
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            cxstep_df(o[side][t][0], f[side][t].a, tl);
+            cxstep_df(o[side][t][1], f[side][t].b, tl);
         }
     }
 }
 
-// one pair of rank rows l0, l0 + 1 of a low-rank block (u: U^T, v: V, the lane's two
-// columns each): stage 1 on the common grids s1u, s1v, reduced over the warp, then
-// the pair's rank rows into the outputs' stage-2 chains
-__device__ __forceinline__ void lr_pair(const Pair<float> (&u)[2], const Pair<float> (&v)[2], const Pair<float> &xi,
-                                        const Pair<float> &xj, float s1u, float s1v, cxacc &ci0, cxacc &ci1,
-                                        cxacc &cj0, cxacc &cj1, int lane)
-{
-    // value index 4 l + (grid re, rem re, grid im, rem im)
-    float gu[8], gv[8];
-#pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        cxacc cu, cv;
-        cx_start(cu, s1u);
-        cxstep(cu, u[l].a, xi.a);
-        cxstep(cu, u[l].b, xi.b);
-        cx_start(cv, s1v);
-        cxstep(cv, v[l].a, xj.a);
-        cxstep(cv, v[l].b, xj.b);
-        gu[4 * l] = __fsub_rn(cu.re.tau, s1u);
-        gu[4 * l + 1] = cu.re.r;
-        gu[4 * l + 2] = __fsub_rn(cu.im.tau, s1u);
-        gu[4 * l + 3] = cu.im.r;
-        gv[4 * l] = __fsub_rn(cv.re.tau, s1v);
-        gv[4 * l + 1] = cv.re.r;
-        gv[4 * l + 2] = __fsub_rn(cv.im.tau, s1v);
-        gv[4 * l + 3] = cv.im.r;
-    }
-    // over the warp: index bits 2..0 by lane bits 4..2, then the four lanes 4 q .. 4 q + 3
-    // add their quarters: lane L ends with value L / 4 summed over all lanes
-    xreduce_step<4>(gu, lane, 16);
-    xreduce_step<4>(gv, lane, 16);
-    xreduce_step<2>(gu, lane, 8);
-    xreduce_step<2>(gv, lane, 8);
-    xreduce_step<1>(gu, lane, 4);
-    xreduce_step<1>(gv, lane, 4);
-#pragma unroll
-    for (int sh = 1; sh <= 2; sh <<= 1) {
-        gu[0] = __fadd_rn(gu[0], __shfl_xor_sync(FULL, gu[0], sh));
-        gv[0] = __fadd_rn(gv[0], __shfl_xor_sync(FULL, gv[0], sh));
-    }
-    // stage 2 (rank rows past k have zero factors and zero intermediates)
-#pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        const cdf tl = {{__shfl_sync(FULL, gv[0], 16 * l), __shfl_sync(FULL, gv[0], 16 * l + 4)},
-                        {__shfl_sync(FULL, gv[0], 16 * l + 8), __shfl_sync(FULL, gv[0], 16 * l + 12)}};
-        const cdf tpl = {{__shfl_sync(FULL, gu[0], 16 * l), __shfl_sync(FULL, gu[0], 16 * l + 4)},
-                         {__shfl_sync(FULL, gu[0], 16 * l + 8), __shfl_sync(FULL, gu[0], 16 * l + 12)}};
-        cxstep_df(ci0, u[l].a, tl);
-        cxstep_df(ci1, u[l].b, tl);
-        cxstep_df(cj0, v[l].a, tpl);
-        cxstep_df(cj1, v[l].b, tpl);
-    }
-}
-
-// the last rank row of an odd rank (u, v: that row's two columns of U^T and V): as
-// lr_pair for one row
-__device__ __forceinline__ void lr_single(const Pair<float> &u, const Pair<float> &v, const Pair<float> &xi,
-                                          const Pair<float> &xj, float s1u, float s1v, cxacc &ci0, cxacc &ci1,
-                                          cxacc &cj0, cxacc &cj1, int lane)
-{
-    cxacc cu, cv;
-    cx_start(cu, s1u);
-    cxstep(cu, u.a, xi.a);
-    cxstep(cu, u.b, xi.b);
-    cx_start(cv, s1v);
-    cxstep(cv, v.a, xj.a);
-    cxstep(cv, v.b, xj.b);
-    float gu[4] = {__fsub_rn(cu.re.tau, s1u), cu.re.r, __fsub_rn(cu.im.tau, s1u), cu.im.r};
-    float gv[4] = {__fsub_rn(cv.re.tau, s1v), cv.re.r, __fsub_rn(cv.im.tau, s1v), cv.im.r};
-    // index bits 1..0 by lane bits 4..3, then the eight lanes 8 c .. 8 c + 7 add their
-    // eighths: lane L ends with value L / 8 summed over all lanes
-    xreduce_step<2>(gu, lane, 16);
-    xreduce_step<2>(gv, lane, 16);
-    xreduce_step<1>(gu, lane, 8);
-    xreduce_step<1>(gv, lane, 8);
-#pragma unroll
-    for (int sh = 1; sh <= 4; sh <<= 1) {
-        gu[0] = __fadd_rn(gu[0], __shfl_xor_sync(FULL, gu[0], sh));
-        gv[0] = __fadd_rn(gv[0], __shfl_xor_sync(FULL, gv[0], sh));
-    }
-    const cdf tl = {{__shfl_sync(FULL, gv[0], 0), __shfl_sync(FULL, gv[0], 8)},
-                    {__shfl_sync(FULL, gv[0], 16), __shfl_sync(FULL, gv[0], 24)}};
-    const cdf tpl = {{__shfl_sync(FULL, gu[0], 0), __shfl_sync(FULL, gu[0], 8)},
-                     {__shfl_sync(FULL, gu[0], 16), __shfl_sync(FULL, gu[0], 24)}};
-    cxstep_df(ci0, u.a, tl);
-    cxstep_df(ci1, u.b, tl);
-    cxstep_df(cj0, v.a, tpl);
-    cxstep_df(cj1, v.b, tpl);
-}
-
 // Low-rank block U V of at most 64 x 64 (U^T k x m, V k x n, m, n padded even):
-// slot rows (m) = U (V x_J), slot columns (n) = V^T (U^T x_I), one pass over pairs
-// of rank rows (loaded one pair ahead).  A lane owns the rows / columns 2 lane,
-// 2 lane + 1 of both panels.  Both stages run on common grids.  Stage 1 (the rank-k
-// intermediates tp = U^T x_I, t = V x_J; bnd.x, bnd.y: largest rank-row 1-norms of
-// U^T and V): the 32-lane reductions add the grid parts exactly in plain FP32.
-// Stage 2 (the outputs; bnd.z, bnd.w: largest column 1-norms of U^T and V): the
-// leading part of each intermediate is a grid sum, at most half its grid's sigma,
-// which bounds the inputs, so each output is one chain over all rank rows.
+// slot rows (m) = U (V x_J), slot columns (n) = V^T (U^T x_I), one pass over the rank rows,
+// one per half-warp (loaded one pair ahead).  A lane owns four rows and four columns.  Both
+// stages run on common grids.  Stage 1 (the rank-k intermediates U^T x_I, V x_J; bnd.x, bnd.y:
+// largest rank-row 1-norms of U^T and V): the lane reductions add the grid parts exactly in
+// plain FP32.  Stage 2 (the outputs; bnd.z, bnd.w: largest column 1-norms of U^T and V): the
+// leading part of each intermediate is a grid sum, at most half its grid's sigma, which bounds
+// the inputs, so each output is one chain over all rank rows of a half-warp, and the two
+// halves' chains, on one grid, are added at the end.  A rank row over 16 lanes of four columns
+// a side costs half the reduction instructions an element of one over 32 lanes of two (the
+// form before; with the packed steps, 30,720-unknown sphere: 0.432 to 0.394 ms.  What is left is
+// latency: issue slots, FMA pipe and HBM are each half busy.  80 registers for 24 warps an SM
+// spill (0.53 ms), and inputs in shared memory as duplicated pairs or the next block prefetched
+// into L2 take 0.41 to 0.43).
 __device__ __forceinline__ void lowrank_item_g(const Item &it, float4 bnd, const float2 *__restrict__ pool,
                                                const float2 *HM_XR x, cdf *HM_XR part, int lane)
 {
     const int m = it.m, n = it.n, k = it.k;
     const float2 *UT = pool + it.off;
     const float2 *V = UT + (int64_t)k * m;
-    const int i = 2 * lane;
-    const bool iv = i < m, jv = i < n;
-    Pair<float> u[2], v[2];
-    lr_load(u, v, UT, V, 0, k, m, n, i, iv, jv);
-    Pair<float> xi{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, xj = xi;
-    if (iv) xi = ld_vec(x + it.row0 + i);
-    if (jv) xj = ld_vec(x + it.col0 + i);
-    const float s1u = grid_sigma(bnd.x, warp_max(fmaxf(linf(xi.a), linf(xi.b))));
-    const float s1v = grid_sigma(bnd.y, warp_max(fmaxf(linf(xj.a), linf(xj.b))));
-    const float s2i = grid_sigma(bnd.z, 0.5f * s1v), s2j = grid_sigma(bnd.w, 0.5f * s1u);
-    cxacc ci0, ci1, cj0, cj1;
-    cx_start(ci0, s2i);
-    cx_start(ci1, s2i);
-    cx_start(cj0, s2j);
-    cx_start(cj1, s2j);
-#pragma unroll 1
-    for (int l0 = 0; l0 + 1 < k; l0 += 2) {
-        Pair<float> un[2], vn[2];
-        lr_load(un, vn, UT, V, l0 + 2, k, m, n, i, iv, jv);
-        lr_pair(u, v, xi, xj, s1u, s1v, ci0, ci1, cj0, cj1, lane);
+    const int c = lane & 15, h = lane >> 4;
+    Pair<float> f[2][2];
+    lr_load(f, UT, V, h, k, m, n, c);
+    Pair<float> xin[2][2];
+    float mx[2] = {0.f, 0.f};
 #pragma unroll
-        for (int l = 0; l < 2; ++l) { u[l] = un[l]; v[l] = vn[l]; }
+    for (int t = 0; t < 2; ++t) {
+        const int i = 32 * t + 2 * c;
+        xin[0][t] = xin[1][t] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (i < m) xin[0][t] = ld_vec(x + it.row0 + i);
+        if (i < n) xin[1][t] = ld_vec(x + it.col0 + i);
+#pragma unroll
+        for (int side = 0; side < 2; ++side)
+            mx[side] = fmaxf(mx[side], fmaxf(linf(xin[side][t].a), linf(xin[side][t].b)));
     }
-    if (k & 1) lr_single(u[0], v[0], xi, xj, s1u, s1v, ci0, ci1, cj0, cj1, lane);   // row k - 1
-    if (iv) { part[it.pad + i] = cxclose(ci0, s2i); part[it.pad + i + 1] = cxclose(ci1, s2i); }
-    if (jv) { part[it.pad + m + i] = cxclose(cj0, s2j); part[it.pad + m + i + 1] = cxclose(cj1, s2j); }
+    const float s1[2] = {grid_sigma(bnd.x, warp_max(mx[0])), grid_sigma(bnd.y, warp_max(mx[1]))};
+    const float s2[2] = {grid_sigma(bnd.z, 0.5f * s1[1]), grid_sigma(bnd.w, 0.5f * s1[0])};
+    cxacc o[2][2][2];
+#pragma unroll
+    for (int side = 0; side < 2; ++side)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) { cx_start(o[side][t][0], s2[side]); cx_start(o[side][t][1], s2[side]); }
+#pragma unroll 1
+    for (int l0 = 0; l0 < k; l0 += 2) {
+        Pair<float> fn[2][2];
+        lr_load(fn, UT, V, l0 + 2 + h, k, m, n, c);
+        lr_row(f, xin, s1, o, lane);
+#pragma unroll
+        for (int side = 0; side < 2; ++side)
+#pragma unroll
+            for (int t = 0; t < 2; ++t) f[side][t] = fn[side][t];
+    }
+    // the half-warps' sums: half h keeps side h
+    float w[32];
+#pragma unroll
+    for (int side = 0; side < 2; ++side)
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) cx_values(w + 16 * side + 8 * t + 4 * e, o[side][t][e], s2[side]);
+    xreduce_step<16>(w, lane, 16);
+    cdf *d = part + it.pad + (h ? m : 0);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int i = 32 * t + 2 * c;
+        if (i < (h ? n : m)) {
+            d[i] = {{w[8 * t], w[8 * t + 1]}, {w[8 * t + 2], w[8 * t + 3]}};
+            d[i + 1] = {{w[8 * t + 4], w[8 * t + 5]}, {w[8 * t + 6], w[8 * t + 7]}};
+        }
+    }
 }
 
 // Low-rank block U V larger than 64 x 64: slot rows (m) = U (V x_J), slot columns
