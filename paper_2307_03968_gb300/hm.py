@@ -356,8 +356,9 @@ class HMatrix:
         return a.value, b.value, c.value, d.value
 
     def set_tuning(self, nrhs, prod_rb, res_rb):
-        """hm_set_tuning: pin the kernel choice for nrhs's bucket (product 1016 = tensor-core
-        products; residual 1017 = owner-computes FP64-class residual)."""
+        """hm_set_tuning: pin the kernel choice for nrhs's bucket (product 32 = matrix
+        instructions, 1016 = tcgen05 tensor-core products; residual 1017 = owner-computes
+        FP64-class residual)."""
         _check(load().hm_set_tuning(self._h, nrhs, prod_rb, res_rb))
 
     def set_wait_limit(self, polls):
