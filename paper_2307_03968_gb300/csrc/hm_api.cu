@@ -82,22 +82,28 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         HM_CUDA(cudaGetLastError());
         // the product's lists with tall dense blocks cut into row panels, long low-rank ones into rank panels
         std::vector<Item> pw, pa, pb;
-        product_panels(wide, pw);
+        std::vector<Item> cta;
+        for (const Item &it : wide)
+            if (cta_item(it)) cta.push_back(it);
+        product_panels(cta, pw);
         pw = balanced_order(pw, (int64_t)pw.size(), product_cost);
-        L.prod_long = (int64_t)pw.size() >= product_warps(h);
-        if (L.prod_long) pw.clear();
+        const bool fills_warps = (int64_t)pw.size() >= product_warps(h);
+        if (fills_warps) pw.clear();
         L.n_prod_wide = (int64_t)pw.size();
+        L.prod_long = fills_warps || wide.size() > cta.size();
         // the product kernel hands the rest to its warps round-robin: sorted by cost, largest
         // first, with every other round reversed, each warp gets an even share
         auto lists = [&](const std::vector<Item> &in, std::vector<Item> &out) {
-            std::vector<Item> p;
-            product_panels(in, p);
+            std::vector<Item> left, p;
+            for (const Item &it : in)
+                if (fills_warps || !cta_item(it)) left.push_back(it);
+            product_panels(left, p);
             p = balanced_order(p, product_warps(h), product_cost);
             out = pw;
             out.insert(out.end(), p.begin(), p.end());
         };
-        lists(L.prod_long ? L.items : rest, pa);
-        lists(std::vector<Item>(big.begin() + (L.prod_long ? 0 : L.n_wide), big.end()), pb);
+        lists(L.items, pa);
+        lists(big, pb);
         L.n_prod = (int64_t)pa.size();
         L.n_prod_big = (int64_t)pb.size();
         if ((st = upload(h, &L.d_prod, pa, s)) != HM_OK) return st;

@@ -99,9 +99,9 @@ struct LevelList {
     int64_t n_dense = 0, n_lowrank = 0;
     int64_t elems = 0;            // stored complex elements
     // the FP32 product's own copies of the item list and of its big part, long blocks cut into
-    // panels (product_panels): the n_prod_wide panels of long low-rank blocks, a CTA each, then
+    // panels (product_panels): the n_prod_wide panels of low-rank blocks above PROD_CTA_LEN, a CTA each, then
     // the rest, a warp each, in the order that balances the kernel's round-robin warps (largest
-    // first, snake rounds).  Panels that fill the warps by their number go there (prod_long;
+    // first, snake rounds).  Panels that fill the warps by their number, or of shorter blocks, go there (prod_long;
     // plate of 67,200 unknowns: 2.13 ms a solve, a CTA each 2.17).
     Item *d_prod = nullptr, *d_prod_big = nullptr;
     int64_t n_prod = 0, n_prod_big = 0, n_prod_wide = 0;

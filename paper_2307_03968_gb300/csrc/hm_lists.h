@@ -484,12 +484,18 @@ inline bool build_mm_lists(const std::map<int32_t, std::vector<TcProd>> &by_out,
 // themselves a dense item of the same row stride), a low-rank block longer than 64 into panels of
 // PROD_RANK rank rows (their sum is the block's product; the kernel works in steps of that many
 // rank rows anyway, so the panels add no memory traffic).  A low-rank item's pad is half the
-// distance (m and n are even) from its U^T panel to its V panel (panel_voff).  (30,720-unknown sphere, level 2: 80 blocks of 480 x 480 and
-// more took 152 us on 80 warps.)
+// distance (m and n are even) from its U^T panel to its V panel (panel_voff).
+// (30,720-unknown sphere, level 2: 80 blocks of 480 x 480 and more took 152 us on 80 warps.)
 constexpr int PROD_PANEL = 64;
 constexpr int PROD_RANK = 8;
 // low-rank blocks longer than 64 x 64
 inline bool wide_item(const Item &it) { return it.k > 0 && (it.m > 64 || it.n > 64); }
+// of those, the ones whose panels fill a CTA in the product (its 8 warps take 64 columns each).  The
+// panels of shorter ones stay with the warps: 24,120 unknowns in leaves of 95, 125 us a solve (a
+// CTA a panel 152, a whole block a warp 145) and 394 us with four right-hand sides (525, 418); 4,720
+// in leaves of 74, 47 us (55, 46)
+constexpr int PROD_CTA_LEN = 256;
+inline bool cta_item(const Item &it) { return it.k > 0 && (it.m > PROD_CTA_LEN || it.n > PROD_CTA_LEN); }
 HM_HD inline int64_t panel_voff(const Item &it) { return 2 * (int64_t)(uint32_t)it.pad; }
 inline void product_panels(const std::vector<Item> &in, std::vector<Item> &out)
 {
