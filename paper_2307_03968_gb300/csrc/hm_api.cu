@@ -64,6 +64,7 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         }
         L.n_small = (int64_t)small.size();
         L.n_big = (int64_t)big.size();
+        L.disjoint = disjoint_outputs(directed_products(small));
         if ((st = upload(h, &L.d_items, L.items, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_small, small, s)) != HM_OK) return st;
         // the residual's own list (the long low-rank blocks, a CTA each, largest first; then the
@@ -586,14 +587,15 @@ static hm_status ensure_mm(hm_matrix h, int m, int nrhs, bool res, cudaStream_t 
     return HM_OK;
 }
 
-// the owner-computes residual applies when every level 1..m holds only items it takes
+// the owner-computes residual applies when every level 1..m holds only items it takes, in
+// clusters that do not overlap
 static bool own_applies(hm_matrix h, int m)
 {
     bool any = false;
     for (int lev = 1; lev <= m; ++lev) {
         auto it = h->levels.find(lev);
         if (it == h->levels.end() || it->second.items.empty()) continue;
-        if (it->second.n_big > 0) return false;
+        if (it->second.n_big > 0 || !it->second.disjoint) return false;
         any = true;
     }
     return any;

@@ -144,6 +144,20 @@ inline void build_owner_lists(const std::map<int32_t, std::vector<TcProd>> &by_o
     }
 }
 
+// Whether the output clusters of a level's directed products are disjoint or the same (at one
+// start the longest counts).  The clusters of one tree level are; a user's own blocks may couple,
+// on the same level, a leaf and a union that holds it.  The owner-computes residuals store each
+// cluster's sums, so two clusters that share rows would overwrite each other's.
+inline bool disjoint_outputs(const std::map<int32_t, std::vector<TcProd>> &by_out)
+{
+    int64_t end = 0;
+    for (const auto &kv : by_out) {
+        if (kv.first < end) return false;
+        for (const TcProd &p : kv.second) end = std::max<int64_t>(end, (int64_t)kv.first + p.olen);
+    }
+    return true;
+}
+
 // The owner units cut into parts of about equal cost, so that a call has `target` units a
 // right-hand-side group where there are fewer clusters than that (each part sums into an array of
 // its own, which the gather adds in order), parts of at least 8 products; returns the parts.
