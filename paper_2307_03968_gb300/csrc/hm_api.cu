@@ -198,7 +198,7 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
         // about four CTAs an SM for one tile of right-hand sides
         if (!build_mm_lists(directed_products(small_items(L)), 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), mm))
             return fail(HM_ERR_STATE, "matrix-product work lists out of their index bounds");
-        TmpArray sets, chunks, rows, pairs, wscale, rscale;
+        TmpArray sets, chunks, rows, pairs, wexp, rexp;
         struct Undo {   // a level's arrays go again if the last of them cannot be had
             hm_matrix h;
             LevelList &L;
@@ -228,8 +228,8 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
             (st = chunks.make(mm.chunks.data(), mm.chunks.size() * sizeof(MmChunk), s)) != HM_OK ||
             (st = rows.make(mm.rows.data(), mm.rows.size() * sizeof(int64_t), s)) != HM_OK ||
             (st = pairs.make(mm.pairs.data(), mm.pairs.size() * sizeof(MmPair), s)) != HM_OK ||
-            (st = wscale.make(nullptr, 2 * mm.pairs.size() * sizeof(float), s)) != HM_OK ||
-            (st = rscale.make(nullptr, mm.rows.size() * sizeof(float), s)) != HM_OK)
+            (st = wexp.make(nullptr, 2 * mm.pairs.size() * sizeof(int), s)) != HM_OK ||
+            (st = rexp.make(nullptr, mm.rows.size() * sizeof(int), s)) != HM_OK)
             return st;
         L.mm_n_unit = (int64_t)mm.units.size();
         L.mm_n_unit2 = (int64_t)mm.units2.size();
@@ -240,7 +240,7 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
         L.mm_n_tch = mm.n_tch;
         L.mm_parts = mm.n_cl > 0 ? mm.parts : 0;
         launch_mm_pack(L, MmPackArgs{(const MmSet *)sets.p, (const MmChunk *)chunks.p, (const int64_t *)rows.p,
-                                     (const MmPair *)pairs.p, (float *)wscale.p, (float *)rscale.p, (int64_t)mm.sets.size(),
+                                     (const MmPair *)pairs.p, (int *)wexp.p, (int *)rexp.p, (int64_t)mm.sets.size(),
                                      (int64_t)mm.chunks.size(), mm.n_cl},
                        h->d_pool32, s);
         HM_CUDA(cudaGetLastError());

@@ -417,7 +417,7 @@ struct MmPackArgs {
     const MmChunk *chunks;
     const int64_t *rows;
     const MmPair *pairs;
-    float *wscale, *rscale;
+    int *wexp, *rexp;
     int64_t n_sets, n_chunks;
     int n_cl;
 };

@@ -34,10 +34,11 @@
 // what lane (g, t) holds, and 32 bytes per t, so that stage 1 writes whole sectors.
 //
 // Scales (powers of two, exact).  FP16 has 5 exponent bits, so every operand is brought to
-// at most 1: x by 2^ex per right-hand side (k_mm_max), W row l by 2^et(l), |T_l| <= |W_l|_1 |x|_inf
+// at most 1: x by 2^-ex per right-hand side (k_mm_max), W row l by 2^et(l), |T_l| <= |W_l|_1 |x|_inf
 // <= 1 with it, and Y row l (dense blocks: the block) by 2^(E - et(l)), E per output cluster the
 // largest that keeps all its terms at most 1 (k_mm_prep, once per operator).  Sums of one
-// output then share the factor 2^(ex + E).
+// output then share the factor 2^(E - ex).  The scales are exponents, never cut off at a float's
+// range (times_pow2): one that is would be missing from the sum's factor.
 //
 // Product: a = hi + lo, hi = fp16(2^15 a), lo = fp16(2^15 a - hi): 22 bits for a >= 2^-17, an
 // absolute 2^-40 below; hi hi + hi lo + lo hi.  The tensor core truncates its FP32 sums, so each
@@ -119,22 +120,28 @@ __device__ __forceinline__ void split_pair(float a, float al, float b, float bl,
 }
 
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
-// the least e with v <= 2^e (0 for 0 and for values that are not finite), within +-120
+// v 2^e, in two factors so that every exponent a scale of FP32 data can have (below 252 either
+// way) is taken whole: a factor cut off at the range of a float would be missing from the result
+__device__ __forceinline__ float times_pow2(float v, int e)
+{
+    const int h = e / 2;
+    return v * pow2f(h) * pow2f(e - h);
+}
+// the least e with v <= 2^e (0 for 0 and for values that are not finite)
 __device__ __forceinline__ int ceil_exp(float v)
 {
     if (!(v > 0.f) || !isfinite(v)) return 0;
     int e;
     const float f = frexpf(v, &e);
-    if (f == 0.5f) --e;
-    return min(max(e, -120), 120);
+    return f == 0.5f ? e - 1 : e;
 }
 
 // ---- x: scale per right-hand side, operand tiles --------------------------------
 
-// xs[2 r] = 2^ex, xs[2 r + 1] = 2^-ex with 2^ex |x_r|_inf <= 1; one CTA per right-hand side
+// ex[r] = the least e with |x_r|_inf <= 2^e; one CTA per right-hand side
 // (245 KB of x at 30,720 unknowns: a few us beside products of milliseconds)
 __global__ void __launch_bounds__(1024)
-k_mm_max(const float2 *__restrict__ x, int64_t pN, float *__restrict__ xs)
+k_mm_max(const float2 *__restrict__ x, int64_t pN, int *__restrict__ ex)
 {
     __shared__ float sm[32];
     const float4 *v = reinterpret_cast<const float4 *>(x + blockIdx.x * pN);   // pN is even
@@ -148,11 +155,7 @@ k_mm_max(const float2 *__restrict__ x, int64_t pN, float *__restrict__ xs)
     __syncthreads();
     if (threadIdx.x < 32) {
         m = warp_max(sm[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            const int e = ceil_exp(m);
-            xs[2 * blockIdx.x] = pow2f(-e);
-            xs[2 * blockIdx.x + 1] = pow2f(e);
-        }
+        if (threadIdx.x == 0) ex[blockIdx.x] = ceil_exp(m);
     }
 }
 
@@ -160,7 +163,7 @@ k_mm_max(const float2 *__restrict__ x, int64_t pN, float *__restrict__ xs)
 template <bool RES>
 __global__ void __launch_bounds__(128)
 k_mm_split(const XChunk *__restrict__ xch, int n_xch, const float2 *__restrict__ x, int64_t pN, int nrhs,
-           const float *__restrict__ xs, uint32_t *__restrict__ xt)
+           const int *__restrict__ ex, uint32_t *__restrict__ xt)
 {
     const int ch = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     if (ch >= n_xch) return;
@@ -173,8 +176,8 @@ k_mm_split(const XChunk *__restrict__ xch, int n_xch, const float2 *__restrict__
         if (q < nrhs && k < c.len) {
             v = *reinterpret_cast<const float4 *>(x + q * pN + c.off + k);
             if (k + 1 >= c.len) v.z = v.w = 0.f;
-            const float s = xs[2 * q];
-            v.x *= s; v.y *= s; v.z *= s; v.w *= s;
+            const int e = -ex[q];
+            v = make_float4(times_pow2(v.x, e), times_pow2(v.y, e), times_pow2(v.z, e), times_pow2(v.w, e));
         }
         if constexpr (RES) {
             uint32_t re[4], im[4];
@@ -453,7 +456,7 @@ struct MmOutArgs {
     const uint32_t *xt, *tt;
     int n_xch, n_tiles, nrhs;
     int64_t n_tch;
-    const float *xs;
+    const int *ex;           // per right-hand side: its scale's exponent (k_mm_max)
     int groups;              // CTAs of a unit, over the right-hand sides
 };
 
@@ -576,20 +579,19 @@ k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
             for (int m = 0; m < MT; ++m) { acc[m][0].drain(); acc[m][1].drain(); }
         }
     });
-    const float ci = pow2f(-E) * (1.f / (MM_TOP * MM_TOP));
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int r = 16 * (m0 + m) + g + 8 * h;
             if (r >= p.nrhs) continue;
-            const float xi = p.xs[2 * r + 1];
+            const int e = p.ex[r] - E - 30;                // operands are scaled to 2^15
 #pragma unroll
             for (int n = 0; n < 2; ++n) {
                 if (h == 0) acc[m][n].drain();
                 const int i = n0 + 8 * n + 2 * t;
-                const float2 a = make_float2(acc[m][n].s[0][2 * h] * ci * xi, acc[m][n].s[1][2 * h] * ci * xi);
-                const float2 b = make_float2(acc[m][n].s[0][2 * h + 1] * ci * xi, acc[m][n].s[1][2 * h + 1] * ci * xi);
+                const float2 a = make_float2(times_pow2(acc[m][n].s[0][2 * h], e), times_pow2(acc[m][n].s[1][2 * h], e));
+                const float2 b = make_float2(times_pow2(acc[m][n].s[0][2 * h + 1], e), times_pow2(acc[m][n].s[1][2 * h + 1], e));
                 float2 *zz = z + (int64_t)r * pN + U.out0 + i;
                 if (i + 1 < U.mlen) red2(zz, a, b);
                 else if (i < U.mlen) red1(zz, a);
@@ -661,12 +663,11 @@ k_mm_resid(MmOutArgs p, double2 *__restrict__ own, int64_t pstride, int64_t pN)
                 }
     }
     if (kw != 0) return;
-    const double cs = ldexp(1.0, -16 - E);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = 16 * m0 + g + 8 * h;
         if (r >= p.nrhs) continue;
-        const double sc = cs * (double)p.xs[2 * r + 1];
+        const double sc = ldexp(1.0, p.ex[r] - E - 16);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int i = n0 + 2 * t + j, a = 2 * h + j;
@@ -680,11 +681,13 @@ k_mm_resid(MmOutArgs p, double2 *__restrict__ own, int64_t pstride, int64_t pN)
 // ---- scales, once per operator -------------------------------------------------------
 
 // Per directed product (a warp each): low-rank, et of every W row from its 1-norm (FP32, rounded
-// up) into wscale and, negated, into rscale, and E's bound et - exponent(max Y row); dense,
-// E's bound from the block's largest component.
+// up, of the row scaled to 1 so that it cannot overflow) into wexp and, negated, into rexp, and
+// E's bound et - exponent(max Y row); dense, E's bound from the block's largest component.  A
+// row pair whose W row is zero gives nothing: its Y row is packed as zeros (ROW_OFF).
+constexpr int ROW_OFF = -(1 << 20);
 __global__ void __launch_bounds__(256)
-k_mm_prep(const MmSet *__restrict__ sets, int64_t n, const float2 *__restrict__ pool, float *__restrict__ wscale,
-          float *__restrict__ rscale, int *__restrict__ eout)
+k_mm_prep(const MmSet *__restrict__ sets, int64_t n, const float2 *__restrict__ pool, int *__restrict__ wexp,
+          int *__restrict__ rexp, int *__restrict__ eout)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -699,34 +702,37 @@ k_mm_prep(const MmSet *__restrict__ sets, int64_t n, const float2 *__restrict__ 
             if (m > 0.f) bound = -ceil_exp(m);
         }
         for (int l = 0; l < S.rank; ++l) {
-            float a = 0.f, m = 0.f;
+            float w = 0.f, a = 0.f, m = 0.f;
+            for (int j = lane; j < S.wlen; j += 32) w = fmaxf(w, linf(pool[S.w + (int64_t)l * S.w_ld + j]));
+            for (int i = lane; i < S.ylen; i += 32) m = fmaxf(m, linf(pool[S.y + (int64_t)l * S.y_ld + i]));
+            w = warp_max(w);
+            m = warp_max(m);
+            const int ew = -ceil_exp(w);
             for (int j = lane; j < S.wlen; j += 32) {
                 const float2 v = pool[S.w + (int64_t)l * S.w_ld + j];
-                a = __fadd_ru(a, __fadd_ru(fabsf(v.x), fabsf(v.y)));
+                a = __fadd_ru(a, __fadd_ru(fabsf(times_pow2(v.x, ew)), fabsf(times_pow2(v.y, ew))));
             }
-            for (int i = lane; i < S.ylen; i += 32) m = fmaxf(m, linf(pool[S.y + (int64_t)l * S.y_ld + i]));
 #pragma unroll
             for (int s = 16; s >= 1; s >>= 1) a = __fadd_ru(a, __shfl_xor_sync(FULL, a, s));
-            m = warp_max(m);
-            const int et = min(-ceil_exp(a), 100);
+            const int et = ew - ceil_exp(a);
             if (lane == 0) {
-                wscale[2 * (int64_t)S.p0 + l] = pow2f(et);
-                rscale[2 * (int64_t)S.t0 + l] = pow2f(-et);
+                wexp[2 * (int64_t)S.p0 + l] = et;
+                rexp[2 * (int64_t)S.t0 + l] = w == 0.f ? ROW_OFF : -et;
             }
-            if (m > 0.f) bound = min(bound, et - ceil_exp(m));
+            if (m > 0.f && w != 0.f) bound = min(bound, et - ceil_exp(m));
         }
-        if (lane == 0 && bound < 1000) atomicMin(eout + S.cl, min(max(bound, -120), 100));
+        if (lane == 0 && bound < 1000) atomicMin(eout + S.cl, bound);
     }
 }
-// rscale = 2^(E - et) of every T row; clusters with nothing but zeros get E = 0
+// rexp = E - et of every T row; clusters with nothing but zeros get E = 0
 __global__ void __launch_bounds__(256)
-k_mm_rscale(const MmSet *__restrict__ sets, int64_t n, float *__restrict__ rscale, const int *__restrict__ eout)
+k_mm_rexp(const MmSet *__restrict__ sets, int64_t n, int *__restrict__ rexp, const int *__restrict__ eout)
 {
     for (int64_t q = blockIdx.x * 256ll + threadIdx.x; q < n; q += gridDim.x * 256ll) {
         const MmSet S = sets[q];
         for (int l = 0; l < S.rank; ++l) {
-            float &v = rscale[2 * (int64_t)S.t0 + l];
-            v = pow2f(min(eout[S.cl] + ((__float_as_int(v) >> 23) - 127), 110));
+            int &v = rexp[2 * (int64_t)S.t0 + l];
+            if (v != ROW_OFF) v += eout[S.cl];
         }
     }
 }
@@ -738,15 +744,22 @@ __global__ void k_mm_eout(int *eout, int n, int set)
 
 // ---- operand streams, once per operator ---------------------------------------------
 
-__device__ __forceinline__ void pack_tile(float4 *dst, const float2 (&v)[4], const float (&s)[4], int lane)
+// the lane's four values times 2^(e + 15)
+__device__ __forceinline__ void pack_tile(float4 *dst, const float2 (&v)[4], const int (&e)[4], int lane)
 {
-    dst[lane] = make_float4(v[0].x * s[0] * MM_TOP, v[0].y * s[0] * MM_TOP, v[1].x * s[1] * MM_TOP, v[1].y * s[1] * MM_TOP);
-    dst[32 + lane] = make_float4(v[2].x * s[2] * MM_TOP, v[2].y * s[2] * MM_TOP, v[3].x * s[3] * MM_TOP, v[3].y * s[3] * MM_TOP);
+    float f[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        f[2 * q] = ldexpf(v[q].x, e[q] + 15);
+        f[2 * q + 1] = ldexpf(v[q].y, e[q] + 15);
+    }
+    dst[lane] = make_float4(f[0], f[1], f[2], f[3]);
+    dst[32 + lane] = make_float4(f[4], f[5], f[6], f[7]);
 }
 
 // the output stream, a warp per chunk
 __global__ void __launch_bounds__(256)
-k_mm_pack_out(const MmChunk *__restrict__ chunks, int64_t n, const int64_t *__restrict__ rows, const float *__restrict__ rscale,
+k_mm_pack_out(const MmChunk *__restrict__ chunks, int64_t n, const int64_t *__restrict__ rows, const int *__restrict__ rexp,
               const int *__restrict__ eout, const float2 *__restrict__ pool, unsigned char *__restrict__ os,
               int32_t *__restrict__ ca)
 {
@@ -755,12 +768,12 @@ k_mm_pack_out(const MmChunk *__restrict__ chunks, int64_t n, const int64_t *__re
         const MmChunk C = chunks[c];
         if (lane == 0) ca[c] = C.kind == 2 ? -1 - C.a : C.a;
         int64_t off[4];
-        float s[4];
+        int e[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int k = 2 * t + (q & 1) + 8 * (q >> 1);
             off[q] = C.kind == 2 ? rows[C.src + k] : k < C.klen ? C.src + (C.kind == 0 ? k : (int64_t)k * C.ld) : -1;
-            s[q] = C.kind == 2 ? rscale[C.src + k] : pow2f(eout[C.cl]);
+            e[q] = C.kind == 2 ? rexp[C.src + k] : eout[C.cl];
         }
         for (int tl = 0; tl < C.tiles; ++tl) {
             const int i = 8 * tl + g;
@@ -768,14 +781,14 @@ k_mm_pack_out(const MmChunk *__restrict__ chunks, int64_t n, const int64_t *__re
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 v[q] = off[q] >= 0 && i < C.olen ? pool[off[q] + (C.kind == 0 ? (int64_t)i * C.ld : i)] : make_float2(0.f, 0.f);
-            pack_tile(reinterpret_cast<float4 *>(os + ((int64_t)C.pos + tl) * MM_TILE), v, s, lane);
+            pack_tile(reinterpret_cast<float4 *>(os + ((int64_t)C.pos + tl) * MM_TILE), v, e, lane);
         }
     }
 }
 
 // the stage-1 stream, a CTA per batch, a warp per tile of 8 W rows
 __global__ void __launch_bounds__(256)
-k_mm_pack_w(const MmBatch *__restrict__ batches, const MmPair *__restrict__ pairs, const float *__restrict__ wscale,
+k_mm_pack_w(const MmBatch *__restrict__ batches, const MmPair *__restrict__ pairs, const int *__restrict__ wexp,
             const float2 *__restrict__ pool, unsigned char *__restrict__ ws, int32_t *__restrict__ tdst)
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -785,8 +798,7 @@ k_mm_pack_w(const MmBatch *__restrict__ batches, const MmPair *__restrict__ pair
         const int tile = B.tile0 + it;
         const MmPair P = pairs[4 * tile + (g >> 1)];
         const int64_t off = P.w < 0 || ((g & 1) && P.ld == 0) ? -1 : P.w + (g & 1) * (int64_t)P.ld;
-        const float sw = wscale[8 * tile + g];
-        const float s[4] = {sw, sw, sw, sw};
+        const int ew = wexp[8 * tile + g], e[4] = {ew, ew, ew, ew};
         if (lane < 4) tdst[4 * tile + lane] = pairs[4 * tile + lane].dst;
         for (int c = 0; c < nch; ++c) {
             float2 v[4];
@@ -795,27 +807,27 @@ k_mm_pack_w(const MmBatch *__restrict__ batches, const MmPair *__restrict__ pair
                 const int k = c * MM_K + 2 * t + (q & 1) + 8 * (q >> 1);
                 v[q] = off >= 0 && k < B.klen ? pool[off + k] : make_float2(0.f, 0.f);
             }
-            pack_tile(reinterpret_cast<float4 *>(ws + ((int64_t)B.pos + (int64_t)it * nch + c) * MM_TILE), v, s, lane);
+            pack_tile(reinterpret_cast<float4 *>(ws + ((int64_t)B.pos + (int64_t)it * nch + c) * MM_TILE), v, e, lane);
         }
     }
 }
 
 } // namespace
 
-// scales and operand streams of a level's lists (device copies M; wscale, rscale zeroed by the caller)
+// scales and operand streams of a level's lists (device copies M; wexp, rexp zeroed by the caller)
 void launch_mm_pack(const LevelList &L, const MmPackArgs &M, const float2 *pool, cudaStream_t s)
 {
     const int n_cl = M.n_cl;
     if (M.n_sets <= 0 || n_cl <= 0) return;
     k_mm_eout<<<(n_cl + 255) / 256, 256, 0, s>>>(L.d_mm_eout, n_cl, 1);
-    k_mm_prep<<<(unsigned)std::min<int64_t>((M.n_sets + 7) / 8, 152 * 16), 256, 0, s>>>(M.sets, M.n_sets, pool, M.wscale, M.rscale,
+    k_mm_prep<<<(unsigned)std::min<int64_t>((M.n_sets + 7) / 8, 152 * 16), 256, 0, s>>>(M.sets, M.n_sets, pool, M.wexp, M.rexp,
                                                                                       L.d_mm_eout);
     k_mm_eout<<<(n_cl + 255) / 256, 256, 0, s>>>(L.d_mm_eout, n_cl, 0);
-    k_mm_rscale<<<(unsigned)std::min<int64_t>((M.n_sets + 255) / 256, 4096), 256, 0, s>>>(M.sets, M.n_sets, M.rscale, L.d_mm_eout);
+    k_mm_rexp<<<(unsigned)std::min<int64_t>((M.n_sets + 255) / 256, 4096), 256, 0, s>>>(M.sets, M.n_sets, M.rexp, L.d_mm_eout);
     k_mm_pack_out<<<(unsigned)std::min<int64_t>((M.n_chunks + 7) / 8, 152 * 32), 256, 0, s>>>(
-        M.chunks, M.n_chunks, M.rows, M.rscale, L.d_mm_eout, pool, L.d_mm_os, L.d_mm_ca);
+        M.chunks, M.n_chunks, M.rows, M.rexp, L.d_mm_eout, pool, L.d_mm_os, L.d_mm_ca);
     if (L.mm_n_batch > 0)
-        k_mm_pack_w<<<(unsigned)L.mm_n_batch, 256, 0, s>>>(L.d_mm_batch, M.pairs, M.wscale, pool, L.d_mm_ws, L.d_mm_tdst);
+        k_mm_pack_w<<<(unsigned)L.mm_n_batch, 256, 0, s>>>(L.d_mm_batch, M.pairs, M.wexp, pool, L.d_mm_ws, L.d_mm_tdst);
 }
 size_t mm_stream_bytes(int64_t tiles) { return (size_t)tiles * MM_TILE; }
 
@@ -835,7 +847,7 @@ size_t mm_ws_bytes(const LevelList &L, int nrhs, bool res)
     const int pass = mm_pass(L, nrhs, res);
     const size_t tiles = (size_t)(pass + 15) / 16;
     const size_t words = res ? tile_words<true>() : tile_words<false>();
-    return tiles * words * sizeof(uint32_t) * ((size_t)L.mm_n_xch + (size_t)L.mm_n_tch) + 2 * sizeof(float) * (size_t)pass;
+    return tiles * words * sizeof(uint32_t) * ((size_t)L.mm_n_xch + (size_t)L.mm_n_tch) + sizeof(int) * (size_t)pass;
 }
 
 namespace {
@@ -848,12 +860,12 @@ void mm_attr(const void *kern, int smem)
 
 // x of a pass into operand tiles, then stage 1
 template <bool RES>
-int mm_inputs(hm_matrix h, const LevelList &L, const float2 *x, int nr, uint32_t *xt, uint32_t *tt, float *xs, cudaStream_t s)
+int mm_inputs(hm_matrix h, const LevelList &L, const float2 *x, int nr, uint32_t *xt, uint32_t *tt, int *ex, cudaStream_t s)
 {
     const int tiles = (nr + 15) / 16;
-    k_mm_max<<<nr, 1024, 0, s>>>(x, h->pN, xs);
+    k_mm_max<<<nr, 1024, 0, s>>>(x, h->pN, ex);
     k_mm_split<RES><<<dim3((unsigned)((L.mm_n_xch + 3) / 4), (unsigned)tiles), 128, 0, s>>>(L.d_mm_xch, (int)L.mm_n_xch, x,
-                                                                                           h->pN, nr, xs, xt);
+                                                                                           h->pN, nr, ex, xt);
     if (L.mm_n_batch == 0) return 2;
     auto go = [&](auto kern, int mt, int smem) {
         mm_attr((const void *)kern, smem);
@@ -888,15 +900,15 @@ int launch_mm_product(hm_matrix h, const LevelList &L, const float2 *x, float2 *
     const int pass = mm_pass(L, nrhs, false);
     const size_t tiles_max = (size_t)(pass + 15) / 16;
     uint32_t *xt = (uint32_t *)ws, *tt = xt + tiles_max * tile_words<false>() * L.mm_n_xch;
-    float *xs = (float *)(tt + tiles_max * tile_words<false>() * L.mm_n_tch);
+    int *ex = (int *)(tt + tiles_max * tile_words<false>() * L.mm_n_tch);
     for (int r0 = 0; r0 < nrhs; r0 += pass) {
         const int nr = std::min(pass, nrhs - r0), tiles = (nr + 15) / 16;
         const float2 *xp = x + (int64_t)r0 * h->pN;
-        n += mm_inputs<false>(h, L, xp, nr, xt, tt, xs, s) + 1;
+        n += mm_inputs<false>(h, L, xp, nr, xt, tt, ex, s) + 1;
         // tiles of 16 right-hand sides a warp up to 16 of them, 32 above, two such groups a CTA above 32
         const int mw = tiles > 2 ? 2 : 1, mt = tiles > 1 ? 2 : 1, groups = (tiles + mt * mw - 1) / (mt * mw);
         MmOutArgs a{coarse ? L.d_mm_unit2 : L.d_mm_unit, L.d_mm_ca, L.d_mm_eout, L.d_mm_os, xt, tt, (int)L.mm_n_xch,
-                    tiles, nr, L.mm_n_tch, xs, groups};
+                    tiles, nr, L.mm_n_tch, ex, groups};
         float2 *zp = z + (int64_t)r0 * h->pN;
         const unsigned units = (unsigned)(coarse ? L.mm_n_unit2 : L.mm_n_unit);
         auto go = [&](auto kern) {
@@ -919,12 +931,12 @@ int launch_mm_resid(hm_matrix h, const LevelList &L, const float2 *x, double2 *o
     const int pass = mm_pass(L, nrhs, true);
     const size_t tiles_max = (size_t)(pass + 15) / 16;
     uint32_t *xt = (uint32_t *)ws, *tt = xt + tiles_max * tile_words<true>() * L.mm_n_xch;
-    float *xs = (float *)(tt + tiles_max * tile_words<true>() * L.mm_n_tch);
+    int *ex = (int *)(tt + tiles_max * tile_words<true>() * L.mm_n_tch);
     for (int r0 = 0; r0 < nrhs; r0 += pass) {
         const int nr = std::min(pass, nrhs - r0), tiles = (nr + 15) / 16;
-        n += mm_inputs<true>(h, L, x + (int64_t)r0 * h->pN, nr, xt, tt, xs, s) + 1;
+        n += mm_inputs<true>(h, L, x + (int64_t)r0 * h->pN, nr, xt, tt, ex, s) + 1;
         MmOutArgs a{L.d_mm_runit, L.d_mm_ca, L.d_mm_eout, L.d_mm_os, xt, tt, (int)L.mm_n_xch,
-                    tiles, nr, L.mm_n_tch, xs, tiles};
+                    tiles, nr, L.mm_n_tch, ex, tiles};
         mm_attr((const void *)k_mm_resid, MM_SMEM);
         k_mm_resid<<<(unsigned)(tiles * L.mm_n_runit), MMW * 32, MM_SMEM, s>>>(a, own + (int64_t)r0 * h->pN,
                                                                                            pstride, h->pN);
