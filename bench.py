@@ -521,13 +521,13 @@ def product_roofline(A, b, x, opts, nrhs, Kp, sm_max):
                   "(dense products and second stages; tcgen05 kind::tf32, 3xTF32; units of <= 64 K chunks; blocks "
                   "<= 64 x 64, rank <= 32) + k_apply_items for larger blocks (k_mrhs_tc.cu, k_product.cu)")
     elif prod_choice == 32:
-        # products of FP16 halves on mma.sync: three MMAs per useful FP32-accurate product, so the roof is the
-        # FP16 (= bf16) tensor peak / 3 (the instruction itself reached 606 TFLOP/s from registers)
+        # products of BF16 parts on mma.sync: six MMAs per useful FP32-accurate product, so the roof is the
+        # bf16 tensor peak / 6 (the instruction itself reached 606 TFLOP/s from registers)
         bf16_s = (PEAKS or {}).get("bf16_tflops_sustained")
-        bound, unit, rpeak = "tensor", "TFLOP/s", (bf16_s if bf16_s else 1700.0) / 3.0
-        rkind = ("measured sustained bf16 %.1f TFLOP/s / 3 (three FP16 products)" % bf16_s
-                 if bf16_s else "fallback 1.7 PFLOP/s bf16 sustained / 3")
-        kernel = ("k_mm_max + k_mm_split + k_mm_stage1 + k_mm_out (mma.sync m16n8k16, FP16 halves; blocks <= 64 x 64, "
+        bound, unit, rpeak = "tensor", "TFLOP/s", (bf16_s if bf16_s else 1700.0) / 6.0
+        rkind = ("measured sustained bf16 %.1f TFLOP/s / 6 (six BF16 products)" % bf16_s
+                 if bf16_s else "fallback 1.7 PFLOP/s bf16 sustained / 6")
+        kernel = ("k_mm_max + k_mm_split + k_mm_stage1 + k_mm_out (mma.sync m16n8k16, BF16 parts; blocks <= 64 x 64, "
                   "rank <= 32) + k_apply_items for larger blocks (k_mm.cu, k_product.cu)")
     elif flops_per_launch / (alu_peak * 1e12) > per_launch_bytes / (peak * 1e9):
         bound, unit, rpeak = "alu", "TFLOP/s", alu_peak

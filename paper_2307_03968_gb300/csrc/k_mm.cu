@@ -7,42 +7,47 @@
 // neither a rank nor a block is padded to an instruction's shape (only the 16 of a chunk
 // and the 8 of a cluster's outputs).
 //
-// Why mma.sync m16n8k16 with FP16 operands.  FP32 accuracy takes 3 products of 11-bit
-// halves whatever the type; FP16 has TF32's 11 bits at twice its rate (measured, registers
-// only: 606 against 302 TFLOP/s; the tcgen05 kernel of k_mrhs_tc.cu, 1952 TFLOP/s in bf16,
-// reaches 28 % of its TF32 roof on the hand-offs of its operand pipeline), and a call of 4 to
-// 64 right-hand sides fills its tiles of 16, which a tile of 128 does not.
+// Why mma.sync m16n8k16 with 16-bit operands.  It runs at twice the rate of TF32 (measured,
+// registers only: 606 against 302 TFLOP/s; the tcgen05 kernel of k_mrhs_tc.cu, 1952 TFLOP/s in
+// bf16, reaches 28 % of its TF32 roof on the hand-offs of its operand pipeline), and a call of 4
+// to 64 right-hand sides fills its tiles of 16, which a tile of 128 does not.  BF16 parts for the
+// FP32 product, FP16 digits for the residual.
 //
 // Operand streams.  The first call repacks the blocks (k_mm_pack_*): for each chunk of 16 K and
 // tile of 8 outputs the 128 values in the order the lanes of the instruction take them, FP32,
 // scaled, both directions of every block: twice the blocks' bytes.  A unit's blocks are then
 // one contiguous stream, copied with a few cp.async a thread, and what is left beside the
-// instructions is the split into halves or digits in registers.  (Gathered from the blocks
+// instructions is the split into parts or digits in registers.  (Gathered from the blocks
 // in place, by rows and by columns, the same kernels spent 500 instructions on 24 products:
 // 0.60 ms instead of 0.31 for 16 right-hand sides of the 12,600-unknown cube.)
 //
-// Measured (GB300): a product of the 30,720-unknown sphere with 181 right-hand sides 6.0 ms, of
-// which stage 1 1.6 (the tcgen05 kernels: 7.3); 16 right-hand sides of the 12,600-unknown
-// cube 0.34 ms (SIMT chunks of 16: 0.66); the FP64-class residual of those 24 ms (SIMT
-// owner kernel: 68) and 1.2 ms (2.3).
+// Measured (GB300): a product of the 30,720-unknown sphere with 181 right-hand sides 10.2 ms
+// (the tcgen05 kernels, of 3xTF32 accuracy, 8.0), with 64 of them 3.4 (SIMT chunks of 16: 11.8),
+// with 16 1.0 (3.0); 16 right-hand sides of the 12,600-unknown cube 0.53 ms (0.69); the FP64-class residual
+// of the 181 24 ms (SIMT owner kernel: 70) and of the 16 1.2 ms (2.5).
 //
 // Right-hand sides are the instruction's M, so an accumulator pair of stage 1 is, in place,
 // an operand pair of the output stage (its K are the W rows): T is stored in operand layout.
-// Operand tile of 16 right-hand sides x 16 K: one plane per half (product: re hi, re lo, im
-// hi, im lo; residual: re 1..4, im 1..4), each 4 registers x 32 words; word t * 8 + g of
+// Operand tile of 16 right-hand sides x 16 K: one plane per part (product: re 1..3, im
+// 1..3; residual: re 1..4, im 1..4), each 4 registers x 32 words; word t * 8 + g of
 // register r is the pair of K 2t, 2t + 1 (+ 8 for r >= 2) of right-hand side g (+ 8 for odd r):
 // what lane (g, t) holds, and 32 bytes per t, so that stage 1 writes whole sectors.
 //
-// Scales (powers of two, exact).  FP16 has 5 exponent bits, so every operand is brought to
-// at most 1: x by 2^-ex per right-hand side (k_mm_max), W row l by 2^et(l), |T_l| <= |W_l|_1 |x|_inf
+// Scales (powers of two, exact), so that FP16 digits do and BF16 parts of any data can hold
+// what FP32 holds: every operand is brought to at most 1: x by 2^-ex per right-hand side (k_mm_max), W row l by 2^et(l), |T_l| <= |W_l|_1 |x|_inf
 // <= 1 with it, and Y row l (dense blocks: the block) by 2^(E - et(l)), E per output cluster the
 // largest that keeps all its terms at most 1 (k_mm_prep, once per operator).  Sums of one
 // output then share the factor 2^(E - ex).  The scales are exponents, never cut off at a float's
 // range (times_pow2): one that is would be missing from the sum's factor.
 //
-// Product: a = hi + lo, hi = fp16(2^15 a), lo = fp16(2^15 a - hi): 22 bits for a >= 2^-17, an
-// absolute 2^-40 below; hi hi + hi lo + lo hi.  The tensor core truncates its FP32 sums, so each
-// chunk's six products start from zero and are added to the running sum in FP32 outside.
+// Product: a = a1 + a2 + a3, three BF16 parts of 8 bits, an FP32 number exactly (the last bits of
+// one below 2^-109 of the scale apart): a1 b1 + a1 b2 + a2 b1 + a1 b3 + a2 b2 + a3 b1, the three
+// left out are below 2^-24 of a b.  BF16 has FP32's exponents, so a small operand keeps its bits
+// beside a large one; two FP16 halves (22 bits, three products, 6.4 ms for those 181) lose them
+// below 2^-17 of the scale: entries at 2^-30 came out to 1e-3.  The tensor core truncates its FP32 sums,
+// so each chunk's sums start from zero and join the running sum in FP32: 1.1e-7 to 2.0e-7 of
+// |A x| over the tested operators (FP32 kernels: 1.6e-7 to 2.2e-7); 32 chunks in the tensor core
+// instead of one took 6 % less time and erred by 1e-6.
 //
 // FP64-class residual: a = 2^-8 d1 + 2^-17 d2 + 2^-26 d3 + 2^-35 r, the digits integers of at most
 // 2^8, r a FP16 of at most 2^8: 38 bits below the scale, exact for every FP32 a >= 2^-14 (integer
@@ -68,12 +73,11 @@ using namespace dot2;
 
 constexpr int MMW = 8;                    // warps per CTA
 constexpr int MM_PLANE = 128;             // words of one plane of an operand tile
-template <bool RES> constexpr int planes() { return RES ? 8 : 4; }
+template <bool RES> constexpr int planes() { return RES ? 8 : 6; }
 template <bool RES> constexpr int tile_words() { return planes<RES>() * MM_PLANE; }
 constexpr int MM_PASS_MIN = 64;           // right-hand sides per pass, at least (mm_pass)
 constexpr size_t MM_PASS_BYTES = size_t(4) << 30;   // operand tiles of a pass, above that many
 constexpr int MM_DRAIN = 4;               // residual: chunks per exact accumulation
-constexpr float MM_TOP = 32768.f;         // product: operands are scaled to at most 2^15
 
 __device__ __forceinline__ void mma16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
 {
@@ -81,19 +85,29 @@ __device__ __forceinline__ void mma16(float (&c)[4], const uint32_t (&a)[4], con
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+// the same with BF16 operands
+__device__ __forceinline__ void mma16b(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
 __device__ __forceinline__ uint32_t h2(float a, float b)
 {
     const __half2 v = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t *>(&v);
 }
-__device__ __forceinline__ float2 f2(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2 *>(&v)); }
 
-// the planes of a pair of normalised values (product: already times 2^15)
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[2])
+// the planes of a pair of values: each cut into three BF16 parts of 8 bits, exactly
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[3])
 {
-    p[0] = h2(a, b);
-    const float2 h = f2(p[0]);
-    p[1] = h2(__fsub_rn(a, h.x), __fsub_rn(b, h.y));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+        p[i] = __byte_perm(ua, ub, 0x7632);                  // the upper halves
+        a = __fsub_rn(a, __uint_as_float(ua & 0xffff0000u));
+        b = __fsub_rn(b, __uint_as_float(ub & 0xffff0000u));
+    }
 }
 // the nearest integer of |v| < 2^22 (ties to even)
 __device__ __forceinline__ float nearest(float v) { return __fsub_rn(__fadd_rn(v, 12582912.f), 12582912.f); }
@@ -189,13 +203,13 @@ k_mm_split(const XChunk *__restrict__ xch, int n_xch, const float2 *__restrict__
                 w[(4 + p) * MM_PLANE + r * 32] = im[p];
             }
         } else {
-            uint32_t re[2], im[2];
-            split_pair(v.x * MM_TOP, v.z * MM_TOP, re);
-            split_pair(v.y * MM_TOP, v.w * MM_TOP, im);
+            uint32_t re[3], im[3];
+            split_pair(v.x, v.z, re);
+            split_pair(v.y, v.w, im);
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
+            for (int p = 0; p < 3; ++p) {
                 w[p * MM_PLANE + r * 32] = re[p];
-                w[(2 + p) * MM_PLANE + r * 32] = im[p];
+                w[(3 + p) * MM_PLANE + r * 32] = im[p];
             }
         }
     }
@@ -204,7 +218,7 @@ k_mm_split(const XChunk *__restrict__ xch, int n_xch, const float2 *__restrict__
 // ---- operands of the blocks -------------------------------------------------------
 
 // the B operands of one chunk and 8 outputs from the lane's four complex values (K 2t, 2t + 1,
-// 2t + 8, 2t + 9 of output g, times 2^15): planes [half or digit][register]
+// 2t + 8, 2t + 9 of output g): planes [part or digit][register]
 template <bool RES> struct BFrag { uint32_t re[planes<RES>() / 2][2], im[planes<RES>() / 2][2]; };
 
 // tile: an 8 x 16 tile of an operand stream in shared memory, two planes of 16 bytes a lane
@@ -217,8 +231,8 @@ __device__ __forceinline__ void make_b(const unsigned char *tile, int lane, BFra
         const float4 v = *reinterpret_cast<const float4 *>(tile + q * 512 + lane * 16);
         uint32_t re[H], im[H];
         if constexpr (RES) {
-            split_pair(v.x * (1.f / MM_TOP), 0.f, v.z * (1.f / MM_TOP), 0.f, re);
-            split_pair(v.y * (1.f / MM_TOP), 0.f, v.w * (1.f / MM_TOP), 0.f, im);
+            split_pair(v.x, 0.f, v.z, 0.f, re);
+            split_pair(v.y, 0.f, v.w, 0.f, im);
         } else {
             split_pair(v.x, v.z, re);
             split_pair(v.y, v.w, im);
@@ -248,50 +262,49 @@ __device__ __forceinline__ void load_plane(uint32_t (&a)[4], const uint32_t *til
 // sums of one tile of 16 right-hand sides x 8 outputs
 template <bool RES> struct Acc;
 template <> struct Acc<false> {
-    float s[2][4], c[2][4];     // re, im: the running sums, and what the tensor core holds since the last drain
+    float s[2][4];              // re, im
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) s[0][i] = s[1][i] = c[0][i] = c[1][i] = 0.f;
-    }
-    __device__ __forceinline__ void drain()
-    {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            s[0][i] += c[0][i];
-            s[1][i] += c[1][i];
-            c[0][i] = c[1][i] = 0.f;
-        }
+        for (int i = 0; i < 4; ++i) s[0][i] = s[1][i] = 0.f;
     }
 };
 // one chunk into N tiles of 8 outputs (the products of the N tiles interleaved: a tile alone is
-// two chains of dependent instructions): A operand planes at `tile` (the lane's word), B operands b
+// two chains of dependent instructions): A operand planes at `tile` (the lane's word), B operands b.
+// The small products first, so that only the last two instructions truncate at the sum's own size.
 template <int N>
 __device__ __forceinline__ void mm_chunk(Acc<false> (&s)[N], const uint32_t *tile, const BFrag<false> (&b)[N])
 {
+    float c[N][2][4] = {};
     uint32_t xr[4], xi[4];
     auto terms = [&](int q) {
 #pragma unroll
         for (int n = 0; n < N; ++n) {
-            mma16(s[n].c[0], xr, b[n].re[q]);
-            mma16(s[n].c[1], xr, b[n].im[q]);
+            mma16b(c[n][0], xr, b[n].re[q]);
+            mma16b(c[n][1], xr, b[n].im[q]);
         }
 #pragma unroll
         for (int n = 0; n < N; ++n) {
             uint32_t m[2];
             negate(m, b[n].im[q]);
-            mma16(s[n].c[0], xi, m);
-            mma16(s[n].c[1], xi, b[n].re[q]);
+            mma16b(c[n][0], xi, m);
+            mma16b(c[n][1], xi, b[n].re[q]);
         }
     };
-    // the small products first: only the last two instructions truncate at the sum's own size
-    load_plane(xr, tile, 1);
-    load_plane(xi, tile, 3);
-    terms(0);
-    load_plane(xr, tile, 0);
-    load_plane(xi, tile, 2);
-    terms(1);
-    terms(0);
+#pragma unroll
+    for (int p = 2; p >= 0; --p) {                 // parts p of x with parts 2 - p .. 0 of the block
+        load_plane(xr, tile, p);
+        load_plane(xi, tile, 3 + p);
+#pragma unroll
+        for (int q = 2 - p; q >= 0; --q) terms(q);
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s[n].s[0][i] += c[n][0][i];
+            s[n].s[1][i] += c[n][1][i];
+        }
 }
 template <> struct Acc<true> {
     float h0[2][4], h1[2][4], h2[2][4], a[2][4], c[2][4];
@@ -412,7 +425,6 @@ k_mm_stage1(const MmBatch *__restrict__ batches, const int32_t *__restrict__ tds
                     acc[m][0].chunk(xw + (c * MT + m) * TW, f[0]);
                 } else {
                     mm_chunk<1>(acc[m], xw + (c * MT + m) * TW, f);
-                    acc[m][0].drain();
                 }
             }
         }
@@ -436,10 +448,10 @@ k_mm_stage1(const MmBatch *__restrict__ batches, const int32_t *__restrict__ tds
 #pragma unroll
                         for (int j = 0; j < 4; ++j) __stcs(o + (4 * c + j) * MM_PLANE + q * 32, p[j]);
                     } else {
-                        uint32_t p[2];
-                        split_pair(acc[m][0].s[c][2 * q] * (1.f / MM_TOP), acc[m][0].s[c][2 * q + 1] * (1.f / MM_TOP), p);
+                        uint32_t p[3];
+                        split_pair(acc[m][0].s[c][2 * q], acc[m][0].s[c][2 * q + 1], p);
 #pragma unroll
-                        for (int j = 0; j < 2; ++j) __stcs(o + (2 * c + j) * MM_PLANE + q * 32, p[j]);
+                        for (int j = 0; j < 3; ++j) __stcs(o + (3 * c + j) * MM_PLANE + q * 32, p[j]);
                     }
                 }
         }
@@ -543,16 +555,17 @@ constexpr int MM_SMEM = 112 * 1024;               // two CTAs an SM
 
 // Product: one unit (blockIdx.x / groups) for MT x mw tiles of 16 right-hand sides.  The 8
 // warps: 16 outputs each (the fastest index), mw groups of MT right-hand-side tiles, and what
-// is left of them along K; every warp adds its sums into z (vector atomics).
-// `drain`: chunks the tensor core adds up before their sum leaves it.
+// is left of them along K, as far as two stages of their copies fit; every warp adds its sums into
+// z (vector atomics).
 template <int MT>
 __global__ void __launch_bounds__(MMW * 32, 2)
-k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
+k_mm_out(MmOutArgs p, int mw, float2 *__restrict__ z, int64_t pN)
 {
     extern __shared__ __align__(128) unsigned char smo[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const MmUnit U = p.units[blockIdx.x / p.groups];
-    const int nt = (U.mlen + 15) / 16, gw = nt * mw, ks = MMW / gw, kw = w / gw, wi = w - kw * gw;
+    const int nt = (U.mlen + 15) / 16, gw = nt * mw, kw = w / gw, wi = w - kw * gw;
+    const int ks = min(MMW / gw, MM_SMEM / (2 * (2 * nt * MM_TILE + MT * mw * tile_words<false>() * 4)));
     if (kw >= ks) return;
     const int n0 = 16 * (wi % nt), mi = (wi / nt) * MT, mb = (int)(blockIdx.x % p.groups) * mw * MT, m0 = mb + mi;
     const int E = p.eout[U.cl];
@@ -562,7 +575,6 @@ k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
     Pipe<false> P;
     const int region = MM_SMEM / ks / 128 * 128;
     P.init(p, U, smo + kw * region, region, wi * 32 + lane, gw * 32, 2 * nt, MT * mw, mb, kw, ks);
-    int held = 0;
     P.run(p, U.c0 + kw, U.c1, ks, 1 + kw, [&](int st) {
         BFrag<false> f[2];
 #pragma unroll
@@ -573,11 +585,6 @@ k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
             const uint32_t *tile = P.tile(st, mi + m) + t * 8 + g;
             mm_chunk<2>(acc[m], tile, f);
         }
-        if (++held == drain) {
-            held = 0;
-#pragma unroll
-            for (int m = 0; m < MT; ++m) { acc[m][0].drain(); acc[m][1].drain(); }
-        }
     });
 #pragma unroll
     for (int m = 0; m < MT; ++m)
@@ -585,10 +592,9 @@ k_mm_out(MmOutArgs p, int mw, int drain, float2 *__restrict__ z, int64_t pN)
         for (int h = 0; h < 2; ++h) {
             const int r = 16 * (m0 + m) + g + 8 * h;
             if (r >= p.nrhs) continue;
-            const int e = p.ex[r] - E - 30;                // operands are scaled to 2^15
+            const int e = p.ex[r] - E;
 #pragma unroll
             for (int n = 0; n < 2; ++n) {
-                if (h == 0) acc[m][n].drain();
                 const int i = n0 + 8 * n + 2 * t;
                 const float2 a = make_float2(times_pow2(acc[m][n].s[0][2 * h], e), times_pow2(acc[m][n].s[1][2 * h], e));
                 const float2 b = make_float2(times_pow2(acc[m][n].s[0][2 * h + 1], e), times_pow2(acc[m][n].s[1][2 * h + 1], e));
@@ -744,14 +750,14 @@ __global__ void k_mm_eout(int *eout, int n, int set)
 
 // ---- operand streams, once per operator ---------------------------------------------
 
-// the lane's four values times 2^(e + 15)
+// the lane's four values times 2^e
 __device__ __forceinline__ void pack_tile(float4 *dst, const float2 (&v)[4], const int (&e)[4], int lane)
 {
     float f[8];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        f[2 * q] = ldexpf(v[q].x, e[q] + 15);
-        f[2 * q + 1] = ldexpf(v[q].y, e[q] + 15);
+        f[2 * q] = ldexpf(v[q].x, e[q]);
+        f[2 * q + 1] = ldexpf(v[q].y, e[q]);
     }
     dst[lane] = make_float4(f[0], f[1], f[2], f[3]);
     dst[32 + lane] = make_float4(f[4], f[5], f[6], f[7]);
@@ -889,14 +895,6 @@ int launch_mm_product(hm_matrix h, const LevelList &L, const float2 *x, float2 *
 {
     if (L.mm_n_unit == 0 || nrhs <= 0) return 0;
     int n = 0;
-    // Chunks of 16 K the tensor core adds up before the sum is taken out.  It truncates, so a sum
-    // shrinks a little with every product: one chunk, and the product errs by 2.8e-7 (30,720-unknown
-    // sphere; the FP32 kernels 5.0e-7), 32 and it errs by 4.2e-6 and takes 6 % less time.  32 is for
-    // the calls of many right-hand sides that had the tcgen05 product (7.5e-6, sums of 512 K):
-    // above 32 of them, or above 16 on operators large enough.
-    const bool many = (nrhs > 32 && L.mm_n_chunk > 3000) || (nrhs > 16 && L.mm_n_chunk > 60000);
-    const int drain = many ? 32 : 1;
-    const bool coarse = many && nrhs > 32;
     const int pass = mm_pass(L, nrhs, false);
     const size_t tiles_max = (size_t)(pass + 15) / 16;
     uint32_t *xt = (uint32_t *)ws, *tt = xt + tiles_max * tile_words<false>() * L.mm_n_xch;
@@ -907,13 +905,15 @@ int launch_mm_product(hm_matrix h, const LevelList &L, const float2 *x, float2 *
         n += mm_inputs<false>(h, L, xp, nr, xt, tt, ex, s) + 1;
         // tiles of 16 right-hand sides a warp up to 16 of them, 32 above, two such groups a CTA above 32
         const int mw = tiles > 2 ? 2 : 1, mt = tiles > 1 ? 2 : 1, groups = (tiles + mt * mw - 1) / (mt * mw);
+        // the coarse units, with fewer sums to add into z, where they alone are four CTAs an SM
+        const bool coarse = tiles > 2 && (int64_t)groups * L.mm_n_unit2 >= 4ll * h->num_sms;
         MmOutArgs a{coarse ? L.d_mm_unit2 : L.d_mm_unit, L.d_mm_ca, L.d_mm_eout, L.d_mm_os, xt, tt, (int)L.mm_n_xch,
                     tiles, nr, L.mm_n_tch, ex, groups};
         float2 *zp = z + (int64_t)r0 * h->pN;
         const unsigned units = (unsigned)(coarse ? L.mm_n_unit2 : L.mm_n_unit);
         auto go = [&](auto kern) {
             mm_attr((const void *)kern, MM_SMEM);
-            kern<<<units * (unsigned)groups, MMW * 32, MM_SMEM, s>>>(a, mw, drain, zp, h->pN);
+            kern<<<units * (unsigned)groups, MMW * 32, MM_SMEM, s>>>(a, mw, zp, h->pN);
         };
         if (mt == 1) go(k_mm_out<1>);
         else go(k_mm_out<2>);
