@@ -191,7 +191,7 @@ def parse():
     p.add_argument("--pin-product", type=int, default=None,
                    help="pin the many-RHS product kernel (0, 8, 16, 32 = matrix instructions, 1016 = tcgen05) instead of autotuning")
     p.add_argument("--pin-residual", type=int, default=None,
-                   help="pin the many-RHS residual kernel (0, 8, 16, 1017 = owner-computes)")
+                   help="pin the many-RHS residual kernel (0, 8, 16, 1017 = owner-computes, 1018 = the same on the matrix instructions)")
     return p.parse_args()
 
 

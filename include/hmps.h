@@ -438,9 +438,9 @@ hm_status hm_get_info(hm_matrix h, hm_info *info);
  * 1017 (residual only, where every level of the call holds only such blocks) =
  * owner-computes FP64-class products, one CTA per output cluster and group of 16
  * right-hand sides, no partial slots.  A refined solve whose levels hold only such blocks and
- * whose choice is not pinned has a choice of its own: the owner-computes form on the matrix
- * instructions (exact integer digits; errors relative to an output cluster's largest
- * terms; reported as 1017), above 16 right-hand sides always.  res_ms of the owner kernel covers all
+ * whose choice is not pinned has a choice of its own: 1018 = the owner-computes form on the matrix
+ * instructions (exact integer digits), above 16 right-hand sides always; it is reported as res_rb
+ * until an hm_residual or hm_apply has made its own choice.  res_ms of the owner kernel covers all
  * nrhs right-hand sides at once, of the others one chunk of at most 16.
  * prod_ms / res_ms: the measured time of one leaf-level launch of the choice.
  * Any output pointer may be NULL.  HM_ERR_STATE if no call with that nrhs has
@@ -457,8 +457,9 @@ hm_status hm_get_tuning(hm_matrix h, int nrhs, int *prod_rb, int *res_rb, double
  * the first call that runs it allocates its stage-1 workspace: the low-rank
  * intermediates, 8 KB per 8 rank rows of every low-rank block side and per tile,
  * counted in hm_info.device_bytes);
- * res_rb 0, 8, 16 or 1017 (owner-computes; calls whose levels hold larger blocks
- * fall back to the partial-slot kernel of one right-hand side at a time).  Drops captured solve graphs.  HM_ERR_ARG for nrhs < 4 or
+ * res_rb 0, 8, 16, 1017 (owner-computes) or 1018 (the same on the matrix instructions; it packs the
+ * blocks as choice 32 does); calls whose levels hold larger blocks, or clusters that overlap, run the
+ * partial-slot kernels instead of these two.  Drops captured solve graphs.  HM_ERR_ARG for nrhs < 4 or
  * another value.
  */
 hm_status hm_set_tuning(hm_matrix h, int nrhs, int prod_rb, int res_rb);

@@ -1055,8 +1055,15 @@ static hm_status use_tuning(SolveCtx &c, bool residual)
         c.prod_rb = -1;
         st = HM_OK;
     }
-    if (st != HM_OK || !residual || c.res_rb != RB_OWN || !own_applies(c.h, c.m)) return st;
-    return ensure_own(c.h, c.m, false, c.s);
+    if (st != HM_OK || !residual || (c.res_rb != RB_OWN && c.res_rb != RB_MM) || !own_applies(c.h, c.m)) return st;
+    if (c.res_rb == RB_OWN) return ensure_own(c.h, c.m, false, c.s);
+    st = ensure_mm(c.h, c.m, c.nrhs, true, c.s);
+    if (st == HM_OK) st = ensure_own(c.h, c.m, true, c.s);
+    if (st == HM_ERR_OOM) {   // no room for the operand streams: the partial-slot kernels
+        c.res_rb = -1;
+        st = HM_OK;
+    }
+    return st;
 }
 
 // the residual kernel of a refined solve on levels of small blocks that is not pinned: the matrix
@@ -1787,8 +1794,8 @@ hm_status hm_set_tuning(hm_matrix h, int nrhs, int prod_rb, int res_rb)
     if (!h) return fail(HM_ERR_ARG, "null handle");
     if (nrhs < MRHS_MIN_RHS) return fail(HM_ERR_ARG, "kernel choices apply from 4 right-hand sides on");
     const bool pok = prod_rb == 0 || prod_rb == 8 || prod_rb == 16 || prod_rb == 32 || prod_rb == RB_TC;
-    const bool rok = res_rb == 0 || res_rb == 8 || res_rb == 16 || res_rb == RB_OWN;
-    if (!pok || !rok) return fail(HM_ERR_ARG, "prod_rb must be 0, 8, 16, 32 or 1016 and res_rb 0, 8, 16 or 1017");
+    const bool rok = res_rb == 0 || res_rb == 8 || res_rb == 16 || res_rb == RB_OWN || res_rb == RB_MM;
+    if (!pok || !rok) return fail(HM_ERR_ARG, "prod_rb must be 0, 8, 16, 32 or 1016 and res_rb 0, 8, 16, 1017 or 1018");
     hm_matrix_s::Tune t;
     t.prod_rb = prod_rb;
     t.res_rb = res_rb;
@@ -1813,9 +1820,8 @@ hm_status hm_get_tuning(hm_matrix h, int nrhs, int *prod_rb, int *res_rb, double
     auto it = nrhs < MRHS_MIN_RHS ? h->tune.end() : h->tune.find(tune_bucket(nrhs));
     if (it == h->tune.end()) return fail(HM_ERR_STATE, "no tuned kernel choice for this right-hand-side count");
     if (prod_rb) *prod_rb = it->second.prod_rb;
-    // a choice made for refined solves alone: the matrix-instruction form is the owner-computes one
-    const int solve_rb = it->second.solve_rb == RB_MM ? RB_OWN : it->second.solve_rb;
-    if (res_rb) *res_rb = it->second.res_rb < 0 ? solve_rb : it->second.res_rb;
+    // the choice of hm_residual and hm_apply, or, where only refined solves have run, theirs
+    if (res_rb) *res_rb = it->second.res_rb < 0 ? it->second.solve_rb : it->second.res_rb;
     if (prod_ms) *prod_ms = it->second.prod_ms;
     if (res_ms) *res_ms = it->second.res_ms;
     return HM_OK;

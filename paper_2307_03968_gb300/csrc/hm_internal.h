@@ -32,7 +32,7 @@ constexpr int RESID_CHUNK = 16;     // right-hand sides per chunk of the FP64-cl
 constexpr int RB_TC = 1016;         // product choice: tensor-core products of the small items, RHS tiles of 128
 constexpr int TC_MIN_RHS = 32;      // the autotuner times the tensor-core product from this many RHS on
 constexpr int RB_OWN = 1017;        // residual choice: owner-computes FP64-class products (levels of small items)
-constexpr int RB_MM = 1018;         // the same on the matrix instructions (refined solves; not a choice of hm_set_tuning)
+constexpr int RB_MM = 1018;         // residual choice: the same on the matrix instructions (timed for refined solves only)
 
 // Double-float numbers of the FP64-class residual (hi + lo, |lo| a few ulps of hi at
 // most): a real one, and a complex one of 16 bytes, which is also the element of

@@ -358,7 +358,7 @@ class HMatrix:
     def set_tuning(self, nrhs, prod_rb, res_rb):
         """hm_set_tuning: pin the kernel choice for nrhs's bucket (product 32 = matrix
         instructions, 1016 = tcgen05 tensor-core products; residual 1017 = owner-computes
-        FP64-class residual)."""
+        FP64-class residual, 1018 = the same on the matrix instructions)."""
         _check(load().hm_set_tuning(self._h, nrhs, prod_rb, res_rb))
 
     def set_wait_limit(self, polls):
