@@ -208,7 +208,8 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
                 if (L.mm_built) return;
                 void **p[] = {(void **)&L.d_mm_unit, (void **)&L.d_mm_unit2, (void **)&L.d_mm_runit, (void **)&L.d_mm_batch,
                               (void **)&L.d_mm_xch, (void **)&L.d_mm_ca, (void **)&L.d_mm_tdst, (void **)&L.d_mm_eout,
-                              (void **)&L.d_mm_os, (void **)&L.d_mm_ws};
+                              (void **)&L.d_mm_os, (void **)&L.d_mm_ws, (void **)&L.d_mm_orow, (void **)&L.d_mm_wrow,
+                              (void **)&L.d_mm_tin};
                 for (void **q : p) {
                     if (*q) cudaFree(*q);
                     *q = nullptr;
@@ -224,6 +225,9 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
             (st = dev_alloc(h, (void **)&L.d_mm_eout, sizeof(int) * (size_t)mm.n_cl)) != HM_OK ||
             (st = dev_alloc(h, (void **)&L.d_mm_os, mm_stream_bytes(mm.n_out))) != HM_OK ||
             (st = dev_alloc(h, (void **)&L.d_mm_ws, mm_stream_bytes(mm.n_w))) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_orow, sizeof(int) * 8 * (size_t)mm.n_out)) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_wrow, sizeof(int) * 8 * (size_t)mm.n_w)) != HM_OK ||
+            (st = dev_alloc(h, (void **)&L.d_mm_tin, sizeof(int32_t) * (MM_K / 2) * (size_t)mm.n_tch)) != HM_OK ||
             (st = sets.make(mm.sets.data(), mm.sets.size() * sizeof(MmSet), s)) != HM_OK ||
             (st = chunks.make(mm.chunks.data(), mm.chunks.size() * sizeof(MmChunk), s)) != HM_OK ||
             (st = rows.make(mm.rows.data(), mm.rows.size() * sizeof(int64_t), s)) != HM_OK ||
@@ -293,7 +297,7 @@ static void free_handle(hm_matrix h)
         if (kv.second.d_xch) cudaFree(kv.second.d_xch);
         const LevelList &L = kv.second;
         void *mm[] = {L.d_rcu, L.d_rcp, L.d_rcb, L.d_mm_unit, L.d_mm_unit2, L.d_mm_runit, L.d_mm_batch, L.d_mm_xch, L.d_mm_ca, L.d_mm_tdst,
-                      L.d_mm_eout, L.d_mm_os, L.d_mm_ws};
+                      L.d_mm_eout, L.d_mm_os, L.d_mm_ws, L.d_mm_orow, L.d_mm_wrow, L.d_mm_tin};
         for (void *p : mm)
             if (p) cudaFree(p);
     }
@@ -944,9 +948,9 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
 // owner-computes), and keep the fastest of each.  The candidates compute the same
 // sums up to FP32 rounding, so the choice changes speed only.  It runs before any graph
 // capture, so captured solves replay the chosen kernels.  A refined solve's residual on levels
-// of small blocks is on the matrix instructions above 16 right-hand sides (faster at every
-// size measured, 300 to 30,720 unknowns: 76 against 83 us the solve to 8.8 against 16.6 ms at
-// 32) and up to 16 timed against the partial-slot kernels (use_solve_residual).
+// of small blocks is on the matrix instructions above 16 right-hand sides (the fastest, or within 4 %
+// of it, at every size measured: 300 unknowns and 32 right-hand sides 74 against 84 us the solve,
+// 7,500 727 against 886, and with 17 119 against 116 at 700) and up to 16 timed against the partial-slot kernels (use_solve_residual).
 // right-hand-side counts share a kernel choice per power-of-two bucket
 static int tune_bucket(int nrhs)
 {

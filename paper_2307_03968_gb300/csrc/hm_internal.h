@@ -90,6 +90,8 @@ struct LevelList {
     XChunk *d_mm_xch = nullptr;
     int32_t *d_mm_ca = nullptr, *d_mm_tdst = nullptr;   // per chunk its operand tile, per stage-1 pair its T pair
     unsigned char *d_mm_os = nullptr, *d_mm_ws = nullptr;   // output and stage-1 streams
+    int *d_mm_orow = nullptr, *d_mm_wrow = nullptr;         // per tile of them its 8 rows' exponents
+    int32_t *d_mm_tin = nullptr;                            // per T pair its input cluster's x chunks (k_mm_tscale)
     int *d_mm_eout = nullptr;
     int64_t mm_n_unit = 0, mm_n_unit2 = 0, mm_n_runit = 0, mm_n_chunk = 0, mm_n_batch = 0, mm_n_xch = 0, mm_n_tch = 0;
     int mm_parts = 0;
