@@ -565,9 +565,10 @@ static hm_status ensure_tct(hm_matrix h, cudaStream_t s)
     return HM_OK;
 }
 
-// operand tiles of the matrix-instruction products for nrhs right-hand sides (a pass of them),
-// levels 1..m; allocated only by the calls that run them, before any capture
-static hm_status ensure_mm(hm_matrix h, int m, int nrhs, bool res, cudaStream_t s)
+// operand tiles of the matrix-instruction products for the workspace's right-hand sides (a pass of
+// them; not the call's, so that a later call of the same bucket of sizes allocates nothing and can be
+// captured), levels 1..m; allocated only by the calls that run them, before any capture
+static hm_status ensure_mm(hm_matrix h, int m, bool res, cudaStream_t s)
 {
     hm::Workspace &ws = h->ws;
     const hm_status st = ensure_mm_lists(h, m, s);
@@ -575,7 +576,7 @@ static hm_status ensure_mm(hm_matrix h, int m, int nrhs, bool res, cudaStream_t 
     size_t bytes = 0;
     for (int lev = 1; lev <= m; ++lev) {
         auto it = h->levels.find(lev);
-        if (it != h->levels.end() && it->second.n_small > 0) bytes = std::max(bytes, mm_ws_bytes(it->second, nrhs, res));
+        if (it != h->levels.end() && it->second.n_small > 0) bytes = std::max(bytes, mm_ws_bytes(it->second, ws.nrhs, res));
     }
     if (bytes == 0 || (ws.d_mm && ws.mm_bytes >= bytes)) return HM_OK;
     clear_graphs(h);   // graphs hold the old pointer
@@ -1006,7 +1007,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
         if (rb < 16 ? nrhs > 8 : rb == 16 && (nrhs <= 8 || (nrhs > 16 && L.elems > 4000000))) continue;
         double ms = 0;
         if (rb == 32) {
-            st = ensure_mm(h, m, nrhs, false, s);
+            st = ensure_mm(h, m, false, s);
             if (st == HM_ERR_OOM) { st = HM_OK; continue; }   // no room for the operand streams: the other kernels
             if (st != HM_OK) break;
         }
@@ -1054,14 +1055,14 @@ static hm_status use_tuning(SolveCtx &c, bool residual)
     }
     hm_status st = HM_OK;
     if (c.prod_rb == RB_TC) st = ensure_tct(c.h, c.s);
-    else if (c.prod_rb == 32) st = ensure_mm(c.h, c.m, c.nrhs, false, c.s);
+    else if (c.prod_rb == 32) st = ensure_mm(c.h, c.m, false, c.s);
     if (st == HM_ERR_OOM && c.prod_rb == 32) {   // no room for the operand streams: chunks in shared memory
         c.prod_rb = -1;
         st = HM_OK;
     }
     if (st != HM_OK || !residual || (c.res_rb != RB_OWN && c.res_rb != RB_MM) || !own_applies(c.h, c.m)) return st;
     if (c.res_rb == RB_OWN) return ensure_own(c.h, c.m, false, c.s);
-    st = ensure_mm(c.h, c.m, c.nrhs, true, c.s);
+    st = ensure_mm(c.h, c.m, true, c.s);
     if (st == HM_OK) st = ensure_own(c.h, c.m, true, c.s);
     if (st == HM_ERR_OOM) {   // no room for the operand streams: the partial-slot kernels
         c.res_rb = -1;
@@ -1078,7 +1079,7 @@ static hm_status use_solve_residual(SolveCtx &c)
     hm_matrix h = c.h;
     hm_matrix_s::Tune &t = h->tune[tune_bucket(c.nrhs)];
     c.res_rb = t.solve_rb;
-    hm_status st = c.res_rb < 0 || c.res_rb == RB_MM ? ensure_mm(h, c.m, c.nrhs, true, c.s) : HM_OK;
+    hm_status st = c.res_rb < 0 || c.res_rb == RB_MM ? ensure_mm(h, c.m, true, c.s) : HM_OK;
     if (st == HM_OK && (c.res_rb < 0 || c.res_rb == RB_MM)) st = ensure_own(h, c.m, true, c.s);
     const bool room = st != HM_ERR_OOM;
     if (st == HM_ERR_OOM) st = HM_OK;
