@@ -428,8 +428,8 @@ hm_status hm_get_info(hm_matrix h, hm_info *info);
  * counterpart in the paper: it concerns how this GPU implementation batches the
  * block products of eqs. 6 and 8).  Right-hand-side counts share a choice per
  * bucket (the next power of two >= nrhs, at least 4).  The first complex64
- * solve, product or residual in a bucket on an operator times the candidate
- * kernels on that operator at the bucket's size (with CUDA events on the
+ * solve, product or residual in a bucket on an operator times the candidates of the kernels
+ * it runs on that operator at the bucket's size (with CUDA events on the
  * caller's stream, which it synchronises once) and keeps the fastest: 0 = one right-hand side at
  * a time, 8 / 16 = blocks staged once in shared memory per chunk of that many right-hand sides,
  * 32 (product only) = the blocks of at most 64 x 64 (rank <= 32) on the matrix instructions, in
@@ -442,7 +442,8 @@ hm_status hm_get_info(hm_matrix h, hm_info *info);
  * instructions (exact integer digits), above 16 right-hand sides always; it is reported as res_rb
  * until an hm_residual or hm_apply has made its own choice.  res_ms of the owner kernel covers all
  * nrhs right-hand sides at once, of the others one chunk of at most 16.
- * prod_ms / res_ms: the measured time of one leaf-level launch of the choice.
+ * prod_ms / res_ms: the measured time of one leaf-level launch of the choice (0: not timed, as
+ * prod_ms while only residuals have been formed; prod_rb is then the default chunk).
  * Any output pointer may be NULL.  HM_ERR_STATE if no call with that nrhs has
  * been made yet (or nrhs < 4, which needs no choice).
  */

@@ -960,26 +960,31 @@ static int tune_bucket(int nrhs)
     return b;
 }
 
-static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool residual)
+// product, residual: whether the call runs FP32 products, and a residual of hm_residual's kind; a call
+// that runs no products times none, and packs no operand streams for them
+static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool product, bool residual)
 {
     if (nrhs_req < MRHS_MIN_RHS) return HM_OK;
     const int nrhs = tune_bucket(nrhs_req);              // timed at the bucket's size
     auto have = h->tune.find(nrhs);
-    if (have != h->tune.end() && (!residual || have->second.res_rb >= 0)) return HM_OK;
+    if (have != h->tune.end() && (!product || have->second.prod_timed) && (!residual || have->second.res_rb >= 0))
+        return HM_OK;
     auto it1 = h->levels.find(1);
     hm_matrix_s::Tune t;
     if (it1 == h->levels.end() || it1->second.items.empty() || it1->second.n_small == 0) {
         t.prod_rb = 0;
         t.res_rb = 0;
+        t.prod_timed = true;
         h->tune[nrhs] = t;
         return HM_OK;
     }
-    const bool do_prod = have == h->tune.end();
-    if (!do_prod) t = have->second;
+    if (have != h->tune.end()) t = have->second;
+    else t.prod_rb = nrhs <= 8 ? 8 : 16;
+    const bool do_prod = product && !t.prod_timed, do_res = residual && t.res_rb < 0;
     const LevelList &L = it1->second, *Lp = &L;
     hm_status st = ensure_workspace(h, nrhs, m);
     if (st != HM_OK) return st;
-    if (residual && (st = ensure_partials(h)) != HM_OK) return st;
+    if (do_res && (st = ensure_partials(h)) != HM_OK) return st;
     float2 *x = (float2 *)h->ws.vec32[0], *z = (float2 *)h->ws.vec32[1];
     HM_CUDA(cudaMemsetAsync(x, 0, sizeof(float2) * h->pN * nrhs, s));
     cudaEvent_t e0, e1;
@@ -1020,7 +1025,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     best = 1e30;
     const int res_c[] = {0, 8, 16, RB_OWN};
     for (int rb : res_c) {
-        if (st != HM_OK || !residual) break;
+        if (st != HM_OK || !do_res) break;
         if (rb == RB_OWN) {
             if (!own_applies(h, m)) continue;
             if ((st = ensure_own(h, m, false, s)) != HM_OK) break;
@@ -1039,13 +1044,14 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != HM_OK) return st;
+    t.prod_timed |= do_prod;
     h->tune[nrhs] = t;
     return HM_OK;
 }
 
 // the autotuner's (or hm_set_tuning's) kernel choices for the call, with the
-// workspace the chosen product needs
-static hm_status use_tuning(SolveCtx &c, bool residual)
+// workspace the chosen kernels need where the call runs them
+static hm_status use_tuning(SolveCtx &c, bool product, bool residual)
 {
     if (c.nrhs < MRHS_MIN_RHS) return HM_OK;
     auto tn = c.h->tune.find(tune_bucket(c.nrhs));
@@ -1054,8 +1060,8 @@ static hm_status use_tuning(SolveCtx &c, bool residual)
         c.res_rb = tn->second.res_rb;
     }
     hm_status st = HM_OK;
-    if (c.prod_rb == RB_TC) st = ensure_tct(c.h, c.s);
-    else if (c.prod_rb == 32) st = ensure_mm(c.h, c.m, false, c.s);
+    if (product && c.prod_rb == RB_TC) st = ensure_tct(c.h, c.s);
+    else if (product && c.prod_rb == 32) st = ensure_mm(c.h, c.m, false, c.s);
     if (st == HM_ERR_OOM && c.prod_rb == 32) {   // no room for the operand streams: chunks in shared memory
         c.prod_rb = -1;
         st = HM_OK;
@@ -1203,8 +1209,8 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     const bool persist = (o->persistent || rec_out) && !c.fp64 && persist_supported(h);
     if (rec_out && !persist) return fail(HM_ERR_ARG, "the operator does not fit the one-launch solve");
     if (!c.fp64 && !persist) {
-        if ((st = autotune(h, nrhs, c.m, s, resid && !own_applies(h, c.m))) != HM_OK) return st;
-        if ((st = use_tuning(c, resid)) != HM_OK) return st;
+        if ((st = autotune(h, nrhs, c.m, s, true, resid && !own_applies(h, c.m))) != HM_OK) return st;
+        if ((st = use_tuning(c, true, resid)) != HM_OK) return st;
         if (resid && (st = ensure_partials(h)) != HM_OK) return st;   // the tuning may have grown the workspace
         if (resid && nrhs >= MRHS_MIN_RHS && own_applies(h, c.m)) {
             auto tn = h->tune.find(tune_bucket(nrhs));
@@ -1693,8 +1699,9 @@ hm_status hm_apply(hm_matrix h, const void *x, int64_t ldx, void *y, int64_t ldy
     hm_status st = ensure_workspace(h, nrhs, c.m);
     if (st != HM_OK) return st;
     if (fp64_accumulate && (st = ensure_partials(h)) != HM_OK) return st;
-    if ((st = autotune(h, nrhs, c.m, s, fp64_accumulate != 0)) != HM_OK) return st;
-    if ((st = use_tuning(c, fp64_accumulate != 0)) != HM_OK) return st;
+    const bool res = fp64_accumulate != 0;
+    if ((st = autotune(h, nrhs, c.m, s, !res, res)) != HM_OK) return st;
+    if ((st = use_tuning(c, !res, res)) != HM_OK) return st;
     void *xt = h->ws.vec32[0], *yt = h->ws.vec32[1];
     launch_permute_in(x, ldx, xt, h->pN, h->d_pperm, nrhs, false, s);
     if (fp64_accumulate) {
@@ -1725,8 +1732,8 @@ hm_status hm_residual(hm_matrix h, const void *b, int64_t ldb, const void *x, in
     hm_status st = ensure_workspace(h, nrhs, c.m);
     if (st != HM_OK) return st;
     if ((st = ensure_partials(h)) != HM_OK) return st;
-    if ((st = autotune(h, nrhs, c.m, s, true)) != HM_OK) return st;
-    if ((st = use_tuning(c, true)) != HM_OK) return st;
+    if ((st = autotune(h, nrhs, c.m, s, false, true)) != HM_OK) return st;
+    if ((st = use_tuning(c, false, true)) != HM_OK) return st;
     void *bt = h->ws.vec32[0], *xt = h->ws.vec32[1], *rt = h->ws.vec32[3];
     launch_permute_in(b, ldb, bt, h->pN, h->d_pperm, nrhs, false, s);
     launch_permute_in(x, ldx, xt, h->pN, h->d_pperm, nrhs, false, s);
@@ -1804,7 +1811,7 @@ hm_status hm_set_tuning(hm_matrix h, int nrhs, int prod_rb, int res_rb)
     hm_matrix_s::Tune t;
     t.prod_rb = prod_rb;
     t.res_rb = res_rb;
-    t.pinned = true;
+    t.pinned = t.prod_timed = true;
     h->tune[tune_bucket(nrhs)] = t;
     clear_graphs(h);   // captured solves hold the previous choice
     return HM_OK;

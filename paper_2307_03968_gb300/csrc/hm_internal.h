@@ -287,7 +287,12 @@ struct hm_matrix_s {
     unsigned *d_bar = nullptr;
 
     // kernel choices measured on this operator per right-hand-side count (hm_api.cu autotune)
-    struct Tune { int prod_rb = -1, res_rb = -1; double prod_ms = 0.0, res_ms = 0.0; bool pinned = false; int solve_rb = -1; };   // res_rb < 0: not tuned; solve_rb: a refined solve's residual
+    struct Tune {
+        int prod_rb = -1, res_rb = -1;          // res_rb < 0: not tuned
+        double prod_ms = 0.0, res_ms = 0.0;
+        bool pinned = false, prod_timed = false;
+        int solve_rb = -1;                      // a refined solve's residual
+    };
     std::map<int, Tune> tune;
 
     // estimates of the level operators U_l = D^{-1} M_l (index l - 1), made by hm_factor_leaf /
