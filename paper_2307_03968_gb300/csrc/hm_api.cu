@@ -1005,11 +1005,11 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     };
     double best = 1e30;
     // candidates: up to 8 right-hand sides one at a time, chunks of 8 and the matrix instructions;
-    // above, those and (up to 16, or on small operators, where launches count) chunks of 16
+    // above, those and chunks of 16
     const int prod_c[] = {0, 8, 16, 32};
     for (int rb : prod_c) {
         if (!do_prod) break;
-        if (rb < 16 ? nrhs > 8 : rb == 16 && (nrhs <= 8 || (nrhs > 16 && L.elems > 4000000))) continue;
+        if (rb < 16 ? nrhs > 8 : rb == 16 && nrhs <= 8) continue;
         double ms = 0;
         if (rb == 32) {
             st = ensure_mm(h, m, false, s);
