@@ -186,10 +186,47 @@ struct TmpArray {
     }
 };
 
+static void free_mm(LevelList &L)
+{
+    void **p[] = {(void **)&L.d_mm_unit, (void **)&L.d_mm_unit2, (void **)&L.d_mm_runit, (void **)&L.d_mm_batch,
+                  (void **)&L.d_mm_xch,  (void **)&L.d_mm_ca,    (void **)&L.d_mm_tdst,  (void **)&L.d_mm_eout,
+                  (void **)&L.d_mm_os,   (void **)&L.d_mm_ws,    (void **)&L.d_mm_orow,  (void **)&L.d_mm_wrow,
+                  (void **)&L.d_mm_tin};
+    for (void **q : p) {
+        if (*q) cudaFree(*q);
+        *q = nullptr;
+    }
+    L.mm_built = false;
+}
+
+// Whether the matrix-instruction kernels may take `bytes` more of the device.  They are an
+// addition to an operator that is held anyway, so they leave half of what is free to others
+// (another operator, a framework on the same GPU).  A refusal is kept until the next bucket of
+// right-hand sides is tuned or a choice is pinned: asking again costs a call to the driver.
+static hm_status mm_room(hm_matrix h, size_t bytes)
+{
+    size_t free = 0, total = 0;
+    if (!h->mm_refused) {
+        HM_CUDA(cudaMemGetInfo(&free, &total));
+        h->mm_refused = bytes > free / 2;
+    }
+    return h->mm_refused ? fail(HM_ERR_OOM, "no room for the operand streams of the matrix-instruction kernels") : HM_OK;
+}
+
 // the matrix-instruction products' lists and operand streams, made by the first call that runs them
 static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
 {
     hm_status st;
+    size_t need = 0;   // of the levels to come, at least: both directions of their small blocks in FP32
+    for (int lev = 1; lev <= m; ++lev) {
+        auto it = h->levels.find(lev);
+        if (it == h->levels.end() || it->second.mm_built || it->second.n_small == 0) continue;
+        LevelList &L = it->second;
+        if (L.mm_need == 0)
+            for (const Item &q : small_items(L)) L.mm_need += 2 * sizeof(float2) * (size_t)item_elems(q);
+        need += L.mm_need;
+    }
+    if (need > 0 && (st = mm_room(h, need)) != HM_OK) return st;
     for (int lev = 1; lev <= m; ++lev) {
         auto it = h->levels.find(lev);
         if (it == h->levels.end() || it->second.mm_built || it->second.n_small == 0) continue;
@@ -198,6 +235,9 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
         // about four CTAs an SM for one tile of right-hand sides
         if (!build_mm_lists(directed_products(small_items(L)), 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), mm))
             return fail(HM_ERR_STATE, "matrix-product work lists out of their index bounds");
+        // what the level takes, exactly (its lists beside the streams are a few per cent of it)
+        L.mm_need = (mm_stream_bytes(1) + 8 * sizeof(int)) * (size_t)(mm.n_out + mm.n_w);
+        if ((st = mm_room(h, L.mm_need)) != HM_OK) return st;
         TmpArray sets, chunks, rows, pairs, wexp, rexp;
         struct Undo {   // a level's arrays go again if the last of them cannot be had
             hm_matrix h;
@@ -206,15 +246,9 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
             ~Undo()
             {
                 if (L.mm_built) return;
-                void **p[] = {(void **)&L.d_mm_unit, (void **)&L.d_mm_unit2, (void **)&L.d_mm_runit, (void **)&L.d_mm_batch,
-                              (void **)&L.d_mm_xch, (void **)&L.d_mm_ca, (void **)&L.d_mm_tdst, (void **)&L.d_mm_eout,
-                              (void **)&L.d_mm_os, (void **)&L.d_mm_ws, (void **)&L.d_mm_orow, (void **)&L.d_mm_wrow,
-                              (void **)&L.d_mm_tin};
-                for (void **q : p) {
-                    if (*q) cudaFree(*q);
-                    *q = nullptr;
-                }
+                free_mm(L);
                 h->device_bytes = bytes;
+                h->mm_refused = true;
             }
         } undo{h, L, h->device_bytes};
         if ((st = upload(h, &L.d_mm_unit, mm.units, s)) != HM_OK || (st = upload(h, &L.d_mm_unit2, mm.units2, s)) != HM_OK ||
@@ -295,11 +329,10 @@ static void free_handle(hm_matrix h)
         if (kv.second.d_tcr) cudaFree(kv.second.d_tcr);
         if (kv.second.d_tcc) cudaFree(kv.second.d_tcc);
         if (kv.second.d_xch) cudaFree(kv.second.d_xch);
-        const LevelList &L = kv.second;
-        void *mm[] = {L.d_rcu, L.d_rcp, L.d_rcb, L.d_mm_unit, L.d_mm_unit2, L.d_mm_runit, L.d_mm_batch, L.d_mm_xch, L.d_mm_ca, L.d_mm_tdst,
-                      L.d_mm_eout, L.d_mm_os, L.d_mm_ws, L.d_mm_orow, L.d_mm_wrow, L.d_mm_tin};
-        for (void *p : mm)
+        LevelList &L = kv.second;
+        for (void *p : {(void *)L.d_rcu, (void *)L.d_rcp, (void *)L.d_rcb})
             if (p) cudaFree(p);
+        free_mm(L);
     }
     for (void *p : h->ws.vec32) if (p) cudaFree(p);
     for (void *p : h->ws.vec64) if (p) cudaFree(p);
@@ -571,7 +604,7 @@ static hm_status ensure_tct(hm_matrix h, cudaStream_t s)
 static hm_status ensure_mm(hm_matrix h, int m, bool res, cudaStream_t s)
 {
     hm::Workspace &ws = h->ws;
-    const hm_status st = ensure_mm_lists(h, m, s);
+    hm_status st = ensure_mm_lists(h, m, s);
     if (st != HM_OK) return st;
     size_t bytes = 0;
     for (int lev = 1; lev <= m; ++lev) {
@@ -579,6 +612,7 @@ static hm_status ensure_mm(hm_matrix h, int m, bool res, cudaStream_t s)
         if (it != h->levels.end() && it->second.n_small > 0) bytes = std::max(bytes, mm_ws_bytes(it->second, ws.nrhs, res));
     }
     if (bytes == 0 || (ws.d_mm && ws.mm_bytes >= bytes)) return HM_OK;
+    if ((st = mm_room(h, bytes - (ws.d_mm ? ws.mm_bytes : 0))) != HM_OK) return st;
     clear_graphs(h);   // graphs hold the old pointer
     if (ws.d_mm) {
         cudaFree(ws.d_mm);
@@ -586,7 +620,9 @@ static hm_status ensure_mm(hm_matrix h, int m, bool res, cudaStream_t s)
     }
     ws.d_mm = nullptr;
     ws.mm_bytes = 0;
+    h->mm_refused = true;                       // unless the allocation succeeds
     HM_CUDA(cudaMalloc(&ws.d_mm, bytes));
+    h->mm_refused = false;
     ws.mm_bytes = bytes;
     ws.dev_bytes += (int64_t)bytes;
     return HM_OK;
@@ -981,6 +1017,7 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
     if (have != h->tune.end()) t = have->second;
     else t.prod_rb = nrhs <= 8 ? 8 : 16;
     const bool do_prod = product && !t.prod_timed, do_res = residual && t.res_rb < 0;
+    h->mm_refused = false;                               // a new choice: ask for room again
     const LevelList &L = it1->second, *Lp = &L;
     hm_status st = ensure_workspace(h, nrhs, m);
     if (st != HM_OK) return st;
@@ -1079,21 +1116,28 @@ static hm_status use_tuning(SolveCtx &c, bool product, bool residual)
 
 // the residual kernel of a refined solve on levels of small blocks that is not pinned: the matrix
 // instructions, up to 16 right-hand sides if faster than the partial-slot kernels (one right-hand
-// side at a time, chunks of 8 or 16), timed with the gather; without room for them, those
+// side at a time, chunks of 8 or 16), timed with the gather; without room for them, above 16 the
+// owner-computes kernel on the FP32 pipes, up to 16 those
 static hm_status use_solve_residual(SolveCtx &c)
 {
     hm_matrix h = c.h;
     hm_matrix_s::Tune &t = h->tune[tune_bucket(c.nrhs)];
     c.res_rb = t.solve_rb;
-    hm_status st = c.res_rb < 0 || c.res_rb == RB_MM ? ensure_mm(h, c.m, true, c.s) : HM_OK;
-    if (st == HM_OK && (c.res_rb < 0 || c.res_rb == RB_MM)) st = ensure_own(h, c.m, true, c.s);
-    const bool room = st != HM_ERR_OOM;
-    if (st == HM_ERR_OOM) st = HM_OK;
-    if (st != HM_OK) return st;
-    if (c.res_rb == RB_MM && !room) c.res_rb = -1;
-    if (t.solve_rb >= 0) return HM_OK;
+    bool room = true;
+    if (c.res_rb < 0 || c.res_rb == RB_MM || c.nrhs > 16) {
+        hm_status st = ensure_mm(h, c.m, true, c.s);
+        if (st == HM_OK) st = ensure_own(h, c.m, true, c.s);
+        if (st != HM_OK && st != HM_ERR_OOM) return st;
+        room = st == HM_OK;
+    }
     if (c.nrhs > 16) {
-        c.res_rb = t.solve_rb = room ? RB_MM : -1;
+        c.res_rb = t.solve_rb = room ? RB_MM : RB_OWN;
+        const hm_status st = room ? HM_OK : ensure_own(h, c.m, false, c.s);
+        if (st == HM_ERR_OOM) c.res_rb = -1;             // the partial-slot kernels
+        return st == HM_ERR_OOM ? HM_OK : st;
+    }
+    if (t.solve_rb >= 0) {
+        if (!room) c.res_rb = -1;
         return HM_OK;
     }
     float2 *x = (float2 *)h->ws.vec32[0], *r = (float2 *)h->ws.vec32[1];
@@ -1812,6 +1856,7 @@ hm_status hm_set_tuning(hm_matrix h, int nrhs, int prod_rb, int res_rb)
     t.prod_rb = prod_rb;
     t.res_rb = res_rb;
     t.pinned = t.prod_timed = true;
+    h->mm_refused = false;
     h->tune[tune_bucket(nrhs)] = t;
     clear_graphs(h);   // captured solves hold the previous choice
     return HM_OK;

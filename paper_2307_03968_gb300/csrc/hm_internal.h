@@ -85,6 +85,7 @@ struct LevelList {
     // hm_lists.h build_mm_lists): product units, residual units (mm_parts a cluster at most), scales
     // and operand streams, made by the first call that runs them
     bool mm_built = false;
+    size_t mm_need = 0;           // device bytes the streams take (a lower bound before the lists are made)
     MmUnit *d_mm_unit = nullptr, *d_mm_unit2 = nullptr, *d_mm_runit = nullptr;
     MmBatch *d_mm_batch = nullptr;
     XChunk *d_mm_xch = nullptr;
@@ -251,6 +252,7 @@ struct hm_matrix_s {
     int *h_status = nullptr;          // pinned mirror
     hm::Workspace ws;
     int64_t device_bytes = 0;
+    bool mm_refused = false;          // the matrix-instruction kernels' streams found no room (hm_api.cu mm_room)
     int num_sms = 0;
     int64_t tc_max_xch = 0;           // largest split-x chunk count over the levels
     int64_t tc_max_tchunk = 0;        // largest T chunk count over the levels
