@@ -186,6 +186,8 @@ struct TmpArray {
     }
 };
 
+static void clear_graphs(hm_matrix h);
+
 static void free_mm(LevelList &L)
 {
     void **p[] = {(void **)&L.d_mm_unit, (void **)&L.d_mm_unit2, (void **)&L.d_mm_runit, (void **)&L.d_mm_batch,
@@ -199,18 +201,49 @@ static void free_mm(LevelList &L)
     L.mm_built = false;
 }
 
+static int64_t held_bytes(hm_matrix h) { return h->device_bytes + h->ws.dev_bytes + (int64_t)h->ws.d_io_bytes; }
+
+// device bytes of the matrix-instruction kernels' streams, lists and operand tiles
+int64_t mm_held(hm_matrix h)
+{
+    int64_t b = h->ws.d_mm ? (int64_t)h->ws.mm_bytes : 0;
+    for (const auto &kv : h->levels)
+        if (kv.second.mm_built) b += kv.second.mm_bytes;
+    return b;
+}
+
+// gives them back (no call of the handle in flight)
+void release_mm(hm_matrix h)
+{
+    if (mm_held(h) == 0) return;
+    clear_graphs(h);   // graphs hold the old pointers
+    for (auto &kv : h->levels)
+        if (kv.second.mm_built) {
+            free_mm(kv.second);
+            h->device_bytes -= kv.second.mm_bytes;
+        }
+    if (h->ws.d_mm) {
+        cudaFree(h->ws.d_mm);
+        h->ws.dev_bytes -= (int64_t)h->ws.mm_bytes;
+    }
+    h->ws.d_mm = nullptr;
+    h->ws.mm_bytes = 0;
+}
+
 // Whether the matrix-instruction kernels may take `bytes` more of the device.  They are an
-// addition to an operator that is held anyway, so they leave half of what is free to others
-// (another operator, a framework on the same GPU).  A refusal is kept until the next bucket of
-// right-hand sides is tuned or a choice is pinned: asking again costs a call to the driver.
+// addition to an operator that is held anyway, so they keep the handle below its limit (a server's
+// budget) and leave half of what is free to others (another operator, a framework on the same
+// GPU).  The second refusal is kept until the next bucket of right-hand sides is tuned or a choice
+// is pinned: asking again costs a call to the driver.
 static hm_status mm_room(hm_matrix h, size_t bytes)
 {
     size_t free = 0, total = 0;
-    if (!h->mm_refused) {
+    const bool over = h->byte_limit >= 0 && held_bytes(h) + (int64_t)bytes > h->byte_limit;
+    if (!over && !h->mm_refused) {
         HM_CUDA(cudaMemGetInfo(&free, &total));
         h->mm_refused = bytes > free / 2;
     }
-    return h->mm_refused ? fail(HM_ERR_OOM, "no room for the operand streams of the matrix-instruction kernels") : HM_OK;
+    return over || h->mm_refused ? fail(HM_ERR_OOM, "no room for the operand streams of the matrix-instruction kernels") : HM_OK;
 }
 
 // the matrix-instruction products' lists and operand streams, made by the first call that runs them
@@ -283,6 +316,7 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
                        h->d_pool32, s);
         HM_CUDA(cudaGetLastError());
         HM_CUDA(cudaStreamSynchronize(s));        // the lists end here
+        L.mm_bytes = h->device_bytes - undo.bytes;
         L.mm_built = true;
     }
     return HM_OK;
@@ -1246,7 +1280,10 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     c.h = h; c.nrhs = nrhs; c.K = o->n_terms; c.fp64 = o->fp64 != 0; c.s = s;
     c.m = clamp_levels(h, o->n_levels);
     c.vbytes = es * h->pN * nrhs;
-    hm_status st = ensure_workspace(h, nrhs, c.m);
+    // at the size of the bucket where the autotuner is going to run, so that what the solve needs is
+    // there (and counted) before anything optional is
+    const bool tunes = !o->fp64 && nrhs >= MRHS_MIN_RHS && !h->tune.count(tune_bucket(nrhs));
+    hm_status st = ensure_workspace(h, tunes && !o->persistent && !rec_out ? tune_bucket(nrhs) : nrhs, c.m);
     if (st != HM_OK) return st;
     const bool resid = !o->fp64 && (o->refine || info);
     if (resid && (st = ensure_partials(h)) != HM_OK) return st;
@@ -1913,7 +1950,7 @@ hm_status hm_get_info(hm_matrix h, hm_info *info)
     info->max_rank = h->max_rank;
     info->factored = h->factored;
     info->has_fp64 = h->has_fp64 ? 1 : 0;
-    info->device_bytes = h->device_bytes + h->ws.dev_bytes + (int64_t)h->ws.d_io_bytes;
+    info->device_bytes = held_bytes(h);
     for (int l = 0; l < 16; ++l) {
         info->norm_est[l] = h->norm_est[l];
         info->rho_est[l] = h->rho_est[l];

@@ -85,6 +85,7 @@ struct LevelList {
     // hm_lists.h build_mm_lists): product units, residual units (mm_parts a cluster at most), scales
     // and operand streams, made by the first call that runs them
     bool mm_built = false;
+    int64_t mm_bytes = 0;         // device bytes of the arrays below
     size_t mm_need = 0;           // device bytes the streams take (a lower bound before the lists are made)
     MmUnit *d_mm_unit = nullptr, *d_mm_unit2 = nullptr, *d_mm_runit = nullptr;
     MmBatch *d_mm_batch = nullptr;
@@ -252,6 +253,7 @@ struct hm_matrix_s {
     int *h_status = nullptr;          // pinned mirror
     hm::Workspace ws;
     int64_t device_bytes = 0;
+    int64_t byte_limit = -1;          // device bytes that the matrix-instruction kernels' streams keep the handle below (-1: none; a server's)
     bool mm_refused = false;          // the matrix-instruction kernels' streams found no room (hm_api.cu mm_room)
     int num_sms = 0;
     int64_t tc_max_xch = 0;           // largest split-x chunk count over the levels
@@ -345,6 +347,9 @@ void launch_item_bounds(const Item *items, int64_t n, const float2 *pool, float4
 // the kernels enqueued
 int launch_apply_items_partials(hm_matrix h, const LevelList *const *L, int n, const float2 *x, dot2::cdf *part,
                                 int64_t pstride, int nrhs, cudaStream_t s, int rb = -1);
+// device bytes that the matrix-instruction kernels hold beside the operator, and giving them back (hm_api.cu)
+int64_t mm_held(hm_matrix h);
+void release_mm(hm_matrix h);
 // the levels 1..m that have blocks
 std::vector<const LevelList *> used_levels(hm_matrix h, int m);
 // per leaf: acc = D x + sum of the leaf's partial slots of levels 1..m (double-float, fixed order);

@@ -17,7 +17,10 @@
 // batches in flight (its workspace is per handle).  When the resident operators
 // exceed the HBM budget (every operator was busy at admission), idle operators
 // with no queued requests are evicted, least recently used first, as soon as
-// batches retire.
+// batches retire.  The operand streams that the many-right-hand-side kernels pack beside
+// an operator (twice its blocks) are taken only within the budget, and given back, idle
+// operators' first, before any operator is evicted: a stream costs milliseconds to pack again,
+// an operator a build.
 #include "hm_internal.h"
 
 #include <algorithm>
@@ -136,23 +139,47 @@ hm_status slot_reserve(Slot &s, size_t elems)
     return HM_OK;
 }
 
+// the operator's device bytes as they are now, into the sums
+void account(hm_server_s *S, int op)
+{
+    hm_info info;
+    if (!S->ops[op].h || hm_get_info(S->ops[op].h, &info) != HM_OK) return;
+    S->resident_bytes += info.device_bytes - S->ops[op].bytes;
+    S->ops[op].bytes = info.device_bytes;
+    S->peak_resident = std::max(S->peak_resident, S->resident_bytes);
+}
+
+// frees memory until `need` more bytes fit the budget: idle operators' operand streams, then idle
+// operators, least recently used first, those with queued requests only if `queued`; stops where
+// nothing is left to free
+void make_room(hm_server_s *S, int64_t need, bool queued)
+{
+    while (S->resident_bytes + need > S->budget) {
+        int victim = -1, packed = -1;
+        auto older = [&](int i, int j) { return j < 0 || S->ops[i].last_use < S->ops[j].last_use; };
+        for (int i = 0; i < (int)S->ops.size(); ++i) {
+            const Operator &c = S->ops[i];
+            if (!c.h || c.busy || !(queued || c.queue.empty())) continue;
+            if (older(i, victim)) victim = i;
+            if (mm_held(c.h) > 0 && older(i, packed)) packed = i;
+        }
+        if (packed >= 0) {
+            release_mm(S->ops[packed].h);
+            account(S, packed);
+            continue;
+        }
+        if (victim < 0) return;
+        drop_operator(S, victim);
+        S->evictions++;
+    }
+}
+
 // make operator op resident, evicting idle LRU operators to respect the budget
 hm_status make_resident(hm_server_s *S, int op)
 {
     Operator &o = S->ops[op];
     if (o.h) return HM_OK;
-    const int64_t need = o.bytes;
-    while (S->resident_bytes + need > S->budget) {
-        int victim = -1;
-        for (int i = 0; i < (int)S->ops.size(); ++i) {
-            const Operator &c = S->ops[i];
-            if (c.h && !c.busy && (victim < 0 || c.last_use < S->ops[victim].last_use)) victim = i;
-        }
-        if (victim < 0) break;   // everything resident is in use: admit anyway, the budget is a target
-        drop_operator(S, victim);
-        S->resident_bytes -= S->ops[victim].bytes;
-        S->evictions++;
-    }
+    make_room(S, o.bytes, true);   // what is in use stays, the budget is a target
     const int per = o.basis == HM_SWG ? 4 : 3;
     hm_mesh mesh{o.basis, (int64_t)o.xyz.size() / 3, o.xyz.data(), (int64_t)o.cells.size() / per, o.cells.data(),
                  o.eps_r.empty() ? nullptr : o.eps_r.data(), o.wavelength};
@@ -190,12 +217,7 @@ void retire(hm_server_s *S, Slot &s)
         r.done = true;
     }
     // the operator's footprint grows with its workspace (right-hand-side vectors)
-    hm_info info;
-    if (hm_get_info(S->ops[s.op].h, &info) == HM_OK) {
-        S->resident_bytes += info.device_bytes - S->ops[s.op].bytes;
-        S->ops[s.op].bytes = info.device_bytes;
-        S->peak_resident = std::max(S->peak_resident, S->resident_bytes);
-    }
+    account(S, s.op);
     S->ops[s.op].busy = false;
     S->ops[s.op].last_use = now;
     S->solved_rhs += s.nrhs;
@@ -279,9 +301,12 @@ hm_status loop_stop(hm_server_s *S, std::unique_lock<std::mutex> &lk)
     return HM_OK;
 }
 
-// destroys an operator's handle; its recorded phase lists go with it
+// destroys an operator's handle; its recorded phase lists go with it.  The bytes it is admitted by
+// next time are those it needs, without its operand streams.
 void drop_operator(hm_server_s *S, int op)
 {
+    S->resident_bytes -= S->ops[op].bytes;
+    S->ops[op].bytes -= mm_held(S->ops[op].h);
     hm_destroy(S->ops[op].h);
     S->ops[op].h = nullptr;
     for (auto it = S->recorded.begin(); it != S->recorded.end();)
@@ -354,14 +379,7 @@ void loop_device(hm_server_s *S)
                 }
                 return v;
             };
-            if (idle && victim_of() >= 0 && loop_stop(S, lk) == HM_OK) {
-                int v;
-                while (S->resident_bytes > S->budget && (v = victim_of()) >= 0) {
-                    drop_operator(S, v);
-                    S->resident_bytes -= S->ops[v].bytes;
-                    S->evictions++;
-                }
-            }
+            if (idle && victim_of() >= 0 && loop_stop(S, lk) == HM_OK) make_room(S, 0, false);
         }
         // 2. a loop that left on an error (a bounded wait gave up) leaves its current batch unserved
         loop_reap(S);
@@ -423,14 +441,7 @@ void loop_device(hm_server_s *S)
                     if ((st = persist_phases(o.h, slot.d_b, slot.d_x, b, &o.so, &ph, &n)) == HM_OK)
                         S->recorded[k2] = {ph, n};
                 }
-                if (st == HM_OK) {
-                    hm_info info;
-                    if (hm_get_info(o.h, &info) == HM_OK) {
-                        S->resident_bytes += info.device_bytes - o.bytes;
-                        o.bytes = info.device_bytes;
-                        S->peak_resident = std::max(S->peak_resident, S->resident_bytes);
-                    }
-                }
+                if (st == HM_OK) account(S, op);
             }
             if (st != HM_OK) {
                 for (int64_t id : take) { S->reqs[id].status = st; S->reqs[id].done = true; }
@@ -521,20 +532,7 @@ void loop(hm_server_s *S)
         if (progressed) {
             S->cv_done.notify_all();
             // shrink to the budget: evict idle operators without queued requests, LRU first
-            while (S->resident_bytes > S->budget) {
-                int victim = -1;
-                for (int i = 0; i < (int)S->ops.size(); ++i) {
-                    const Operator &c = S->ops[i];
-                    if (c.h && !c.busy && c.queue.empty() &&
-                        (victim < 0 || c.last_use < S->ops[victim].last_use))
-                        victim = i;
-                }
-                if (victim < 0) break;
-                hm_destroy(S->ops[victim].h);
-                S->ops[victim].h = nullptr;
-                S->resident_bytes -= S->ops[victim].bytes;
-                S->evictions++;
-            }
+            make_room(S, 0, false);
         }
         // 2. launch new batches.  While one is in flight and a burst is still arriving, the next
         // ones wait for its end: few full batches instead of many small ones, and the same ones
@@ -586,7 +584,9 @@ void loop(hm_server_s *S)
                 col += r.nrhs;
             }
             cudaMemcpyAsync(slot->d_b, slot->h_buf, sizeof(float2) * N * nrhs, cudaMemcpyHostToDevice, slot->stream);
+            o.h->byte_limit = std::max<int64_t>(0, S->budget - (S->resident_bytes - o.bytes));
             st = hm_powerseries_solve(o.h, slot->d_b, N, slot->d_x, N, nrhs, &o.so, slot->stream, nullptr);
+            account(S, op);
             if (st != HM_OK) {
                 for (int64_t id : take) { S->reqs[id].status = st; S->reqs[id].done = true; }
                 S->cv_done.notify_all();
