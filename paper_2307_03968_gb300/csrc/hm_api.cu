@@ -122,6 +122,23 @@ static std::vector<Item> small_items(const LevelList &L)
     return small;
 }
 
+// device arrays that are made together: unless all of them are (keep), they go again
+struct Together {
+    hm_matrix h;
+    std::vector<void **> arrays;
+    int64_t bytes = h->device_bytes;
+    bool keep = false;
+    ~Together()
+    {
+        if (keep) return;
+        for (void **p : arrays) {
+            if (*p) cudaFree(*p);
+            *p = nullptr;
+        }
+        h->device_bytes = bytes;
+    }
+};
+
 // the tcgen05 product's lists, made by the first call that runs it (a pinned choice)
 static hm_status ensure_tc_lists(hm_matrix h, cudaStream_t s)
 {
@@ -138,6 +155,8 @@ static hm_status ensure_tc_lists(hm_matrix h, cudaStream_t s)
         L.n_tcb = (int64_t)tc.batches.size();
         L.n_tcr = (int64_t)tc.rows.size();
         L.n_tchunk = tc.n_tchunk;
+        Together made{h, {(void **)&L.d_xch, (void **)&L.d_tcu, (void **)&L.d_tco, (void **)&L.d_tcb, (void **)&L.d_tcr,
+                          (void **)&L.d_tcc}};
         if ((st = upload(h, &L.d_xch, tc.xch, s)) != HM_OK || (st = upload(h, &L.d_tcu, tc.units, s)) != HM_OK ||
             (st = upload(h, &L.d_tco, tc.ops, s)) != HM_OK || (st = upload(h, &L.d_tcb, tc.batches, s)) != HM_OK ||
             (st = upload(h, &L.d_tcr, tc.rows, s)) != HM_OK || (st = upload(h, &L.d_tcc, tc.tchunks, s)) != HM_OK)
@@ -145,7 +164,7 @@ static hm_status ensure_tc_lists(hm_matrix h, cudaStream_t s)
         HM_CUDA(cudaStreamSynchronize(s));        // the host lists end here
         h->tc_max_xch = std::max(h->tc_max_xch, L.n_xch);
         h->tc_max_tchunk = std::max(h->tc_max_tchunk, L.n_tchunk);
-        L.tc_built = true;
+        L.tc_built = made.keep = true;
     }
     return HM_OK;
 }
@@ -163,12 +182,13 @@ static hm_status ensure_own_lists(hm_matrix h, cudaStream_t s)
         std::vector<RcUnit> parts;
         L.own_parts = split_owner_units(rcu, rcp, 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), parts);
         L.n_rcu = (int64_t)parts.size();
+        Together made{h, {(void **)&L.d_rcu, (void **)&L.d_rcp, (void **)&L.d_rcb}};
         if ((st = upload(h, &L.d_rcu, parts, s)) != HM_OK || (st = upload(h, &L.d_rcp, rcp, s)) != HM_OK ||
             (st = dev_alloc(h, (void **)&L.d_rcb, sizeof(float2) * rcp.size())) != HM_OK)
             return st;
         launch_prod_bounds(L.d_rcp, (int64_t)rcp.size(), h->d_pool32, L.d_rcb, s);
         HM_CUDA(cudaStreamSynchronize(s));        // the host lists end here
-        L.own_built = true;
+        L.own_built = made.keep = true;
     }
     return HM_OK;
 }
@@ -1099,7 +1119,9 @@ static hm_status autotune(hm_matrix h, int nrhs_req, int m, cudaStream_t s, bool
         if (st != HM_OK || !do_res) break;
         if (rb == RB_OWN) {
             if (!own_applies(h, m)) continue;
-            if ((st = ensure_own(h, m, false, s)) != HM_OK) break;
+            st = ensure_own(h, m, false, s);
+            if (st == HM_ERR_OOM) { st = HM_OK; continue; }   // no room for its lists or sums: the other kernels
+            if (st != HM_OK) break;
         } else if (rb > 8 && rb / 2 >= nr) {
             continue;
         }
