@@ -428,11 +428,9 @@ void launch_gather_own(hm_matrix h, const float2 *x, int arrays, const double2 *
     const bool four = h->n_leaves * groups >= h->num_sms;
     const auto kern = four ? k_gather_own<4> : k_gather_own<1>;
     const size_t sm = sizeof(float4) * (four ? 2 : 1) * (size_t)std::max<int64_t>(maxnp, 1);
-    static bool attr = false;
-    if (sm > 32 * 1024 && !attr) {
-        cudaFuncSetAttribute(k_gather_own<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-        attr = true;
-    }
+    // the attribute is of the current device, so it is set by every call that needs it (leaves of more
+    // than 1,024 unknowns; the longest, 1,536, take 48 KB beside the 16 KB of sums)
+    if (sm > 32 * 1024) cudaFuncSetAttribute(k_gather_own<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     kern<<<dim3((unsigned)h->n_leaves, (unsigned)(four ? groups : nrhs)), 256, sm, s>>>(
         h->d_pleaf_off, h->d_dinv_off, h->d_self32, x, h->pN, nrhs, arrays, own, lstride, b, out, norms);
 }
