@@ -92,7 +92,6 @@ struct hm_server_s {
     std::vector<Operator> ops;
     std::map<int64_t, Request> reqs;
     int64_t next_id = 1;
-    clk::time_point last_submit;
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::thread worker;
@@ -503,9 +502,6 @@ void loop_device(hm_server_s *S)
     loop_stop(S, lk);
 }
 
-// a burst is over when no request has come for BURST_GAP; no request is held longer than BURST_HOLD
-constexpr auto BURST_GAP = std::chrono::microseconds(100), BURST_HOLD = std::chrono::microseconds(1000);
-
 void loop(hm_server_s *S)
 {
     cudaSetDevice(S->device);
@@ -534,19 +530,10 @@ void loop(hm_server_s *S)
             // shrink to the budget: evict idle operators without queued requests, LRU first
             make_room(S, 0, false);
         }
-        // 2. launch new batches.  While one is in flight and a burst is still arriving, the next
-        // ones wait for its end: few full batches instead of many small ones, and the same ones
-        // whatever the threads' timing
-        bool in_flight = false;
-        for (const Slot &s : S->slots) in_flight |= s.busy;
-        const auto now = clk::now();
-        const bool arriving = in_flight && now - S->last_submit < BURST_GAP;
+        // 2. launch new batches
         for (int op = 0; op < (int)S->ops.size(); ++op) {
             Operator &o = S->ops[op];
             if (o.busy || o.queue.empty()) continue;
-            int queued = 0;
-            for (int64_t id : o.queue) queued += S->reqs[id].nrhs;
-            if (arriving && queued < S->max_batch_rhs && now - S->reqs[o.queue.front()].t_submit < BURST_HOLD) continue;
             Slot *slot = nullptr;
             for (Slot &s : S->slots)
                 if (!s.busy) { slot = &s; break; }
@@ -557,17 +544,14 @@ void loop(hm_server_s *S)
                 S->cv_done.notify_all();
                 continue;
             }
-            // take requests in arrival order up to max_batch_rhs right-hand sides; a longer queue in
-            // batches of about equal size (36 and 50 of 86 at 64 a batch, not 55 and 31)
-            const int parts = (queued + S->max_batch_rhs - 1) / S->max_batch_rhs, even = (queued + parts - 1) / parts;
+            // take requests in arrival order up to max_batch_rhs right-hand sides
             std::vector<int64_t> take;
             int nrhs = 0;
             while (!o.queue.empty()) {
                 const Request &r = S->reqs[o.queue.front()];
-                const int with = nrhs + r.nrhs;
-                if (!take.empty() && (with > S->max_batch_rhs || with - even > even - nrhs)) break;
+                if (!take.empty() && nrhs + r.nrhs > S->max_batch_rhs) break;
                 take.push_back(o.queue.front());
-                nrhs = with;
+                nrhs += r.nrhs;
                 o.queue.pop_front();
             }
             const int64_t N = o.n;
@@ -736,7 +720,7 @@ hm_status hm_server_submit(hm_server S, int op_id, const void *b, int64_t n, int
     r.op = op_id;
     r.nrhs = nrhs;
     r.b.assign((const float2 *)b, (const float2 *)b + (size_t)n * nrhs);
-    r.t_submit = S->last_submit = clk::now();
+    r.t_submit = clk::now();
     const int64_t id = r.id;
     S->reqs.emplace(id, std::move(r));
     S->ops[op_id].queue.push_back(id);
