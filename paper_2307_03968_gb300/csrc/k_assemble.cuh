@@ -723,13 +723,28 @@ struct TmpBuffers {
     }
 };
 
-// each double as the pair (hi, lo) of floats, hi the nearest float, lo the nearest to the rest
-inline std::vector<float2> float_pairs(const std::vector<double> &v)
+// the middle of the points' bounding box
+inline std::array<double, 3> middle(const std::vector<double> &v)
+{
+    std::array<double, 3> c{};
+    for (int d = 0; d < 3; ++d) {
+        double lo = v[d], hi = v[d];
+        for (size_t i = d; i < v.size(); i += 3) { lo = std::min(lo, v[i]); hi = std::max(hi, v[i]); }
+        c[d] = 0.5 * lo + 0.5 * hi;
+    }
+    return c;
+}
+
+// points relative to c, each coordinate as the pair (hi, lo) of floats, hi the nearest float, lo the
+// nearest to the rest: 49 bits of the object's size, wherever it lies (only differences of two such
+// points are used)
+inline std::vector<float2> float_pairs(const std::vector<double> &v, const std::array<double, 3> &c)
 {
     std::vector<float2> r(v.size());
     for (size_t i = 0; i < v.size(); ++i) {
-        r[i].x = (float)v[i];
-        r[i].y = (float)(v[i] - (double)r[i].x);
+        const double x = v[i] - c[i % 3];
+        r[i].x = (float)x;
+        r[i].y = (float)(x - (double)r[i].x);
     }
     return r;
 }

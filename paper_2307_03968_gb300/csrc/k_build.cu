@@ -35,7 +35,7 @@ struct Geo {
     const double *elen;   // ne
     const int32_t *perm;  // tree position -> original edge index
     double k, eta;
-    // the same points as pairs of floats (hi, lo), hi + lo within 2^-49 of the double, for the
+    // the same points, relative to the mesh's middle, as pairs of floats (hi, lo), within 2^-49, for the
     // FP32 entries: their local coordinates p - o are then formed without the FP64 pipe, which
     // runs at 1/64 of the FP32 rate here and which 96 subtractions and conversions per triangle
     // pair made the bound of the fill and of the ACA
@@ -418,7 +418,8 @@ hm_status build_from_mesh(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
     g.k = 2.0 * 3.14159265358979323846 / mesh->wavelength;
     g.eta = 376.730313461770655;
     float2 *d_vtx32, *d_qpd32;
-    if ((st = tmp.up(&d_vtx32, float_pairs(vtx), s)) || (st = tmp.up(&d_qpd32, float_pairs(qpd), s))) return st;
+    const std::array<double, 3> mid = middle(vtx);
+    if ((st = tmp.up(&d_vtx32, float_pairs(vtx, mid), s)) || (st = tmp.up(&d_qpd32, float_pairs(qpd, mid), s))) return st;
     g.vtx32 = d_vtx32;
     g.qpd32 = d_qpd32;
     g.kf = (float)g.k;

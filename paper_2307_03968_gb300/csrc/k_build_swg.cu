@@ -63,7 +63,7 @@ struct VGeo {
     static constexpr int PARTS = 1;
     static constexpr bool BLOCK_FILL = true;
     // for the near fill by blocks (k_fill_swg)
-    const float2 *vtx32, *tqp32, *fqp32;   // the points as pairs of floats (hi, lo)
+    const float2 *vtx32, *tqp32, *fqp32;   // the points relative to the mesh's middle, as pairs of floats (hi, lo)
     const double *fgeo;     // nf x FGEO: vertices, unit normal away from T+'s free vertex, per edge direction and outward in-plane normal
     const double *tgeo;     // nt x TGEO: vertices; per face (opposite vertex a): outward normal, per edge of the face its outward in-plane normal; the 6 edge directions and lengths
     hm_status fill_near(const std::vector<FillJob> &jobs, float2 *pool, TmpBuffers &tmp, cudaStream_t s) const;
@@ -978,8 +978,9 @@ hm_status build_from_tets(const hm_mesh *mesh, const hm_build_opts *o, cudaStrea
     g.k = 2.0 * 3.14159265358979323846 / mesh->wavelength;
     float2 *d_vtx32, *d_tqp32, *d_fqp32;
     double *d_fgeo, *d_tgeo;
-    if ((st = tmp.up(&d_vtx32, float_pairs(vtx), s)) || (st = tmp.up(&d_tqp32, float_pairs(tqp), s)) ||
-        (st = tmp.up(&d_fqp32, float_pairs(fqp), s)) || (st = tmp.up(&d_fgeo, fgeo, s)) || (st = tmp.up(&d_tgeo, tgeo, s)))
+    const std::array<double, 3> mid = middle(vtx);
+    if ((st = tmp.up(&d_vtx32, float_pairs(vtx, mid), s)) || (st = tmp.up(&d_tqp32, float_pairs(tqp, mid), s)) ||
+        (st = tmp.up(&d_fqp32, float_pairs(fqp, mid), s)) || (st = tmp.up(&d_fgeo, fgeo, s)) || (st = tmp.up(&d_tgeo, tgeo, s)))
         return st;
     g.vtx32 = d_vtx32; g.tqp32 = d_tqp32; g.fqp32 = d_fqp32; g.fgeo = d_fgeo; g.tgeo = d_tgeo;
 
