@@ -433,8 +433,9 @@ hm_status hm_get_info(hm_matrix h, hm_info *info);
  * caller's stream, which it synchronises once) and keeps the fastest: 0 = one right-hand side at
  * a time, 8 / 16 = blocks staged once in shared memory per chunk of that many right-hand sides,
  * 32 (product only) = the blocks of at most 64 x 64 (rank <= 32) on the matrix instructions, in
- * three BF16 parts (FP32 accuracy) and tiles of 16 or 32 right-hand sides (its first call packs the blocks a second
- * time, twice their bytes, counted in hm_info.device_bytes, with its workspace);
+ * three BF16 parts (FP32 accuracy) and tiles of 16 or 32 right-hand sides (its first call packs
+ * the blocks a second time, twice their bytes, counted in hm_info.device_bytes, with its
+ * workspace, where half of the free device memory holds that; else the other kernels run);
  * 1017 (residual only, where every level of the call holds only such blocks) =
  * owner-computes FP64-class products, one CTA per output cluster and group of 16
  * right-hand sides, no partial slots.  A refined solve whose levels hold only such blocks and

@@ -587,9 +587,6 @@ static hm_status ensure_workspace(hm_matrix h, int nrhs, int m)
     return HM_OK;
 }
 
-// FP64 owner sums of the owner-computes residual ([level][part][RHS][pN] for the
-// workspace's RHS count and m levels); allocated only by the calls that form a
-// residual with that kernel, before any capture
 // owner-sum arrays of levels 1..m: a level's own_parts, or its mm_parts on the matrix instructions
 static int own_arrays(hm_matrix h, int m, bool mm)
 {
@@ -605,6 +602,9 @@ static size_t own_bytes(hm_matrix h, int m, int nrhs, bool mm)
     return sizeof(double2) * (size_t)std::max(own_arrays(h, m, mm), 1) * (size_t)nrhs * (size_t)h->pN;
 }
 
+// FP64 owner sums of the owner-computes residual ([level][part][RHS][pN] for the
+// workspace's RHS count and m levels); allocated only by the calls that form a
+// residual with that kernel, before any capture
 static hm_status ensure_own(hm_matrix h, int m, bool mm, cudaStream_t s)
 {
     hm::Workspace &ws = h->ws;
@@ -950,6 +950,16 @@ static int clamp_levels(hm_matrix h, int n_levels)
     return std::max(m, 1);
 }
 
+// whether levels 1..m have their operand streams and operand tiles
+static bool mm_ready(hm_matrix h, int m)
+{
+    for (int lev = 1; lev <= m; ++lev) {
+        auto it = h->levels.find(lev);
+        if (it != h->levels.end() && it->second.n_small > 0 && !it->second.mm_built) return false;
+    }
+    return h->ws.d_mm != nullptr;
+}
+
 // out = b - A_m x (with |r|^2, |b|^2 per column into norms) when b is given, else
 // out = A_m x; complex64 blocks, FP64 products and sums, deterministic order:
 // every block writes its double-float partial slots, then each leaf gathers its slots.
@@ -961,7 +971,7 @@ static void residual64(SolveCtx &c, const float2 *xt, const float2 *bt, float2 *
 {
     hm_matrix h = c.h;
     const bool mm = c.res_rb == RB_MM;
-    if (!c.rec && (mm || c.res_rb == RB_OWN) && h->ws.d_own && h->ws.own_bytes >= own_bytes(h, c.m, c.nrhs, mm) &&
+    if (!c.rec && ((mm && mm_ready(h, c.m)) || c.res_rb == RB_OWN) && h->ws.d_own && h->ws.own_bytes >= own_bytes(h, c.m, c.nrhs, mm) &&
         own_applies(h, c.m)) {
         // owner-computes: each level's sums into its own FP64 [part][RHS][pN] arrays, then one gather
         const int64_t lstride = (int64_t)c.nrhs * h->pN;

@@ -30,7 +30,6 @@ namespace hm {
 constexpr int MRHS_MIN_RHS = 4;     // from this many right-hand sides on, the multi-RHS kernels take the small blocks
 constexpr int RESID_CHUNK = 16;     // right-hand sides per chunk of the FP64-class residual (partial slots held)
 constexpr int RB_TC = 1016;         // product choice: tensor-core products of the small items, RHS tiles of 128
-constexpr int TC_MIN_RHS = 32;      // the autotuner times the tensor-core product from this many RHS on
 constexpr int RB_OWN = 1017;        // residual choice: owner-computes FP64-class products (levels of small items)
 constexpr int RB_MM = 1018;         // residual choice: the same on the matrix instructions (timed for refined solves only)
 

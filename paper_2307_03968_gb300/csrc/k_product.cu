@@ -159,7 +159,7 @@ int launch_apply_items(hm_matrix h, const LevelList &L, const void *x, void *z, 
             if (L.n_prod_big == 0) return launched;
         } else if (rb > 0 && nrhs > 1 && L.n_small > 0) {
             // many right-hand sides: on the matrix instructions, or blocks staged in shared memory once per chunk
-            if (rb == 32 && h->ws.d_mm && h->ws.mm_bytes >= mm_ws_bytes(L, nrhs, false)) {
+            if (rb == 32 && L.mm_built && h->ws.d_mm && h->ws.mm_bytes >= mm_ws_bytes(L, nrhs, false)) {
                 launched += launch_mm_product(h, L, (const float2 *)x, (float2 *)z, nrhs, h->ws.d_mm, s);
             } else {
                 launch_apply_items_mrhs(h, L, (const float2 *)x, (float2 *)z, nrhs, std::min(rb, 16), s);
