@@ -45,12 +45,15 @@
 //
 // Product: a = a1 + a2 + a3, three BF16 parts of 8 bits, an FP32 number exactly (the last bits of
 // one below 2^-109 of the scale apart): a1 b1 + a1 b2 + a2 b1 + a1 b3 + a2 b2 + a3 b1, the three
-// left out are below 2^-24 of a b.  BF16 has FP32's exponents, so a small operand keeps its bits
+// left out are below 2^-25 of a b and of either sign, the parts being rounded to nearest (cut off,
+// they leave out terms of one sign: the refined solve of a 3,001-unknown import erred by 2.7e-7, so by
+// 1.8e-7, with the FP32 kernels by 1.9e-7).  BF16 has FP32's exponents, so a small operand keeps its bits
 // beside a large one; two FP16 halves (22 bits, three products, 6.4 ms for those 181) lose them
 // below 2^-17 of the scale: entries at 2^-30 came out to 1e-3.  The tensor core truncates its FP32 sums,
-// so each chunk's sums start from zero and join the running sum in FP32: 1.1e-7 to 2.0e-7 of
-// |A x| over the tested operators (FP32 kernels: 1.6e-7 to 2.2e-7); 32 chunks in the tensor core
-// instead of one took 6 % less time and erred by 1e-6.
+// so each chunk's sums start from zero and join the running sum in FP32; 32 chunks in the tensor
+// core instead of one took 6 % less time and erred by 1e-6 of |A x| (5e-6 in that solve).  What is left
+// is the mean of the truncation, 5e-9 of |A x|; adding every second chunk times 1 + 2^-23 takes it back
+// (1.4e-7) but makes exact products inexact, so it is not done.
 //
 // FP64-class residual: a = 2^-8 d1 + 2^-17 d2 + 2^-26 d3 + 2^-35 d4 + 2^-44 r, the digits integers of at
 // most 2^8 (a unit or two more for T), r a FP16 of at most 2^8: 48 bits below the scale, exact for every FP32
@@ -101,17 +104,17 @@ __device__ __forceinline__ uint32_t h2(float a, float b)
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
-// the planes of a pair of values: each cut into three BF16 parts of 8 bits, exactly
+// the planes of a pair of values (the smaller K in the lower half): each in three BF16 parts, rounded to nearest, exactly
 __device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[3])
 {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-        p[i] = __byte_perm(ua, ub, 0x7632);                  // the upper halves
-        a = __fsub_rn(a, __uint_as_float(ua & 0xffff0000u));
-        b = __fsub_rn(b, __uint_as_float(ub & 0xffff0000u));
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[i]) : "f"(b), "f"(a));
+        a = __fsub_rn(a, __uint_as_float(p[i] << 16));
+        b = __fsub_rn(b, __uint_as_float(p[i] & 0xffff0000u));
     }
 }
+
 // The digit and sum steps run on packed pairs (k_dot2.cuh fma2, add2, sub2): two operations an
 // issue slot, which is what bounds them beside the matrix instructions.
 // the nearest integers of |v| < 2^22 (ties to even)

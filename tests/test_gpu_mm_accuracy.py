@@ -7,7 +7,7 @@ so that neither a large part nor a large cluster hides a small one: right-hand s
 size, an excitation of one leaf with everything else at 2^-30 of it, entries spread over 2^-30, and blocks with
 imaginary parts of 2^-30 of the real ones (fine meshes have them), with real vectors.
 
-Bounds: three parts of 8 bits hold an FP32 number exactly; the products left out are 2^-24 of a
+Bounds: three parts of 8 bits hold an FP32 number exactly; the products left out are 2^-25 of a
 term, the tensor core truncates the last two of twelve sums of a chunk of 16 K at the chunk's own
 size (2 x 2^-23), and the chunks add in FP32 (about sqrt(300) x 2^-24 over the 300 chunks of a
 cluster here): 1.3e-6 with every error at its largest, held to 2e-6, a hundred times less on the
