@@ -64,7 +64,6 @@ hm_status upload_item_lists(hm_matrix h, cudaStream_t s)
         }
         L.n_small = (int64_t)small.size();
         L.n_big = (int64_t)big.size();
-        L.disjoint = disjoint_outputs(directed_products(small));
         if ((st = upload(h, &L.d_items, L.items, s)) != HM_OK) return st;
         if ((st = upload(h, &L.d_small, small, s)) != HM_OK) return st;
         // the residual's own list (the long low-rank blocks, a CTA each, largest first; then the
@@ -690,7 +689,10 @@ static bool own_applies(hm_matrix h, int m)
     for (int lev = 1; lev <= m; ++lev) {
         auto it = h->levels.find(lev);
         if (it == h->levels.end() || it->second.items.empty()) continue;
-        if (it->second.n_big > 0 || !it->second.disjoint) return false;
+        LevelList &L = it->second;
+        if (L.n_big > 0) return false;
+        if (L.disjoint < 0) L.disjoint = disjoint_clusters(L.items, h->pN);
+        if (!L.disjoint) return false;
         any = true;
     }
     return any;
@@ -1322,7 +1324,7 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     const bool persist = (o->persistent || rec_out) && !c.fp64 && persist_supported(h);
     if (rec_out && !persist) return fail(HM_ERR_ARG, "the operator does not fit the one-launch solve");
     if (!c.fp64 && !persist) {
-        if ((st = autotune(h, nrhs, c.m, s, true, resid && !own_applies(h, c.m))) != HM_OK) return st;
+        if ((st = autotune(h, nrhs, c.m, s, true, resid && nrhs >= MRHS_MIN_RHS && !own_applies(h, c.m))) != HM_OK) return st;
         if ((st = use_tuning(c, true, resid)) != HM_OK) return st;
         if (resid && (st = ensure_partials(h)) != HM_OK) return st;   // the tuning may have grown the workspace
         if (resid && nrhs >= MRHS_MIN_RHS && own_applies(h, c.m)) {

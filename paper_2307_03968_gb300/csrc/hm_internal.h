@@ -52,7 +52,7 @@ struct LevelList {
     // in shared memory, and the rest
     Item *d_small = nullptr, *d_big = nullptr;
     int64_t n_small = 0, n_big = 0;
-    bool disjoint = true;         // the small items' clusters (hm_lists.h disjoint_outputs)
+    int disjoint = -1;            // the small items' clusters (hm_lists.h disjoint_clusters; -1: not looked at yet)
     // the FP64-class residual's copy of the item list: n_wide long low-rank blocks (wide_item;
     // also the first n_wide of d_big), then the rest in the order that balances its
     // round-robin warps; and per item of it / of d_big the block bounds of the

@@ -144,17 +144,25 @@ inline void build_owner_lists(const std::map<int32_t, std::vector<TcProd>> &by_o
     }
 }
 
-// Whether the output clusters of a level's directed products are disjoint or the same (at one
-// start the longest counts).  The clusters of one tree level are; a user's own blocks may couple,
-// on the same level, a leaf and a union that holds it.  The owner-computes residuals store each
-// cluster's sums, so two clusters that share rows would overwrite each other's.
-inline bool disjoint_outputs(const std::map<int32_t, std::vector<TcProd>> &by_out)
+// Whether the clusters of a level's small items (sides of at most MRHS_MAX_DIM, padded positions below
+// pN) are disjoint or the same; at one start the longest counts.  The clusters of one tree level are;
+// a user's own blocks may couple, on the same level, a leaf and a union that holds it.  The
+// owner-computes residuals store each cluster's sums, so two clusters that share rows would
+// overwrite each other's.
+inline bool disjoint_clusters(const std::vector<Item> &items, int64_t pN)
 {
+    std::vector<int32_t> len((size_t)pN, 0);
+    for (const Item &it : items)
+        if (it.m <= MRHS_MAX_DIM && it.n <= MRHS_MAX_DIM && it.k <= MRHS_MAX_RANK) {
+            len[it.row0] = std::max(len[it.row0], it.m);
+            len[it.col0] = std::max(len[it.col0], it.n);
+        }
     int64_t end = 0;
-    for (const auto &kv : by_out) {
-        if (kv.first < end) return false;
-        for (const TcProd &p : kv.second) end = std::max<int64_t>(end, (int64_t)kv.first + p.olen);
-    }
+    for (int64_t p = 0; p < pN; ++p)
+        if (len[p] > 0) {
+            if (p < end) return false;
+            end = p + len[p];
+        }
     return true;
 }
 
