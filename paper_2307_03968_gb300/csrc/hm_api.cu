@@ -287,8 +287,11 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
         // about four CTAs an SM for one tile of right-hand sides
         if (!build_mm_lists(directed_products(small_items(L)), 4 * (int64_t)(h->num_sms > 0 ? h->num_sms : 1), mm))
             return fail(HM_ERR_STATE, "matrix-product work lists out of their index bounds");
-        // what the level takes, exactly (its lists beside the streams are a few per cent of it)
-        L.mm_need = (mm_stream_bytes(1) + 8 * sizeof(int)) * (size_t)(mm.n_out + mm.n_w);
+        // what the level takes (its lists beside the streams are a few per cent of it), with the operand
+        // tiles that follow, without which the streams would be of no use
+        L.mm_n_xch = (int64_t)mm.xch.size();
+        L.mm_n_tch = mm.n_tch;
+        L.mm_need = (mm_stream_bytes(1) + 8 * sizeof(int)) * (size_t)(mm.n_out + mm.n_w) + mm_ws_bytes(L, h->ws.nrhs, true);
         if ((st = mm_room(h, L.mm_need)) != HM_OK) return st;
         TmpArray sets, chunks, rows, pairs, wexp, rexp;
         struct Undo {   // a level's arrays go again if the last of them cannot be had
@@ -326,8 +329,6 @@ static hm_status ensure_mm_lists(hm_matrix h, int m, cudaStream_t s)
         L.mm_n_chunk = (int64_t)mm.chunks.size();
         L.mm_n_runit = (int64_t)mm.runits.size();
         L.mm_n_batch = (int64_t)mm.batches.size();
-        L.mm_n_xch = (int64_t)mm.xch.size();
-        L.mm_n_tch = mm.n_tch;
         L.mm_parts = mm.n_cl > 0 ? mm.parts : 0;
         launch_mm_pack(L, MmPackArgs{(const MmSet *)sets.p, (const MmChunk *)chunks.p, (const int64_t *)rows.p,
                                      (const MmPair *)pairs.p, (int *)wexp.p, (int *)rexp.p, (int64_t)mm.sets.size(),
@@ -1284,6 +1285,19 @@ static void check_vec(SolveCtx &c, const void *x)
     launch_check_finite(x, c.h->pN * c.nrhs, c.fp64, c.h->d_status, c.s);
 }
 
+int64_t solve_growth(hm_matrix h, int nrhs, const hm_solve_opts *o)
+{
+    const Workspace &ws = h->ws;
+    const int r = std::max(nrhs < MRHS_MIN_RHS ? nrhs : tune_bucket(nrhs), ws.nrhs), m = clamp_levels(h, o->n_levels);
+    const size_t vecs = 4 * (size_t)(m + 1) + 8;
+    const bool grows = ws.nrhs < r || ws.vec32.size() < vecs;
+    int64_t need = 0;
+    if (grows) need += (int64_t)(sizeof(float2) * (size_t)h->pN * r * (vecs - (ws.nrhs < r ? 0 : ws.vec32.size())));
+    if (o->refine && (grows || !ws.d_part))
+        need += (int64_t)(sizeof(dot2::cdf) * (size_t)std::max<int64_t>(h->partial_elems, 1) * std::min(r, RESID_CHUNK));
+    return need;
+}
+
 // rec_out: record (or find) the one-launch phase list of this solve and return it
 // without launching anything (the serving loop runs it)
 static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, int64_t ldx, int nrhs,
@@ -1316,8 +1330,10 @@ static hm_status solve_device(hm_matrix h, const void *b, int64_t ldb, void *x, 
     c.vbytes = es * h->pN * nrhs;
     // at the size of the bucket where the autotuner is going to run, so that what the solve needs is
     // there (and counted) before anything optional is
-    const bool tunes = !o->fp64 && nrhs >= MRHS_MIN_RHS && !h->tune.count(tune_bucket(nrhs));
-    hm_status st = ensure_workspace(h, tunes && !o->persistent && !rec_out ? tune_bucket(nrhs) : nrhs, c.m);
+    const auto lev1 = h->levels.find(1);
+    const bool tunes = !o->fp64 && !o->persistent && !rec_out && nrhs >= MRHS_MIN_RHS &&
+                       !h->tune.count(tune_bucket(nrhs)) && lev1 != h->levels.end() && lev1->second.n_small > 0;
+    hm_status st = ensure_workspace(h, tunes ? tune_bucket(nrhs) : nrhs, c.m);
     if (st != HM_OK) return st;
     const bool resid = !o->fp64 && (o->refine || info);
     if (resid && (st = ensure_partials(h)) != HM_OK) return st;

@@ -85,7 +85,7 @@ struct LevelList {
     // and operand streams, made by the first call that runs them
     bool mm_built = false;
     int64_t mm_bytes = 0;         // device bytes of the arrays below
-    size_t mm_need = 0;           // device bytes the streams take (a lower bound before the lists are made)
+    size_t mm_need = 0;           // device bytes the streams and operand tiles take (a lower bound before the lists are made)
     MmUnit *d_mm_unit = nullptr, *d_mm_unit2 = nullptr, *d_mm_runit = nullptr;
     MmBatch *d_mm_batch = nullptr;
     XChunk *d_mm_xch = nullptr;
@@ -346,6 +346,8 @@ void launch_item_bounds(const Item *items, int64_t n, const float2 *pool, float4
 // the kernels enqueued
 int launch_apply_items_partials(hm_matrix h, const LevelList *const *L, int n, const float2 *x, dot2::cdf *part,
                                 int64_t pstride, int nrhs, cudaStream_t s, int rb = -1);
+// device bytes that a complex64 solve allocates for its vectors and partial slots, about (hm_api.cu)
+int64_t solve_growth(hm_matrix h, int nrhs, const hm_solve_opts *o);
 // device bytes that the matrix-instruction kernels hold beside the operator, and giving them back (hm_api.cu)
 int64_t mm_held(hm_matrix h);
 void release_mm(hm_matrix h);

@@ -148,10 +148,10 @@ void account(hm_server_s *S, int op)
     S->peak_resident = std::max(S->peak_resident, S->resident_bytes);
 }
 
-// frees memory until `need` more bytes fit the budget: idle operators' operand streams, then idle
-// operators, least recently used first, those with queued requests only if `queued`; stops where
-// nothing is left to free
-void make_room(hm_server_s *S, int64_t need, bool queued)
+// frees memory until `need` more bytes fit the budget: idle operators' operand streams, then (if
+// `evict`) idle operators, least recently used first, those with queued requests only if `queued`;
+// stops where nothing is left to free
+void make_room(hm_server_s *S, int64_t need, bool queued, bool evict = true)
 {
     while (S->resident_bytes + need > S->budget) {
         int victim = -1, packed = -1;
@@ -167,7 +167,7 @@ void make_room(hm_server_s *S, int64_t need, bool queued)
             account(S, packed);
             continue;
         }
-        if (victim < 0) return;
+        if (victim < 0 || !evict) return;
         drop_operator(S, victim);
         S->evictions++;
     }
@@ -568,6 +568,9 @@ void loop(hm_server_s *S)
                 col += r.nrhs;
             }
             cudaMemcpyAsync(slot->d_b, slot->h_buf, sizeof(float2) * N * nrhs, cudaMemcpyHostToDevice, slot->stream);
+            o.busy = true;                        // its own streams stay
+            make_room(S, solve_growth(o.h, nrhs, &o.so), true, false);
+            o.busy = false;
             o.h->byte_limit = std::max<int64_t>(0, S->budget - (S->resident_bytes - o.bytes));
             st = hm_powerseries_solve(o.h, slot->d_b, N, slot->d_x, N, nrhs, &o.so, slot->stream, nullptr);
             account(S, op);
