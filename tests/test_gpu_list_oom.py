@@ -4,6 +4,7 @@ holds exactly what one holds that never failed, with the same result.
 """
 
 import ctypes
+import gc
 
 import pytest
 
@@ -14,17 +15,23 @@ class Full:
     """Takes the device's memory but for `left` pieces of 2 MB."""
 
     def __init__(self, left):
+        import torch
         from paper_2307_03968_gb300.hm import load
+        gc.collect()                                       # nothing of earlier tests is given back in between
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
         self.rt, self.held = load(), []
-        for size in (1 << 30, 64 << 20, 2 << 20):
+        for size in (1 << 30, 64 << 20, 2 << 20, 64 << 10):
             while True:
                 p = ctypes.c_void_p()
                 if self.rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) != 0:
                     self.rt.cudaGetLastError()
                     break
+                p.size = size
                 self.held.append(p)
-        for _ in range(left):
-            self.rt.cudaFree(self.held.pop())
+        for p, _ in zip([q for q in self.held if q.size == 2 << 20], range(left)):
+            self.held.remove(p)
+            self.rt.cudaFree(p)
 
     def close(self):
         while self.held:

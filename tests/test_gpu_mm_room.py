@@ -4,6 +4,8 @@ take the rest of the device from others.  Without them the calls run the other k
 results (1e-5 of each other: FP32 sums in another order), and keep to them; a pinned choice asks again.
 """
 
+import gc
+
 import pytest
 
 from test_gpu_mm_accuracy import Operator
@@ -28,7 +30,9 @@ def test_streams_leave_room(left):
     assert T.tuning(nrhs)[1] == 1018
     streams = 2 * 8 * (A.info().near_elems + sum(A.info().far_elems))
     vectors = 16 * 8 * 64 * (P.n + 64)                     # the product's work vectors at the bucket's 64 right-hand sides
+    gc.collect()                                           # nothing of earlier tests is given back in between
     torch.cuda.synchronize()
+    torch.cuda.empty_cache()
     held, free = A.info().device_bytes, torch.cuda.mem_get_info()[0]
     more = torch.empty(512 << 20, dtype=torch.uint8, device="cuda")
     fill = torch.empty(free - more.numel() - vectors - left * streams // 10, dtype=torch.uint8, device="cuda")

@@ -40,4 +40,5 @@ def test_idle_operator_is_not_held():
         for q in queued:
             srv.wait(q)
     srv.close()
-    assert best < 0.6e-3, best
+    print("launched after %.0f us" % (1e6 * best))
+    assert best < 0.6e-3
